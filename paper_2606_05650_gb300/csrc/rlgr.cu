@@ -26,40 +26,119 @@ namespace {
 
 constexpr int kUnaryEsc = 24;
 
-// Bits are appended LSB first to a 32-bit word (cur, nacc bits used); a value
-// that straddles the word boundary leaves its upper part in the next word via
-// one funnel shift.  Words beyond `cap` are counted but not stored.
+// Bits are appended LSB first to a 64-bit accumulator holding nacc < 32 bits:
+// one wide multiply-add by 2^nacc places a value (its bits are free there), a
+// full low word is stored.  Words beyond `cap` are counted but not stored.
 struct BitWriter {
-    uint32_t cur;
+    uint64_t acc;
     uint32_t nacc;
+    uint32_t unit;  // 2^nacc
     uint32_t nw;
     uint32_t *out;
     uint32_t cap;
-    __device__ __forceinline__ void emit(uint32_t w)
-    {
-        if (nw < cap) out[nw] = w;
-        ++nw;
-    }
+    __device__ __forceinline__ BitWriter(uint32_t *o, uint32_t c) : acc(0), nacc(0), unit(1), nw(0), out(o), cap(c) {}
     __device__ __forceinline__ void put(uint32_t v, uint32_t n)  // n <= 32, v < 2^n
     {
-        const uint32_t spill = __funnelshift_l(v, 0u, nacc);  // bits of v above the word, if any
-        cur |= v << nacc;  // nacc < 32
+        acc += (uint64_t)v * unit;
         nacc += n;
-        if (nacc >= 32u) {
-            emit(cur);
-            cur = spill;
-            nacc -= 32u;
-        }
+        const bool full = nacc >= 32u;
+        asm volatile("{\n.reg .pred f;\nsetp.ge.u32 f, %4, 32;\nsetp.lt.and.u32 f, %1, %2, f;\n@f st.global.u32 [%0], %3;\n}" ::"l"(
+                         out + nw),
+                     "r"(nw), "r"(cap), "r"((uint32_t)acc), "r"(nacc)
+                     : "memory");  // one predicated store, no branch
+        nw += full ? 1u : 0u;
+        acc = full ? acc >> 32 : acc;
+        nacc &= 31u;
+        unit = 1u << nacc;
     }
     __device__ __forceinline__ void flush()
     {
-        if (nacc) {
-            emit(cur);
-            cur = 0;
-            nacc = 0;
-        }
+        if (nacc) put(0u, 32u - nacc);
     }
 };
+
+// Golomb-Rice codewords by table.  The encoder's entry, for the mode, the
+// parameter k (row) and column 2 t + s (magnitude t, sign s; zigzag index
+// u = 2 t - s, or 0), is the codeword of u (of u - 1 in run mode; 16 bits),
+// the change of KR (8 bits, signed) and the codeword's length n (8 bits); the
+// decoder's, for k and the next 10 stream bits, is n, the changes of KR and K
+// (signed) and the value + 128 that the codeword stands for in Golomb-Rice
+// mode, 8 bits each.  Entry 0 sends the symbol to the general path: codewords
+// longer than 16 (encoder) or 10 bits (decoder) and values that do not fit.
+// One shared-memory load replaces the prefix and remainder arithmetic and the
+// adaptation's comparisons.  The coders are bound by instruction issue, most
+// of it on the half-rate integer pipe: one serial stream per thread, every
+// stream slot of the SM filled.
+constexpr uint32_t kEncRows = 8, kEncCols = 256;   // per mode: k 0 .. 7
+constexpr uint32_t kEncMax = kEncCols / 2 - 1;     // magnitudes below; kEncMax stands for every larger one
+constexpr uint32_t kEncMode = kEncRows * kEncCols;  // entries of one mode
+constexpr uint32_t kDecRows = 8, kDecBits = 10;    // k 0 .. 7
+
+struct EncTable {
+    uint32_t e[2 * kEncMode];
+};
+struct DecTable {
+    uint32_t e[kDecRows << kDecBits];
+};
+
+constexpr int kr_change(uint32_t p) { return p >= 2 ? (int)p + 1 : (p == 1 ? 0 : -2); }
+
+constexpr EncTable make_enc_table()
+{
+    EncTable t{};
+    for (uint32_t run = 0; run < 2; ++run)
+        for (uint32_t k = 0; k < kEncRows; ++k)
+            for (uint32_t i = 0; i < 2 * kEncMax; ++i) {
+                const uint32_t m = i >> 1, u = (i & 1u) && m ? 2 * m - 1 : 2 * m;
+                uint32_t &e = t.e[run * kEncMode + k * kEncCols + i];
+                if (run && u == 0) {  // a zero of a run: no codeword (not an entry of the general path either)
+                    e = 1u << 24;
+                    continue;
+                }
+                const uint32_t v = u - run, p = v >> k, n = p + 1 + k, low = v & ((1u << k) - 1u);
+                if (n > 16) continue;
+                e = ((((low << 1) | 1u) << p) - 1u) | (((uint32_t)kr_change(p) & 0xFFu) << 16) | (n << 24);
+            }
+    return t;
+}
+
+constexpr DecTable make_dec_table()
+{
+    DecTable t{};
+    for (uint32_t k = 0; k < kDecRows; ++k)
+        for (uint32_t x = 0; x < (1u << kDecBits); ++x) {
+            uint32_t p = 0;
+            while (p < kDecBits && ((x >> p) & 1u)) ++p;
+            const uint32_t n = p + 1 + k;
+            if (n > kDecBits) continue;
+            const uint32_t u = (p << k) | ((x >> (p + 1)) & ((1u << k) - 1u));
+            const int q = (u & 1u) ? -(int)(u >> 1) - 1 : (int)(u >> 1);
+            if (q < -128 || q > 127) continue;
+            t.e[(k << kDecBits) | x] = n | (((uint32_t)kr_change(p) & 0xFFu) << 8) |
+                                       (((uint32_t)(u == 0 ? 3 : -3) & 0xFFu) << 16) | ((uint32_t)(q + 128) << 24);
+        }
+    return t;
+}
+
+__device__ const EncTable g_enc_table = make_enc_table();
+__device__ const DecTable g_dec_table = make_dec_table();
+
+template <int BYTE>
+__device__ __forceinline__ int signed_byte(uint32_t e)
+{
+    int r;
+    asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r) : "r"(e), "n"(BYTE | (0x888 | (BYTE * 0x111)) << 4));
+    return r;
+}
+
+template <typename Table>
+__device__ __forceinline__ void stage_table(Table *dst, const Table *src)
+{
+    static_assert(sizeof(Table) % 16 == 0, "copied in 16-byte words");
+    uint4 *d = reinterpret_cast<uint4 *>(dst);
+    const uint4 *q = reinterpret_cast<const uint4 *>(src);
+    for (uint32_t i = threadIdx.x; i < sizeof(Table) / 16; i += blockDim.x) d[i] = __ldg(q + i);
+}
 
 __device__ __forceinline__ uint32_t zz(int32_t q)
 {
@@ -98,35 +177,104 @@ __device__ __forceinline__ void gr_put(BitWriter &bw, uint32_t v, uint32_t k, in
     adapt_kr(p, KR);
 }
 
-// Streaming RLGR coder state of one block.
+// A value that is the same in every lane, in a register of each: left to
+// itself the compiler reloads it for every symbol.
+__device__ __forceinline__ uint32_t in_register(uint32_t x) { return __shfl_sync(0xFFFFFFFFu, x, 0); }
+__device__ __forceinline__ float in_register(float x) { return __shfl_sync(0xFFFFFFFFu, x, 0); }
+
+__device__ __forceinline__ uint32_t shared_address(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// from a table (not written after the CTA's first barrier)
+__device__ __forceinline__ uint32_t table_load(uint32_t a)
+{
+    uint32_t v;
+    asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+
+// Table column 2 t + s of a coefficient, t its magnitude by quantize_f32 up to
+// kEncMax, plus kColBias: the floor by adding 2^23 rounded towards zero, the
+// sign bit shifted in below it.
+constexpr uint32_t kColBias = 2u * 0x4B000000u;
+
+__device__ __forceinline__ uint32_t column_f32(float y, float inv_step, float tau)
+{
+    const float t = fminf(__fadd_rn(__fmul_rn(fabsf(y), inv_step), tau), (float)kEncMax);  // a NaN: kEncMax
+    return __funnelshift_l(__float_as_uint(y), __float_as_uint(__fadd_rz(t, 8388608.0f)), 1);
+}
+
+__device__ __forceinline__ uint32_t column_i32(int32_t q)
+{
+    const uint32_t m = q < 0 ? 0u - (uint32_t)q : (uint32_t)q;
+    return kColBias + 2u * min(m, kEncMax) + (q < 0 ? 1u : 0u);
+}
+
+// RLGR coder of one block.
 struct Rlgr {
     int K, KR;
-    uint32_t z;  // pending zeros of an open run
-    __device__ __forceinline__ void init()
+    uint32_t z;    // pending zeros of an open run
+    uint32_t tab;  // shared-memory address of the table, less the bias of its columns
+    __device__ __forceinline__ void init(const EncTable &t)
     {
         K = 0;
         KR = 32;
         z = 0;
+        tab = in_register(shared_address(t.e) - 4u * kColBias);
     }
-    __device__ __forceinline__ void code(BitWriter &bw, uint32_t u)
+    static __device__ __forceinline__ int next_kr(int kr, uint32_t e)
+    {
+        return __viaddmin_s32_relu(kr, signed_byte<2>(e), 384);
+    }
+    // Two symbols in Golomb-Rice mode (K < 16: no cap at 240), appended by one write; false, with nothing changed,
+    // when the table does not hold one of the codewords.  Wants ready(): the first symbol raises K by 3 and KR by 16
+    // at most, which leaves the second in Golomb-Rice mode and in the table's rows.
+    __device__ __forceinline__ bool ready() const { return K < 13 && KR < 16 * (int)kEncRows - 16; }
+    __device__ __forceinline__ bool pair(BitWriter &bw, uint32_t a, uint32_t b)
+    {
+        const uint32_t e0 = table_load((uint32_t)(KR & 0x1F0) * (kEncCols / 4) + tab + 4u * a);
+        const int kr1 = next_kr(KR, e0);
+        const uint32_t e1 = table_load((uint32_t)(kr1 & 0x1F0) * (kEncCols / 4) + tab + 4u * b);
+        if (e0 == 0u || e1 == 0u) return false;
+        KR = next_kr(kr1, e1);
+        K = __viaddmax_s32(K, a < kColBias + 2u ? 3 : -3, 0);
+        K = __viaddmax_s32(K, b < kColBias + 2u ? 3 : -3, 0);
+        const uint32_t n0 = e0 >> 24;
+        bw.put((e0 & 0xFFFFu) + (e1 & 0xFFFFu) * (1u << n0), n0 + (e1 >> 24));
+        return true;
+    }
+    // One symbol in either mode, without branches for the mode; false, with nothing changed, when the table does not
+    // hold its codeword.  In run mode (k > 0) a nonzero is bit 1, the run length in k bits (z < 2^k, k <= 15), then
+    // its codeword; in Golomb-Rice mode k and z are 0.  The 2^k-th zero of a run is bit 0.
+    __device__ __forceinline__ bool one(BitWriter &bw, uint32_t a)
+    {
+        const uint32_t k = (uint32_t)K >> 4, run = min(k, 1u);
+        const uint32_t e = table_load((uint32_t)(KR & 0x70) * (kEncCols / 4) + run * (4u * kEncMode) + tab + 4u * a);
+        if (e == 0u || KR >= 16 * (int)kEncRows) return false;
+        const bool zero = a < kColBias + 2u, more = zero && K >= 16;
+        const uint32_t z1 = z + 1u, full = z1 >> k;  // used in a run only: z1 <= 2^k
+        const uint32_t npre = k + run, c = ((e & 0xFFFFu) << npre) + (2u * z + run), n = npre + (e >> 24);
+        const int dk = zero ? (more ? 4 * (int)full : 3) : -3 - 3 * (int)run;
+        K = __viaddmin_s32_relu(K, dk, 240);
+        KR = next_kr(KR, e);
+        z = more && !full ? z1 : 0u;
+        bw.put(more ? 0u : c, more ? full : n);
+        return true;
+    }
+    // any symbol, by its zigzag index
+    __device__ __forceinline__ void any(BitWriter &bw, uint32_t u)
     {
         const uint32_t k = (uint32_t)K >> 4;
-        if (__builtin_expect(k == 0, 1)) {  // Golomb-Rice mode
-            gr_put(bw, u, (uint32_t)KR >> 4, KR);
-            K = u == 0 ? K + 3 : (K >= 3 ? K - 3 : 0);  // Golomb-Rice mode runs while K < 16: no cap at 240
-        } else if (u == 0) {
+        if (k != 0 && u == 0) {
             if (++z == (1u << k)) {
                 bw.put(0, 1);
-                K += 4;
-                if (K > 240) K = 240;
+                K = min(K + 4, 240);
                 z = 0;
             }
-        } else {
-            bw.put(1u | (z << 1), 1u + k);  // bit 1, then the run length in k bits (z < 2^k, k <= 15)
-            gr_put(bw, u - 1u, (uint32_t)KR >> 4, KR);
-            K = K >= 6 ? K - 6 : 0;
-            z = 0;
+            return;
         }
+        if (k != 0) bw.put(1u | (z << 1), 1u + k);
+        gr_put(bw, k ? u - 1u : u, (uint32_t)KR >> 4, KR);
+        K = max(k ? K - 6 : K + (u == 0 ? 3 : -3), 0);
+        z = 0;
     }
     __device__ __forceinline__ void finish(BitWriter &bw)
     {
@@ -136,18 +284,20 @@ struct Rlgr {
 };
 
 // ---- encoder: one CTA per rb row blocks; thread = (row block, rung, channel) --
-// Each thread reads its channel's coefficients straight from global memory
-// (lanes of a warp are consecutive channels of a row, so a warp's load is one
-// contiguous run of the row) with the next kPrefetch rows in flight in
-// registers while the current ones are coded; threads never wait for each
-// other after the CTA's one barrier.  Threads of the other rungs of a row
-// read the same words (served by L1).
+// Each thread copies its channel's coefficients into a ring of its own in
+// shared memory by cp.async (lanes of a warp are consecutive channels of a
+// row, so a warp's copy of a row is one contiguous run), kRing - kPrefetch
+// rows ahead of the one being coded: registers for that many rows would cost
+// more resident warps than they hide.  Threads never wait for each other after
+// the CTA's one barrier.  Threads of the other rungs of a row read the same
+// words (served by L1).
 struct EncJobs {
     RlgrJob j;
     const uint64_t *job_off;  // F + 1: first job (row block) of each frame
 };
 
-constexpr uint32_t kPrefetch = 4;
+constexpr uint32_t kPrefetch = 4;  // rows copied and coded at a time; even, for the rows are coded in pairs
+constexpr uint32_t kRing = 16;     // rows of a ring
 
 // Row blocks per CTA: enough that rb * W (W = rungs x channels threads per
 // row block) fills whole warps (rb = 32 / gcd(W, 32)), at most 512 threads.
@@ -160,49 +310,83 @@ __host__ __device__ inline uint32_t row_blocks_per_cta(uint32_t W)
     return rb;
 }
 
+// asynchronous copy of the word p[r * step] to shared memory at dst + OFF; a load from at + OFF
+template <uint32_t OFF>
+__device__ __forceinline__ void copy_word(uint32_t dst, const uint32_t *p, uint32_t r, uint32_t step)
+{
+    asm volatile("{\n.reg .u64 a;\nmad.wide.u32 a, %1, %2, %3;\ncp.async.ca.shared.global [%0+%4], [a], 4;\n}" ::"r"(dst),
+                 "r"(r), "r"(4u * step), "l"(p), "n"(OFF)
+                 : "memory");
+}
+template <uint32_t OFF>
+__device__ __forceinline__ uint32_t ring_load(uint32_t at)
+{
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(at), "n"(OFF) : "memory");
+    return v;
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copies_wait()  // all but the latest N groups have arrived
+{
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ uint32_t shared_load(uint32_t a)
+{
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
+
 struct EncBlock {  // one row block of a CTA
     uint64_t gbase;  // first coefficient (row-major) of the block
     uint32_t f, b, nb, len;
 };
 
-template <bool FROM_INT, bool DIST>
-__global__ void __launch_bounds__(512) rlgr_encode_kernel(EncJobs E, const int32_t *qin, uint32_t rb)
+// row block `job` of the batch (length 0 past the last)
+__device__ __forceinline__ EncBlock enc_block(const EncJobs &E, uint64_t job)
 {
+    const RlgrJob &j = E.j;
+    EncBlock e{0, 0, 0, 0, 0};
+    if (job < E.job_off[j.F]) {
+        uint32_t lo = 0, hi = j.F;
+        while (hi - lo > 1) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if (E.job_off[mid] <= job) lo = mid; else hi = mid;
+        }
+        const uint32_t vs = j.vstart[lo], nv = j.vstart[lo + 1] - vs;
+        e.f = lo;
+        e.b = (uint32_t)(job - E.job_off[lo]);
+        e.nb = (nv + j.B - 1) / j.B;
+        const uint32_t row0 = e.b * j.B;
+        e.len = (nv - row0) < j.B ? (nv - row0) : j.B;
+        e.gbase = ((uint64_t)vs + row0) * j.C;
+    }
+    return e;
+}
+
+// PITCH: threads of a CTA at most
+template <bool FROM_INT, bool DIST, uint32_t PITCH>
+__global__ void __launch_bounds__(PITCH, 1024 / PITCH) rlgr_encode_kernel(EncJobs E, const int32_t *qin, uint32_t rb)
+{
+    extern __shared__ uint32_t ring[];  // kRing x PITCH
     __shared__ EncBlock blk_info[32];
+    __shared__ __align__(16) EncTable tab;
+    stage_table(&tab, &g_enc_table);
     const RlgrJob &j = E.j;
     const uint32_t C = j.C, W = j.R * C;
-    const uint64_t njobs = E.job_off[j.F];
     const uint32_t t = threadIdx.x;
-    if (t < rb) {  // describe the CTA's row blocks
-        EncBlock e{0, 0, 0, 0, 0};
-        const uint64_t job = (uint64_t)blockIdx.x * rb + t;
-        if (job < njobs) {
-            uint32_t lo = 0, hi = j.F;
-            while (hi - lo > 1) {
-                const uint32_t mid = (lo + hi) >> 1;
-                if (E.job_off[mid] <= job) lo = mid; else hi = mid;
-            }
-            const uint32_t vs = j.vstart[lo], nv = j.vstart[lo + 1] - vs;
-            e.f = lo;
-            e.b = (uint32_t)(job - E.job_off[lo]);
-            e.nb = (nv + j.B - 1) / j.B;
-            const uint32_t row0 = e.b * j.B;
-            e.len = (nv - row0) < j.B ? (nv - row0) : j.B;
-            e.gbase = ((uint64_t)vs + row0) * C;
-        }
-        blk_info[t] = e;
-    }
+    if (t < rb) blk_info[t] = enc_block(E, (uint64_t)blockIdx.x * rb + t);
     __syncthreads();
-    const uint32_t jl = t / W;
-    if (jl >= rb) return;
+    // lanes past the last stream do that stream's work once more and write nothing
+    const bool spare = t >= rb * W;
+    const uint32_t tt = spare ? rb * W - 1u : t, jl = tt / W, w = tt - jl * W;
     const EncBlock me = blk_info[jl];
-    if (me.len == 0) return;
-    const uint32_t w = t - jl * W;
     const uint32_t r = w / C, c = w - r * C;
     const uint64_t blk = j.blk_off[me.f] + ((uint64_t)r * me.nb + me.b) * C + c;
-    BitWriter bw{0u, 0u, 0u, j.slots + blk * j.slot_words, j.slot_words};
+    BitWriter bw(j.slots + blk * j.slot_words, spare ? 0u : j.slot_words);
     Rlgr st;
-    st.init();
+    st.init(tab);
     const float inv = FROM_INT ? 0.f : j.inv_step[r * C + c];
     const float stp = DIST ? j.step[r * C + c] : 0.f;
     float sq = 0.f;
@@ -211,67 +395,245 @@ __global__ void __launch_bounds__(512) rlgr_encode_kernel(EncJobs E, const int32
     const uint32_t *col = src + me.gbase + c;  // row i of this channel at col[i * C]
     const uint32_t len = me.len;
     uint32_t i = 0;
-    if (!FROM_INT && j.dc && me.b == 0) {  // the frame's DC: quantised from its FP64 value
+    if (!FROM_INT && j.dc && me.b == 0 && me.len) {  // the frame's DC: quantised from its FP64 value
         const double y = j.dc[(uint64_t)me.f * C + c], st64 = j.steps_rg[r * j.G + j.groups[c]];
         const int32_t q = quantize_f64(y, st64, j.tau64);
-        st.code(bw, zz(q));
+        st.any(bw, zz(q));
         if (DIST) {
             const double e = __dsub_rn(y, __dmul_rn((double)q, st64));
             dc_err = __dmul_rn(e, e);
         }
         i = 1;
     }
-    auto code_one = [&](uint32_t x) {
-        if (DIST) {  // squared error of the dequantised coefficient (Parseval: of the attributes)
-            const float y = __uint_as_float(x);
-            const int32_t q = quantize_f32(y, inv, j.tau);
-            const float e = __fsub_rn(y, __fmul_rn((float)q, stp));
-            sq = __fadd_rn(sq, __fmul_rn(e, e));
-            st.code(bw, zz(q));
-        } else {
-            st.code(bw, FROM_INT ? zz((int32_t)x) : quantize_zz_f32(__uint_as_float(x), inv, j.tau));
+    const float tau = in_register(j.tau);
+    auto index_of = [&](uint32_t x) {
+        return FROM_INT ? zz((int32_t)x) : quantize_zz_f32(__uint_as_float(x), inv, tau);
+    };
+    auto column_of = [&](uint32_t x) {
+        return FROM_INT ? column_i32((int32_t)x) : column_f32(__uint_as_float(x), inv, tau);
+    };
+    auto distort = [&](uint32_t x) {  // squared error of the dequantised coefficient (Parseval: of the attributes)
+        const float y = __uint_as_float(x);
+        const float e = __fsub_rn(y, __fmul_rn((float)quantize_f32(y, inv, tau), stp));
+        sq = __fadd_rn(sq, __fmul_rn(e, e));
+    };
+    // a lane's whole groups of kPrefetch rows; the warp stays together to the end of its longest block (a frame's
+    // last block is shorter)
+    const uint32_t groups = (len - i) / kPrefetch;
+    const uint32_t common = __reduce_min_sync(0xFFFFFFFFu, groups), longest = __reduce_max_sync(0xFFFFFFFFu, groups);
+    constexpr uint32_t kRow = 4u * PITCH, kGroup = kPrefetch * kRow, kBytes = kRing * kRow;  // bytes in the ring
+    const uint32_t mine = in_register(shared_address(ring)) + 4u * t;
+    uint32_t next = 0, slot = 0;  // group to copy, and its place
+    auto copy_group = [&] {
+        if (next < groups) {
+            const uint32_t at = mine + slot, r = i + next * kPrefetch;
+            copy_word<0>(at, col, r, C);
+            copy_word<kRow>(at, col, r + 1, C);
+            copy_word<2 * kRow>(at, col, r + 2, C);
+            copy_word<3 * kRow>(at, col, r + 3, C);
+        }
+        static_assert(kPrefetch == 4, "copies of a group");
+        copies_commit();
+        ++next;
+        slot = (slot + kGroup) % kBytes;
+    };
+    auto code_group = [&](bool live) {
+        copies_wait<kRing / kPrefetch - 2>();
+        const uint32_t from = mine + (slot + kGroup) % kBytes;
+        const uint32_t x[kPrefetch] = {ring_load<0>(from), ring_load<kRow>(from), ring_load<2 * kRow>(from),
+                                       ring_load<3 * kRow>(from)};
+        copy_group();  // over the group before this one
+#pragma unroll
+        for (uint32_t d = 0; d < kPrefetch; d += 2) {
+            // one lane in run mode (or near it) takes its warp through the path for either mode
+            bool done = __all_sync(0xFFFFFFFFu, !live || st.ready());
+            if (!live) continue;
+            const uint32_t a = column_of(x[d]), b = column_of(x[d + 1]);
+            if (done) done = st.pair(bw, a, b);
+            if (!done) {
+                uint32_t h = st.one(bw, a) ? (st.one(bw, b) ? 2u : 1u) : 0u;
+#pragma unroll 1
+                for (; h < 2u; ++h)  // what the table does not hold: rare
+                    if (!st.one(bw, h ? b : a)) st.any(bw, index_of(h ? x[d + 1] : x[d]));
+            }
+            if (DIST) {
+                distort(x[d]);
+                distort(x[d + 1]);
+            }
         }
     };
-    uint32_t cur[kPrefetch];
 #pragma unroll
-    for (uint32_t d = 0; d < kPrefetch; ++d) cur[d] = (i + d < len) ? __ldg(col + (uint64_t)(i + d) * C) : 0u;
-    for (; i + kPrefetch <= len; i += kPrefetch) {
-        uint32_t nx[kPrefetch];
-        const uint32_t *q = col + (uint64_t)(i + kPrefetch) * C;
+    for (uint32_t g = 0; g + 1 < kRing / kPrefetch; ++g) copy_group();
+    for (uint32_t g = 0; g < common; ++g) code_group(true);
+    for (uint32_t g = common; g < longest; ++g) code_group(g < groups);
+    copies_wait<0>();
+    i += groups * kPrefetch;
+    if (i < len) {  // fewer than kPrefetch rows
+        uint32_t x[kPrefetch - 1];
 #pragma unroll
-        for (uint32_t d = 0; d < kPrefetch; ++d) nx[d] = (i + kPrefetch + d < len) ? __ldg(q + d * C) : 0u;
-#pragma unroll
-        for (uint32_t d = 0; d < kPrefetch; ++d) code_one(cur[d]);
-#pragma unroll
-        for (uint32_t d = 0; d < kPrefetch; ++d) cur[d] = nx[d];
+        for (uint32_t d = 0; d + 1 < kPrefetch; ++d) x[d] = i + d < len ? __ldg(col + (uint64_t)(i + d) * C) : 0u;
+#pragma unroll 1
+        for (uint32_t d = 0; i < len; ++i, ++d) {
+            const uint32_t y = d == 0 ? x[0] : (d == 1 ? x[1] : x[2]);
+            if (!st.one(bw, column_of(y))) st.any(bw, index_of(y));
+            if (DIST) distort(y);
+        }
     }
-#pragma unroll
-    for (uint32_t d = 0; d < kPrefetch; ++d)
-        if (i + d < len) code_one(cur[d]);
+    if (len == 0 || spare) return;
     st.finish(bw);
     j.block_words[blk] = bw.nw;
     if (bw.nw > j.slot_words) atomicExch(j.overflow, 1u);
     if (DIST) atomicAdd(j.sq_err + ((uint64_t)me.f * j.R + r) * C + c, __dadd_rn((double)sq, dc_err));
 }
 
+// ---- encoder for few streams ----------------------------------------------------
+// Where the streams do not fill the GPU, a launch takes as long as one thread
+// takes for its block, and what counts is the length of a symbol's dependent
+// chain, not its instructions over all paths: each lane branches to its own
+// path, and a zero of a run is three instructions.  A point cloud of 1M points
+// (C = 3, 2,900 streams, mostly runs): 88 us against 129 us by the kernel
+// above; a frame of 250k Gaussians (27k streams, few runs): 90 against 81 us.
+constexpr uint64_t kFewStreams = 20000;
+
+struct RlgrFew {
+    int K, KR;
+    uint32_t z;  // pending zeros of an open run
+    __device__ __forceinline__ void code(BitWriter &bw, uint32_t u)
+    {
+        const uint32_t k = (uint32_t)K >> 4;
+        if (__builtin_expect(k == 0, 1)) {  // Golomb-Rice mode
+            gr_put(bw, u, (uint32_t)KR >> 4, KR);
+            K = max(K + (u == 0 ? 3 : -3), 0);
+        } else if (u == 0) {
+            if (++z == (1u << k)) {
+                bw.put(0, 1);
+                K = min(K + 4, 240);
+                z = 0;
+            }
+        } else {
+            bw.put(1u | (z << 1), 1u + k);  // bit 1, then the run length in k bits (z < 2^k, k <= 15)
+            gr_put(bw, u - 1u, (uint32_t)KR >> 4, KR);
+            K = max(K - 6, 0);
+            z = 0;
+        }
+    }
+};
+
+__global__ void __launch_bounds__(512) rlgr_encode_few_kernel(EncJobs E, uint32_t rb)
+{
+    __shared__ EncBlock blk_info[32];
+    const RlgrJob &j = E.j;
+    const uint32_t C = j.C, W = j.R * C, t = threadIdx.x;
+    if (t < rb) blk_info[t] = enc_block(E, (uint64_t)blockIdx.x * rb + t);
+    __syncthreads();
+    const uint32_t jl = t / W;
+    if (jl >= rb) return;
+    const EncBlock me = blk_info[jl];
+    if (me.len == 0) return;
+    const uint32_t w = t - jl * W, r = w / C, c = w - r * C;
+    const uint64_t blk = j.blk_off[me.f] + ((uint64_t)r * me.nb + me.b) * C + c;
+    BitWriter bw(j.slots + blk * j.slot_words, j.slot_words);
+    RlgrFew st{0, 32, 0u};
+    const float inv = j.inv_step[r * C + c], tau = j.tau;
+    const float *col = j.Y + me.gbase + c;  // row i of this channel at col[i * C]
+    const uint32_t len = me.len;
+    uint32_t i = 0;
+    if (j.dc && me.b == 0) {  // the frame's DC: quantised from its FP64 value
+        st.code(bw, zz(quantize_f64(j.dc[(uint64_t)me.f * C + c], j.steps_rg[r * j.G + j.groups[c]], j.tau64)));
+        i = 1;
+    }
+    float cur[kPrefetch];
+#pragma unroll
+    for (uint32_t d = 0; d < kPrefetch; ++d) cur[d] = (i + d < len) ? __ldg(col + (uint64_t)(i + d) * C) : 0.f;
+    for (; i + kPrefetch <= len; i += kPrefetch) {
+        float nx[kPrefetch];
+        const float *q = col + (uint64_t)(i + kPrefetch) * C;
+#pragma unroll
+        for (uint32_t d = 0; d < kPrefetch; ++d) nx[d] = (i + kPrefetch + d < len) ? __ldg(q + d * C) : 0.f;
+#pragma unroll
+        for (uint32_t d = 0; d < kPrefetch; ++d) st.code(bw, quantize_zz_f32(cur[d], inv, tau));
+#pragma unroll
+        for (uint32_t d = 0; d < kPrefetch; ++d) cur[d] = nx[d];
+    }
+#pragma unroll
+    for (uint32_t d = 0; d < kPrefetch; ++d)
+        if (i + d < len) st.code(bw, quantize_zz_f32(cur[d], inv, tau));
+    if (st.z) bw.put(0, 1);
+    bw.flush();
+    j.block_words[blk] = bw.nw;
+    if (bw.nw > j.slot_words) atomicExch(j.overflow, 1u);
+}
+
 // ---- decoder ------------------------------------------------------------------
 // Bits are looked at through a 32-bit window over two consecutive words
-// (cur, nxt) at bit offset pos: one funnel shift per look and one word load
-// every 32 bits consumed.  Words past the end of a stream read as zero, so a
-// malformed stream cannot make the reader leave it; whether the stream was
-// overrun is checked once, after its last coefficient, from the bits consumed.
+// (cur, nxt) at bit offset pos; the word after them (ahead) is in a register
+// too, so that no lane's refill makes the warp wait for a load.  The words
+// come from a ring of four 16-byte pieces per thread in shared memory that the
+// thread tops up by cp.async (top_up, every four symbols); a stream that drains
+// it in between is read from global memory.  Words past the end of a stream
+// read as zero, so a malformed stream cannot make the reader leave it; whether
+// the stream was overrun is checked once, after its last coefficient, from the
+// bits consumed.  Word numbers count from the 16-byte boundary at or below the
+// stream's first word.
+constexpr uint32_t kRingWords = 16, kPieces = kRingWords / 4;
+
 struct WinReader {
-    const uint32_t *w;
-    uint32_t nw, cur, nxt, pos, idx;
-    __device__ __forceinline__ void init(const uint32_t *p, uint32_t n)
+    const uint32_t *base;  // the 16-byte boundary
+    uint32_t ring;         // shared-memory address of the ring (aligned to its size)
+    uint32_t lead, end;    // byte offsets of the stream's first word and of its end
+    uint32_t cur, nxt, ahead, pos;
+    uint32_t at;      // byte offset of the word after `ahead`
+    uint32_t issued;  // pieces asked for; and as that was at the ends of the last three calls of top_up
+    uint32_t issued1, issued2, issued3;
+    uint32_t ready;   // bytes below have arrived
+
+    __device__ __forceinline__ uint32_t ring_word(uint32_t o) const
     {
-        w = p;
-        nw = n;
-        cur = n > 0 ? p[0] : 0u;
-        nxt = n > 1 ? p[1] : 0u;
-        pos = 0;
-        idx = 2;
+        return shared_load(ring | (o & (4u * kRingWords - 4u)));
     }
+    __device__ __forceinline__ void issue()
+    {
+        const uint32_t bytes = (uint32_t)min(max((int)end - 16 * (int)issued, 0), 16);  // the rest: zeros
+        const uint32_t dst = ring | (16u * (issued & (kPieces - 1u)));
+        const uint32_t *src = base + 4 * (bytes ? issued : 0u);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+        ++issued;
+    }
+    __device__ __forceinline__ void init(const uint32_t *p, uint32_t n, const uint32_t *r)
+    {
+        lead = (uint32_t)((uintptr_t)p & 12u);
+        base = p - lead / 4;
+        ring = shared_address(r);
+        end = lead + 4u * n;
+        issued = 0;
+#pragma unroll
+        for (uint32_t k = 0; k < kPieces; ++k) issue();
+        copies_commit();
+        copies_wait<0>();
+        issued1 = issued2 = issued3 = issued;
+        ready = 16u * issued;
+        cur = ring_word(lead);
+        nxt = ring_word(lead + 4u);
+        ahead = ring_word(lead + 8u);
+        pos = 0;
+        at = lead + 12u;
+    }
+    // Asks for the piece that the reader comes to next, once the one whose place it takes has been read; a piece is
+    // taken to have arrived at the third call after.  True when the ring holds the two words that may be wanted
+    // before the next call (skip_ready).
+    __device__ __forceinline__ bool top_up()
+    {
+        copies_wait<2>();
+        ready = 16u * issued3;
+        issued3 = issued2;
+        issued2 = issued1;
+        issued = max(issued, at >> 4);
+        if (at + 16u * (kPieces - 1u) >= 16u * issued) issue();
+        issued1 = issued;
+        copies_commit();
+        return stocked();
+    }
+    __device__ __forceinline__ bool stocked() const { return at + 8u <= ready; }
     __device__ __forceinline__ uint32_t peek() const { return __funnelshift_r(cur, nxt, pos); }
     __device__ __forceinline__ void skip(uint32_t n)  // n <= 32
     {
@@ -279,16 +641,27 @@ struct WinReader {
         if (pos >= 32u) {
             pos -= 32u;
             cur = nxt;
-            nxt = idx < nw ? w[idx] : 0u;
-            ++idx;
+            nxt = ahead;
+            ahead = at < ready ? ring_word(at) : (at < end ? base[at >> 2] : 0u);
+            at += 4u;
         }
+    }
+    // the same when the ring holds the next word: no branch
+    __device__ __forceinline__ void skip_ready(uint32_t n)
+    {
+        pos += n;
+        asm volatile("{\n.reg .pred f;\n.reg .u32 a;\nsetp.ge.u32 f, %4, 32;\n"
+                     "@f mov.u32 %0, %1;\n@f mov.u32 %1, %2;\n"
+                     "lop3.b32 a, %3, %6, %5, 0xEA;\n@f ld.shared.u32 %2, [a];\n@f add.u32 %3, %3, 4;\n}"
+                     : "+r"(cur), "+r"(nxt), "+r"(ahead), "+r"(at)
+                     : "r"(pos), "r"(ring), "n"(4 * kRingWords - 4));
+        pos &= 31u;
     }
     __device__ __forceinline__ bool overrun() const
     {
-        return (uint64_t)(idx - 2u) * 32u + pos > (uint64_t)nw * 32u;
+        return (uint64_t)(at - 12u - lead) * 8u + pos > (uint64_t)(end - lead) * 8u;
     }
 };
-
 
 // Rare path of gr_read: the remainder crosses the window, or the escape code.
 __device__ __forceinline__ uint32_t gr_read_slow(WinReader &r, uint32_t k, uint32_t p, bool &bad)
@@ -332,77 +705,96 @@ __device__ __forceinline__ uint32_t gr_read(WinReader &r, uint32_t k, int &KR, b
 }
 
 // Decodes one block stream (len coefficients of one channel) to out[i * C],
-// i < len: dequantised (times sc) or as indices.  Runs are kept as pending
-// zeros (and the nonzero that ends a partial run as a pending value), so a
-// lane writes one or two rows per iteration: a lane that ends an iteration in
-// Golomb-Rice mode decodes a second symbol in the same iteration (fewer loop
-// and mode tests per symbol).
+// i < len: dequantised (times sc) or as indices.  A Golomb-Rice symbol whose
+// codeword the table holds takes the short path; run mode (runs are kept as
+// pending zeros, and the nonzero that ends a partial run as a pending value)
+// and longer codewords the general one.
+constexpr int kRunLeft = 1 << 16;  // flags in K: zeros or a value of an earlier run are still to be written,
+constexpr int kDrained = 1 << 17;  // the ring may not hold the next words: only the general path, which checks
+
 template <bool TO_INT>
-__device__ __forceinline__ void decode_stream(const uint32_t *wp, uint32_t nw, uint32_t len, uint32_t C, float sc,
-                                              float *yout, int32_t *qout, DevState *st)
+__device__ __forceinline__ void decode_stream(const DecTable &tab, uint32_t *ring, const uint32_t *wp, uint32_t nw,
+                                              uint32_t len, uint32_t C, float sc, float *yout, int32_t *qout,
+                                              DevState *st)
 {
     WinReader r;
-    r.init(wp, nw);
+    r.init(wp, nw, ring);
     int K = 0, KR = 32;
     uint32_t zeros = 0;
-    bool has_pending = false, bad = false;
-    int32_t pending = 0;
-    for (uint32_t i = 0; i < len; ++i) {
-        int32_t q = 0;
-        const uint32_t k = (uint32_t)K >> 4;
-        if (__builtin_expect(!(zeros | (uint32_t)has_pending | k), 1)) {  // the common case: Golomb-Rice mode
-            const uint32_t u = gr_read(r, (uint32_t)KR >> 4, KR, bad);
-            q = unzz(u);
-            K = u == 0 ? K + 3 : (K >= 3 ? K - 3 : 0);  // Golomb-Rice mode runs while K < 16: no cap at 240
-        } else if (zeros) {
-            --zeros;
-        } else if (has_pending) {
-            q = pending;
-            has_pending = false;
-        } else {
-            const uint32_t x = r.peek();
-            if (!(x & 1u)) {  // a full run of 2^k zeros (clamped at the block end)
-                r.skip(1);
-                const uint32_t run = 1u << k;
-                zeros = (run < len - i ? run : len - i) - 1;
-                K += 4;
-                if (K > 240) K = 240;
-            } else {  // r < 2^k zeros, then a nonzero
-                const uint32_t rr = (x >> 1) & ((1u << k) - 1u);
-                r.skip(1u + k);
-                const uint32_t v = gr_read(r, (uint32_t)KR >> 4, KR, bad);
-                if (rr >= len - i || v == 0xFFFFFFFFu) bad = true;
-                K = K >= 6 ? K - 6 : 0;
-                if (rr == 0) {
-                    q = unzz(v + 1u);
-                } else {
-                    zeros = rr - 1;
-                    pending = unzz(v + 1u);
-                    has_pending = true;
-                }
-            }
-        }
-        if (TO_INT) {
-            *qout = q;
-            qout += C;
-        } else {
-            *yout = __fmul_rn((float)q, sc);
-            yout += C;
-        }
-        if (i + 1 < len && !(zeros | (uint32_t)has_pending | ((uint32_t)K >> 4))) {  // a second GR-mode symbol
-            const uint32_t u = gr_read(r, (uint32_t)KR >> 4, KR, bad);
-            const int32_t q2 = unzz(u);
-            K = u == 0 ? K + 3 : (K >= 3 ? K - 3 : 0);
-            ++i;
-            if (TO_INT) {
-                *qout = q2;
-                qout += C;
+    bool bad = false;
+    int32_t pending = 0;  // written after the zeros; 0: nothing (a pending value is a nonzero)
+    auto general = [&](uint32_t left) -> int32_t {  // left: coefficients of the block from this one on
+        if (K & kRunLeft) {
+            int32_t q = 0;
+            if (zeros) {
+                --zeros;
             } else {
-                *yout = __fmul_rn((float)q2, sc);
-                yout += C;
+                q = pending;
+                pending = 0;
             }
+            if (!zeros && !pending) K &= ~kRunLeft;
+            return q;
         }
+        K &= ~kDrained;
+        const uint32_t k = (uint32_t)K >> 4;
+        if (k == 0) {
+            const uint32_t u = gr_read(r, (uint32_t)KR >> 4, KR, bad);
+            K = max(K + (u == 0 ? 3 : -3), 0);
+            return unzz(u);
+        }
+        const uint32_t x = r.peek();
+        if (!(x & 1u)) {  // a full run of 2^k zeros (clamped at the block end)
+            r.skip(1);
+            zeros = min(1u << k, left) - 1u;
+            K = min(K + 4, 240);
+            if (zeros) K |= kRunLeft;
+            return 0;
+        }
+        const uint32_t rr = (x >> 1) & ((1u << k) - 1u);  // rr < 2^k zeros, then a nonzero
+        r.skip(1u + k);
+        const uint32_t v = gr_read(r, (uint32_t)KR >> 4, KR, bad);
+        if (rr >= left || v == 0xFFFFFFFFu) bad = true;
+        K = max(K - 6, 0);
+        const int32_t q = unzz(v + 1u);
+        if (rr == 0) return q;
+        zeros = rr - 1;
+        pending = q;
+        if (zeros | (uint32_t)pending) K |= kRunLeft;
+        return 0;
+    };
+    const uint32_t ta = shared_address(tab.e);
+    auto symbol = [&](uint32_t i) {
+        const uint32_t e = table_load((uint32_t)(KR & 0x70) * (4u << (kDecBits - 4)) + ta +
+                                      4u * (r.peek() & ((1u << kDecBits) - 1u)));
+        int32_t q;
+        float y;
+        // Golomb-Rice mode (K < 16, no flag set), a row and a codeword of the table
+        if (__builtin_expect(e != 0u && K < 16 && KR < 16 * (int)kDecRows, 1)) {
+            q = (int32_t)(e >> 24) - 128;
+            y = __fadd_rn(__uint_as_float(__byte_perm(e, 0x4B000000u, 0x7443)), -8388736.0f);  // 2^23 + (q + 128)
+            KR = __viaddmin_s32_relu(KR, signed_byte<1>(e), 384);
+            K = __viaddmax_s32(K, signed_byte<2>(e), 0);
+            r.skip_ready(e & 0xFFu);
+        } else {
+            q = general(len - i);
+            y = (float)q;
+            if (!r.stocked()) K |= kDrained;
+        }
+        if (TO_INT)
+            qout[(uint64_t)i * C] = q;
+        else
+            yout[(uint64_t)i * C] = __fmul_rn(y, sc);
+    };
+    uint32_t i = 0;
+    for (; i + 4 <= len; i += 4) {
+        K = r.top_up() ? K & ~kDrained : K | kDrained;
+#pragma unroll
+        for (uint32_t h = 0; h < 4; ++h) symbol(i + h);
     }
+    K = r.top_up() ? K & ~kDrained : K | kDrained;
+#pragma unroll 1
+    for (; i < len; ++i) symbol(i);
+    copies_wait<0>();
     if (bad || r.overrun()) set_error(&st->err, kErrCorrupt);
 }
 
@@ -410,12 +802,16 @@ __device__ __forceinline__ void decode_stream(const uint32_t *wp, uint32_t nw, u
 // b = x * rb + jl of channel c.  Streams at block_off[b*C+c] (words) when
 // block_off is given, else at (b*C+c) * stride.
 template <bool TO_INT>
-__global__ void __launch_bounds__(512, 4) rlgr_decode_kernel(const uint32_t *payload, uint64_t payload_words,
+__global__ void __launch_bounds__(512, 2) rlgr_decode_kernel(const uint32_t *payload, uint64_t payload_words,
                                                           const uint32_t *block_words, const uint64_t *block_off,
                                                           uint32_t stride, uint32_t nv, uint32_t C, uint32_t B,
                                                           uint32_t rb, const float *step, float *Y, int32_t *qout,
                                                           DevState *st)
 {
+    extern __shared__ __align__(128) uint32_t ring[];  // kRingWords per thread
+    __shared__ __align__(16) DecTable tab;
+    stage_table(&tab, &g_dec_table);
+    __syncthreads();
     const uint32_t jl = threadIdx.x / C;
     if (jl >= rb) return;
     const uint32_t c = threadIdx.x - jl * C;
@@ -424,22 +820,27 @@ __global__ void __launch_bounds__(512, 4) rlgr_decode_kernel(const uint32_t *pay
     if (row0 >= nv) return;
     const uint32_t len = (nv - row0) < B ? (uint32_t)(nv - row0) : B;
     const uint64_t blk = b * C + c;
-    const uint64_t off = block_off ? block_off[blk] : blk * stride;
+    uint64_t off = block_off ? block_off[blk] : blk * stride;
     uint32_t nw = block_words[blk];
     if (off + nw > payload_words) {
         set_error(&st->err, kErrCorrupt);
         nw = 0;
+        off = 0;
     }
-    decode_stream<TO_INT>(payload + off, nw, len, C, TO_INT ? 0.f : step[c], TO_INT ? nullptr : Y + row0 * C + c,
+    decode_stream<TO_INT>(tab, ring + threadIdx.x * kRingWords, payload + off, nw, len, C, TO_INT ? 0.f : step[c], TO_INT ? nullptr : Y + row0 * C + c,
                           TO_INT ? qout + row0 * C + c : nullptr, st);
 }
 
 // All frames of a batch: row blocks numbered across frames (job_off), rb per CTA.
-__global__ void __launch_bounds__(512, 4) rlgr_decode_batch_kernel(const DecFrame *fr, uint32_t F,
+__global__ void __launch_bounds__(512, 2) rlgr_decode_batch_kernel(const DecFrame *fr, uint32_t F,
                                                                 const uint64_t *job_off, const uint32_t *bw_all,
                                                                 const uint64_t *boff_all, const float *steps_all,
                                                                 uint32_t C, uint32_t rb, float *Y, DevState *st)
 {
+    extern __shared__ __align__(128) uint32_t ring[];  // kRingWords per thread
+    __shared__ __align__(16) DecTable tab;
+    stage_table(&tab, &g_dec_table);
+    __syncthreads();
     const uint32_t jl = threadIdx.x / C;
     if (jl >= rb) return;
     const uint32_t c = threadIdx.x - jl * C;
@@ -456,13 +857,14 @@ __global__ void __launch_bounds__(512, 4) rlgr_decode_batch_kernel(const DecFram
     const uint32_t len = (d.nv - row0) < d.B ? (d.nv - row0) : d.B;
     const uint64_t base = boff_all[d.blk_off];
     const uint64_t blk = d.blk_off + (uint64_t)b * C + c;
-    const uint64_t off = boff_all[blk] - base;
+    uint64_t off = boff_all[blk] - base;
     uint32_t nw = bw_all[blk];
     if (off + nw > d.payload_words) {
         set_error(&st->err, kErrCorrupt);
         nw = 0;
+        off = 0;
     }
-    decode_stream<false>(d.payload + off, nw, len, C, steps_all[(uint64_t)lo * C + c],
+    decode_stream<false>(tab, ring + threadIdx.x * kRingWords, d.payload + off, nw, len, C, steps_all[(uint64_t)lo * C + c],
                          Y + ((uint64_t)d.vstart + row0) * C + c, nullptr, st);
 }
 
@@ -482,7 +884,24 @@ __global__ void job_offsets_kernel(const uint32_t *vstart, uint32_t F, uint32_t 
     blk_off[F] = bo;
 }
 
+// dynamic shared memory of a kernel's rings (beside its table it may pass the 48 KB that need no opt-in)
+template <typename Kernel>
+size_t ring_smem(Kernel k, size_t bytes)
+{
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    return bytes;
+}
+
 }  // namespace
+
+template <bool FROM_INT, bool DIST>
+static void launch_encode(const EncJobs &E, const int32_t *q, uint32_t rb, uint32_t threads, uint64_t jobs, cudaStream_t s)
+{
+    const uint32_t grid = (uint32_t)((jobs + rb - 1) / rb);
+    auto k = threads <= 256 ? rlgr_encode_kernel<FROM_INT, DIST, 256> : rlgr_encode_kernel<FROM_INT, DIST, 512>;
+    k<<<grid, threads, ring_smem(k, 4 * (size_t)kRing * (threads <= 256 ? 256 : 512)), s>>>(E, q, rb);
+    count_launch();
+}
 
 // A slot holds 16 bits per coefficient on average (ample for quantised
 // attribute coefficients); the worst case is 78 bits per coefficient.
@@ -502,13 +921,18 @@ void launch_rlgr_encode(const RlgrJob &j, const uint64_t *job_off, uint64_t jobs
 {
     if (jobs_bound == 0 || j.C == 0) return;
     EncJobs E{j, job_off};
-    const uint32_t rb = row_blocks_per_cta(j.R * j.C);
-    const uint32_t threads = (rb * j.R * j.C + 31) / 32 * 32;
+    const uint32_t W = j.R * j.C;
+    const uint32_t rb = row_blocks_per_cta(W);
+    const uint32_t threads = (rb * W + 31) / 32 * 32;
+    if (!j.sq_err && jobs_bound * W <= kFewStreams) {
+        rlgr_encode_few_kernel<<<(uint32_t)((jobs_bound + rb - 1) / rb), threads, 0, s>>>(E, rb);
+        count_launch();
+        return;
+    }
     if (j.sq_err)
-        rlgr_encode_kernel<false, true><<<(uint32_t)((jobs_bound + rb - 1) / rb), threads, 0, s>>>(E, nullptr, rb);
+        launch_encode<false, true>(E, nullptr, rb, threads, jobs_bound, s);
     else
-        rlgr_encode_kernel<false, false><<<(uint32_t)((jobs_bound + rb - 1) / rb), threads, 0, s>>>(E, nullptr, rb);
-    count_launch();
+        launch_encode<false, false>(E, nullptr, rb, threads, jobs_bound, s);
 }
 
 void launch_rlgr_encode_indices(const int32_t *q, const uint32_t *vstart, uint32_t C, uint32_t B, uint32_t *slots,
@@ -530,8 +954,7 @@ void launch_rlgr_encode_indices(const int32_t *q, const uint32_t *vstart, uint32
     EncJobs E{j, job_off};
     const uint32_t rb = row_blocks_per_cta(C);
     const uint32_t threads = (rb * C + 31) / 32 * 32;
-    rlgr_encode_kernel<true, false><<<(uint32_t)((jobs_bound + rb - 1) / rb), threads, 0, s>>>(E, q, rb);
-    count_launch();
+    launch_encode<true, false>(E, q, rb, threads, jobs_bound, s);
 }
 
 void launch_rlgr_decode(const uint32_t *payload, uint64_t payload_words, const uint32_t *block_words,
@@ -541,9 +964,8 @@ void launch_rlgr_decode(const uint32_t *payload, uint64_t payload_words, const u
     if (nv == 0 || C == 0) return;
     const uint64_t nb = (nv + B - 1) / B;
     const uint32_t rb = row_blocks_per_cta(C);
-    // Streams are read in place: staging them in shared memory would cap the
-    // number of resident threads, and this sequential decoder needs them all.
-    rlgr_decode_kernel<false><<<(uint32_t)((nb + rb - 1) / rb), rb * C, 0, s>>>(
+    const size_t smem = ring_smem(rlgr_decode_kernel<false>, 4 * kRingWords * rb * C);
+    rlgr_decode_kernel<false><<<(uint32_t)((nb + rb - 1) / rb), rb * C, smem, s>>>(
         payload, payload_words, block_words, block_off, 0u, (uint32_t)nv, C, B, rb, step, Y, nullptr, st);
     count_launch();
 }
@@ -554,7 +976,8 @@ void launch_rlgr_decode_batch(const DecFrame *fr, uint32_t F, const uint64_t *jo
 {
     if (jobs_bound == 0 || C == 0) return;
     const uint32_t rb = row_blocks_per_cta(C);
-    rlgr_decode_batch_kernel<<<(uint32_t)((jobs_bound + rb - 1) / rb), rb * C, 0, s>>>(
+    const size_t smem = ring_smem(rlgr_decode_batch_kernel, 4 * kRingWords * rb * C);
+    rlgr_decode_batch_kernel<<<(uint32_t)((jobs_bound + rb - 1) / rb), rb * C, smem, s>>>(
         fr, F, job_off, bw_all, boff_all, steps_all, C, rb, Y, st);
     count_launch();
 }
@@ -565,7 +988,8 @@ void launch_rlgr_decode_indices(const uint32_t *words, uint64_t total_words, con
     if (nv == 0 || C == 0) return;
     const uint64_t nb = (nv + B - 1) / B;
     const uint32_t rb = row_blocks_per_cta(C);
-    rlgr_decode_kernel<true><<<(uint32_t)((nb + rb - 1) / rb), rb * C, 0, s>>>(
+    const size_t smem = ring_smem(rlgr_decode_kernel<true>, 4 * kRingWords * rb * C);
+    rlgr_decode_kernel<true><<<(uint32_t)((nb + rb - 1) / rb), rb * C, smem, s>>>(
         words, total_words, bw, nullptr, stride, (uint32_t)nv, C, B, rb, nullptr, nullptr, q, st);
     count_launch();
 }
