@@ -1038,6 +1038,15 @@ gsnfs_status encode_impl(gsnfs_ctx *ctx, cudaStream_t s, EncodeReq &rq, bool wor
         fs.J = L.Jd;
         fs.grid = L.grid;
 
+        // the attributes' centres and colour transforms depend on the input rows alone: beside a1-a3, on the
+        // high-priority stream that a6-a9 follow on
+        cudaStream_t sa = s;
+        if (C) {
+            const gsnfs_status fst = fork_hi_begin(ctx, s, &sa);
+            if (fst) return fst;
+            launch_frame_centres(L.attrp, L.poff, F, C, L.center, sa);
+            if (q->color) launch_color_klt(L.attrp, L.poff, F, L.klt, L.center, L.kltpart, sa);
+        }
         // a1: voxelise + Morton
         stage_begin(s, kStVoxelize);
         launch_voxelize(fs, dst, N, nmax, L.keys, L.vals, sms, s);
@@ -1057,9 +1066,8 @@ gsnfs_status encode_impl(gsnfs_ctx *ctx, cudaStream_t s, EncodeReq &rq, bool wor
                      C ? svals : nullptr, L.row0);
         stage_end(s, kStDedup);
         // a4 + a5 (geometry) run on s beside a6-a9 (attributes, the longer branch) on the high-priority stream
-        cudaStream_t sa = s;
         if (C) {
-            const gsnfs_status fst = fork_hi_begin(ctx, s, &sa);
+            const gsnfs_status fst = stream_wait(ctx, sa, s);
             if (fst) return fst;
         }
         // a4: octree occupancy
@@ -1079,8 +1087,6 @@ gsnfs_status encode_impl(gsnfs_ctx *ctx, cudaStream_t s, EncodeReq &rq, bool wor
             stage_begin(sa, kStPrelude);
             launch_raht_prelude(L.plan, L.gap, dst, nullptr, sms, sa);
             stage_end(sa, kStPrelude);
-            launch_frame_centres(L.attrp, L.poff, F, C, L.center, sa);
-            if (q->color) launch_color_klt(L.attrp, L.poff, F, L.klt, L.center, L.kltpart, sa);
             RahtIO io{};
             io.C = C;
             io.seg = L.seg;
