@@ -2947,54 +2947,53 @@ gsnfs_status gsnfs_render(gsnfs_ctx *ctx, void *stream, const float *d_pos, cons
     for (int c = 0; c < 3; ++c) rc.bg[c] = (float)cam->background[c];
     const uint64_t tiles = (uint64_t)rc.TX * rc.TY;
     const uint64_t m = n ? n : 1;
-    auto carve1 = [&](Carve &cv, void **sp, float **depth, int4 **rect, uint32_t **count, uint64_t **offs,
-                      uint64_t **part, uint2 **ranges) {
-        *sp = cv.take<unsigned char>(m * render_splat_bytes());
-        *depth = cv.take<float>(m);
-        *rect = cv.take<int4>(m);
-        *count = cv.take<uint32_t>(m);
-        *offs = cv.take<uint64_t>(m + 2);
-        *part = cv.take<uint64_t>(scan_partial_words(m, sms) + 1);
-        *ranges = cv.take<uint2>(tiles);
+    RenderBuffers rb;
+    uint2 *ranges;
+    auto carve1 = [&](Carve &cv) {
+        rb.splats = cv.take<unsigned char>(m * render_splat_bytes());
+        rb.depth = cv.take<uint32_t>(m);
+        rb.depth_alt = cv.take<uint32_t>(m);
+        rb.idx = cv.take<uint32_t>(m);
+        rb.idx_alt = cv.take<uint32_t>(m);
+        rb.rect = cv.take<ushort4>(m);
+        rb.count = cv.take<uint32_t>(m);
+        rb.count_sorted = cv.take<uint32_t>(m);
+        rb.offs = cv.take<uint64_t>(m + 2);
+        rb.partials = cv.take<uint64_t>(scan_partial_words(m, sms) + 1);
+        rb.hist = cv.take<uint32_t>(radix_sort_hist_words(m, sms));
+        ranges = cv.take<uint2>(tiles);
         return cv.off;
     };
-    void *sp;
-    float *depth;
-    int4 *rect;
-    uint32_t *count;
-    uint64_t *offs, *part;
-    uint2 *ranges;
     Carve m1(nullptr);
-    gsnfs_status st = grow(&ctx->rnd, &ctx->rnd_cap, carve1(m1, &sp, &depth, &rect, &count, &offs, &part, &ranges));
+    gsnfs_status st = grow(&ctx->rnd, &ctx->rnd_cap, carve1(m1));
     if (st) return st;
     Carve c1(ctx->rnd);
-    carve1(c1, &sp, &depth, &rect, &count, &offs, &part, &ranges);
+    carve1(c1);
+    const uint32_t *order = nullptr;
     uint64_t total = 0;
     if (n) {
-        launch_render_prepare(d_pos, d_attr, n, rc, sp, depth, rect, count, offs, part, sms, s);
+        launch_render_prepare(d_pos, d_attr, n, rc, rb, &order, sms, s);
         CK(cudaGetLastError());
-        CK(cudaMemcpyAsync(&total, offs + n, 8, cudaMemcpyDeviceToHost, s));
+        CK(cudaMemcpyAsync(&total, rb.offs + n, 8, cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
         if (total >= (1ull << 32)) return GSNFS_ERR_CAPACITY;
     }
     const uint64_t mt = total ? total : 1;
-    auto carve2 = [&](Carve &cv, uint64_t **k, uint32_t **v, uint64_t **ka, uint32_t **va, uint32_t **hist) {
-        *k = cv.take<uint64_t>(mt);
-        *ka = cv.take<uint64_t>(mt);
-        *v = cv.take<uint32_t>(mt);
-        *va = cv.take<uint32_t>(mt);
-        *hist = cv.take<uint32_t>(radix_sort_hist_words(mt, sms));
+    uint32_t *ltile, *ltile_alt, *lval, *lval_alt, *hist;
+    auto carve2 = [&](Carve &cv) {
+        ltile = cv.take<uint32_t>(mt);
+        ltile_alt = cv.take<uint32_t>(mt);
+        lval = cv.take<uint32_t>(mt);
+        lval_alt = cv.take<uint32_t>(mt);
+        hist = cv.take<uint32_t>(radix_sort_hist_words(mt, sms));
         return cv.off;
     };
-    uint64_t *keys, *keys_alt;
-    uint32_t *vals, *vals_alt, *hist;
     Carve m2(nullptr);
-    st = grow(&ctx->rkeys, &ctx->rkeys_cap, carve2(m2, &keys, &vals, &keys_alt, &vals_alt, &hist));
+    st = grow(&ctx->rkeys, &ctx->rkeys_cap, carve2(m2));
     if (st) return st;
     Carve c2(ctx->rkeys);
-    carve2(c2, &keys, &vals, &keys_alt, &vals_alt, &hist);
-    launch_render_tiles(n, rect, depth, count, offs, total, rc, sp, keys, vals, keys_alt, vals_alt, hist, ranges,
-                        d_image, sms, s);
+    carve2(c2);
+    launch_render_tiles(n, rb, order, total, rc, ltile, lval, ltile_alt, lval_alt, hist, ranges, d_image, sms, s);
     CK(cudaGetLastError());
     return GSNFS_OK;
 }

@@ -36,8 +36,9 @@ void launch_voxelize(const FrameSet &fs, DevState *st, uint64_t n_total, uint64_
 
 // ---- sort.cu: LSD radix sort of (key, value) over bits [0, nbits) -------
 // Returns true when the result is in (keys_alt, vals_alt).
-bool radix_sort(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt, uint32_t *hist,
-                uint64_t n, uint32_t nbits, int num_sms, cudaStream_t s);
+template <typename Key>  // uint64_t or uint32_t
+bool radix_sort(Key *keys, uint32_t *vals, Key *keys_alt, uint32_t *vals_alt, uint32_t *hist, uint64_t n,
+                uint32_t nbits, int num_sms, cudaStream_t s);
 // histogram words for n keys (room for `segments` extra CTAs of a segmented sort)
 uint64_t radix_sort_hist_words(uint64_t n, int num_sms, uint32_t segments = 0);
 // Segmented sort: segment f = elements [seg_lo[f], seg_lo[f + 1]) is sorted on its own (keys never leave it).
@@ -331,13 +332,23 @@ struct RenderCam {  // camera in FP64: the per-Gaussian projection is evaluated 
     float bg[3];
 };
 size_t render_splat_bytes();
-void launch_render_prepare(const float *pos, const float *attr, uint64_t n, const RenderCam &cam, void *splats,
-                           float *depth, int4 *rect, uint32_t *count, uint64_t *offs, uint64_t *partials,
-                           int num_sms, cudaStream_t s);
-void launch_render_tiles(uint64_t n, const int4 *rect, const float *depth, const uint32_t *count,
-                         const uint64_t *offs, uint64_t total, const RenderCam &cam, const void *splats,
-                         uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt, uint32_t *hist,
-                         uint2 *ranges, float *image, int num_sms, cudaStream_t s);
+struct RenderBuffers {  // per Gaussian
+    void *splats;
+    uint32_t *depth, *depth_alt;  // float bits of the depth: sort keys
+    uint32_t *idx, *idx_alt;      // Gaussians by (depth, index)
+    ushort4 *rect;                // tile rectangle: x0, x1, y0, y1
+    uint32_t *count;              // its tiles, and the same by (depth, index)
+    uint32_t *count_sorted;
+    uint64_t *offs;               // exclusive sums of count_sorted; offs[n] the total
+    uint64_t *partials;
+    uint32_t *hist;               // sort histograms
+};
+// projection, depth order and list offsets; *order receives the sorted Gaussian indices (idx or idx_alt)
+void launch_render_prepare(const float *pos, const float *attr, uint64_t n, const RenderCam &cam,
+                           const RenderBuffers &b, const uint32_t **order, int num_sms, cudaStream_t s);
+void launch_render_tiles(uint64_t n, const RenderBuffers &b, const uint32_t *order, uint64_t total,
+                         const RenderCam &cam, uint32_t *tiles, uint32_t *vals, uint32_t *tiles_alt,
+                         uint32_t *vals_alt, uint32_t *hist, uint2 *ranges, float *image, int num_sms, cudaStream_t s);
 
 // ---- scan.cu / api.cu helpers -------------------------------------------
 // exclusive scan of n u32 values into u64 offsets (out has n + 1 entries)

@@ -2,10 +2,11 @@
 // 3DGS forward pass, from its definition): per Gaussian, the projected mean,
 // the EWA 2-D covariance J R S S^T R^T J^T + 0.3 I and its inverse (conic),
 // a footprint square of radius ceil(3 sqrt(largest eigenvalue)), opacity
-// sigmoid(logit) and a degree-3 real-SH colour at the viewing direction; one
-// key per overlapped 16 x 16 tile, (tile << 32 | depth bits), sorted stably
-// (so a tile's list is by depth, then input index); one CTA per tile
-// composites its list front to back for its 256 pixels.  Attributes are the
+// sigmoid(logit) and a degree-3 real-SH colour at the viewing direction; the
+// Gaussians are sorted by depth, each then lists the 16 x 16 tiles it overlaps
+// and the list is sorted stably by tile (so a tile's list is by depth, then
+// input index); one CTA per tile composites its list front to back for its 256
+// pixels.  Attributes are the
 // 56-channel 3DGS rows: log-scale 0-2, rotation (w, x, y, z) 3-6, opacity
 // logit 7, SH DC RGB 8-10, SH AC 11-55 as R[15] G[15] B[15].
 //
@@ -61,10 +62,13 @@ __device__ __forceinline__ void sh_basis_d(double x, double y, double z, double 
 
 __global__ void __launch_bounds__(256) preprocess_kernel(const float *__restrict__ pos,
                                                          const float *__restrict__ attr, uint64_t n, RenderCam cam,
-                                                         Splat *sp, float *depth, int4 *rect, uint32_t *count)
+                                                         Splat *sp, uint32_t *depth, uint32_t *idx,
+                                                         ushort4 *rect, uint32_t *count)
 {
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
         count[i] = 0;
+        depth[i] = 0xFFFFFFFFu;
+        idx[i] = (uint32_t)i;
         const float *p = pos + 3 * i, *a = attr + 56 * i;
         double pc[3];
         for (int r = 0; r < 3; ++r)
@@ -142,35 +146,60 @@ __global__ void __launch_bounds__(256) preprocess_kernel(const float *__restrict
         s.b = col[2];
         s.pad = 0.f;
         sp[i] = s;
-        depth[i] = (float)z;
-        rect[i] = make_int4(tx0, tx1, ty0, ty1);
+        depth[i] = __float_as_uint((float)z);  // positive: integer order = float order
+        rect[i] = make_ushort4((unsigned short)tx0, (unsigned short)tx1, (unsigned short)ty0, (unsigned short)ty1);
         count[i] = (uint32_t)((tx1 - tx0 + 1) * (ty1 - ty0 + 1));
     }
 }
 
-__global__ void emit_kernel(uint64_t n, const int4 *rect, const float *depth, const uint32_t *count,
-                            const uint64_t *offs, int TX, uint64_t *keys, uint32_t *vals)
+__global__ void gather_counts_kernel(const uint32_t *order, const uint32_t *count, uint64_t n, uint32_t *out)
 {
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-        if (!count[i]) continue;
-        const int4 r = rect[i];
-        const uint32_t db = __float_as_uint(depth[i]);  // positive: integer order = float order
-        uint64_t o = offs[i];
-        for (int ty = r.z; ty <= r.w; ++ty)
-            for (int tx = r.x; tx <= r.y; ++tx) {
-                keys[o] = ((uint64_t)(uint32_t)(ty * TX + tx) << 32) | db;
-                vals[o] = (uint32_t)i;
-                ++o;
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
+        out[i] = count[order[i]];
+}
+
+// The tile lists, in depth order: a warp writes the tiles of 32 consecutive
+// Gaussians, whose entries are contiguous, one entry per lane (a thread per
+// Gaussian would scatter its stores over the others' ranges).
+__global__ void __launch_bounds__(256) emit_kernel(uint64_t n, const uint32_t *order, const ushort4 *rect,
+                                                   const uint64_t *offs, int TX, uint32_t *tiles, uint32_t *vals)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
+    for (uint64_t w = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w * 32 < n; w += warps) {
+        const uint64_t k = w * 32 + lane, last = w * 32 + 32 < n ? w * 32 + 32 : n;
+        const uint64_t base = offs[w * 32], total = offs[last] - base;
+        if (total == 0) continue;
+        const uint32_t i = k < n ? order[k] : 0u;
+        const uint64_t off = (k < n ? offs[k] : offs[n]) - base;
+        const ushort4 r = k < n ? rect[i] : make_ushort4(0, 0, 0, 0);
+        const uint32_t xs = r.x | ((uint32_t)r.y << 16), y0 = r.z;
+        for (uint64_t e0 = 0; e0 < total; e0 += 32) {
+            const uint64_t e = e0 + lane;
+            uint32_t g = 0;  // the last Gaussian that starts at or before entry e
+#pragma unroll
+            for (uint32_t st = 16; st; st >>= 1) {
+                const uint64_t o = __shfl_sync(0xFFFFFFFFu, off, g + st);  // g + st < 32
+                if (o <= e) g += st;
             }
+            const uint32_t rel = (uint32_t)(e - __shfl_sync(0xFFFFFFFFu, off, g));
+            const uint32_t gxs = __shfl_sync(0xFFFFFFFFu, xs, g), gy = __shfl_sync(0xFFFFFFFFu, y0, g);
+            const uint32_t gi = __shfl_sync(0xFFFFFFFFu, i, g);
+            const uint32_t x0 = gxs & 0xFFFFu, width = (gxs >> 16) - x0 + 1u, row = rel / width;
+            if (e < total) {
+                tiles[base + e] = (gy + row) * (uint32_t)TX + x0 + (rel - row * width);
+                vals[base + e] = gi;
+            }
+        }
     }
 }
 
-__global__ void ranges_kernel(const uint64_t *keys, uint64_t total, uint2 *ranges)
+__global__ void ranges_kernel(const uint32_t *tiles, uint64_t total, uint2 *ranges)
 {
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (uint64_t)gridDim.x * blockDim.x) {
-        const uint32_t tile = (uint32_t)(keys[i] >> 32);
-        if (i == 0 || (uint32_t)(keys[i - 1] >> 32) != tile) ranges[tile].x = (uint32_t)i;
-        if (i + 1 == total || (uint32_t)(keys[i + 1] >> 32) != tile) ranges[tile].y = (uint32_t)(i + 1);
+        const uint32_t tile = tiles[i];
+        if (i == 0 || tiles[i - 1] != tile) ranges[tile].x = (uint32_t)i;
+        if (i + 1 == total || tiles[i + 1] != tile) ranges[tile].y = (uint32_t)(i + 1);
     }
 }
 
@@ -226,36 +255,40 @@ uint32_t rgrid(uint64_t n, int num_sms)
 
 size_t render_splat_bytes() { return sizeof(Splat); }
 
-void launch_render_prepare(const float *pos, const float *attr, uint64_t n, const RenderCam &cam, void *splats,
-                           float *depth, int4 *rect, uint32_t *count, uint64_t *offs, uint64_t *partials,
-                           int num_sms, cudaStream_t s)
+void launch_render_prepare(const float *pos, const float *attr, uint64_t n, const RenderCam &cam,
+                           const RenderBuffers &b, const uint32_t **order, int num_sms, cudaStream_t s)
 {
-    preprocess_kernel<<<rgrid(n, num_sms), 256, 0, s>>>(pos, attr, n, cam, (Splat *)splats, depth, rect, count);
+    preprocess_kernel<<<rgrid(n, num_sms), 256, 0, s>>>(pos, attr, n, cam, (Splat *)b.splats, b.depth, b.idx, b.rect,
+                                                        b.count);
     count_launch();
-    launch_scan_u32_to_u64(count, n, offs, partials, num_sms, s);
+    // Depth first, over the Gaussians; then only the tile bits over the many times longer list of their tiles.
+    // Sorting that list by (tile, depth) at once took six passes of 12-byte pairs, 3.3 ms of 6.6 with the emission at
+    // 1M Gaussians and 960 x 540 (24M entries); the whole call is 4.6 ms this way.
+    const bool alt = radix_sort(b.depth, b.idx, b.depth_alt, b.idx_alt, b.hist, n, 32u, num_sms, s);
+    *order = alt ? b.idx_alt : b.idx;
+    gather_counts_kernel<<<rgrid(n, num_sms), 256, 0, s>>>(*order, b.count, n, b.count_sorted);
+    count_launch();
+    launch_scan_u32_to_u64(b.count_sorted, n, b.offs, b.partials, num_sms, s);
 }
 
-void launch_render_tiles(uint64_t n, const int4 *rect, const float *depth, const uint32_t *count,
-                         const uint64_t *offs, uint64_t total, const RenderCam &cam, const void *splats,
-                         uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt, uint32_t *hist,
-                         uint2 *ranges, float *image, int num_sms, cudaStream_t s)
+void launch_render_tiles(uint64_t n, const RenderBuffers &b, const uint32_t *order, uint64_t total,
+                         const RenderCam &cam, uint32_t *tiles, uint32_t *vals, uint32_t *tiles_alt,
+                         uint32_t *vals_alt, uint32_t *hist, uint2 *ranges, float *image, int num_sms, cudaStream_t s)
 {
-    const uint32_t tiles = (uint32_t)(cam.TX * cam.TY);
-    dev_memset(ranges, 0, sizeof(uint2) * tiles, s);
+    const uint32_t ntiles = (uint32_t)(cam.TX * cam.TY);
+    dev_memset(ranges, 0, sizeof(uint2) * ntiles, s);
+    const uint32_t *sv = vals;
     if (total) {
-        emit_kernel<<<rgrid(n, num_sms), 256, 0, s>>>(n, rect, depth, count, offs, cam.TX, keys, vals);
+        emit_kernel<<<rgrid(n, num_sms), 256, 0, s>>>(n, order, b.rect, b.offs, cam.TX, tiles, vals);
         count_launch();
         uint32_t tb = 0;
-        while ((1u << tb) < tiles) ++tb;
-        const bool alt = radix_sort(keys, vals, keys_alt, vals_alt, hist, total, 32 + tb, num_sms, s);
-        const uint64_t *sk = alt ? keys_alt : keys;
-        const uint32_t *sv = alt ? vals_alt : vals;
-        ranges_kernel<<<rgrid(total, num_sms), 256, 0, s>>>(sk, total, ranges);
+        while ((1u << tb) < ntiles) ++tb;
+        const bool alt = radix_sort(tiles, vals, tiles_alt, vals_alt, hist, total, tb, num_sms, s);
+        if (alt) sv = vals_alt;
+        ranges_kernel<<<rgrid(total, num_sms), 256, 0, s>>>(alt ? tiles_alt : tiles, total, ranges);
         count_launch();
-        render_kernel<<<dim3(cam.TX, cam.TY), 256, 0, s>>>(ranges, sv, (const Splat *)splats, cam, image);
-    } else {
-        render_kernel<<<dim3(cam.TX, cam.TY), 256, 0, s>>>(ranges, vals, (const Splat *)splats, cam, image);
     }
+    render_kernel<<<dim3(cam.TX, cam.TY), 256, 0, s>>>(ranges, sv, (const Splat *)b.splats, cam, image);
     count_launch();
 }
 

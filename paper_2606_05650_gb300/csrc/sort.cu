@@ -1,5 +1,6 @@
 // LSD radix sort of (64-bit Morton key, 32-bit point index) pairs
-// (Algorithm 1: "RadixSort" of the Morton codes).  Only the 3J significant
+// (Algorithm 1: "RadixSort" of the Morton codes), and of pairs with 32-bit
+// keys (the rasteriser's depths and tiles).  Only the 3J significant
 // key bits are sorted, 8 bits per pass; the frames of a batch, which arrive
 // grouped, are sorted as separate segments so that their id bits need no pass.
 //
@@ -51,7 +52,8 @@ __device__ __forceinline__ void cta_range(const uint64_t *cta_lo, uint64_t chunk
     }
 }
 
-__global__ void __launch_bounds__(kThreads) upsweep_kernel(const uint64_t *__restrict__ keys, uint64_t n,
+template <typename Key>
+__global__ void __launch_bounds__(kThreads) upsweep_kernel(const Key *__restrict__ keys, uint64_t n,
                                                            uint32_t shift, uint64_t chunk, uint32_t *hist,
                                                            const uint64_t *__restrict__ cta_lo)
 {
@@ -82,11 +84,12 @@ __global__ void __launch_bounds__(256) scan_cols_kernel(uint32_t *hist, uint32_t
     if (lane == 0) hist[(uint64_t)kRadix * P + d] = run;
 }
 
-__global__ void __launch_bounds__(kThreads, kCtasPerSm) downsweep_kernel(const uint64_t *__restrict__ keys,
+template <typename Key>
+__global__ void __launch_bounds__(kThreads, kCtasPerSm) downsweep_kernel(const Key *__restrict__ keys,
                                                              const uint32_t *__restrict__ vals, uint64_t n,
                                                              uint32_t shift, uint64_t chunk,
                                                              const uint32_t *__restrict__ hist,
-                                                             uint64_t *__restrict__ keys_out,
+                                                             Key *__restrict__ keys_out,
                                                              uint32_t *__restrict__ vals_out,
                                                              const uint64_t *__restrict__ cta_lo,
                                                              const uint32_t *__restrict__ cta_seg)
@@ -94,7 +97,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) downsweep_kernel(const u
     __shared__ uint32_t s_base[kRadix];
     __shared__ uint32_t s_wcnt[kWarps][kRadix];
     __shared__ uint32_t s_toff[kRadix];
-    __shared__ uint64_t s_keys[kTile];
+    __shared__ Key s_keys[kTile];
     __shared__ uint32_t s_vals[kTile];
     __shared__ uint32_t s_scan[33];
 
@@ -122,14 +125,14 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) downsweep_kernel(const u
     for (int ww = 0; ww < kWarps; ++ww) s_wcnt[ww][tid] = 0;
     __syncthreads();
     for (uint64_t t0 = cb; t0 < ce; t0 += kTile) {
-        uint64_t k[kKeysPerThread];
+        Key k[kKeysPerThread];
         uint32_t v[kKeysPerThread], rk[kKeysPerThread];
         uint32_t dg[kKeysPerThread];
 #pragma unroll
         for (int r = 0; r < kKeysPerThread; ++r) {
             uint64_t p = t0 + (uint64_t)w * (32 * kKeysPerThread) + (uint64_t)r * 32 + lane;
             bool ok = p < ce;
-            k[r] = ok ? keys[p] : 0ull;
+            k[r] = ok ? keys[p] : Key(0);
             v[r] = ok ? vals[p] : 0u;
             uint32_t d = ok ? (uint32_t)((k[r] >> shift) & 0xFF) : (kRadix + lane);
             dg[r] = d;
@@ -171,7 +174,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) downsweep_kernel(const u
         for (int ww = 0; ww < kWarps; ++ww) s_wcnt[ww][tid] = 0;
         uint32_t cnt = (uint32_t)((ce - t0) < (uint64_t)kTile ? (ce - t0) : (uint64_t)kTile);
         for (uint32_t slot = tid; slot < cnt; slot += kThreads) {
-            uint64_t key = s_keys[slot];
+            const Key key = s_keys[slot];
             uint32_t d = (uint32_t)((key >> shift) & 0xFF);
             uint64_t op = (uint64_t)s_base[d] + (slot - s_toff[d]);
             keys_out[op] = key;
@@ -208,11 +211,12 @@ uint32_t radix_sort_segment_table(const uint64_t *seg_lo, uint32_t segments, int
     return P;
 }
 
-static bool sort_passes(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt, uint32_t *hist,
+template <typename Key>
+static bool sort_passes(Key *keys, uint32_t *vals, Key *keys_alt, uint32_t *vals_alt, uint32_t *hist,
                         uint64_t n, uint32_t nbits, uint32_t P, uint64_t chunk, const uint64_t *cta_lo,
                         const uint32_t *cta_seg, cudaStream_t s)
 {
-    uint64_t *ki = keys, *ko = keys_alt;
+    Key *ki = keys, *ko = keys_alt;
     uint32_t *vi = vals, *vo = vals_alt;
     bool flipped = false;
     for (uint32_t shift = 0; shift < nbits; shift += 8) {
@@ -222,7 +226,7 @@ static bool sort_passes(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint
         count_launch();
         downsweep_kernel<<<P, kThreads, 0, s>>>(ki, vi, n, shift, chunk, hist, ko, vo, cta_lo, cta_seg);
         count_launch();
-        uint64_t *tk = ki;
+        Key *tk = ki;
         ki = ko;
         ko = tk;
         uint32_t *tv = vi;
@@ -233,13 +237,18 @@ static bool sort_passes(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint
     return flipped;
 }
 
-bool radix_sort(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt, uint32_t *hist,
-                uint64_t n, uint32_t nbits, int num_sms, cudaStream_t s)
+template <typename Key>
+bool radix_sort(Key *keys, uint32_t *vals, Key *keys_alt, uint32_t *vals_alt, uint32_t *hist, uint64_t n,
+                uint32_t nbits, int num_sms, cudaStream_t s)
 {
     if (n <= 1 || nbits == 0) return false;
     const SortGeom g = sort_geom(n, num_sms);
     return sort_passes(keys, vals, keys_alt, vals_alt, hist, n, nbits, g.P, g.chunk, nullptr, nullptr, s);
 }
+template bool radix_sort<uint64_t>(uint64_t *, uint32_t *, uint64_t *, uint32_t *, uint32_t *, uint64_t, uint32_t, int,
+                                   cudaStream_t);
+template bool radix_sort<uint32_t>(uint32_t *, uint32_t *, uint32_t *, uint32_t *, uint32_t *, uint64_t, uint32_t, int,
+                                   cudaStream_t);
 
 bool radix_sort_segments(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt, uint32_t *hist,
                          uint64_t n, uint32_t nbits, uint32_t ctas, const uint64_t *cta_lo, const uint32_t *cta_seg,
