@@ -32,7 +32,7 @@ struct Splat {
     float u, ulo, v, vlo;  // projected centre as hi + lo
     float l1, l2, l3;      // Cholesky factor of the conic
     float opacity, r, g, b;
-    float pad;
+    uint32_t reach;        // pixels from the centre, in x and (upper half) in y, past which alpha stays below the cut
 };
 
 __device__ __forceinline__ void sh_basis_d(double x, double y, double z, double Y[16])
@@ -113,8 +113,23 @@ __global__ void __launch_bounds__(256) preprocess_kernel(const float *__restrict
         const double lmax = mid + sqrt(disc > 0.1 ? disc : 0.1);
         const double rad = ceil(3.0 * sqrt(lmax));
         const double u = cam.fx * pc[0] / z + cam.cx, v = cam.fy * pc[1] / z + cam.cy;
-        int tx0 = (int)floor((u - rad) / kTile), tx1 = (int)floor((u + rad) / kTile);
-        int ty0 = (int)floor((v - rad) / kTile), ty1 = (int)floor((v + rad) / kTile);
+        const float opacity = (float)(1.0 / (1.0 + exp(-(double)a[7])));
+        // Past |d_x| = sqrt(c cov_xx) the exponent d^T conic d is above c whatever d_y is, so with
+        // c = 2 ln(255 opacity) alpha stays below 1/255 there and the splat changes no pixel; likewise in y.  The
+        // margins cover the FP32 rounding of the per-pixel exponent, whose relative error grows with
+        // cov_xx cov_yy / det (1e-7 sqrt(of it)): very elongated footprints keep the square of radius rad alone.
+        double rx = rad, ry = rad;
+        float reach_x = 65535.f, reach_y = 65535.f;
+        if (ca * cc < 1e8 * det) {
+            if (opacity * 255.f < 0.9999f) continue;
+            const float c = 2.04f * fmaxf(logf(opacity * 255.f), 0.f) + 0.1f;
+            reach_x = sqrtf(c * (float)ca) * 1.0001f;
+            reach_y = sqrtf(c * (float)cc) * 1.0001f;
+            rx = fmin(rad, (double)reach_x);
+            ry = fmin(rad, (double)reach_y);
+        }
+        int tx0 = (int)floor((u - rx) / kTile), tx1 = (int)floor((u + rx) / kTile);
+        int ty0 = (int)floor((v - ry) / kTile), ty1 = (int)floor((v + ry) / kTile);
         tx0 = max(tx0, 0);
         ty0 = max(ty0, 0);
         tx1 = min(tx1, cam.TX - 1);
@@ -128,7 +143,7 @@ __global__ void __launch_bounds__(256) preprocess_kernel(const float *__restrict
         s.l1 = (float)l1;
         s.l2 = (float)l2;
         s.l3 = (float)l3;
-        s.opacity = (float)(1.0 / (1.0 + exp(-(double)a[7])));
+        s.opacity = opacity;
         double d[3] = {(double)p[0] - cam.campos[0], (double)p[1] - cam.campos[1], (double)p[2] - cam.campos[2]};
         const double dn = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
         const double id = dn > 0.0 ? 1.0 / dn : 1.0;
@@ -144,7 +159,7 @@ __global__ void __launch_bounds__(256) preprocess_kernel(const float *__restrict
         s.r = col[0];
         s.g = col[1];
         s.b = col[2];
-        s.pad = 0.f;
+        s.reach = (uint32_t)fminf(ceilf(reach_x) + 1.f, 65535.f) | ((uint32_t)fminf(ceilf(reach_y) + 1.f, 65535.f) << 16);
         sp[i] = s;
         depth[i] = __float_as_uint((float)z);  // positive: integer order = float order
         rect[i] = make_ushort4((unsigned short)tx0, (unsigned short)tx1, (unsigned short)ty0, (unsigned short)ty1);
@@ -203,43 +218,84 @@ __global__ void ranges_kernel(const uint32_t *tiles, uint64_t total, uint2 *rang
     }
 }
 
-// one CTA per tile, thread per pixel; the tile's splats in batches of 256 through shared memory
+__device__ __forceinline__ void copy16(void *smem, const void *gmem)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem)
+                 : "memory");
+}
+
+// One CTA per tile, a thread per pixel, a warp per 8 x 4 pixels; the tile's
+// splats in batches of 256 through shared memory, the next batch landing while
+// one is composited.  A warp first finds, a splat per lane, which of 32 splats
+// reach its pixels (Splat::reach), then composites those in order: most of a
+// tile's list does not reach a given 8 x 4 block, and the skipped ones would
+// have failed the alpha cut at every pixel, so the image is the same.  With the
+// tile rectangles cut to the reach as well: 1M Gaussians at 960 x 540
+// 4.6 -> 2.9 ms (a thread per pixel evaluating its tile's whole list before).
+constexpr int kBatch = 256;
+
 __global__ void __launch_bounds__(256) render_kernel(const uint2 *ranges, const uint32_t *vals, const Splat *sp,
                                                      RenderCam cam, float *image)
 {
-    __shared__ Splat batch[256];
-    const int tx = blockIdx.x, ty = blockIdx.y;
-    const int lx = threadIdx.x & 15, ly = threadIdx.x >> 4;
-    const int px = tx * kTile + lx, py = ty * kTile + ly;
+    static_assert(sizeof(Splat) == 48, "copied in 16-byte words");
+    __shared__ __align__(16) Splat batch[2][kBatch];
+    const int tx = blockIdx.x, ty = blockIdx.y, t = threadIdx.x;
+    const uint32_t lane = t & 31, w = t >> 5;
+    const int bx = tx * kTile + (int)(w & 1) * 8, by = ty * kTile + (int)(w >> 1) * 4;  // the warp's block
+    const int px = bx + (int)(lane & 7), py = by + (int)(lane >> 3);
+    const float mx = bx + 4.f, my = by + 2.f;  // its centre
     const bool inside = px < cam.W && py < cam.H;
     const uint2 rg = ranges[ty * cam.TX + tx];
     const float fxp = px + 0.5f, fyp = py + 0.5f;
     float T = 1.f, col[3] = {0.f, 0.f, 0.f};
     bool done = !inside;
-    for (uint32_t b0 = rg.x; b0 < rg.y; b0 += 256) {
+    auto fetch = [&](uint32_t b0, uint32_t val) {  // splat `val` of the batch at b0
+        if (b0 + t < rg.y) {
+            Splat *d = &batch[((b0 - rg.x) / kBatch) & 1][t];
+            const char *q = reinterpret_cast<const char *>(sp + val);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) copy16(reinterpret_cast<char *>(d) + 16 * k, q + 16 * k);
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    auto val_at = [&](uint32_t b0) { return b0 < rg.y && b0 + t < rg.y ? vals[b0 + t] : 0u; };
+    fetch(rg.x, val_at(rg.x));
+    uint32_t next = val_at(rg.x + kBatch);
+    for (uint32_t b0 = rg.x; b0 < rg.y; b0 += kBatch) {
+        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
         if (__syncthreads_count(done ? 0 : 1) == 0) break;  // every pixel of the tile has finished
-        const uint32_t k = b0 + threadIdx.x;
-        if (k < rg.y) batch[threadIdx.x] = sp[vals[k]];
-        __syncthreads();
-        const uint32_t cnt = (rg.y - b0) < 256u ? (rg.y - b0) : 256u;
-        for (uint32_t j = 0; j < cnt && !done; ++j) {
-            const Splat s = batch[j];
-            const float dx = (s.u - fxp) + s.ulo, dy = (s.v - fyp) + s.vlo;
-            const float e0 = fmaf(s.l1, dx, s.l2 * dy), e1 = s.l3 * dy;
-            const float power = -0.5f * fmaf(e0, e0, e1 * e1);
-            const float alpha = fminf(0.99f, s.opacity * expf(power));
-            if (alpha < 1.f / 255.f) continue;
-            const float tn = T * (1.f - alpha);
-            if (tn < 1e-4f) {
-                done = true;
-                break;
+        fetch(b0 + kBatch, next);  // over the batch before this one
+        next = val_at(b0 + 2 * kBatch);
+        const Splat *B = batch[((b0 - rg.x) / kBatch) & 1];
+        const uint32_t cnt = (rg.y - b0) < (uint32_t)kBatch ? (rg.y - b0) : (uint32_t)kBatch;
+        for (uint32_t j0 = 0; j0 < cnt; j0 += 32) {
+            if (__all_sync(0xFFFFFFFFu, done)) break;
+            bool hit = false;
+            if (j0 + lane < cnt) {
+                const Splat &s = B[j0 + lane];
+                hit = fabsf(s.u - mx) <= (float)(s.reach & 0xFFFFu) + 4.f && fabsf(s.v - my) <= (float)(s.reach >> 16) + 2.f;
             }
-            col[0] += s.r * alpha * T;
-            col[1] += s.g * alpha * T;
-            col[2] += s.b * alpha * T;
-            T = tn;
+            for (uint32_t m = __ballot_sync(0xFFFFFFFFu, hit); m; m &= m - 1) {
+                if (done) continue;
+                const Splat &s = B[j0 + __ffs(m) - 1];
+                const float dx = (s.u - fxp) + s.ulo, dy = (s.v - fyp) + s.vlo;
+                const float e0 = fmaf(s.l1, dx, s.l2 * dy), e1 = s.l3 * dy;
+                const float power = -0.5f * fmaf(e0, e0, e1 * e1);
+                const float alpha = fminf(0.99f, s.opacity * expf(power));
+                if (alpha < 1.f / 255.f) continue;
+                const float tn = T * (1.f - alpha);
+                if (tn < 1e-4f) {
+                    done = true;
+                    continue;
+                }
+                col[0] += s.r * alpha * T;
+                col[1] += s.g * alpha * T;
+                col[2] += s.b * alpha * T;
+                T = tn;
+            }
         }
     }
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     if (inside)
         for (int c = 0; c < 3; ++c) image[((uint64_t)py * cam.W + px) * 3 + c] = col[c] + T * cam.bg[c];
 }
@@ -263,7 +319,7 @@ void launch_render_prepare(const float *pos, const float *attr, uint64_t n, cons
     count_launch();
     // Depth first, over the Gaussians; then only the tile bits over the many times longer list of their tiles.
     // Sorting that list by (tile, depth) at once took six passes of 12-byte pairs, 3.3 ms of 6.6 with the emission at
-    // 1M Gaussians and 960 x 540 (24M entries); the whole call is 4.6 ms this way.
+    // 1M Gaussians and 960 x 540 (24M entries); the whole call was 4.6 ms this way.
     const bool alt = radix_sort(b.depth, b.idx, b.depth_alt, b.idx_alt, b.hist, n, 32u, num_sms, s);
     *order = alt ? b.idx_alt : b.idx;
     gather_counts_kernel<<<rgrid(n, num_sms), 256, 0, s>>>(*order, b.count, n, b.count_sorted);
