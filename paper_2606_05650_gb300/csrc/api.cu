@@ -327,28 +327,68 @@ gsnfs_status stream_wait(gsnfs_ctx *ctx, cudaStream_t waiter, cudaStream_t from)
 // Small transfers between the pinned staging buffer and the device (a call's
 // parameters and results) run as a kernel over the staging buffer's unified
 // address instead of on the copy engines, so they never queue behind a
-// caller's bulk copies in flight on other streams.
-__global__ void stage_copy_kernel(unsigned char *dst, const unsigned char *src, uint64_t n)
+// caller's bulk copies in flight on other streams.  A call's transfers that
+// are ready together go in one launch (a null source fills with zeros): each
+// launch of a small frame's chain costs 2.5 us, and a call has a dozen.
+struct CopyList {
+    static constexpr uint32_t kMax = 16;
+    struct Item {
+        unsigned char *dst;
+        const unsigned char *src;
+        uint64_t n;
+    } item[kMax];
+    uint32_t count;
+};
+
+__global__ void __launch_bounds__(256) stage_copy_kernel(CopyList l)
 {
+    const CopyList::Item c = l.item[blockIdx.y];
     const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (uint64_t)gridDim.x * blockDim.x;
-    if ((((uintptr_t)dst | (uintptr_t)src | n) & 3) == 0) {
-        uint32_t *d = reinterpret_cast<uint32_t *>(dst);
-        const uint32_t *q = reinterpret_cast<const uint32_t *>(src);
-        for (uint64_t i = t; i < n / 4; i += nt) d[i] = q[i];
+    if ((((uintptr_t)c.dst | (uintptr_t)c.src | c.n) & 3) == 0) {
+        uint32_t *d = reinterpret_cast<uint32_t *>(c.dst);
+        const uint32_t *q = reinterpret_cast<const uint32_t *>(c.src);
+        for (uint64_t i = t; i < c.n / 4; i += nt) d[i] = q ? q[i] : 0u;
     } else {
-        for (uint64_t i = t; i < n; i += nt) dst[i] = src[i];
+        for (uint64_t i = t; i < c.n; i += nt) c.dst[i] = c.src ? c.src[i] : (unsigned char)0;
     }
 }
 
+class StageCopies {
+public:
+    explicit StageCopies(cudaStream_t s) : s_(s) { l_.count = 0; }
+    cudaError_t add(void *dst, const void *src, size_t n)
+    {
+        if (n == 0) return cudaSuccess;
+        if (l_.count == CopyList::kMax) {
+            const cudaError_t e = flush();
+            if (e != cudaSuccess) return e;
+        }
+        l_.item[l_.count++] = {static_cast<unsigned char *>(dst), static_cast<const unsigned char *>(src), n};
+        longest_ = std::max<uint64_t>(longest_, n);
+        return cudaSuccess;
+    }
+    cudaError_t flush()
+    {
+        if (!l_.count) return cudaSuccess;
+        const uint64_t blocks = std::min<uint64_t>((longest_ / 4 + 255) / 256, 128);
+        stage_copy_kernel<<<dim3((uint32_t)std::max<uint64_t>(blocks, 1), l_.count), 256, 0, s_>>>(l_);
+        count_launch();
+        l_.count = 0;
+        longest_ = 0;
+        return cudaGetLastError();
+    }
+
+private:
+    cudaStream_t s_;
+    CopyList l_;
+    uint64_t longest_ = 0;
+};
+
 cudaError_t stage_copy(void *dst, const void *src, size_t n, cudaStream_t s)
 {
-    if (n == 0) return cudaSuccess;
-    const uint64_t words = (n + 3) / 4;
-    const uint32_t blocks = (uint32_t)std::min<uint64_t>((words + 255) / 256, 128);
-    stage_copy_kernel<<<blocks, 256, 0, s>>>(static_cast<unsigned char *>(dst), static_cast<const unsigned char *>(src),
-                                             n);
-    count_launch();
-    return cudaGetLastError();
+    StageCopies c(s);
+    c.add(dst, src, n);
+    return c.flush();
 }
 
 __host__ __device__ inline uint64_t pad8(uint64_t x) { return (x + 7) & ~7ull; }
@@ -1011,21 +1051,24 @@ gsnfs_status encode_impl(gsnfs_ctx *ctx, cudaStream_t s, EncodeReq &rq, bool wor
     // ---- device work: stream-ordered and sized from host values only, so it
     // can be captured once per request shape and replayed as a CUDA graph
     auto enqueue = [&](cudaStream_t s) -> gsnfs_status {
-        CK(stage_copy((void *)L.posp, hp + o_pos, 8 * F, s));
-        CK(stage_copy((void *)L.attrp, hp + o_attr, 8 * F, s));
-        CK(stage_copy(L.poff, hp + o_poff, 8 * (F + 1), s));
-        CK(stage_copy(L.Jd, hp + o_J, 4 * F, s));
+        StageCopies up(s);
+        CK(up.add((void *)L.posp, hp + o_pos, 8 * F));
+        CK(up.add((void *)L.attrp, hp + o_attr, 8 * F));
+        CK(up.add(L.poff, hp + o_poff, 8 * (F + 1)));
+        CK(up.add(L.Jd, hp + o_J, 4 * F));
         if (C) {
-            CK(stage_copy(L.inv_step, hp + o_inv, 4 * (size_t)R * C, s));
-            CK(stage_copy(L.step, hp + o_step, 4 * (size_t)R * C, s));
-            CK(stage_copy(L.steps_rg, hp + o_srg, 8 * (size_t)R * G, s));
-            CK(stage_copy(L.groups, hp + o_grp, C, s));
+            CK(up.add(L.inv_step, hp + o_inv, 4 * (size_t)R * C));
+            CK(up.add(L.step, hp + o_step, 4 * (size_t)R * C));
+            CK(up.add(L.steps_rg, hp + o_srg, 8 * (size_t)R * G));
+            CK(up.add(L.groups, hp + o_grp, C));
         }
         if (sort_ctas) {
-            CK(stage_copy(L.cta_lo, hp + o_ctalo, 8 * ((size_t)sort_ctas + 1), s));
-            CK(stage_copy(L.cta_seg, hp + o_ctaseg, 8 * (size_t)sort_ctas, s));
+            CK(up.add(L.cta_lo, hp + o_ctalo, 8 * ((size_t)sort_ctas + 1)));
+            CK(up.add(L.cta_seg, hp + o_ctaseg, 8 * (size_t)sort_ctas));
         }
-        CK(dev_memset(L.overflow, 0, 16, s));
+        CK(up.add(L.overflow, nullptr, 16));
+        if (rq.dist) CK(up.add(L.sq_err, nullptr, 8 * (size_t)F * R * C));
+        CK(up.flush());
 
         DevState *dst = ctx->st;
         const int sms = ctx->num_sms;
@@ -1121,7 +1164,6 @@ gsnfs_status encode_impl(gsnfs_ctx *ctx, cudaStream_t s, EncodeReq &rq, bool wor
             j.overflow = L.overflow;
             j.dc = L.dc;
             if (rq.dist) {
-                CK(dev_memset(L.sq_err, 0, 8 * (size_t)F * R * C, sa));
                 j.sq_err = L.sq_err;
                 j.step = L.step;
             }
@@ -1181,10 +1223,12 @@ gsnfs_status encode_impl(gsnfs_ctx *ctx, cudaStream_t s, EncodeReq &rq, bool wor
         stage_end(s, kStRecon);
         CK(cudaGetLastError());
         // results
-        CK(stage_copy(res, &dst->err, 8, s));
-        CK(stage_copy(res + 1, &dst->nv_total, 16, s));
-        CK(stage_copy(res + 3, L.overflow, 4, s));
-        if (dist_bytes) CK(stage_copy(hp + o_dist, L.sq_err, dist_bytes, s));
+        StageCopies down(s);
+        CK(down.add(res, &dst->err, 8));
+        CK(down.add(res + 1, &dst->nv_total, 16));
+        CK(down.add(res + 3, L.overflow, 4));
+        CK(down.add(hp + o_dist, L.sq_err, dist_bytes));
+        CK(down.flush());
         return GSNFS_OK;
     };
     std::vector<Profiler::Rec> gstages;  // the replayed graph's stage events
@@ -1342,19 +1386,32 @@ gsnfs_status parse_sections(const uint8_t *occ_hdr, const uint8_t *attr_hdr, Par
 
 gsnfs_status read_headers(gsnfs_ctx *ctx, cudaStream_t s, const uint8_t *d_in, uint64_t bytes, ParsedHeader &P)
 {
-    gsnfs_status st = grow_pinned(ctx, 8192);
+    gsnfs_status st = grow_pinned(ctx, 2 * 8192);
     if (st) return st;
     CK(cudaStreamSynchronize(s));
     uint8_t *hp = ctx->pinned;
     if (bytes < 96) return GSNFS_ERR_CORRUPT;
-    CK(stage_copy(hp, d_in, 96, s));
+    // the stream's header record in one launch and one wait
+    RecLaunch a;
+    a.in = d_in;
+    a.rec = hp;
+    a.stride = 8192;
+    a.f0 = 0;
+    a.off[0] = 0;
+    a.off[1] = bytes;
+    stream_records_kernel<<<1, 256, 0, s>>>(a);
+    count_launch();
+    CK(cudaGetLastError());
     CK(cudaStreamSynchronize(s));
     st = parse_fixed(hp, bytes, P);
     if (st) return st;
-    CK(stage_copy(hp, d_in, P.hb, s));
-    CK(stage_copy(hp + 4096, d_in + P.hb, 24, s));
-    if (P.attr_bytes >= 8) CK(stage_copy(hp + 4096 + 64, d_in + P.hb + P.occ_bytes, 8, s));
-    CK(cudaStreamSynchronize(s));
+    if (P.hb > 4096) {  // a record leaves out the sections' heads then
+        StageCopies heads(s);
+        CK(heads.add(hp + 4096, d_in + P.hb, 24));
+        if (P.attr_bytes >= 8) CK(heads.add(hp + 4096 + 64, d_in + P.hb + P.occ_bytes, 8));
+        CK(heads.flush());
+        CK(cudaStreamSynchronize(s));
+    }
     st = parse_tables(hp, P);
     if (st) return st;
     return parse_sections(hp + 4096, hp + 4096 + 64, P);
@@ -1445,12 +1502,14 @@ gsnfs_status decode_impl(gsnfs_ctx *ctx, cudaStream_t s, const uint8_t *d_in, ui
     const uint32_t vst_h[2] = {0u, (uint32_t)P.nv};
     memcpy(hp + 192, vst_h, 8);
     for (uint32_t c = 0; c < P.C; ++c) ((float *)(hp + 256))[c] = (float)P.steps[P.groups[c]];
-    CK(stage_copy(L.grid, hp, sizeof(g), s));
-    CK(stage_copy(L.nvdev, hp + 128, 8, s));
-    CK(stage_copy(L.vst, hp + 192, 8, s));
-    if (P.color) CK(stage_copy(L.klt, d_in + P.klt_off, 4 * kKltFloats, s));
-    if (P.C) CK(stage_copy(L.step, hp + 256, 4 * P.C, s));
-    CK(dev_memset(dst, 0, 8, s));
+    StageCopies up(s);
+    CK(up.add(L.grid, hp, sizeof(g)));
+    CK(up.add(L.nvdev, hp + 128, 8));
+    CK(up.add(L.vst, hp + 192, 8));
+    if (P.color) CK(up.add(L.klt, d_in + P.klt_off, 4 * kKltFloats));
+    if (P.C) CK(up.add(L.step, hp + 256, 4 * P.C));
+    CK(up.add(dst, nullptr, 8));
+    CK(up.flush());
     const int sms = ctx->num_sms;
     // a12's RLGR decode needs only the block tables: it runs on s beside a11 and the schedule (the longer
     // branch), which run on the context's high-priority stream sg and take the RLGR branch's results last
@@ -1627,8 +1686,10 @@ gsnfs_status lod_from_voxels(gsnfs_ctx *ctx, cudaStream_t s, cudaStream_t cs, co
         if (fst) return fst;
     }
     uint32_t *hres = reinterpret_cast<uint32_t *>(ctx->pinned + 1024);
-    CK(stage_copy(hres, &dst->err, 4, cs));
-    if (room) CK(stage_copy(hn, offs + nv, 8, cs));
+    StageCopies down(cs);
+    CK(down.add(hres, &dst->err, 4));
+    if (room) CK(down.add(hn, offs + nv, 8));
+    CK(down.flush());
     CK(cudaStreamSynchronize(cs));
     if (room) *lod.out_nodes = *hn;
     return map_dev_error(hres[0]);
@@ -1903,22 +1964,24 @@ gsnfs_status decode_batch_impl(gsnfs_ctx *ctx, cudaStream_t s, uint32_t F, const
         level_tiles[lv] = run;
     }
     memcpy(tp + o_nv, &N, 8);
-    CK(stage_copy(L.fr, tp + o_fr, sizeof(DecFrame) * F, s));
-    CK(stage_copy(L.vstart, tp + o_vs, 4 * (F + 1), s));
-    CK(stage_copy(L.lvl_pref, tp + o_lp, 8 * (size_t)(Jmax + 1) * (F + 1), s));
-    CK(stage_copy(L.job_off, tp + o_jo, 8 * (F + 1), s));
-    CK(stage_copy(L.blk_pref, tp + o_bp, 8 * (F + 1), s));
-    CK(stage_copy(L.nvdev, tp + o_nv, 8, s));
-    if (Jmax) CK(stage_copy(L.tile_pref, tp + o_tp, 4 * (size_t)Jmax * (F + 1), s));
-    if (C) CK(stage_copy(L.steps, tp + o_st, 4 * (size_t)F * C, s));
+    DevState *dst = ctx->st;
+    StageCopies up(s);
+    CK(up.add(L.fr, tp + o_fr, sizeof(DecFrame) * F));
+    CK(up.add(L.vstart, tp + o_vs, 4 * (F + 1)));
+    CK(up.add(L.lvl_pref, tp + o_lp, 8 * (size_t)(Jmax + 1) * (F + 1)));
+    CK(up.add(L.job_off, tp + o_jo, 8 * (F + 1)));
+    CK(up.add(L.blk_pref, tp + o_bp, 8 * (F + 1)));
+    CK(up.add(L.nvdev, tp + o_nv, 8));
+    if (Jmax) CK(up.add(L.tile_pref, tp + o_tp, 4 * (size_t)Jmax * (F + 1)));
+    if (C) CK(up.add(L.steps, tp + o_st, 4 * (size_t)F * C));
+    CK(up.add(dst, nullptr, 8));
     if (any_color) {
-        CK(stage_copy(L.fcolor, tp + o_fc, 4 * (size_t)F, s));
+        CK(up.add(L.fcolor, tp + o_fc, 4 * (size_t)F));
         for (uint32_t f = 0; f < F; ++f)
             if (P[f].color)
-                CK(stage_copy(L.klt + (uint64_t)f * kKltFloats, d_in + offs[f] + P[f].klt_off, 4 * kKltFloats, s));
+                CK(up.add(L.klt + (uint64_t)f * kKltFloats, d_in + offs[f] + P[f].klt_off, 4 * kKltFloats));
     }
-    DevState *dst = ctx->st;
-    CK(dev_memset(dst, 0, 8, s));
+    CK(up.flush());
     const int sms = ctx->num_sms;
 
     // a12's RLGR decode needs only the streams' block tables: it runs on s beside a11 and the prelude (the
