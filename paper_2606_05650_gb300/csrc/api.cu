@@ -1128,7 +1128,7 @@ gsnfs_status encode_impl(gsnfs_ctx *ctx, cudaStream_t s, EncodeReq &rq, bool wor
         if (C) {
             // a6: RAHT prelude; a7: forward transform with the cluster average fused into the first pass
             stage_begin(sa, kStPrelude);
-            launch_raht_prelude(L.plan, L.gap, dst, nullptr, sms, sa);
+            launch_raht_prelude(L.plan, L.gap, dst, nullptr, N, sms, sa);
             stage_end(sa, kStPrelude);
             RahtIO io{};
             io.C = C;
@@ -1548,7 +1548,7 @@ gsnfs_status decode_impl(gsnfs_ctx *ctx, cudaStream_t s, const uint8_t *d_in, ui
     if (attrs) {
         stage_begin(sg, kStPrelude);
         launch_gap_levels(L.codes, P.nv, L.gap, sg);
-        launch_raht_prelude(L.plan, L.gap, dst, L.nvdev, sms, sg);
+        launch_raht_prelude(L.plan, L.gap, dst, L.nvdev, P.nv, sms, sg);
         stage_end(sg, kStPrelude);
         st = stream_wait(ctx, sg, s);  // the coefficients
         if (st) return st;
@@ -1646,7 +1646,7 @@ gsnfs_status lod_from_voxels(gsnfs_ctx *ctx, cudaStream_t s, cudaStream_t cs, co
             L.plan.pos0 = pos0;
             L.plan.end0 = end0;
             stage_begin(s, kStPrelude);
-            launch_raht_prelude(L.plan, gap0, dst, offs + nv, sms, s);
+            launch_raht_prelude(L.plan, gap0, dst, offs + nv, nn, sms, s);
             stage_end(s, kStPrelude);
         }
     }
@@ -2013,7 +2013,7 @@ gsnfs_status decode_batch_impl(gsnfs_ctx *ctx, cudaStream_t s, uint32_t F, const
     // a12: RAHT schedule, then (after the RLGR branch) the inverse RAHT
     if (attrs) {
         stage_begin(sg, kStPrelude);
-        launch_raht_prelude(L.plan, L.gap, dst, L.nvdev, sms, sg);
+        launch_raht_prelude(L.plan, L.gap, dst, L.nvdev, N, sms, sg);
         stage_end(sg, kStPrelude);
         st = fork_hi_end(ctx, s);
         if (st) return st;
@@ -2711,7 +2711,7 @@ gsnfs_status gsnfs_raht_plan_create(gsnfs_ctx *ctx, void *stream, const uint64_t
     CK(dev_memset(pl->st, 0, sizeof(DevState), s));
     CK(cudaMemcpyAsync(nvd, &pl->nv, 8, cudaMemcpyHostToDevice, s));
     if (nv) launch_gap_levels(d_codes, nv, gap, s);
-    launch_raht_prelude(pl->dev, gap, pl->st, nvd, ctx->num_sms, s);
+    launch_raht_prelude(pl->dev, gap, pl->st, nvd, nv, ctx->num_sms, s);
     CK(cudaStreamSynchronize(s));
     e = cudaGetLastError();
     if (e != cudaSuccess) {

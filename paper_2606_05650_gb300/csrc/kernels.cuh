@@ -143,8 +143,9 @@ struct RahtPlanDev {  // device pointers of a plan
 
 uint32_t raht_tile_size(uint32_t C);
 void raht_plan_sizes(uint64_t nv_cap, uint32_t T, uint64_t *elems, uint64_t *tiles, uint64_t *surv_rows);
-void launch_raht_prelude(const RahtPlanDev &p, const uint8_t *gap, const DevState *st, const uint64_t *nv_host,
-                         int num_sms, cudaStream_t s);
+// nv_dev: voxel count on the device (or null: st's); nv_bound: at least that, for the launch shapes
+void launch_raht_prelude(const RahtPlanDev &p, const uint8_t *gap, const DevState *st, const uint64_t *nv_dev,
+                         uint64_t nv_bound, int num_sms, cudaStream_t s);
 
 template <typename S>
 struct RahtIOT {  // S = float (codec) or double (FP64 instantiation of the same kernels)

@@ -315,22 +315,24 @@ __global__ void __launch_bounds__(kThreads) prelude_init_kernel(RahtPlanDev p, c
     }
 }
 
-// tiles of at most 256 elements: one warp per tile; larger tiles: one CTA per tile
+// Tiles of at most 256 elements: one warp per tile where there are tiles for
+// every warp, else (and for larger tiles) one CTA per tile, whose phases are
+// eight times shorter.
 template <int TMAX>
 constexpr bool kWarpTiles = TMAX <= 256;
 
-template <int TMAX>
+template <int TMAX, bool WARP>
 constexpr size_t prelude_smem_bytes()
 {
-    return (kWarpTiles<TMAX> ? (size_t)(kThreads / 32) : (size_t)1) * sizeof(PreludeSmem<TMAX>);
+    return (WARP ? (size_t)(kThreads / 32) : (size_t)1) * sizeof(PreludeSmem<TMAX>);
 }
 
-template <int TMAX>
+template <int TMAX, bool WARP>
 __global__ void __launch_bounds__(kThreads) prelude_tiles_kernel(PreludeArgs a, int q)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const RahtPass ps = a.p.passes[q];
-    if constexpr (kWarpTiles<TMAX>) {
+    if constexpr (WARP) {
         const uint32_t wid = threadIdx.x >> 5;
         PreludeSmem<TMAX> &S = reinterpret_cast<PreludeSmem<TMAX> *>(smem_raw)[wid];
         const WarpGroup G{threadIdx.x & 31u, 0u};
@@ -1435,22 +1437,40 @@ void raht_plan_sizes(uint64_t nv_cap, uint32_t T, uint64_t *elems, uint64_t *til
     *surv_rows = nv_cap + 128 * (kRahtMaxPasses + 1);
 }
 
+template <int TMAX, bool WARP>
+void prelude_tiles(const PreludeArgs &a, int q, uint32_t grid, cudaStream_t s)
+{
+    const size_t smem = prelude_smem_bytes<TMAX, WARP>();
+    cudaFuncSetAttribute(prelude_tiles_kernel<TMAX, WARP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    prelude_tiles_kernel<TMAX, WARP><<<grid, kThreads, smem, s>>>(a, q);
+    count_launch();
+}
+
 template <int TMAX>
 void prelude_launches(const PreludeArgs &a, const RahtPlanDev &p, const DevState *st, const uint64_t *nv_dev,
-                      int num_sms, cudaStream_t s)
+                      uint64_t nv_bound, int num_sms, cudaStream_t s)
 {
-    const size_t smem = prelude_smem_bytes<TMAX>();
-    cudaFuncSetAttribute(prelude_tiles_kernel<TMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = prelude_smem_bytes<TMAX, kWarpTiles<TMAX>>();
     cudaFuncSetAttribute(prelude_finish_kernel<TMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     prelude_init_kernel<<<1, 32, 0, s>>>(p, st, nv_dev);
     count_launch();
-    uint32_t grid = (uint32_t)num_sms * (p.pgrid_mult ? p.pgrid_mult : 8u);
-    for (int q = 0; q < kRahtMultiPasses; ++q) {
-        prelude_tiles_kernel<TMAX><<<grid, kThreads, smem, s>>>(a, q);
-        count_launch();
+    const uint32_t grid = (uint32_t)num_sms * (p.pgrid_mult ? p.pgrid_mult : 8u);
+    // A pass's sequence is about a fifth of the one before it (its length is known on the device only).  A CTA per
+    // tile while that makes at most kCtaWaves waves of CTAs: a tile takes a warp 18 us and a CTA 4, but a CTA's
+    // barriers cost more in all.  Prelude of one frame, a warp / a CTA per tile: 10k Gaussians 98 / 70 us, 250k
+    // 124 / 96 us, 1M 155 / 146 us; 16 frames of 1M take the warps (0.39 ms).
+    constexpr uint64_t kCtaWaves = 4;
+    uint64_t tiles = (nv_bound + p.T - 1) / p.T;
+    for (int q = 0; q < kRahtMultiPasses; ++q, tiles = tiles / 4 + 1) {
+        const bool few = tiles <= (uint64_t)grid * kCtaWaves;
+        const uint32_t g = few && tiles < grid ? (uint32_t)tiles : grid;
+        if (kWarpTiles<TMAX> && !few)
+            prelude_tiles<TMAX, kWarpTiles<TMAX>>(a, q, grid, s);
+        else
+            prelude_tiles<TMAX, false>(a, q, g < 1 ? 1 : g, s);
         prelude_scan_kernel<<<1, 1024, 0, s>>>(p, q);
         count_launch();
-        prelude_compact_kernel<<<grid, kThreads, 0, s>>>(a, q);
+        prelude_compact_kernel<<<g < 1 ? 1 : g, kThreads, 0, s>>>(a, q);
         count_launch();
     }
     prelude_finish_kernel<TMAX><<<1, kThreads, smem, s>>>(a, kRahtMultiPasses);
@@ -1458,18 +1478,18 @@ void prelude_launches(const PreludeArgs &a, const RahtPlanDev &p, const DevState
 }
 
 void launch_raht_prelude(const RahtPlanDev &p, const uint8_t *gap, const DevState *st, const uint64_t *nv_dev,
-                         int num_sms, cudaStream_t s)
+                         uint64_t nv_bound, int num_sms, cudaStream_t s)
 {
     PreludeArgs a;
     a.p = p;
     a.gap0 = gap;
     a.st = st;
     if (p.T <= 256)
-        prelude_launches<256>(a, p, st, nv_dev, num_sms, s);
+        prelude_launches<256>(a, p, st, nv_dev, nv_bound, num_sms, s);
     else if (p.T <= 1024)
-        prelude_launches<1024>(a, p, st, nv_dev, num_sms, s);
+        prelude_launches<1024>(a, p, st, nv_dev, nv_bound, num_sms, s);
     else
-        prelude_launches<4096>(a, p, st, nv_dev, num_sms, s);
+        prelude_launches<4096>(a, p, st, nv_dev, nv_bound, num_sms, s);
 }
 
 template <typename S>
