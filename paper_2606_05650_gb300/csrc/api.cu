@@ -1418,7 +1418,6 @@ gsnfs_status read_headers(gsnfs_ctx *ctx, cudaStream_t s, const uint8_t *d_in, u
 }
 
 struct DecLayout {
-    uint32_t *tabs;
     uint8_t *occ, *gap;
     uint64_t *nodes, *codes, *nvdev, *block_off, *spart;
     uint32_t *pref, *ppart;
@@ -1431,7 +1430,6 @@ struct DecLayout {
 size_t carve_decode(Carve &cv, DecLayout &L, const ParsedHeader &P, int num_sms, const uint32_t *tune)
 {
     L.grid = cv.take<FrameGrid>(1);
-    L.tabs = cv.take<uint32_t>(rans_table_words());
     L.nvdev = cv.take<uint64_t>(1);
     L.step = cv.take<float>(P.C + 1);
     L.occ = cv.take<uint8_t>(P.n_occ + 8);
@@ -1537,7 +1535,7 @@ gsnfs_status decode_impl(gsnfs_ctx *ctx, cudaStream_t s, const uint8_t *d_in, ui
     else if (P.occ_mode == 2)
         launch_fill(L.occ, P.n_occ, (uint8_t)P.occ_aux, sg);
     else
-        launch_rans_decode(sec, P.occ_bytes, P.n_occ, P.occ_aux, P.chunk, L.occ, L.tabs, dst, sms, sg);
+        launch_rans_decode(sec, P.occ_bytes, P.n_occ, P.occ_aux, P.chunk, L.occ, dst, sms, sg);
     stage_end(sg, kStOccDecode);
     stage_begin(sg, kStOctreeDecode);
     launch_octree_decode(occ, P.n_occ, P.J, P.lsz, L.nodes, L.pref, L.ppart, L.codes, dst, sms, sg);
@@ -2655,13 +2653,7 @@ gsnfs_status gsnfs_occupancy_section_decode(gsnfs_ctx *ctx, void *stream, const 
     } else if (P.occ_mode == 2) {
         launch_fill(d_out, n, (uint8_t)P.occ_aux, s);
     } else {
-        Carve m(nullptr);
-        m.take<uint32_t>(rans_table_words());
-        st = grow_arena(ctx, m.off, s);
-        if (st) return st;
-        Carve cv(ctx->arena);
-        uint32_t *tabs = cv.take<uint32_t>(rans_table_words());
-        launch_rans_decode(d_sec, sec_bytes, n, P.occ_aux, P.chunk, d_out, tabs, ctx->st, ctx->num_sms, s);
+        launch_rans_decode(d_sec, sec_bytes, n, P.occ_aux, P.chunk, d_out, ctx->st, ctx->num_sms, s);
     }
     CK(cudaMemcpyAsync(hp + 64, ctx->st, 4, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));

@@ -42,34 +42,11 @@ __global__ void __launch_bounds__(1024) tables_kernel(const DecFrame *fr, uint32
     const DecFrame &d = fr[blockIdx.x];
     if (d.mode != 1) return;
     uint32_t *tab = tabs + (uint64_t)blockIdx.x * tab_words;
-    __shared__ uint32_t s_cm[256];
-    __shared__ uint32_t s_fc[256];
-    const uint8_t *ftab = d.occ_sec + 24;
-    if (threadIdx.x < 32) {
-        uint32_t run = 0;
-        for (int b = 0; b < 256; b += 32) {
-            const int s2 = b + threadIdx.x;
-            const uint32_t v = (uint32_t)(ftab[2 * s2] | (ftab[2 * s2 + 1] << 8));
-            const uint32_t inc = warp_inclusive_sum(v);
-            s_cm[s2] = run + inc - v;
-            s_fc[s2] = (v << 16) | ((run + inc - v) & 0xFFFFu);
-            run += __shfl_sync(0xFFFFFFFFu, inc, 31);
-        }
-        if (threadIdx.x == 0) {
-            tab[kM / 4 + 256] = (run != kM);
-            if (run != kM) set_error(&st->err, kErrCorrupt);
-        }
-    }
-    __syncthreads();
-    for (uint32_t t = threadIdx.x; t < 256; t += blockDim.x) tab[kM / 4 + t] = s_fc[t];
-    uint8_t *slot2sym = reinterpret_cast<uint8_t *>(tab);
-    for (uint32_t t = threadIdx.x; t < kM; t += blockDim.x) {
-        uint32_t lo = 0, hi = 256;
-        while (hi - lo > 1) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (s_cm[mid] <= t) lo = mid; else hi = mid;
-        }
-        slot2sym[t] = (uint8_t)lo;
+    __shared__ uint32_t cum[257];
+    const bool ok = ransdec::build_tables(d.occ_sec + 24, tab, cum);
+    if (threadIdx.x == 0) {
+        tab[kM / 4 + 256] = !ok;
+        if (!ok) set_error(&st->err, kErrCorrupt);
     }
     // chunk offsets: after the section header, the frequency table and the size table (8-byte aligned)
     __shared__ uint64_t sh64[33];
@@ -90,8 +67,7 @@ __global__ void __launch_bounds__(1024) tables_kernel(const DecFrame *fr, uint32
     }
 }
 
-// grid (chunk groups, frames): warp per chunk of frame blockIdx.y, the chunk read in place (its words are
-// consumed in order, so they come from L1 after the first lane of a sector asks), the tables in shared memory
+// grid (chunk groups, frames): warp per chunk of frame blockIdx.y, the chunk read in place, the tables in shared memory
 constexpr uint32_t kRansWarps = 8;
 
 __global__ void __launch_bounds__(32 * kRansWarps) rans_batch_kernel(const DecFrame *fr, const uint32_t *tabs,
@@ -117,7 +93,7 @@ __global__ void __launch_bounds__(32 * kRansWarps) rans_batch_kernel(const DecFr
         const uint64_t start = cstart[d.chunk_off + c];
         const uint8_t *cp = ctab + 4 * c;
         const uint32_t cbytes = (uint32_t)cp[0] | ((uint32_t)cp[1] << 8) | ((uint32_t)cp[2] << 16) | ((uint32_t)cp[3] << 24);
-        if (cbytes < 128 || (cbytes & 3) || cbytes > 128 + 2 * chunk + 2 || start + cbytes > d.occ_bytes) {
+        if (cbytes < 128 || (cbytes & 3) || (start & 3) || cbytes > 128 + 2 * chunk + 2 || start + cbytes > d.occ_bytes) {
             if (lane == 0) set_error(&st->err, kErrCorrupt);
             continue;
         }

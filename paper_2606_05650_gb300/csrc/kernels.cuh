@@ -276,7 +276,7 @@ uint64_t rans_chunk_slot_bytes(uint32_t chunk);
 void launch_rans_encode(const RansFrames &r, DevState *st, uint64_t max_chunks, int num_sms, cudaStream_t s);
 uint64_t rans_table_words();
 void launch_rans_decode(const uint8_t *sec, uint64_t sec_bytes, uint64_t n, uint32_t nch, uint32_t chunk,
-                        uint8_t *out, uint32_t *tabs, DevState *st, int num_sms, cudaStream_t s);
+                        uint8_t *out, DevState *st, int num_sms, cudaStream_t s);
 void launch_fill(uint8_t *out, uint64_t n, uint8_t v, cudaStream_t s);
 
 // ---- batchdec.cu: batch-wide decoding steps --------------------------------

@@ -265,61 +265,25 @@ __global__ void __launch_bounds__(256) section_size_kernel(const uint64_t *occ_o
     if (lane == 0) sec_bytes[f] = raw;
 }
 
-// ---- decoder: warp per chunk of one frame; the chunk (states and words) is
-// copied to shared memory with coalesced loads, then decoded from there.
-
-// slot -> symbol table (kM bytes) and freq << 16 | cum (256 words) of one
-// section, followed by a corruption flag; one CTA of 1024 threads
-__global__ void __launch_bounds__(1024) table_kernel(const uint8_t *__restrict__ sec, uint32_t *tabs, DevState *st)
-{
-    __shared__ uint32_t s_cm[256];
-    __shared__ uint32_t s_fc[256];
-    uint8_t *slot2sym = reinterpret_cast<uint8_t *>(tabs);
-    const uint8_t *ftab = sec + 24;
-    if (threadIdx.x < 32) {
-        uint32_t run = 0;
-        for (int b = 0; b < 256; b += 32) {
-            const int s2 = b + threadIdx.x;
-            const uint32_t v = (uint32_t)(ftab[2 * s2] | (ftab[2 * s2 + 1] << 8));
-            const uint32_t inc = warp_inclusive_sum(v);
-            s_cm[s2] = run + inc - v;
-            s_fc[s2] = (v << 16) | ((run + inc - v) & 0xFFFFu);
-            run += __shfl_sync(0xFFFFFFFFu, inc, 31);
-        }
-        if (threadIdx.x == 0) {
-            tabs[kM / 4 + 256] = (run != kM);
-            if (run != kM) set_error(&st->err, kErrCorrupt);
-        }
-    }
-    __syncthreads();
-    for (uint32_t t = threadIdx.x; t < 256; t += blockDim.x) tabs[kM / 4 + t] = s_fc[t];
-    for (uint32_t t = threadIdx.x; t < kM; t += blockDim.x) {  // symbol of each slot: last s with cum[s] <= t
-        uint32_t lo = 0, hi = 256;
-        while (hi - lo > 1) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (s_cm[mid] <= t) lo = mid; else hi = mid;
-        }
-        slot2sym[t] = (uint8_t)lo;
-    }
-}
-
-// One frame's chunks, a warp per chunk read in place (its words are consumed
-// in order, so they come from L1).  Each CTA first turns the chunk size table
-// into chunk offsets in shared memory (one block scan per 1,024 chunks) when
-// they fit (kSmemChunks), else each warp sums the sizes before its chunk.
+// ---- decoder
+// One frame's chunks, a warp per chunk read in place.  Each CTA first builds
+// the decoding tables in shared memory and turns the chunk size table into
+// chunk offsets there (one block scan per 256 chunks) when they fit
+// (kSmemChunks), else each warp sums the sizes before its chunk.  (One CTA
+// building the tables for all of them in a launch before: 19 us more.)
 constexpr uint32_t kSmemChunks = 4096;
 
 __global__ void __launch_bounds__(32 * ransdec::kMaxWarps) decode_kernel(const uint8_t *__restrict__ sec,
                                                                          uint64_t sec_bytes, uint64_t n, uint32_t nch,
-                                                                         uint32_t chunk, uint8_t *out, DevState *st,
-                                                                         const uint32_t *tabs)
+                                                                         uint32_t chunk, uint8_t *out, DevState *st)
 {
     using namespace ransdec;
     extern __shared__ __align__(16) unsigned char dsm[];
-    __shared__ uint32_t sh[33];
-    // decoding tables built once by table_kernel: copy them in
-    if (tabs[kTabWords] != 0) return;  // frequencies did not sum to M (reported by table_kernel)
-    load_tables(reinterpret_cast<uint32_t *>(dsm), tabs);
+    __shared__ uint32_t sh[33], cum[257];
+    if (!build_tables(sec + 24, reinterpret_cast<uint32_t *>(dsm), cum)) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) set_error(&st->err, kErrCorrupt);
+        return;
+    }
     const uint8_t *ctab = sec + 24 + 512;
     const uint64_t table = (16 + 8 + 512 + 4 * (uint64_t)nch + 7) & ~7ull;
     const bool local = nch <= kSmemChunks && sec_bytes < (1ull << 32);
@@ -347,7 +311,7 @@ __global__ void __launch_bounds__(32 * ransdec::kMaxWarps) decode_kernel(const u
         const uint64_t start = local ? s_start[c] : table + chunk_offset(ctab, c, lane);
         const uint8_t *cp = ctab + 4 * c;
         const uint32_t cbytes = (uint32_t)cp[0] | ((uint32_t)cp[1] << 8) | ((uint32_t)cp[2] << 16) | ((uint32_t)cp[3] << 24);
-        if (cbytes < 128 || (cbytes & 3) || cbytes > 128 + 2 * chunk + 2 || start + cbytes > sec_bytes) {
+        if (cbytes < 128 || (cbytes & 3) || (start & 3) || cbytes > 128 + 2 * chunk + 2 || start + cbytes > sec_bytes) {
             if (lane == 0) set_error(&st->err, kErrCorrupt);
             continue;
         }
@@ -398,17 +362,15 @@ void launch_rans_encode(const RansFrames &r, DevState *st, uint64_t max_chunks, 
 uint64_t rans_table_words() { return kM / 4 + 256 + 4; }
 
 void launch_rans_decode(const uint8_t *sec, uint64_t sec_bytes, uint64_t n, uint32_t nch, uint32_t chunk,
-                        uint8_t *out, uint32_t *tabs, DevState *st, int num_sms, cudaStream_t s)
+                        uint8_t *out, DevState *st, int num_sms, cudaStream_t s)
 {
     if (nch == 0) return;
-    table_kernel<<<1, 1024, 0, s>>>(sec, tabs, st);
-    count_launch();
     const uint32_t warps = ransdec::kMaxWarps;
     uint32_t blocks = (nch + warps - 1) / warps;
     if (blocks > (uint32_t)num_sms * 4) blocks = (uint32_t)num_sms * 4;
     const size_t smem = (size_t)ransdec::kTabWords * 4 + 4 * (size_t)kSmemChunks;
     cudaFuncSetAttribute(decode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    decode_kernel<<<blocks, 32 * warps, smem, s>>>(sec, sec_bytes, n, nch, chunk, out, st, tabs);
+    decode_kernel<<<blocks, 32 * warps, smem, s>>>(sec, sec_bytes, n, nch, chunk, out, st);
     count_launch();
 }
 
