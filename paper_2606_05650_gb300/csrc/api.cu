@@ -822,7 +822,8 @@ void carve_plan(Carve &cv, RahtPlanDev &p, uint64_t nv_cap, uint32_t T, const ui
     p.npasses = cv.take<uint32_t>(1);
     p.pos0 = nullptr;
     p.end0 = nullptr;
-    p.pipe_ctr = cv.take<uint32_t>(2);
+    p.pipe_ctr = cv.take<uint32_t>(3);
+    p.cta_carry = cv.take<uint32_t>(kRahtMaxPreludeCtas);
 }
 
 size_t carve_encode(Carve &cv, EncLayout &L, const EncodeReq &rq, int num_sms, bool worst_slots,

@@ -100,6 +100,7 @@ constexpr uint32_t kRahtCarrySlots = 128;  // survivors of a tile: at most 2 x 6
                                            // from either tile edge)
 constexpr int kRahtMultiPasses = 3;  // passes launched grid-wide; the rest run in one CTA
 constexpr int kRahtMaxPasses = 40;
+constexpr uint32_t kRahtMaxPreludeCtas = 8192;  // 32 per SM (GSNFS_TUNE_PRELUDE_GRID), at most 256 SMs
 
 struct RahtPass {  // device-resident description of one pass
     uint32_t n;        // elements in this pass
@@ -129,7 +130,8 @@ struct RahtPlanDev {  // device pointers of a plan
     uint32_t *bf_idx;      // per tile x T: i0 | i1 << 16
     float2 *bf_ab;         // per tile x T: FP32 coefficients (a, b)
     uint2 *bf_w;           // per tile x T: integer weights (w0, w1), or null (not recorded)
-    uint32_t *tile_carry;  // per tile carried count, then exclusive base
+    uint32_t *tile_carry;  // per tile carried count, then that of the earlier tiles of its CTA
+    uint32_t *cta_carry;   // per CTA of a prelude pass: carried count of the earlier CTAs (kRahtMaxPreludeCtas)
     uint16_t *carry_list;  // per tile x kRahtCarrySlots: in-tile index of each carried survivor, by rank
     RahtPass *passes;      // kRahtMaxPasses
     uint32_t *npasses;     // device counter
@@ -137,8 +139,9 @@ struct RahtPlanDev {  // device pointers of a plan
     // (a coarser sequence: the nodes of an octree depth, each a run of voxels, for level-of-detail decoding)
     const uint32_t *pos0;
     const uint32_t *end0;
-    uint32_t *pipe_ctr;    // 2 words: tiles claimed and CTAs finished in the pipelined first transform pass
-                           // (zeroed by the prelude; the last CTA of every launch puts them back to zero)
+    uint32_t *pipe_ctr;    // 3 words: tiles claimed and CTAs finished in the pipelined first transform pass, CTAs
+                           // finished in a prelude pass (zeroed by the prelude; the last CTA of every launch puts
+                           // them back to zero)
 };
 
 uint32_t raht_tile_size(uint32_t C);

@@ -312,6 +312,7 @@ __global__ void __launch_bounds__(kThreads) prelude_init_kernel(RahtPlanDev p, c
         *p.npasses = n ? 1u : 0u;
         p.pipe_ctr[0] = 0;
         p.pipe_ctr[1] = 0;
+        p.pipe_ctr[2] = 0;
     }
 }
 
@@ -327,21 +328,79 @@ constexpr size_t prelude_smem_bytes()
     return (WARP ? (size_t)(kThreads / 32) : (size_t)1) * sizeof(PreludeSmem<TMAX>);
 }
 
+// pass q + 1 of `carried` elements
+__device__ void prelude_next_pass(const RahtPlanDev &p, int q, const RahtPass &ps, uint32_t carried)
+{
+    if (q + 1 >= kRahtMaxPasses) return;
+    RahtPass nx = {};
+    nx.n = carried;
+    nx.ntiles = (carried + p.T - 1) / p.T;
+    nx.seq_off = ps.seq_off + ps.n + 1;
+    nx.tile_off = ps.tile_off + ps.ntiles;
+    nx.surv_off = (q == 0) ? 0u : ps.surv_off + ps.n;
+    p.passes[q + 1] = nx;
+    if (carried) *p.npasses = (uint32_t)(q + 2);
+}
+
+// tiles of a CTA of the grid-wide prelude passes: a contiguous run, so that their carried counts are summed within
+// the CTA
+__device__ __forceinline__ uint32_t tiles_per_cta(uint32_t ntiles, uint32_t ctas) { return (ntiles + ctas - 1) / ctas; }
+
+// Schedules of a pass's tiles, then the places of their carried survivors: per
+// tile the count of the CTA's earlier tiles (tile_carry), per CTA the count of
+// the earlier CTAs (cta_carry), the latter by the CTA that finishes last.  (A
+// launch of one CTA that scanned all tiles: 20 us at 62,500 tiles, and up to
+// 80 us of waiting for an SM beside the other branch's kernels.)
 template <int TMAX, bool WARP>
 __global__ void __launch_bounds__(kThreads) prelude_tiles_kernel(PreludeArgs a, int q)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const RahtPass ps = a.p.passes[q];
+    __shared__ uint32_t sh[33];
+    __shared__ bool last;
+    const RahtPlanDev &p = a.p;
+    const RahtPass ps = p.passes[q];
+    if (ps.n == 0) return;
+    const uint32_t per = tiles_per_cta(ps.ntiles, gridDim.x);
+    const uint32_t t0 = min(blockIdx.x * per, ps.ntiles), t1 = min(t0 + per, ps.ntiles);
     if constexpr (WARP) {
         const uint32_t wid = threadIdx.x >> 5;
         PreludeSmem<TMAX> &S = reinterpret_cast<PreludeSmem<TMAX> *>(smem_raw)[wid];
         const WarpGroup G{threadIdx.x & 31u, 0u};
-        const uint32_t nw = gridDim.x * (kThreads / 32);
-        for (uint32_t t = blockIdx.x * (kThreads / 32) + wid; t < ps.ntiles; t += nw) prelude_tile(a, S, q, ps, t, G);
+        for (uint32_t t = t0 + wid; t < t1; t += kThreads / 32) prelude_tile(a, S, q, ps, t, G);
     } else {
         PreludeSmem<TMAX> &S = *reinterpret_cast<PreludeSmem<TMAX> *>(smem_raw);
         const CtaGroup G{threadIdx.x, threadIdx.x >> 5};
-        for (uint32_t t = blockIdx.x; t < ps.ntiles; t += gridDim.x) prelude_tile(a, S, q, ps, t, G);
+        for (uint32_t t = t0; t < t1; ++t) prelude_tile(a, S, q, ps, t, G);
+    }
+    __syncthreads();
+    uint32_t *tc = p.tile_carry + ps.tile_off;
+    uint32_t run = 0;
+    for (uint32_t b = t0; b < t1; b += kThreads) {  // this CTA's own writes
+        const uint32_t t = b + threadIdx.x, c = t < t1 ? tc[t] : 0u;
+        uint32_t tot;
+        const uint32_t ex = block_exclusive_sum<uint32_t>(c, sh, &tot);
+        if (t < t1) tc[t] = run + ex;
+        run += tot;
+    }
+    if (threadIdx.x == 0) {
+        p.cta_carry[blockIdx.x] = run;
+        __threadfence();
+        last = atomicAdd(p.pipe_ctr + 2, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    run = 0;
+    for (uint32_t b = 0; b < gridDim.x; b += kThreads) {
+        const uint32_t x = b + threadIdx.x, c = x < gridDim.x ? __ldcg(p.cta_carry + x) : 0u;
+        uint32_t tot;
+        const uint32_t ex = block_exclusive_sum<uint32_t>(c, sh, &tot);
+        if (x < gridDim.x) p.cta_carry[x] = run + ex;
+        run += tot;
+    }
+    if (threadIdx.x == 0) {
+        p.pipe_ctr[2] = 0;  // for the next launch
+        prelude_next_pass(p, q, ps, run);
     }
 }
 
@@ -349,56 +408,35 @@ __global__ void __launch_bounds__(kThreads) prelude_tiles_kernel(PreludeArgs a, 
 __device__ void prelude_scan_body(const RahtPlanDev &p, int q, uint32_t *sh)
 {
     const RahtPass ps = p.passes[q];
-    // each thread sums a contiguous run of tiles (all its loads in flight together), one block scan of the
-    // run totals, then each thread writes its run's prefixes
-    const uint32_t per = (ps.ntiles + blockDim.x - 1) / blockDim.x;
-    const uint32_t b = threadIdx.x * per < ps.ntiles ? threadIdx.x * per : ps.ntiles;
-    const uint32_t e = b + per < ps.ntiles ? b + per : ps.ntiles;
     uint32_t *tc = p.tile_carry + ps.tile_off;
-    uint32_t sum = 0;
-    for (uint32_t t = b; t < e; ++t) sum += tc[t];
-    uint32_t run;
-    uint32_t pre = block_exclusive_sum<uint32_t>(sum, sh, &run);
-    for (uint32_t t = b; t < e; ++t) {
-        const uint32_t c = tc[t];
-        tc[t] = pre;
-        pre += c;
+    uint32_t run = 0;
+    for (uint32_t b = 0; b < ps.ntiles; b += blockDim.x) {
+        const uint32_t t = b + threadIdx.x, c = t < ps.ntiles ? tc[t] : 0u;
+        uint32_t tot;
+        const uint32_t ex = block_exclusive_sum<uint32_t>(c, sh, &tot);
+        if (t < ps.ntiles) tc[t] = run + ex;
+        run += tot;
     }
     if (threadIdx.x == 0) {
-        RahtPass nx = {};
-        if (q + 1 < kRahtMaxPasses) {
-            nx.n = run;
-            nx.ntiles = (run + p.T - 1) / p.T;
-            nx.seq_off = ps.seq_off + ps.n + 1;
-            nx.tile_off = ps.tile_off + ps.ntiles;
-            nx.surv_off = (q == 0) ? 0u : ps.surv_off + ps.n;
-            p.passes[q + 1] = nx;
-            if (run) *p.npasses = (uint32_t)(q + 2);
-        }
+        p.cta_carry[0] = 0;
+        prelude_next_pass(p, q, ps, run);
     }
     __syncthreads();
-}
-
-__global__ void __launch_bounds__(1024) prelude_scan_kernel(RahtPlanDev p, int q)
-{
-    __shared__ uint32_t sh[33];
-    if (p.passes[q].n == 0) return;
-    prelude_scan_body(p, q, sh);
 }
 
 // carried elements: global index, next sequence arrays, sentinel.  A warp
 // per tile walks the tile's list of carried survivors (their global index is
 // the tile's scanned base plus their rank), so elements that are not carried
-// are never read.
-__device__ void prelude_compact_body(const PreludeArgs &a, int q, uint32_t warp0, uint32_t nwarps)
+// are never read.  per: tiles of each entry of cta_carry.
+__device__ void prelude_compact_body(const PreludeArgs &a, int q, uint32_t warp0, uint32_t nwarps, uint32_t per)
 {
     const RahtPlanDev &p = a.p;
     const RahtPass ps = p.passes[q];
     const RahtPass nx = p.passes[q + 1];
     const uint32_t lane = threadIdx.x & 31;
     for (uint32_t t = warp0; t < ps.ntiles; t += nwarps) {
-        const uint32_t b0 = p.tile_carry[ps.tile_off + t];
-        const uint32_t b1 = t + 1 < ps.ntiles ? p.tile_carry[ps.tile_off + t + 1] : nx.n;
+        const uint32_t b0 = p.tile_carry[ps.tile_off + t] + p.cta_carry[t / per];
+        const uint32_t b1 = t + 1 < ps.ntiles ? p.tile_carry[ps.tile_off + t + 1] + p.cta_carry[(t + 1) / per] : nx.n;
         for (uint32_t r = lane; r < b1 - b0 && r < kRahtCarrySlots; r += 32) {
             const uint32_t i = p.carry_list[(uint64_t)(ps.tile_off + t) * kRahtCarrySlots + r];
             const uint64_t j = (uint64_t)t * p.T + i;
@@ -415,10 +453,11 @@ __device__ void prelude_compact_body(const PreludeArgs &a, int q, uint32_t warp0
     }
 }
 
-__global__ void __launch_bounds__(kThreads) prelude_compact_kernel(PreludeArgs a, int q)
+__global__ void __launch_bounds__(kThreads) prelude_compact_kernel(PreludeArgs a, int q, uint32_t tile_ctas)
 {
     if (a.p.passes[q].n == 0 || q + 1 >= kRahtMaxPasses) return;
-    prelude_compact_body(a, q, blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5), gridDim.x * (kThreads / 32));
+    prelude_compact_body(a, q, blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5), gridDim.x * (kThreads / 32),
+                         tiles_per_cta(a.p.passes[q].ntiles, tile_ctas));
 }
 
 // remaining passes inside one CTA
@@ -441,7 +480,7 @@ __global__ void __launch_bounds__(kThreads) prelude_finish_kernel(PreludeArgs a,
         __syncthreads();
         prelude_scan_body(a.p, q, S[0].scan);
         __syncthreads();
-        prelude_compact_body(a, q, threadIdx.x >> 5, kThreads / 32);
+        prelude_compact_body(a, q, threadIdx.x >> 5, kThreads / 32, ps.ntiles);
         __syncthreads();
     }
 }
@@ -1463,14 +1502,12 @@ void prelude_launches(const PreludeArgs &a, const RahtPlanDev &p, const DevState
     uint64_t tiles = (nv_bound + p.T - 1) / p.T;
     for (int q = 0; q < kRahtMultiPasses; ++q, tiles = tiles / 4 + 1) {
         const bool few = tiles <= (uint64_t)grid * kCtaWaves;
-        const uint32_t g = few && tiles < grid ? (uint32_t)tiles : grid;
+        const uint32_t g = few && tiles < grid ? (tiles ? (uint32_t)tiles : 1u) : grid;
         if (kWarpTiles<TMAX> && !few)
-            prelude_tiles<TMAX, kWarpTiles<TMAX>>(a, q, grid, s);
+            prelude_tiles<TMAX, kWarpTiles<TMAX>>(a, q, g, s);
         else
-            prelude_tiles<TMAX, false>(a, q, g < 1 ? 1 : g, s);
-        prelude_scan_kernel<<<1, 1024, 0, s>>>(p, q);
-        count_launch();
-        prelude_compact_kernel<<<g < 1 ? 1 : g, kThreads, 0, s>>>(a, q);
+            prelude_tiles<TMAX, false>(a, q, g, s);
+        prelude_compact_kernel<<<g, kThreads, 0, s>>>(a, q, g);
         count_launch();
     }
     prelude_finish_kernel<TMAX><<<1, kThreads, smem, s>>>(a, kRahtMultiPasses);
