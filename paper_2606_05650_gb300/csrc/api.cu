@@ -536,32 +536,35 @@ __device__ __forceinline__ void wr64(uint8_t *p, uint64_t v)
     for (int i = 0; i < 8; ++i) p[i] = (uint8_t)(v >> (8 * i));
 }
 
-__global__ void sizes_kernel(HdrParams hp, const uint32_t *J, const uint32_t *vstart, const uint64_t *sec_bytes,
-                             const uint64_t *blk_off, const uint64_t *block_off, StreamInfo *si, DevState *st)
+// one CTA, a thread per stream
+__global__ void __launch_bounds__(kMaxFrames * kMaxRungs) sizes_kernel(HdrParams hp, const uint32_t *J, const uint32_t *vstart,
+                                                                       const uint64_t *sec_bytes, const uint64_t *blk_off,
+                                                                       const uint64_t *block_off, StreamInfo *si,
+                                                                       DevState *st)
 {
-    if (threadIdx.x != 0) return;
-    uint64_t run = 0;
-    for (uint32_t f = 0; f < hp.F; ++f) {
+    __shared__ uint64_t sh[33];
+    const uint32_t i = threadIdx.x;
+    StreamInfo x{0, 0, 0, 0};
+    if (i < hp.F * hp.R) {
+        const uint32_t f = i / hp.R, r = i - f * hp.R;
         const uint64_t nv = vstart[f + 1] - vstart[f];
         const uint64_t nb = (nv + hp.B - 1) / hp.B;
-        for (uint32_t r = 0; r < hp.R; ++r) {
-            StreamInfo x;
-            x.hb = header_bytes(J[f], hp.C, hp.C ? hp.G : 0, hp.color);
-            x.occ = sec_bytes[f];
-            x.attr = 0;
-            if (hp.C && nv) {
-                const uint64_t b0 = blk_off[f] + (uint64_t)r * hp.C * nb;
-                const uint64_t words = block_off[b0 + hp.C * nb] - block_off[b0];
-                x.attr = pad8(8 + 4 * hp.C * nb + 4 * words);
-            }
-            x.off = run;
-            run += x.hb + x.occ + x.attr;
-            si[f * hp.R + r] = x;
+        x.hb = header_bytes(J[f], hp.C, hp.C ? hp.G : 0, hp.color);
+        x.occ = sec_bytes[f];
+        if (hp.C && nv) {
+            const uint64_t b0 = blk_off[f] + (uint64_t)r * hp.C * nb;
+            const uint64_t words = block_off[b0 + hp.C * nb] - block_off[b0];
+            x.attr = pad8(8 + 4 * hp.C * nb + 4 * words);
         }
     }
-    si[hp.F * hp.R].off = run;
-    st->total_bytes = run;
-    if (run > hp.capacity) set_error(&st->err, kErrCapacity);
+    uint64_t run;
+    x.off = block_exclusive_sum<uint64_t>(x.hb + x.occ + x.attr, sh, &run);
+    if (i < hp.F * hp.R) si[i] = x;
+    if (i == 0) {
+        si[hp.F * hp.R].off = run;
+        st->total_bytes = run;
+        if (run > hp.capacity) set_error(&st->err, kErrCapacity);
+    }
 }
 
 __global__ void header_kernel(HdrParams hp, const uint32_t *J, const uint32_t *vstart, const FrameGrid *grid,
@@ -706,19 +709,21 @@ __global__ void attr_copy_kernel(HdrParams hp, AttrCopyArgs a, const StreamInfo 
     const uint64_t base = a.block_off[b0];
     const uint32_t lane = threadIdx.x & 31;
     const uint64_t wid = tid >> 5, nwarps = nt >> 5;
-    // a warp takes 32 consecutive block streams: their sizes and offsets in one
-    // load, then four streams at a time, the first 96 words of all four loaded
+    // a warp takes up to 32 consecutive block streams: their sizes and offsets in
+    // one load, then four streams at a time, the first 96 words of all four loaded
     // before any is stored (a stream is ~75 words at the headline's rates)
     constexpr uint32_t kGroup = 4, kPerLane = 3;
-    for (uint64_t k0 = wid * 32; k0 < nblk; k0 += nwarps * 32) {
+    // 32 streams per turn, fewer (in groups of four) when that leaves warps without any
+    const uint32_t per = (uint32_t)min((uint64_t)32, max((nblk + nwarps - 1) / nwarps + kGroup - 1, (uint64_t)kGroup) / kGroup * kGroup);
+    for (uint64_t k0 = wid * per; k0 < nblk; k0 += nwarps * per) {
         const uint64_t k = k0 + lane;
         uint32_t wl = 0;
         uint64_t ol = 0;
-        if (k < nblk) {
+        if (k < nblk && lane < per) {
             wl = a.block_words[b0 + k];
             ol = a.block_off[b0 + k] - base;
         }
-        const uint32_t cnt = (nblk - k0) < 32 ? (uint32_t)(nblk - k0) : 32u;
+        const uint32_t cnt = (nblk - k0) < per ? (uint32_t)(nblk - k0) : per;
         for (uint32_t j0 = 0; j0 < cnt; j0 += kGroup) {
             uint32_t w[kGroup], v[kGroup][kPerLane];
             uint64_t o[kGroup];
@@ -1117,7 +1122,7 @@ gsnfs_status encode_impl(gsnfs_ctx *ctx, cudaStream_t s, EncodeReq &rq, bool wor
         // a4: octree occupancy
         OccupancyOut oo{L.occ, L.occ_cap, L.lsz, L.occ_off, L.hoff, L.opart};
         stage_begin(s, kStOccupancy);
-        launch_occupancy(L.codes, L.gap, L.vstart, L.Jd, F, frame_shift, oo, dst, sms, s);
+        launch_occupancy(L.codes, L.gap, L.vstart, L.Jd, F, nmax, oo, dst, sms, s);
         stage_end(s, kStOccupancy);
         // a5: occupancy rANS
         RansFrames rf{F, L.occ, L.occ_off, q->rans_chunk, L.chunk_off, L.freq, L.cum, L.mode, L.chunk_words,
@@ -1183,7 +1188,7 @@ gsnfs_status encode_impl(gsnfs_ctx *ctx, cudaStream_t s, EncodeReq &rq, bool wor
         }
         // a10: container
         stage_begin(s, kStContainer);
-        sizes_kernel<<<1, 32, 0, s>>>(hpar, L.Jd, L.vstart, L.sec_bytes, L.blk_off, L.block_off, L.si, dst);
+        sizes_kernel<<<1, (F * R + 31) / 32 * 32, 0, s>>>(hpar, L.Jd, L.vstart, L.sec_bytes, L.blk_off, L.block_off, L.si, dst);
         count_launch();
         header_kernel<<<F * R, 128, 0, s>>>(hpar, L.Jd, L.vstart, L.grid, L.lsz, L.groups, L.steps_rg, L.klt, L.si, dst,
                                             rq.out);
@@ -2516,7 +2521,7 @@ gsnfs_status gsnfs_octree_encode(gsnfs_ctx *ctx, void *stream, const uint64_t *d
     if (nv) CK(cudaMemcpyAsync(L.codes, d_codes, 8 * nv, cudaMemcpyDeviceToDevice, s));
     launch_gap_levels(L.codes, nv, L.gap, s);
     OccupancyOut oo{L.occ, (ob + 64) & ~(uint64_t)63, L.lsz, L.occ_off, L.hoff, L.opart};
-    launch_occupancy(L.codes, L.gap, L.vstart, L.Jd, 1, 64, oo, ctx->st, ctx->num_sms, s);
+    launch_occupancy(L.codes, L.gap, L.vstart, L.Jd, 1, nv, oo, ctx->st, ctx->num_sms, s);
     CK(cudaMemcpyAsync(hp + 256, L.lsz, 4 * 22, cudaMemcpyDeviceToHost, s));
     CK(cudaMemcpyAsync(hp + 512, L.occ_off, 16, cudaMemcpyDeviceToHost, s));
     CK(cudaMemcpyAsync(hp + 640, ctx->st, 4, cudaMemcpyDeviceToHost, s));

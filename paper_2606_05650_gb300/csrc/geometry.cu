@@ -86,15 +86,26 @@ __global__ void __launch_bounds__(kThreads) dedup_down_kernel(const uint64_t *__
     }
 }
 
-__global__ void dedup_fix_kernel(const uint32_t *partials, uint32_t P, uint32_t *vstart, uint32_t F,
-                                 DevState *st)
+// One warp: empty frames (no voxel marked their start) start where the next one does.
+__global__ void __launch_bounds__(32) dedup_fix_kernel(const uint32_t *partials, uint32_t P, uint32_t *vstart,
+                                                       uint32_t F, DevState *st)
 {
     // partials were scanned in place; the total is the last prefix plus the last count
-    uint32_t nv = partials[P];
-    vstart[F] = nv;
-    for (int f = (int)F - 1; f >= 0; --f)
-        if (vstart[f] == 0xFFFFFFFFu) vstart[f] = vstart[f + 1];
-    st->nv_total = nv;
+    const uint32_t nv = partials[P], lane = threadIdx.x;
+    uint32_t next = nv;  // start of the frame after the group
+    for (int g = ((int)F - 1) / 32; g >= 0; --g) {
+        const uint32_t f = 32u * (uint32_t)g + lane;
+        uint32_t v = f < F ? vstart[f] : next;
+        const uint32_t known = __ballot_sync(0xFFFFFFFFu, v != 0xFFFFFFFFu), at = known & ~lanemask_lt();
+        const uint32_t from = __shfl_sync(0xFFFFFFFFu, v, at ? __ffs(at) - 1 : 0);
+        if (v == 0xFFFFFFFFu) v = at ? from : next;
+        if (f < F) vstart[f] = v;
+        next = __shfl_sync(0xFFFFFFFFu, v, 0);
+    }
+    if (lane == 0) {
+        vstart[F] = nv;
+        st->nv_total = nv;
+    }
 }
 
 // exclusive scan of P words with the total appended at [P] (one CTA)
@@ -151,13 +162,18 @@ __global__ void __launch_bounds__(32 * kH) occ_scan_kernel(uint32_t *partials, u
     __shared__ uint32_t tot[kH];
     const uint32_t f = blockIdx.x, lane = threadIdx.x & 31, h = threadIdx.x >> 5;
     uint32_t *row = partials + ((uint64_t)f * kH + h) * X;
-    uint32_t run = 0;
-    for (uint32_t b = 0; b < X; b += 32) {
-        const uint32_t x = b + lane;
-        const uint32_t v = (x < X) ? row[x] : 0u;
-        const uint32_t inc = warp_inclusive_sum(v);
-        if (x < X) row[x] = run + inc - v;
-        run += __shfl_sync(0xFFFFFFFFu, inc, 31);
+    // a contiguous run of counts per lane: all its loads in flight, one warp scan, then its prefixes
+    const uint32_t per = (X + 31) / 32, b0 = min(lane * per, X), b1 = min(b0 + per, X);
+    uint32_t sum = 0;
+#pragma unroll 8
+    for (uint32_t x = b0; x < b1; ++x) sum += row[x];
+    const uint32_t inc = warp_inclusive_sum(sum), run = __shfl_sync(0xFFFFFFFFu, inc, 31);
+    uint32_t pre = inc - sum;
+#pragma unroll 8
+    for (uint32_t x = b0; x < b1; ++x) {
+        const uint32_t v = __ldcg(row + x);
+        row[x] = pre;
+        pre += v;
     }
     if (lane == 0) tot[h] = run;
     __syncthreads();
@@ -177,15 +193,14 @@ __global__ void __launch_bounds__(32 * kH) occ_scan_kernel(uint32_t *partials, u
     }
 }
 
-__global__ void occ_offsets_kernel(const uint64_t *nocc, uint32_t F, uint64_t *occ_off)
+__global__ void __launch_bounds__(kMaxFrames) occ_offsets_kernel(const uint64_t *nocc, uint32_t F, uint64_t *occ_off)
 {
-    if (threadIdx.x) return;
-    uint64_t run = 0;
-    for (uint32_t f = 0; f < F; ++f) {
-        occ_off[f] = run;
-        run += nocc[f];
-    }
-    occ_off[F] = run;
+    __shared__ uint64_t sh[33];
+    const uint32_t f = threadIdx.x;
+    uint64_t tot;
+    const uint64_t off = block_exclusive_sum<uint64_t>(f < F ? nocc[f] : 0ull, sh, &tot);
+    if (f < F) occ_off[f] = off;
+    if (f == 0) occ_off[F] = tot;
 }
 
 __global__ void zero_words_kernel(uint32_t *p, const uint64_t *nbytes_at, uint64_t cap_words)
@@ -539,10 +554,13 @@ Chunks popc_chunks(uint64_t n, int num_sms)
     return c;
 }
 
-uint32_t occ_x(uint32_t F, int num_sms)
+// CTAs per frame: to fill the GPU, but no more than tiles of the longest frame (n_max voxels at most)
+uint32_t occ_x(uint32_t F, int num_sms, uint64_t n_max = ~0ull)
 {
     uint32_t X = (uint32_t)(num_sms * 8) / F;
-    return X < 16 ? 16 : X;
+    if (X < 16) X = 16;
+    const uint64_t tiles = n_max / kThreads + 1;
+    return tiles < X ? (uint32_t)tiles : X;
 }
 
 }  // namespace
@@ -572,25 +590,23 @@ void launch_dedup(const uint64_t *keys, uint64_t n, uint32_t frame_shift, uint32
                                                    vstart, vals, row0);
         count_launch();
     }
-    dedup_fix_kernel<<<1, 1, 0, s>>>(partials, c.P, vstart, F, st);
+    dedup_fix_kernel<<<1, 32, 0, s>>>(partials, c.P, vstart, F, st);
     count_launch();
 }
 
 uint64_t occupancy_partial_words(uint32_t F, int num_sms) { return (uint64_t)F * occ_x(F, num_sms) * kH + 2 * kMaxFrames + 8; }
 
 void launch_occupancy(const uint64_t *codes, const uint8_t *gap, const uint32_t *vstart, const uint32_t *J,
-                      uint32_t F, uint32_t frame_shift, const OccupancyOut &o, DevState *st, int num_sms,
-                      cudaStream_t s)
+                      uint32_t F, uint64_t n_max, const OccupancyOut &o, DevState *st, int num_sms, cudaStream_t s)
 {
-    (void)frame_shift;
-    uint32_t X = occ_x(F, num_sms);
+    uint32_t X = occ_x(F, num_sms, n_max);
     dim3 grid(X, F);
     occ_up_kernel<<<grid, kThreads, 0, s>>>(gap, vstart, J, o.partials);
     count_launch();
     uint64_t *nocc = reinterpret_cast<uint64_t *>(o.partials + (uint64_t)F * X * kH + ((F * X * kH) & 1u));
     occ_scan_kernel<<<F, 32 * kH, 0, s>>>(o.partials, X, vstart, J, o.level_sizes, o.hoff, nocc);
     count_launch();
-    occ_offsets_kernel<<<1, 32, 0, s>>>(nocc, F, o.occ_off);
+    occ_offsets_kernel<<<1, kMaxFrames, 0, s>>>(nocc, F, o.occ_off);
     count_launch();
     zero_words_kernel<<<num_sms * 2, 256, 0, s>>>((uint32_t *)o.occ, o.occ_off + F, o.occ_capacity / 4);
     count_launch();

@@ -72,8 +72,8 @@ struct OccupancyOut {
     uint32_t *partials;      // scratch
 };
 void launch_occupancy(const uint64_t *codes, const uint8_t *gap, const uint32_t *vstart, const uint32_t *J,
-                      uint32_t F, uint32_t frame_shift, const OccupancyOut &o, DevState *st, int num_sms,
-                      cudaStream_t s);
+                      uint32_t F, uint64_t n_max, const OccupancyOut &o, DevState *st, int num_sms,
+                      cudaStream_t s);  // n_max: voxels of any frame at most
 uint64_t occupancy_partial_words(uint32_t F, int num_sms);
 // the same bound for one frame on a GPU with at most max_sms SMs
 constexpr uint64_t occupancy_partial_words_one_frame(int max_sms) { return 8ull * max_sms * 22 + 2 * kMaxFrames + 8; }

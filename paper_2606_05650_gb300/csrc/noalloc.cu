@@ -112,7 +112,7 @@ extern "C" gsnfs_status gsnfs_octree_encode_static(void *stream, const uint64_t 
     static_init_kernel<<<1, 32, 0, s>>>(dst, vstart, Jd, (uint32_t)nv, J);
     launch_gap_levels(d_codes, nv, gap, s);
     OccupancyOut oo{d_occ, occ_capacity & ~(uint64_t)3, lsz, occ_off, hoff, partials};
-    launch_occupancy(d_codes, gap, vstart, Jd, 1, 64, oo, dst, ds->sms, s);
+    launch_occupancy(d_codes, gap, vstart, Jd, 1, nv, oo, dst, ds->sms, s);
     if (cudaGetLastError() != cudaSuccess) return GSNFS_ERR_CUDA;
 
     uint32_t h_lsz[22];

@@ -99,27 +99,16 @@ __global__ void __launch_bounds__(256) norm_kernel(const uint64_t *occ_off, DevS
     if (s == 0) mode[f] = (n == 0) ? 0u : (distinct == 1 ? 2u : 1u);
 }
 
-__global__ void chunk_offsets_kernel(const uint64_t *occ_off, const uint32_t *mode, uint32_t F, uint32_t chunk,
-                                     uint64_t *chunk_off)
+__global__ void __launch_bounds__(kMaxFrames) chunk_offsets_kernel(const uint64_t *occ_off, const uint32_t *mode, uint32_t F,
+                                                                   uint32_t chunk, uint64_t *chunk_off)
 {
-    if (threadIdx.x) return;
-    uint64_t run = 0;
-    for (uint32_t f = 0; f < F; ++f) {
-        chunk_off[f] = run;
-        uint64_t n = occ_off[f + 1] - occ_off[f];
-        if (mode[f] == 1) run += (n + chunk - 1) / chunk;
-    }
-    chunk_off[F] = run;
-}
-
-__device__ __forceinline__ uint32_t frame_of(const uint64_t *off, uint32_t F, uint64_t x)
-{
-    uint32_t lo = 0, hi = F;
-    while (hi - lo > 1) {
-        uint32_t mid = (lo + hi) >> 1;
-        if (off[mid] <= x) lo = mid; else hi = mid;
-    }
-    return lo;
+    __shared__ uint64_t sh[33];
+    const uint32_t f = threadIdx.x;
+    const uint64_t c = f < F && mode[f] == 1 ? (occ_off[f + 1] - occ_off[f] + chunk - 1) / chunk : 0ull;
+    uint64_t tot;
+    const uint64_t off = block_exclusive_sum<uint64_t>(c, sh, &tot);
+    if (f < F) chunk_off[f] = off;
+    if (f == 0) chunk_off[F] = tot;
 }
 
 // warp per chunk; slot layout: u32 state[32] at 0, u16 word stack [128, 128 + 2*chunk).
@@ -227,42 +216,36 @@ __global__ void __launch_bounds__(32 * kEncWarps) encode_kernel(const uint8_t *_
     }
 }
 
-// per frame (one warp each): chunk positions by a warp scan of the chunk
-// sizes, the occupancy section size and the final mode (rANS only when
-// smaller than raw)
-__global__ void __launch_bounds__(256) section_size_kernel(const uint64_t *occ_off, const uint64_t *chunk_off,
-                                                           uint32_t F, const uint32_t *chunk_words,
-                                                           uint32_t *chunk_pos, uint32_t *mode, uint64_t *sec_bytes)
+// per frame (one CTA each): chunk positions by a scan of the chunk sizes, the
+// occupancy section size and the final mode (rANS only when smaller than raw)
+__global__ void __launch_bounds__(512) section_size_kernel(const uint64_t *occ_off, const uint64_t *chunk_off,
+                                                           const uint32_t *chunk_words, uint32_t *chunk_pos,
+                                                           uint32_t *mode, uint64_t *sec_bytes)
 {
-    const uint32_t f = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const uint32_t lane = threadIdx.x & 31;
-    if (f >= F) return;
+    __shared__ uint64_t sh[33];
+    const uint32_t f = blockIdx.x;
     const uint64_t n = occ_off[f + 1] - occ_off[f];
     const uint64_t raw = 16 + ((n + 7) & ~7ull);
     const uint32_t md = mode[f];
-    if (md == 2) {
-        if (lane == 0) sec_bytes[f] = 16;
-        return;
-    }
+    uint64_t size = md == 2 ? 16 : raw;
     if (md == 1) {
         const uint64_t c0 = chunk_off[f], nch = chunk_off[f + 1] - c0;
         uint64_t t = (16 + 8 + 512 + 4 * nch + 7) & ~7ull;
-        for (uint64_t base = 0; base < nch; base += 32) {
-            const uint64_t c = base + lane;
-            const uint32_t sz = c < nch ? (uint32_t)((128 + 2 * (uint64_t)chunk_words[c0 + c] + 3) & ~3ull) : 0u;
-            const uint32_t inc = warp_inclusive_sum(sz);
-            if (c < nch) chunk_pos[c0 + c] = (uint32_t)(t + inc - sz);
-            t += __shfl_sync(0xFFFFFFFFu, inc, 31);
+        for (uint64_t base = 0; base < nch; base += blockDim.x) {
+            const uint64_t c = base + threadIdx.x;
+            const uint64_t sz = c < nch ? (128 + 2 * (uint64_t)chunk_words[c0 + c] + 3) & ~3ull : 0ull;
+            uint64_t tot;
+            const uint64_t ex = block_exclusive_sum<uint64_t>(sz, sh, &tot);
+            if (c < nch) chunk_pos[c0 + c] = (uint32_t)(t + ex);
+            t += tot;
         }
         t = (t + 7) & ~7ull;
-        if (t < raw) {
-            if (lane == 0) sec_bytes[f] = t;
-            return;
-        }
-        __syncwarp();
-        if (lane == 0) mode[f] = 0;
+        if (t < raw)
+            size = t;
+        else if (threadIdx.x == 0)
+            mode[f] = 0;
     }
-    if (lane == 0) sec_bytes[f] = raw;
+    if (threadIdx.x == 0) sec_bytes[f] = size;
 }
 
 // ---- decoder
@@ -341,7 +324,7 @@ void launch_rans_encode(const RansFrames &r, DevState *st, uint64_t max_chunks, 
     count_launch();
     norm_kernel<<<r.F, 256, 0, s>>>(r.occ_off, st, r.freq, r.cum, r.mode);
     count_launch();
-    chunk_offsets_kernel<<<1, 32, 0, s>>>(r.occ_off, r.mode, r.F, r.chunk, r.chunk_off);
+    chunk_offsets_kernel<<<1, kMaxFrames, 0, s>>>(r.occ_off, r.mode, r.F, r.chunk, r.chunk_off);
     count_launch();
     if (max_chunks) {
         // per frame: enough CTAs to fill the GPU when every frame has chunks, at most one chunk per warp
@@ -354,8 +337,7 @@ void launch_rans_encode(const RansFrames &r, DevState *st, uint64_t max_chunks, 
                                                         r.chunk_top);
         count_launch();
     }
-    section_size_kernel<<<(r.F + 7) / 8, 256, 0, s>>>(r.occ_off, r.chunk_off, r.F, r.chunk_words, r.chunk_pos,
-                                                      r.mode, r.sec_bytes);
+    section_size_kernel<<<r.F, 512, 0, s>>>(r.occ_off, r.chunk_off, r.chunk_words, r.chunk_pos, r.mode, r.sec_bytes);
     count_launch();
 }
 

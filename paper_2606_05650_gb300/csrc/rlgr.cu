@@ -868,20 +868,22 @@ __global__ void __launch_bounds__(512, 2) rlgr_decode_batch_kernel(const DecFram
                          Y + ((uint64_t)d.vstart + row0) * C + c, nullptr, st);
 }
 
-__global__ void job_offsets_kernel(const uint32_t *vstart, uint32_t F, uint32_t B, uint32_t R, uint32_t C,
-                                   uint64_t *job_off, uint64_t *blk_off)
+__global__ void __launch_bounds__(kMaxFrames) job_offsets_kernel(const uint32_t *vstart, uint32_t F, uint32_t B, uint32_t R,
+                                                                 uint32_t C, uint64_t *job_off, uint64_t *blk_off)
 {
-    if (threadIdx.x != 0) return;
-    uint64_t jo = 0, bo = 0;
-    for (uint32_t f = 0; f < F; ++f) {
+    __shared__ uint64_t sh[33];
+    const uint32_t f = threadIdx.x;
+    const uint64_t nb = f < F ? ((uint64_t)(vstart[f + 1] - vstart[f]) + B - 1) / B : 0ull;
+    uint64_t tot;
+    const uint64_t jo = block_exclusive_sum<uint64_t>(nb, sh, &tot);
+    if (f < F) {
         job_off[f] = jo;
-        blk_off[f] = bo;
-        uint64_t nb = ((uint64_t)(vstart[f + 1] - vstart[f]) + B - 1) / B;
-        jo += nb;
-        bo += nb * R * C;
+        blk_off[f] = jo * R * C;
     }
-    job_off[F] = jo;
-    blk_off[F] = bo;
+    if (f == 0) {
+        job_off[F] = tot;
+        blk_off[F] = tot * R * C;
+    }
 }
 
 // dynamic shared memory of a kernel's rings (beside its table it may pass the 48 KB that need no opt-in)
@@ -913,7 +915,7 @@ uint32_t rlgr_slot_words(uint32_t B, bool worst_case)
 void launch_rlgr_offsets(const uint32_t *vstart, uint32_t F, uint32_t B, uint32_t R, uint32_t C, uint64_t *job_off,
                          uint64_t *blk_off, cudaStream_t s)
 {
-    job_offsets_kernel<<<1, 32, 0, s>>>(vstart, F, B, R, C, job_off, blk_off);
+    job_offsets_kernel<<<1, kMaxFrames, 0, s>>>(vstart, F, B, R, C, job_off, blk_off);
     count_launch();
 }
 
