@@ -107,8 +107,8 @@ gsnfs_status gsnfs_graph_stats(gsnfs_ctx *ctx, uint64_t *out);
  * whatever the tiling); only the speed does.  Value 0 restores the built-in
  * default.  Changing one drops the context's captured graphs.
  *   GSNFS_TUNE_RAHT_TILE     RAHT tile size in voxels: power of two in
- *                            [256, 4096] (default: largest whose C rows fit
- *                            56 KB of shared memory, at least 256)
+ *                            [256, 4096] (default: largest up to 1024 whose C
+ *                            rows fit 56 KB of shared memory, at least 256)
  *   GSNFS_TUNE_RAHT_GRID     CTAs per SM of the first transform pass, 1..32 (4)
  *   GSNFS_TUNE_PRELUDE_GRID  CTAs per SM of the prelude tile passes, 1..32 (8)
  *   GSNFS_TUNE_RAHT_PIPE     first pass of FP32 transforms, where its
