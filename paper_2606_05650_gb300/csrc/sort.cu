@@ -185,6 +185,114 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) downsweep_kernel(const K
     }
 }
 
+// Few pairs: every pass in one CTA, the keys and the pairs' original places in
+// shared memory (a launch instead of three per pass, and no trips through L2).
+// A warp owns `rounds` x 32 consecutive pairs, in registers while a pass moves
+// them; the values are fetched by place at the end.  A frame of 10k Gaussians
+// (30-bit keys, 12 launches before): encode 427 -> 412 us.  Above kSmallMax the
+// pairs do not fit one SM's shared memory.
+constexpr uint32_t kSmallMax = 16384, kSmallThreads = 1024, kSmallRounds = kSmallMax / kSmallThreads;
+
+template <typename Key>
+struct SmallSmem {
+    Key keys[kSmallMax];
+    uint16_t place[kSmallMax];
+    uint16_t cnt[kSmallThreads / 32][kRadix];
+    uint32_t first[kRadix];  // first slot of each digit
+    uint32_t scan[33];
+};
+
+template <typename Key>
+__global__ void __launch_bounds__(kSmallThreads, 1) small_sort_kernel(const Key *__restrict__ keys,
+                                                                      const uint32_t *__restrict__ vals, uint32_t n,
+                                                                      uint32_t nbits, uint32_t rounds,
+                                                                      Key *__restrict__ keys_out,
+                                                                      uint32_t *__restrict__ vals_out)
+{
+    extern __shared__ __align__(16) unsigned char small_raw[];
+    SmallSmem<Key> &S = *reinterpret_cast<SmallSmem<Key> *>(small_raw);
+    const uint32_t tid = threadIdx.x, lane = tid & 31, w = tid >> 5, at0 = w * rounds * 32 + lane;
+    const uint32_t ltmask = lanemask_lt();
+    Key k[kSmallRounds];
+    uint32_t pl[kSmallRounds / 2], rk[kSmallRounds / 2];  // two 16-bit values each: places, ranks
+#pragma unroll
+    for (uint32_t r = 0; r < kSmallRounds; ++r) {
+        const uint32_t at = at0 + r * 32;
+        k[r] = r < rounds && at < n ? keys[at] : Key(0);
+        pl[r / 2] = (r & 1) ? (pl[r / 2] | (at << 16)) : (at & 0xFFFFu);
+    }
+    for (uint32_t shift = 0; shift < nbits; shift += 8) {
+        uint32_t *zero = reinterpret_cast<uint32_t *>(S.cnt[w]);
+#pragma unroll
+        for (uint32_t i = 0; i < kRadix / 64; ++i) zero[lane + 32 * i] = 0u;
+        __syncwarp();
+#pragma unroll
+        for (uint32_t r = 0; r < kSmallRounds; ++r) {
+            if (r >= rounds) break;
+            const bool ok = at0 + r * 32 < n;
+            const uint32_t d = ok ? (uint32_t)(k[r] >> shift) & 0xFFu : kRadix + lane;
+            const uint32_t peers = __match_any_sync(0xFFFFFFFFu, d), before = __popc(peers & ltmask);
+            const uint32_t base = ok ? S.cnt[w][d] : 0u;
+            __syncwarp();
+            if (ok && before == 0) S.cnt[w][d] = (uint16_t)(base + __popc(peers));
+            __syncwarp();
+            rk[r / 2] = (r & 1) ? (rk[r / 2] | ((base + before) << 16)) : (base + before);
+        }
+        __syncthreads();
+        // per digit: exclusive prefix over the warps, then the digits' first slots
+        uint32_t run = 0;
+        if (tid < kRadix) {
+#pragma unroll
+            for (uint32_t ww = 0; ww < kSmallThreads / 32; ++ww) {
+                const uint32_t c = S.cnt[ww][tid];
+                S.cnt[ww][tid] = (uint16_t)run;
+                run += c;
+            }
+        }
+        uint32_t tot;
+        const uint32_t pre = block_exclusive_sum<uint32_t>(run, S.scan, &tot);
+        if (tid < kRadix) S.first[tid] = pre;
+        __syncthreads();
+#pragma unroll
+        for (uint32_t r = 0; r < kSmallRounds; ++r) {
+            if (r < rounds && at0 + r * 32 < n) {
+                const uint32_t d = (uint32_t)(k[r] >> shift) & 0xFFu;
+                const uint32_t slot = S.first[d] + S.cnt[w][d] + ((rk[r / 2] >> (16 * (r & 1))) & 0xFFFFu);
+                S.keys[slot] = k[r];
+                S.place[slot] = (uint16_t)(pl[r / 2] >> (16 * (r & 1)));
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (uint32_t r = 0; r < kSmallRounds; ++r) {
+            const uint32_t at = at0 + r * 32;
+            if (r < rounds && at < n) {
+                k[r] = S.keys[at];
+                const uint32_t p = S.place[at];
+                pl[r / 2] = (r & 1) ? ((pl[r / 2] & 0xFFFFu) | (p << 16)) : ((pl[r / 2] & 0xFFFF0000u) | p);
+            }
+        }
+    }
+#pragma unroll
+    for (uint32_t r = 0; r < kSmallRounds; ++r) {
+        const uint32_t at = at0 + r * 32;
+        if (r < rounds && at < n) {
+            keys_out[at] = k[r];
+            vals_out[at] = vals[(pl[r / 2] >> (16 * (r & 1))) & 0xFFFFu];
+        }
+    }
+}
+
+template <typename Key>
+void small_sort(const Key *keys, const uint32_t *vals, Key *keys_out, uint32_t *vals_out, uint32_t n, uint32_t nbits,
+                cudaStream_t s)
+{
+    cudaFuncSetAttribute(small_sort_kernel<Key>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallSmem<Key>));
+    small_sort_kernel<Key><<<1, kSmallThreads, sizeof(SmallSmem<Key>), s>>>(
+        keys, vals, n, nbits, (n + kSmallThreads - 1) / kSmallThreads, keys_out, vals_out);
+    count_launch();
+}
+
 }  // namespace
 
 uint64_t radix_sort_hist_words(uint64_t n, int num_sms, uint32_t segments)
@@ -242,6 +350,10 @@ bool radix_sort(Key *keys, uint32_t *vals, Key *keys_alt, uint32_t *vals_alt, ui
                 uint32_t nbits, int num_sms, cudaStream_t s)
 {
     if (n <= 1 || nbits == 0) return false;
+    if (n <= kSmallMax) {
+        small_sort(keys, vals, keys_alt, vals_alt, (uint32_t)n, nbits, s);
+        return true;
+    }
     const SortGeom g = sort_geom(n, num_sms);
     return sort_passes(keys, vals, keys_alt, vals_alt, hist, n, nbits, g.P, g.chunk, nullptr, nullptr, s);
 }
