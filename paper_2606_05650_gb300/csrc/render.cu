@@ -11,9 +11,9 @@
 // logit 7, SH DC RGB 8-10, SH AC 11-55 as R[15] G[15] B[15].
 //
 // Precision: everything per Gaussian (projection, covariance, conic, tile
-// rectangle, opacity, colour) is evaluated in FP64 and rounded once to FP32
-// for the per-pixel loop, which runs in FP32.  The projected centre is kept
-// as an unevaluated sum of two floats, so a pixel's offset from it is exact
+// rectangle, opacity, colour) is evaluated in FP64, or in double-float where
+// nothing cancels, and rounded once to FP32 for the per-pixel loop, which runs
+// in FP32.  The projected centre is kept as an unevaluated sum of two floats, so a pixel's offset from it is exact
 // to FP32 rounding of the offset itself (a single float would carry an
 // absolute error of its ulp at hundreds of pixels).  The conic enters the
 // loop through its Cholesky factor, conic = L^T L with
@@ -35,29 +35,153 @@ struct Splat {
     uint32_t reach;        // pixels from the centre, in x and (upper half) in y, past which alpha stays below the cut
 };
 
-__device__ __forceinline__ void sh_basis_d(double x, double y, double z, double Y[16])
+// Double-float arithmetic (an unevaluated sum h + l of two floats, about 2^-46
+// relative; the error-free sums of Knuth and products of Dekker, by FMA).  An
+// SM issues an FP64 warp instruction in 16 cycles and four FP32 ones a cycle,
+// and the projection was bound by its FP64 instructions (some 640 a Gaussian):
+// what stays in FP64 is what cancels or decides (camera coordinates,
+// covariance, determinant, footprint), some 220; colour, scales and opacity
+// are double-float and round to the same floats as the FP64 expressions but
+// for about one in a million.  1M Gaussians at 960 x 540: this kernel 381 us,
+// the whole call 2.86 -> 2.08 ms.
+struct Df {
+    float h, l;
+};
+__device__ __forceinline__ Df df_quick(float a, float b)  // |a| >= |b|
 {
-    const double pi = 3.14159265358979323846;
-    const double c0 = 0.5 / sqrt(pi), c1 = sqrt(3.0 / (4.0 * pi));
-    const double c2a = 0.5 * sqrt(15.0 / pi), c2b = 0.25 * sqrt(5.0 / pi), c2c = 0.25 * sqrt(15.0 / pi);
-    const double c3a = 0.25 * sqrt(35.0 / (2.0 * pi)), c3b = 0.5 * sqrt(105.0 / pi);
-    const double c3c = 0.25 * sqrt(21.0 / (2.0 * pi)), c3d = 0.25 * sqrt(7.0 / pi), c3e = 0.25 * sqrt(105.0 / pi);
-    Y[0] = c0;
-    Y[1] = -c1 * y;
-    Y[2] = c1 * z;
-    Y[3] = -c1 * x;
-    Y[4] = c2a * x * y;
-    Y[5] = -c2a * y * z;
-    Y[6] = c2b * (2.0 * z * z - x * x - y * y);
-    Y[7] = -c2a * x * z;
-    Y[8] = c2c * (x * x - y * y);
-    Y[9] = -c3a * y * (3.0 * x * x - y * y);
-    Y[10] = c3b * x * y * z;
-    Y[11] = -c3c * y * (4.0 * z * z - x * x - y * y);
-    Y[12] = c3d * z * (2.0 * z * z - 3.0 * x * x - 3.0 * y * y);
-    Y[13] = -c3c * x * (4.0 * z * z - x * x - y * y);
-    Y[14] = c3e * z * (x * x - y * y);
-    Y[15] = -c3a * x * (x * x - 3.0 * y * y);
+    const float s = __fadd_rn(a, b);
+    return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+__device__ __forceinline__ Df df_sum(float a, float b)
+{
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+}
+__device__ __forceinline__ Df operator+(Df a, Df b)
+{
+    Df s = df_sum(a.h, b.h);
+    const Df t = df_sum(a.l, b.l);
+    s = df_quick(s.h, __fadd_rn(s.l, t.h));
+    return df_quick(s.h, __fadd_rn(s.l, t.l));
+}
+__device__ __forceinline__ Df operator-(Df a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ Df operator-(Df a, Df b) { return a + (-b); }
+__device__ __forceinline__ Df operator*(Df a, Df b)
+{
+    const float p = __fmul_rn(a.h, b.h);
+    const float e = __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -p)));
+    return df_quick(p, e);
+}
+__device__ __forceinline__ Df operator*(Df a, float b)
+{
+    const float p = __fmul_rn(a.h, b);
+    return df_quick(p, __fmaf_rn(a.l, b, __fmaf_rn(a.h, b, -p)));
+}
+__device__ __forceinline__ Df df_of(double x)
+{
+    const float h = (float)x;
+    return {h, (float)(x - (double)h)};
+}
+__host__ __device__ constexpr Df df_const(double x)
+{
+    return {(float)x, (float)(x - (double)(float)x)};
+}
+
+// e^x, |x| <= 80: x = k ln 2 + r (Cody and Waite), Taylor's series of e^r with
+// its terms to r^5 in double-float (the rest is below 3e-6 of the sum)
+__device__ __forceinline__ Df df_exp(float x, int &k)
+{
+    const float kf = rintf(__fmul_rn(x, 1.44269504f));
+    k = (int)kf;
+    constexpr float kLn2Hi = 2839.f / 4096.f;  // the first 12 bits of ln 2: kf * kLn2Hi is exact
+    constexpr Df kLn2Lo = df_const(0.693147180559945309417 - 2839.0 / 4096.0);
+    const Df r = Df{__fmaf_rn(-kf, kLn2Hi, x), 0.f} + kLn2Lo * -kf;
+    float t = 1.f / 479001600.f;
+    t = __fmaf_rn(t, r.h, 1.f / 39916800.f);
+    t = __fmaf_rn(t, r.h, 1.f / 3628800.f);
+    t = __fmaf_rn(t, r.h, 1.f / 362880.f);
+    t = __fmaf_rn(t, r.h, 1.f / 40320.f);
+    t = __fmaf_rn(t, r.h, 1.f / 5040.f);
+    t = __fmaf_rn(t, r.h, 1.f / 720.f);
+    Df s = r * t + df_const(1.0 / 120.0);
+    s = s * r + df_const(1.0 / 24.0);
+    s = s * r + df_const(1.0 / 6.0);
+    s = s * r + Df{0.5f, 0.f};
+    s = s * r + Df{1.f, 0.f};
+    return s * r + Df{1.f, 0.f};
+}
+
+// e^(2 a) in FP64 from a float
+__device__ __forceinline__ double exp_twice(float a)
+{
+    if (!(fabsf(a) <= 40.f)) return exp(2.0 * (double)a);
+    int k;
+    const Df e = df_exp(2.f * a, k);
+    const double d = (double)e.h + (double)e.l;  // in [0.7, 1.42]: the exponent has room for k
+    return __hiloint2double(__double2hiint(d) + k * 0x100000, __double2loint(d));
+}
+
+// 1 / (1 + e^-a), rounded once
+__device__ __forceinline__ float sigmoid(float a)
+{
+    if (!(fabsf(a) <= 60.f)) return (float)(1.0 / (1.0 + exp(-(double)a)));
+    int k;
+    Df e = df_exp(-a, k);
+    const float sc = __int_as_float((127 + k) << 23);  // |k| <= 87
+    e = Df{1.f, 0.f} + Df{__fmul_rn(e.h, sc), __fmul_rn(e.l, sc)};
+    const float q = __frcp_rn(e.h);
+    const Df r = Df{1.f, 0.f} - e * q;  // 1 / e = q + q r + ...
+    return df_quick(q, __fmul_rn(q, r.h)).h;
+}
+
+// degree-3 real SH basis at the unit direction (x, y, z), times the three
+// colours' coefficients (DC at a[8 + c], AC at a[11 + 15 c]), plus 0.5
+constexpr double kPi = 3.14159265358979323846;
+__host__ __device__ constexpr double csqrt_(double x)
+{
+    double r = x > 1 ? x : 1;
+    for (int i = 0; i < 60; ++i) r = 0.5 * (r + x / r);
+    return r;
+}
+
+__device__ __forceinline__ void sh_colour(Df x, Df y, Df z, const float *a, float col[3])
+{
+    constexpr Df c0 = df_const(0.5 / csqrt_(kPi)), c1 = df_const(csqrt_(3.0 / (4.0 * kPi)));
+    constexpr Df c2a = df_const(0.5 * csqrt_(15.0 / kPi)), c2b = df_const(0.25 * csqrt_(5.0 / kPi)),
+                 c2c = df_const(0.25 * csqrt_(15.0 / kPi));
+    constexpr Df c3a = df_const(0.25 * csqrt_(35.0 / (2.0 * kPi))), c3b = df_const(0.5 * csqrt_(105.0 / kPi)),
+                 c3c = df_const(0.25 * csqrt_(21.0 / (2.0 * kPi))), c3d = df_const(0.25 * csqrt_(7.0 / kPi)),
+                 c3e = df_const(0.25 * csqrt_(105.0 / kPi));
+    const Df xx = x * x, yy = y * y, zz = z * z, xy = x * y;
+    const Df dm = xx - yy, dz = zz * 4.f - xx - yy;
+    Df sum[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) sum[c] = c0 * a[8 + c] + Df{0.5f, 0.f};
+    auto add = [&](int k, Df Y) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const float v = a[11 + 15 * c + (k - 1)], p = __fmul_rn(Y.h, v);
+            const Df s = df_sum(sum[c].h, p);
+            sum[c] = df_quick(s.h, __fadd_rn(__fadd_rn(s.l, sum[c].l), __fmaf_rn(Y.l, v, __fmaf_rn(Y.h, v, -p))));
+        }
+    };
+    add(1, -(c1 * y));
+    add(2, c1 * z);
+    add(3, -(c1 * x));
+    add(4, c2a * xy);
+    add(5, -(c2a * (y * z)));
+    add(6, c2b * (zz * 2.f - xx - yy));
+    add(7, -(c2a * (x * z)));
+    add(8, c2c * dm);
+    add(9, -(c3a * (y * (xx * 3.f - yy))));
+    add(10, c3b * (xy * z));
+    add(11, -(c3c * (y * dz)));
+    add(12, c3d * (z * (zz * 2.f - (xx + yy) * 3.f)));
+    add(13, -(c3c * (x * dz)));
+    add(14, c3e * (z * dm));
+    add(15, -(c3a * (x * (xx - yy * 3.f))));
+#pragma unroll
+    for (int c = 0; c < 3; ++c) col[c] = sum[c].h > 0.f ? sum[c].h : 0.f;
 }
 
 __global__ void __launch_bounds__(256) preprocess_kernel(const float *__restrict__ pos,
@@ -76,44 +200,54 @@ __global__ void __launch_bounds__(256) preprocess_kernel(const float *__restrict
                     cam.t[r];
         const double z = pc[2];
         if (!(z > cam.znear)) continue;
+        // rotation of the normalised quaternion: I - (2 / |q|^2) (...)
         double qw = a[3], qx = a[4], qy = a[5], qz = a[6];
-        double qn = sqrt(qw * qw + qx * qx + qy * qy + qz * qz);
-        if (!(qn > 0.0)) {
-            qw = 1.0;
+        double q2 = qw * qw + qx * qx + qy * qy + qz * qz;
+        if (!(q2 > 0.0)) {
+            qw = q2 = 1.0;
             qx = qy = qz = 0.0;
-            qn = 1.0;
         }
-        const double w = qw / qn, x = qx / qn, y = qy / qn, zq = qz / qn;
-        const double Rq[9] = {1 - 2 * (y * y + zq * zq), 2 * (x * y - w * zq), 2 * (x * zq + w * y),
-                              2 * (x * y + w * zq), 1 - 2 * (x * x + zq * zq), 2 * (y * zq - w * x),
-                              2 * (x * zq - w * y), 2 * (y * zq + w * x), 1 - 2 * (x * x + y * y)};
-        const double sc[3] = {exp((double)a[0]), exp((double)a[1]), exp((double)a[2])};
-        double M[9], S[9];
-        for (int r = 0; r < 3; ++r)
-            for (int c = 0; c < 3; ++c) M[3 * r + c] = Rq[3 * r + c] * sc[c];
-        for (int r = 0; r < 3; ++r)
-            for (int c = 0; c < 3; ++c) S[3 * r + c] = M[3 * r] * M[3 * c] + M[3 * r + 1] * M[3 * c + 1] + M[3 * r + 2] * M[3 * c + 2];
-        const double J[6] = {cam.fx / z, 0.0, -cam.fx * pc[0] / (z * z), 0.0, cam.fy / z, -cam.fy * pc[1] / (z * z)};
-        double T[6], TS[6];
-        for (int r = 0; r < 2; ++r)
-            for (int c = 0; c < 3; ++c)
-                T[3 * r + c] = J[3 * r] * cam.R[c] + J[3 * r + 1] * cam.R[3 + c] + J[3 * r + 2] * cam.R[6 + c];
-        for (int r = 0; r < 2; ++r)
-            for (int c = 0; c < 3; ++c) TS[3 * r + c] = T[3 * r] * S[c] + T[3 * r + 1] * S[3 + c] + T[3 * r + 2] * S[6 + c];
-        const double ca = TS[0] * T[0] + TS[1] * T[1] + TS[2] * T[2] + 0.3;
-        const double cb = TS[0] * T[3] + TS[1] * T[4] + TS[2] * T[5];
-        const double cc = TS[3] * T[3] + TS[4] * T[4] + TS[5] * T[5] + 0.3;
+        const double s2 = 2.0 / q2;
+        const double sx = s2 * qx, sy = s2 * qy, sz = s2 * qz;
+        const double xx = sx * qx, yy = sy * qy, zz = sz * qz, xy = sx * qy, xz = sx * qz, yz = sy * qz, wx = sx * qw,
+                     wy = sy * qw, wz = sz * qw;
+        const double Rq[9] = {1 - (yy + zz), xy - wz, xz + wy, xy + wz, 1 - (xx + zz), yz - wx, xz - wy, yz + wx,
+                              1 - (xx + yy)};
+        const double v2[3] = {exp_twice(a[0]), exp_twice(a[1]), exp_twice(a[2])};  // squared scales
+        // 2-D covariance N diag(v2) N^T, N = J W Rq
+        const double iz = 1.0 / z, jx = cam.fx * iz, jy = cam.fy * iz;
+        const double ux = jx * pc[0], vy = jy * pc[1], jxz = -ux * iz, jyz = -vy * iz;
+        double N0[3], N1[3], T0[3], T1[3];
+        for (int c = 0; c < 3; ++c) {
+            T0[c] = jx * cam.R[c] + jxz * cam.R[6 + c];
+            T1[c] = jy * cam.R[3 + c] + jyz * cam.R[6 + c];
+        }
+        for (int c = 0; c < 3; ++c) {
+            N0[c] = T0[0] * Rq[c] + T0[1] * Rq[3 + c] + T0[2] * Rq[6 + c];
+            N1[c] = T1[0] * Rq[c] + T1[1] * Rq[3 + c] + T1[2] * Rq[6 + c];
+        }
+        double ca = 0.3, cb = 0.0, cc = 0.3;
+        for (int c = 0; c < 3; ++c) {
+            const double w0 = v2[c] * N0[c], w1 = v2[c] * N1[c];
+            ca += w0 * N0[c];
+            cb += w0 * N1[c];
+            cc += w1 * N1[c];
+        }
         const double det = ca * cc - cb * cb;
         if (!(det > 0.0)) continue;
         // conic Q = [[cc, -cb], [-cb, ca]] / det; Q = L^T L with L = [[l1, l2], [0, l3]]
-        const double q00 = cc / det, q01 = -cb / det;
-        const double l1 = sqrt(q00), l2 = q01 / l1, l3 = sqrt(1.0 / (det * q00));  // det(Q) = 1 / det
-        const double mid = 0.5 * (ca + cc);
-        const double disc = mid * mid - det;
-        const double lmax = mid + sqrt(disc > 0.1 ? disc : 0.1);
-        const double rad = ceil(3.0 * sqrt(lmax));
-        const double u = cam.fx * pc[0] / z + cam.cx, v = cam.fy * pc[1] / z + cam.cy;
-        const float opacity = (float)(1.0 / (1.0 + exp(-(double)a[7])));
+        const double l3 = rsqrt(cc), g = l3 * rsqrt(det);
+        const double l1 = cc * g, l2 = -cb * g;
+        // footprint radius ceil(3 sqrt(largest eigenvalue)): in FP32 unless that is too near an integer to tell
+        const float caf = (float)ca, ccf = (float)cc, cbf = (float)cb, half = 0.5f * (caf - ccf);
+        const float r3 = 3.f * sqrtf(0.5f * (caf + ccf) + sqrtf(fmaxf(half * half + cbf * cbf, 0.1f)));
+        double rad = ceil((double)r3);
+        if (!(fabsf(r3 - rintf(r3)) > 4e-6f * r3 + 1e-6f)) {
+            const double mid = 0.5 * (ca + cc), disc = mid * mid - det;
+            rad = ceil(3.0 * sqrt(mid + sqrt(disc > 0.1 ? disc : 0.1)));
+        }
+        const double u = ux + cam.cx, v = vy + cam.cy;
+        const float opacity = sigmoid(a[7]);
         // Past |d_x| = sqrt(c cov_xx) the exponent d^T conic d is above c whatever d_y is, so with
         // c = 2 ln(255 opacity) alpha stays below 1/255 there and the splat changes no pixel; likewise in y.  The
         // margins cover the FP32 rounding of the per-pixel exponent, whose relative error grows with
@@ -123,13 +257,14 @@ __global__ void __launch_bounds__(256) preprocess_kernel(const float *__restrict
         if (ca * cc < 1e8 * det) {
             if (opacity * 255.f < 0.9999f) continue;
             const float c = 2.04f * fmaxf(logf(opacity * 255.f), 0.f) + 0.1f;
-            reach_x = sqrtf(c * (float)ca) * 1.0001f;
-            reach_y = sqrtf(c * (float)cc) * 1.0001f;
+            reach_x = sqrtf(c * caf) * 1.0001f;
+            reach_y = sqrtf(c * ccf) * 1.0001f;
             rx = fmin(rad, (double)reach_x);
             ry = fmin(rad, (double)reach_y);
         }
-        int tx0 = (int)floor((u - rx) / kTile), tx1 = (int)floor((u + rx) / kTile);
-        int ty0 = (int)floor((v - ry) / kTile), ty1 = (int)floor((v + ry) / kTile);
+        static_assert(kTile == 16, "tile of a pixel coordinate by a shift");
+        int tx0 = __double2int_rd(u - rx) >> 4, tx1 = __double2int_rd(u + rx) >> 4;
+        int ty0 = __double2int_rd(v - ry) >> 4, ty1 = __double2int_rd(v + ry) >> 4;
         tx0 = max(tx0, 0);
         ty0 = max(ty0, 0);
         tx1 = min(tx1, cam.TX - 1);
@@ -144,18 +279,11 @@ __global__ void __launch_bounds__(256) preprocess_kernel(const float *__restrict
         s.l2 = (float)l2;
         s.l3 = (float)l3;
         s.opacity = opacity;
-        double d[3] = {(double)p[0] - cam.campos[0], (double)p[1] - cam.campos[1], (double)p[2] - cam.campos[2]};
-        const double dn = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-        const double id = dn > 0.0 ? 1.0 / dn : 1.0;
-        double Y[16];
-        sh_basis_d(d[0] * id, d[1] * id, d[2] * id, Y);
+        const double d[3] = {(double)p[0] - cam.campos[0], (double)p[1] - cam.campos[1], (double)p[2] - cam.campos[2]};
+        const double d2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+        const double id = d2 > 0.0 ? rsqrt(d2) : 1.0;
         float col[3];
-        for (int c = 0; c < 3; ++c) {
-            double val = Y[0] * (double)a[8 + c];
-            for (int k = 1; k < 16; ++k) val += Y[k] * (double)a[11 + 15 * c + (k - 1)];
-            val += 0.5;
-            col[c] = val > 0.0 ? (float)val : 0.f;
-        }
+        sh_colour(df_of(d[0] * id), df_of(d[1] * id), df_of(d[2] * id), a, col);
         s.r = col[0];
         s.g = col[1];
         s.b = col[2];
