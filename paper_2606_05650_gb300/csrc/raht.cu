@@ -460,7 +460,8 @@ __global__ void __launch_bounds__(kThreads) prelude_compact_kernel(PreludeArgs a
                          tiles_per_cta(a.p.passes[q].ntiles, tile_ctas));
 }
 
-// remaining passes inside one CTA
+// remaining passes inside one CTA: a tile at a time by the whole CTA, or by
+// its warps where a pass has more tiles than that is worth
 template <int TMAX>
 __global__ void __launch_bounds__(kThreads) prelude_finish_kernel(PreludeArgs a, int q0)
 {
@@ -469,10 +470,10 @@ __global__ void __launch_bounds__(kThreads) prelude_finish_kernel(PreludeArgs a,
     for (int q = q0; q + 1 < kRahtMaxPasses; ++q) {
         const RahtPass ps = a.p.passes[q];
         if (ps.n == 0) break;
-        if constexpr (kWarpTiles<TMAX>) {
+        if (kWarpTiles<TMAX> && ps.ntiles > 4) {
             const uint32_t wid = threadIdx.x >> 5;
             const WarpGroup G{threadIdx.x & 31u, 0u};
-            for (uint32_t t = wid; t < ps.ntiles; t += kThreads / 32) prelude_tile(a, S[wid], q, ps, t, G);
+            for (uint32_t t = wid; t < ps.ntiles; t += kThreads / 32) prelude_tile(a, S[kWarpTiles<TMAX> ? wid : 0u], q, ps, t, G);
         } else {
             const CtaGroup G{threadIdx.x, threadIdx.x >> 5};
             for (uint32_t t = 0; t < ps.ntiles; ++t) prelude_tile(a, S[0], q, ps, t, G);
@@ -483,6 +484,19 @@ __global__ void __launch_bounds__(kThreads) prelude_finish_kernel(PreludeArgs a,
         prelude_compact_body(a, q, threadIdx.x >> 5, kThreads / 32, ps.ntiles);
         __syncthreads();
     }
+}
+
+// Passes launched grid-wide, the rest run in one CTA: a pass has about a 26th
+// of the tiles of the one before, so that with at most 64 tiles in the first
+// the later ones are one to three tiles, for which a launch (three in the
+// prelude) costs more than it saves.  10k Gaussians: encode 412 -> 390 us,
+// decode 347 -> 328 us.  Two wide passes up to 2000 tiles lost: the last kernel
+// then walks up to three tiles of 56 channels one by one (500k rows, two
+// forward and two inverse transforms: 375 -> 425 us).
+int grid_passes(uint64_t nv_bound, uint32_t T)
+{
+    const uint64_t tiles = (nv_bound + T - 1) / T;
+    return tiles <= 64 ? 1 : kRahtMultiPasses;
 }
 
 // ----------------------------------------------------------- transform ---
@@ -1396,7 +1410,8 @@ void forward_all(const XformArgs<S> &A, uint64_t nv_bound, int num_sms, cudaStre
     uint64_t tiles = (nv_bound + T - 1) / T;
     const uint64_t gcap = (uint64_t)num_sms * (A.p.xgrid_mult ? A.p.xgrid_mult : 4u);
     uint32_t grid0 = (uint32_t)(tiles < 1 ? 1 : (tiles < gcap ? tiles : gcap));
-    for (int q = 0; q < kRahtMultiPasses; ++q) {
+    const int wide = grid_passes(nv_bound, T);
+    for (int q = 0; q < wide; ++q) {
         uint32_t g = q == 0 ? grid0 : (grid0 < (uint32_t)num_sms ? grid0 : (uint32_t)num_sms);
         if (q == 0) stage_begin(s, kStRahtFwd0);
         size_t psm = 0;
@@ -1417,7 +1432,7 @@ void forward_all(const XformArgs<S> &A, uint64_t nv_bound, int num_sms, cudaStre
             launch_pass<S, false, VEC, false, false>(A, q, g, smem, s);
         if (q == 0) stage_end(s, kStRahtFwd0);
     }
-    launch_finish<S, false, VEC, false>(A, kRahtMultiPasses, smem, s);
+    launch_finish<S, false, VEC, false>(A, wide, smem, s);
 }
 
 template <typename S, int VEC>
@@ -1429,11 +1444,12 @@ void inverse_all(const XformArgs<S> &A, uint64_t nv_bound, int num_sms, cudaStre
     const uint64_t gcap = (uint64_t)num_sms * (A.p.xgrid_mult ? A.p.xgrid_mult : 4u);
     uint32_t grid0 = (uint32_t)(tiles < 1 ? 1 : (tiles < gcap ? tiles : gcap));
     const bool qd = A.io.inv_step != nullptr;
+    const int wide = grid_passes(nv_bound, T);
     if (qd)
-        launch_finish<S, true, VEC, true>(A, kRahtMultiPasses, smem, s);
+        launch_finish<S, true, VEC, true>(A, wide, smem, s);
     else
-        launch_finish<S, true, VEC, false>(A, kRahtMultiPasses, smem, s);
-    for (int q = kRahtMultiPasses - 1; q >= 0; --q) {
+        launch_finish<S, true, VEC, false>(A, wide, smem, s);
+    for (int q = wide - 1; q >= 0; --q) {
         uint32_t g = q == 0 ? grid0 : (grid0 < (uint32_t)num_sms ? grid0 : (uint32_t)num_sms);
         if (q == 0) stage_begin(s, kStRahtInv0);
         size_t psm = 0;
@@ -1503,7 +1519,8 @@ void prelude_launches(const PreludeArgs &a, const RahtPlanDev &p, const DevState
     // 124 / 96 us, 1M 155 / 146 us; 16 frames of 1M take the warps (0.39 ms).
     constexpr uint64_t kCtaWaves = 4;
     uint64_t tiles = (nv_bound + p.T - 1) / p.T;
-    for (int q = 0; q < kRahtMultiPasses; ++q, tiles = tiles / 4 + 1) {
+    const int wide = grid_passes(nv_bound, p.T);
+    for (int q = 0; q < wide; ++q, tiles = tiles / 4 + 1) {
         const bool few = tiles <= (uint64_t)grid * kCtaWaves;
         const uint32_t g = few && tiles < grid ? (tiles ? (uint32_t)tiles : 1u) : grid;
         if (kWarpTiles<TMAX> && !few)
@@ -1513,7 +1530,7 @@ void prelude_launches(const PreludeArgs &a, const RahtPlanDev &p, const DevState
         prelude_compact_kernel<<<g, kThreads, 0, s>>>(a, q, g);
         count_launch();
     }
-    prelude_finish_kernel<TMAX><<<1, kThreads, smem, s>>>(a, kRahtMultiPasses);
+    prelude_finish_kernel<TMAX><<<1, kThreads, smem, s>>>(a, wide);
     count_launch();
 }
 
