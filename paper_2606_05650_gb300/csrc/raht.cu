@@ -941,12 +941,14 @@ __global__ void __launch_bounds__(kXThreads, 3) xform_finish_kernel(XformArgs<S>
 }
 
 // ---- software-pipelined first pass (FP32, whole rows in shared memory) -----
-// A CTA walks its tiles (blockIdx.x + k * gridDim.x) with NR row buffers and
-// NR + 1 metadata buffers, loads issued as cp.async groups ahead of use:
-//   NR = 1 (three CTAs per SM): the metadata of tile k + 1 lands while tile k
-//          is transformed; tile k + 1's rows are issued once tile k is stored;
-//   NR = 3 (one CTA per SM): the rows of tiles k + 1 and k + 2 and the
-//          metadata of tile k + 3 are in flight while tile k is transformed.
+// A CTA walks its tiles with NR row buffers and NR + 1 metadata buffers, loads
+// issued as cp.async groups ahead of use:
+//   NR = 1 (xform_first_kernel, three CTAs per SM): the metadata of tile k + 1
+//          lands while tile k is transformed; tile k + 1's rows are issued once
+//          tile k is stored;
+//   NR = 3 (xform_pipe_kernel, one CTA per SM): the rows of tiles k + 1 and
+//          k + 2 and the metadata of tile k + 3 are in flight while tile k is
+//          transformed.
 // Per tile the arithmetic is that of xform_tile, in the same order, so the
 // results are bit-identical.
 
@@ -1237,7 +1239,7 @@ __device__ void pipe_compute(const XformArgs<float> &A, const RahtPass &ps, cons
 }
 
 template <int NR, bool INV, bool GATHER, bool QDQ>
-__global__ void __launch_bounds__(kXThreads, NR == 1 ? 3 : 1) xform_pipe_kernel(XformArgs<float> A)
+__global__ void __launch_bounds__(kXThreads, 1) xform_pipe_kernel(XformArgs<float> A)
 {
     constexpr uint32_t NM = NR + 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1251,77 +1253,328 @@ __global__ void __launch_bounds__(kXThreads, NR == 1 ? 3 : 1) xform_pipe_kernel(
     auto rows = [&](uint32_t k) { return reinterpret_cast<float *>(smem_raw + (size_t)(k % NR) * rowb); };
     auto meta = [&](uint32_t k) { return pipe_stage(smem_raw + NR * rowb + (size_t)(k % NM) * metab, T); };
     uint32_t klt_fr = 0xFFFFFFFFu;
-    if constexpr (NR == 1) {
-        // Tiles are claimed from a global counter as the CTA goes (the next but one while the current one is
-        // transformed), so a CTA that starts late or runs slow (its SM shared with other work) takes fewer
-        // tiles; the claims ascend, so a claim past the last tile ends the CTA's loop.
-        __shared__ uint32_t s_claim[4];
-        if (threadIdx.x == 0) {
-            s_claim[0] = atomicAdd(A.p.pipe_ctr, 1u);
-            s_claim[1] = atomicAdd(A.p.pipe_ctr, 1u);
-        }
-        __syncthreads();
-        if (s_claim[0] < nt) pipe_issue_meta<GATHER>(A, ps, s_claim[0], meta(0));
-        if (s_claim[1] < nt) pipe_issue_meta<GATHER>(A, ps, s_claim[1], meta(1));
-        cp_async_commit();
-        cp_async_wait<0>();
-        __syncthreads();
-        if (s_claim[0] < nt) pipe_issue_rows<INV, GATHER>(A, ps, nx, s_claim[0], meta(0), rows(0));
-        cp_async_commit();
-        for (uint32_t k = 0;; ++k) {
-            const uint32_t tk = s_claim[k & 3];
-            if (tk >= nt) break;
-            // complete: rows of tile k, metadata of tile k + 1.  Without colour transforms no barrier is needed
-            // here: a thread first touches only the row chunks it copied itself (same thread-to-chunk mapping
-            // for the copy and the finishing step, complete for it after its own wait), tile k's metadata became
-            // visible at the previous tile's first barrier, and the barrier before the rounds orders the rest.
-            cp_async_wait<0>();
-            if (A.io.klt) __syncthreads();  // the colour steps read other threads' rows
-            pipe_compute<INV, GATHER, QDQ>(A, ps, nx, tk, meta(k), rows(k), klt_s, klt_fr);
-            if (threadIdx.x == 0) s_claim[(k + 2) & 3] = atomicAdd(A.p.pipe_ctr, 1u);
-            __syncthreads();  // the row buffer and tile k's metadata are free; the new claim is visible
-            const uint32_t t1 = s_claim[(k + 1) & 3], t2 = s_claim[(k + 2) & 3];
-            if (t2 < nt) pipe_issue_meta<GATHER>(A, ps, t2, meta(k + 2));
-            if (t1 < nt) pipe_issue_rows<INV, GATHER>(A, ps, nx, t1, meta(k + 1), rows(k + 1));
-            cp_async_commit();
-        }
-        cp_async_wait<0>();
-        if (threadIdx.x == 0) {  // the last CTA to finish leaves the counters at zero for the next launch
-            __threadfence();
-            if (atomicAdd(A.p.pipe_ctr + 1, 1u) == gridDim.x - 1) {
-                A.p.pipe_ctr[0] = 0;
-                A.p.pipe_ctr[1] = 0;
-                __threadfence();
-            }
-        }
-        return;
-    }
     // prologue: metadata of tiles 0 .. NR - 1, then the rows of tiles 0 .. NR - 2
-    constexpr uint32_t kMeta0 = NR == 1 ? 2u : NR, kRows0 = NR == 1 ? 1u : NR - 1;
-    for (uint32_t k = 0; k < kMeta0 && k < cnt; ++k) pipe_issue_meta<GATHER>(A, ps, b + k * G, meta(k));
+    for (uint32_t k = 0; k < NR && k < cnt; ++k) pipe_issue_meta<GATHER>(A, ps, b + k * G, meta(k));
     cp_async_commit();
     cp_async_wait<0>();
     __syncthreads();
-    for (uint32_t k = 0; k < kRows0; ++k) {
+    for (uint32_t k = 0; k < NR - 1; ++k) {
         if (k < cnt) pipe_issue_rows<INV, GATHER>(A, ps, nx, b + k * G, meta(k), rows(k));
         cp_async_commit();
     }
     for (uint32_t k = 0; k < cnt; ++k) {
-        if constexpr (NR == 1) {
-            break;  // tiles are claimed dynamically below
-        } else {
-            // complete: rows of tile k, metadata of tile k + NR - 1 (only the rows of k + NR - 2 may still fly)
-            cp_async_wait<1>();
-            __syncthreads();
-            if (k + NR < cnt) pipe_issue_meta<GATHER>(A, ps, b + (k + NR) * G, meta(k + NR));
-            cp_async_commit();
-            if (k + NR - 1 < cnt)
-                pipe_issue_rows<INV, GATHER>(A, ps, nx, b + (k + NR - 1) * G, meta(k + NR - 1), rows(k + NR - 1));
-            cp_async_commit();
-            pipe_compute<INV, GATHER, QDQ>(A, ps, nx, b + k * G, meta(k), rows(k), klt_s, klt_fr);
-        }
+        // complete: rows of tile k, metadata of tile k + NR - 1 (only the rows of k + NR - 2 may still fly)
+        cp_async_wait<1>();
+        __syncthreads();
+        if (k + NR < cnt) pipe_issue_meta<GATHER>(A, ps, b + (k + NR) * G, meta(k + NR));
+        cp_async_commit();
+        if (k + NR - 1 < cnt)
+            pipe_issue_rows<INV, GATHER>(A, ps, nx, b + (k + NR - 1) * G, meta(k + NR - 1), rows(k + NR - 1));
+        cp_async_commit();
+        pipe_compute<INV, GATHER, QDQ>(A, ps, nx, b + k * G, meta(k), rows(k), klt_s, klt_fr);
     }
     cp_async_wait<0>();
+}
+
+// ---- the same with one row buffer (three CTAs per SM), the form the codec runs ----
+// Bound by instruction issue and by the rounds' barriers rather than by HBM:
+// of 28,000 warp instructions a tile (forward, 56 channels) 4,000 were
+// butterflies.  So everything that a thread needs in every tile (its row slot
+// and column, the column's base pointers) is computed once; a tile that lies in
+// one frame, all but one per frame, looks up its frame once, not per row; row
+// slots are a power of two where the columns allow it (56 channels: 32 slots x 14 columns
+// = 448 threads, none idle, and eight more registers a thread than 512 leave).
+// Per tile the arithmetic is that of xform_tile, in the same order, so the
+// results are bit-identical.  16 x 1M frames: forward 2.09 -> 1.70 ms, inverse
+// 1.33 -> 1.21 ms (7.2 GB of rows read and written: 4.2 and 5.9 TB/s).
+struct FirstStage {
+    float2 *ab;      // T: butterfly coefficients
+    uint32_t *io;    // T: row destination (forward) or source (inverse)
+    uint32_t *row0;  // T: input row of the voxel's first point | kCarry (forward gather)
+    uint32_t *idx;   // T: butterfly i0 | i1 << 16
+    uint16_t *re;    // kRounds: end of each round
+    uint32_t *cnt;   // 2: butterflies, rounds
+    uint64_t *code;  // 2: codes of the first and the last voxel (forward gather of several frames)
+};
+
+__host__ __device__ inline size_t first_meta_bytes(uint32_t T) { return ((size_t)20 * T + 2 * kRounds + 32 + 15) & ~(size_t)15; }
+__host__ __device__ inline size_t first_smem(uint32_t T, uint32_t C, bool color)
+{
+    return (size_t)T * C * 4 + 2 * first_meta_bytes(T) + (color ? 4 * (size_t)kKltFloats + 16 : 0);
+}
+
+__device__ __forceinline__ FirstStage first_stage(unsigned char *base, uint32_t T)
+{
+    FirstStage s;
+    s.ab = reinterpret_cast<float2 *>(base);
+    s.io = reinterpret_cast<uint32_t *>(base + 8 * (size_t)T);
+    s.row0 = s.io + T;
+    s.idx = s.row0 + T;
+    s.re = reinterpret_cast<uint16_t *>(base + 20 * (size_t)T);
+    s.cnt = reinterpret_cast<uint32_t *>(base + 20 * (size_t)T + 2 * kRounds);
+    s.code = reinterpret_cast<uint64_t *>(base + 20 * (size_t)T + 2 * kRounds + 16);
+    return s;
+}
+
+template <bool INV, bool GATHER, bool QDQ, bool COLOR, int THREADS>
+__global__ void __launch_bounds__(THREADS, 3) xform_first_kernel(XformArgs<float> A, uint32_t slots)
+{
+    typedef Vec<float, 4> V4;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ uint32_t s_claim[4];
+    const RahtPlanDev &p = A.p;
+    const RahtIO &io = A.io;
+    const RahtPass ps = p.passes[0];
+    const uint32_t T = p.T, C = io.C, nt = ps.ntiles;
+    const uint32_t tid = threadIdx.x, L = C / 4, slot = tid / L, c = 4 * (tid - slot * L);
+    const bool act = slot < slots;
+    const uint32_t rs = 4 * C, sb = smem_addr(smem_raw) + 4 * c;  // row stride and this column's first row, in bytes
+    unsigned char *const meta0 = smem_raw + (size_t)T * rs;
+    const uint32_t metab = (uint32_t)first_meta_bytes(T);
+    float *const rows = reinterpret_cast<float *>(smem_raw);
+    float *const klt_s = reinterpret_cast<float *>(meta0 + 2 * metab);
+    float *const Yc = io.Y + c, *const poolc = io.pool + (uint64_t)p.passes[1].surv_off * C + c;
+    const bool frames = GATHER && io.frame_shift < 64;
+    uint32_t klt_fr = 0xFFFFFFFFu;
+
+    auto meta = [&](uint32_t k) { return first_stage(meta0 + (k & 1u) * metab, T); };
+    auto size_of = [&](uint32_t t) { return min(ps.n - t * T, T); };
+    auto issue_meta = [&](uint32_t t, const FirstStage &M) {
+        const uint32_t m = size_of(t), j0 = t * T;
+        for (uint32_t i = tid; i < T; i += THREADS) {
+            if (i < m) {
+                cp_async_vec<4>(M.io + i, p.dest + j0 + i);
+                if (GATHER) cp_async_vec<4>(M.row0 + i, io.row0 + j0 + i);
+            }
+            // whole schedule arrays: the count is not known yet, the entries past it are never read
+            cp_async_vec<4>(M.idx + i, p.bf_idx + (uint64_t)j0 + i);
+            cp_async_vec<8>(M.ab + i, p.bf_ab + (uint64_t)j0 + i);
+        }
+        if (tid < 2 * kRounds / 16)
+            cp_async_vec<16>(reinterpret_cast<unsigned char *>(M.re) + 16 * tid,
+                             reinterpret_cast<const unsigned char *>(p.round_end + (uint64_t)t * kRounds) + 16 * tid);
+        if (tid == 0) {
+            cp_async_vec<4>(M.cnt, p.tile_nbf + t);
+            cp_async_vec<4>(M.cnt + 1, p.tile_nr + t);
+            if (frames) {
+                cp_async_vec<8>(M.code, io.codes + j0);
+                cp_async_vec<8>(M.code + 1, io.codes + j0 + m - 1);
+            }
+        }
+    };
+    auto frame_of = [&](const FirstStage &M) { return frames ? (uint32_t)(uint8_t)(M.code[0] >> io.frame_shift) : 0u; };
+    auto one_frame = [&](const FirstStage &M) { return !frames || ((M.code[0] ^ M.code[1]) >> io.frame_shift) == 0; };
+    auto row_frame = [&](uint32_t j) { return (uint32_t)(uint8_t)(io.codes[j] >> io.frame_shift); };
+    auto issue_rows = [&](uint32_t t, const FirstStage &M) {
+        if (!act) return;
+        const uint32_t m = size_of(t), j0 = t * T, step = slots * rs;
+        uint32_t sa = sb + slot * rs;
+        if (INV) {
+            for (uint32_t i = slot; i < m; i += slots, sa += step) {
+                const uint32_t d = M.io[i];
+                cp_async16_s(sa, ((d & kCarry) ? poolc : Yc) + (uint64_t)(d & ~kCarry) * C);
+            }
+        } else if (!GATHER) {
+            const float *src = io.in + (uint64_t)(j0 + slot) * C + c;
+            for (uint32_t i = slot; i < m; i += slots, sa += step, src += slots * C) cp_async16_s(sa, src);
+        } else if (one_frame(M)) {
+            const float *base = io.attr[frame_of(M)] + c;
+            for (uint32_t i = slot; i < m; i += slots, sa += step)
+                cp_async16_s(sa, base + (uint64_t)(M.row0[i] & ~kCarry) * C);
+        } else {
+            for (uint32_t i = slot; i < m; i += slots, sa += step)
+                cp_async16_s(sa, io.attr[row_frame(j0 + i)] + c + (uint64_t)(M.row0[i] & ~kCarry) * C);
+        }
+    };
+    // rows of tile t: cluster average and centring (forward), quantise -> dequantise (inverse); each thread on the
+    // 16-byte chunks that it copied
+    auto finish_rows = [&](uint32_t t, const FirstStage &M) {
+        if (!act) return;
+        const uint32_t m = size_of(t), j0 = t * T;
+        if (!INV && GATHER) {
+            const bool centred = io.center != nullptr && !COLOR, one = one_frame(M);
+            uint32_t fr = frame_of(M);
+            float4 ctr = centred ? V4::ld(io.center + (uint64_t)fr * C + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+            for (uint32_t i = slot; i < m; i += slots) {
+                const bool multi = (M.row0[i] & kCarry) != 0;
+                if (!multi && !centred) continue;
+                if (!one) {
+                    fr = row_frame(j0 + i);
+                    if (centred) ctr = V4::ld(io.center + (uint64_t)fr * C + c);
+                }
+                const uint32_t pr = sb + i * rs;
+                float4 acc = lds4(pr);
+                if (multi) {  // voxels holding several points: average in input order
+                    const uint32_t s0 = io.seg[j0 + i], s1 = io.seg[j0 + i + 1];
+                    const float *base = io.attr[fr] + c;
+                    for (uint32_t g = s0 + 1; g < s1; ++g) {
+                        const float4 xv = V4::ld(base + (uint64_t)io.vals[g] * C);
+                        acc = make_float4(add_rn(acc.x, xv.x), add_rn(acc.y, xv.y), add_rn(acc.z, xv.z), add_rn(acc.w, xv.w));
+                    }
+                    const float n = (float)(s1 - s0);
+                    acc = make_float4(div_rn(acc.x, n), div_rn(acc.y, n), div_rn(acc.z, n), div_rn(acc.w, n));
+                }
+                if (centred)  // centred rows keep the low-pass sums small (FP32 accuracy)
+                    acc = make_float4(add_rn(acc.x, -ctr.x), add_rn(acc.y, -ctr.y), add_rn(acc.z, -ctr.z), add_rn(acc.w, -ctr.w));
+                sts4(pr, acc);
+            }
+        } else if (INV && QDQ) {
+            const float4 inv = V4::ld(io.inv_step + c), stp = V4::ld(io.step + c);
+            for (uint32_t i = slot; i < m; i += slots) {
+                if (M.io[i] & kCarry) continue;
+                const uint32_t pr = sb + i * rs;
+                const float4 v = lds4(pr);
+                sts4(pr, make_float4(qdq(v.x, inv.x, stp.x, io.tau), qdq(v.y, inv.y, stp.y, io.tau),
+                                     qdq(v.z, inv.z, stp.z, io.tau), qdq(v.w, inv.w, stp.w, io.tau)));
+            }
+        }
+    };
+    // colour mode: the KLT of the tile's first frame, staged once per change of frame
+    auto stage_klt = [&](uint32_t kfr) {
+        if (kfr == klt_fr) return;
+        __syncthreads();  // the previous tile's readers of klt_s are done
+        for (uint32_t k = tid; k < (uint32_t)kKltFloats; k += THREADS) klt_s[k] = io.klt[(uint64_t)kfr * kKltFloats + k];
+        klt_fr = kfr;
+        __syncthreads();
+    };
+    auto klt_of = [&](uint32_t fr, uint32_t ch) {
+        return (fr == klt_fr ? klt_s : io.klt + (uint64_t)fr * kKltFloats) + ch * kKltN * kKltN;
+    };
+    auto colour_forward = [&](uint32_t t, const FirstStage &M) {  // of whole rows, then centring
+        const uint32_t m = size_of(t), j0 = t * T;
+        const bool one = one_frame(M);
+        const uint32_t f0 = frame_of(M);
+        __syncthreads();
+        for (uint32_t e = tid; e < m * 16; e += THREADS) color_yuv_task(rows + (uint64_t)(e >> 4) * C, (int)(e & 15), kYuvFwd);
+        __syncthreads();
+        for (uint32_t e = tid; e < m * 3; e += THREADS) {
+            const uint32_t i = e / 3, ch = e - 3 * i;
+            color_klt_task<false>(rows + (uint64_t)i * C, (int)ch, klt_of(one ? f0 : row_frame(j0 + i), ch));
+        }
+        if (io.center) {
+            __syncthreads();
+            for (uint32_t e = tid; e < m * C; e += THREADS) {
+                const uint32_t i = e / C, cc = e - i * C;
+                const uint32_t fr = one ? f0 : row_frame(j0 + i);
+                rows[e] = __fadd_rn(rows[e], -io.center[(uint64_t)fr * C + cc]);
+            }
+        }
+    };
+    auto colour_inverse = [&](uint32_t t) {
+        const uint32_t m = size_of(t), j0 = t * T;
+        for (uint32_t e = tid; e < m * 3; e += THREADS) {
+            const uint32_t i = e / 3, ch = e - 3 * i;
+            const uint32_t fr = frame_of_voxel(io.vstart, io.F, j0 + i);
+            if (io.frame_color && !io.frame_color[fr]) continue;
+            color_klt_task<true>(rows + (uint64_t)i * C, (int)ch, klt_of(fr, ch));
+        }
+        __syncthreads();
+        for (uint32_t e = tid; e < m * 16; e += THREADS) {
+            const uint32_t i = e >> 4;
+            const uint32_t fr = io.F > 1 ? frame_of_voxel(io.vstart, io.F, j0 + i) : 0u;
+            if (io.frame_color && !io.frame_color[fr]) continue;
+            color_yuv_task(rows + (uint64_t)i * C, (int)(e & 15), io.yuv_inv.m);
+        }
+        __syncthreads();
+    };
+    auto rounds = [&](const FirstStage &M) {
+        const uint32_t nr = M.cnt[1];
+        uint32_t edge = INV ? M.cnt[0] : 0u;  // one past the round's last butterfly (inverse) or its first
+        for (uint32_t r = 0; r < nr; ++r) {
+            uint32_t kb, ke;
+            if (INV) {
+                ke = edge;
+                edge = kb = r + 1 < nr ? M.re[nr - 2 - r] : 0u;
+            } else {
+                kb = edge;
+                edge = ke = M.re[r];
+            }
+            if (act) {
+                for (uint32_t k = kb + slot; k < ke; k += slots) {
+                    const uint32_t ix = M.idx[k];
+                    const float2 ab = M.ab[k];
+                    const uint32_t r0 = sb + (ix & 0xFFFFu) * rs, r1 = sb + (ix >> 16) * rs;
+                    float4 y0 = lds4(r0), y1 = lds4(r1);
+                    rot<INV>(ab.x, ab.y, y0, y1);
+                    sts4(r0, y0);
+                    sts4(r1, y1);
+                }
+            }
+            __syncthreads();
+        }
+    };
+    auto store_rows = [&](uint32_t t, const FirstStage &M) {  // the buffer is refilled only after a later barrier
+        if (!act) return;
+        const uint32_t m = size_of(t), j0 = t * T, step = slots * rs;
+        uint32_t sa = sb + slot * rs;
+        if (!INV) {
+            for (uint32_t i = slot; i < m; i += slots, sa += step) {
+                const uint32_t d = M.io[i];
+                V4::st(((d & kCarry) ? poolc : Yc) + (uint64_t)(d & ~kCarry) * C, lds4(sa));
+            }
+        } else {
+            float *dst = io.out + (uint64_t)(j0 + slot) * C + c;
+            for (uint32_t i = slot; i < m; i += slots, sa += step, dst += slots * C) {
+                float4 v = lds4(sa);
+                if (io.lod_mean) {
+                    const float dv = lod_divisor<float>(p, j0 + i);
+                    v = make_float4(__fdiv_rn(v.x, dv), __fdiv_rn(v.y, dv), __fdiv_rn(v.z, dv), __fdiv_rn(v.w, dv));
+                }
+                V4::st(dst, v);
+            }
+        }
+    };
+
+    // Tiles are claimed from a global counter as the CTA goes (the next but one while the current one is
+    // transformed), so a CTA that starts late or runs slow (its SM shared with other work) takes fewer
+    // tiles; the claims ascend, so a claim past the last tile ends the CTA's loop.
+    if (tid == 0) {
+        s_claim[0] = atomicAdd(p.pipe_ctr, 1u);
+        s_claim[1] = atomicAdd(p.pipe_ctr, 1u);
+    }
+    __syncthreads();
+    if (s_claim[0] < nt) issue_meta(s_claim[0], meta(0));
+    if (s_claim[1] < nt) issue_meta(s_claim[1], meta(1));
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncthreads();
+    if (s_claim[0] < nt) issue_rows(s_claim[0], meta(0));
+    cp_async_commit();
+    for (uint32_t k = 0;; ++k) {
+        const uint32_t t = s_claim[k & 3];
+        if (t >= nt) break;
+        const FirstStage M = meta(k);
+        // complete: rows of tile k, metadata of tile k + 1.  Without colour transforms no barrier is needed
+        // here: a thread first touches only the row chunks it copied itself (complete for it after its own
+        // wait), tile k's metadata became visible at the previous tile's first barrier, and the barrier before
+        // the rounds orders the rest.
+        cp_async_wait<0>();
+        if (COLOR) {
+            __syncthreads();  // the colour steps read other threads' rows
+            stage_klt(INV ? frame_of_voxel(io.vstart, io.F, t * T) : frame_of(M));
+        }
+        finish_rows(t, M);
+        if (COLOR && !INV) colour_forward(t, M);
+        __syncthreads();
+        rounds(M);
+        if (COLOR && INV) colour_inverse(t);
+        store_rows(t, M);
+        if (tid == 0) s_claim[(k + 2) & 3] = atomicAdd(p.pipe_ctr, 1u);
+        __syncthreads();  // the row buffer and tile k's metadata are free; the new claim is visible
+        const uint32_t t1 = s_claim[(k + 1) & 3], t2 = s_claim[(k + 2) & 3];
+        if (t2 < nt) issue_meta(t2, meta(k + 2));
+        if (t1 < nt) issue_rows(t1, meta(k + 1));
+        cp_async_commit();
+    }
+    cp_async_wait<0>();
+    if (tid == 0) {  // the last CTA to finish leaves the counters at zero for the next launch
+        __threadfence();
+        if (atomicAdd(p.pipe_ctr + 1, 1u) == gridDim.x - 1) {
+            p.pipe_ctr[0] = 0;
+            p.pipe_ctr[1] = 0;
+            __threadfence();
+        }
+    }
 }
 
 int max_optin_smem()
@@ -1333,40 +1586,62 @@ int max_optin_smem()
 }
 
 // The pipelined first pass applies to FP32 transforms with 4-float vectors and
-// whole rows per tile whose buffers fit one CTA's shared memory.  Returns NR, or
-// 0 for the plain passes.
+// whole rows per tile whose buffers fit one CTA's shared memory.  Returns the
+// row buffers (1, or 3 for the deep pipeline), or 0 for the plain passes.
 template <typename S, int VEC>
 int pipe_depth(const XformArgs<S> &A, size_t *smem)
 {
     if (!std::is_same<S, float>::value || VEC != 4 || A.p.xpipe_off == 1) return 0;
     if (A.Cg != A.io.C || A.io.C % 4 || A.io.C / 4 > (uint32_t)kXThreads) return 0;
     const int nr = A.p.xpipe_off == 2 ? 3 : 1;
-    *smem = pipe_smem(nr, A.p.T, A.io.C, A.io.klt != nullptr);
+    *smem = nr == 1 ? first_smem(A.p.T, A.io.C, A.io.klt != nullptr) : pipe_smem(nr, A.p.T, A.io.C, A.io.klt != nullptr);
     return *smem <= (size_t)max_optin_smem() ? nr : 0;
 }
 
-template <int NR, bool INV, bool GATHER, bool QDQ>
-void launch_pipe(const XformArgs<float> &A, uint64_t nv_bound, size_t smem, int num_sms, cudaStream_t s)
+template <typename Kernel>
+uint32_t one_wave(Kernel k, int threads, uint64_t tiles, size_t smem, int num_sms)  // and the kernel's opt-in
 {
-    auto k = xform_pipe_kernel<NR, INV, GATHER, QDQ>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int per_sm = 0;  // resident CTAs per SM with this shared memory (one wave)
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kXThreads, smem) != cudaSuccess || per_sm < 1)
+    int per_sm = 0;  // resident CTAs per SM with this shared memory
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem) != cudaSuccess || per_sm < 1)
         per_sm = 1;
-    const uint64_t tiles = (nv_bound + A.p.T - 1) / A.p.T;
     const uint64_t cap = (uint64_t)num_sms * (uint64_t)per_sm;
-    const uint32_t grid = (uint32_t)(tiles < 1 ? 1 : (tiles < cap ? tiles : cap));
-    k<<<grid, kXThreads, smem, s>>>(A);
+    return (uint32_t)(tiles < 1 ? 1 : (tiles < cap ? tiles : cap));
+}
+
+template <bool INV, bool GATHER, bool QDQ, bool COLOR>
+void launch_first(const XformArgs<float> &A, uint64_t tiles, size_t smem, int num_sms, cudaStream_t s)
+{
+    const uint32_t L = A.io.C / 4;
+    uint32_t slots = 512 / L, pow2 = 1;
+    while (2 * pow2 <= slots) pow2 *= 2;
+    if (pow2 * L >= 384) slots = pow2;  // whole sweeps over a tile's rows
+    if (slots * L <= 448) {
+        auto k = xform_first_kernel<INV, GATHER, QDQ, COLOR, 448>;
+        const uint32_t grid = one_wave(k, 448, tiles, smem, num_sms);
+        k<<<grid, 448, smem, s>>>(A, slots);
+    } else {
+        auto k = xform_first_kernel<INV, GATHER, QDQ, COLOR, 512>;
+        const uint32_t grid = one_wave(k, 512, tiles, smem, num_sms);
+        k<<<grid, 512, smem, s>>>(A, slots);
+    }
     count_launch();
 }
 
 template <bool INV, bool GATHER, bool QDQ>
 void launch_pipe_nr(int nr, const XformArgs<float> &A, uint64_t nv_bound, size_t smem, int num_sms, cudaStream_t s)
 {
-    if (nr == 3)
-        launch_pipe<3, INV, GATHER, QDQ>(A, nv_bound, smem, num_sms, s);
-    else
-        launch_pipe<1, INV, GATHER, QDQ>(A, nv_bound, smem, num_sms, s);
+    const uint64_t tiles = (nv_bound + A.p.T - 1) / A.p.T;
+    if (nr == 3) {
+        auto k = xform_pipe_kernel<3, INV, GATHER, QDQ>;
+        const uint32_t grid = one_wave(k, kXThreads, tiles, smem, num_sms);
+        k<<<grid, kXThreads, smem, s>>>(A);
+        count_launch();
+    } else if (A.io.klt && (INV || GATHER)) {
+        launch_first<INV, GATHER, QDQ, INV || GATHER>(A, tiles, smem, num_sms, s);
+    } else {
+        launch_first<INV, GATHER, QDQ, false>(A, tiles, smem, num_sms, s);
+    }
 }
 
 uint32_t channel_group(uint32_t C, uint32_t T, uint32_t elem)

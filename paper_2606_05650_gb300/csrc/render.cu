@@ -13,9 +13,9 @@
 // Precision: everything per Gaussian (projection, covariance, conic, tile
 // rectangle, opacity, colour) is evaluated in FP64, or in double-float where
 // nothing cancels, and rounded once to FP32 for the per-pixel loop, which runs
-// in FP32.  The projected centre is kept as an unevaluated sum of two floats, so a pixel's offset from it is exact
-// to FP32 rounding of the offset itself (a single float would carry an
-// absolute error of its ulp at hundreds of pixels).  The conic enters the
+// in FP32.  The projected centre is kept as an unevaluated sum of two floats,
+// so a pixel's offset from it is exact to FP32 rounding of the offset itself (a
+// single float would carry an absolute error of its ulp at hundreds of pixels).  The conic enters the
 // loop through its Cholesky factor, conic = L^T L with
 // L = [[l1, l2], [0, l3]]: the exponent is -(|L d|^2) / 2, a sum of two
 // squares, which FP32 evaluates without cancellation even for elongated
