@@ -5,7 +5,7 @@
 // sigmoid(logit) and a degree-3 real-SH colour at the viewing direction; the
 // Gaussians are sorted by depth, each then lists the 16 x 16 tiles it overlaps
 // and the list is sorted stably by tile (so a tile's list is by depth, then
-// input index); one CTA per tile composites its list front to back for its 256
+// input index); a warp composites its tile's list front to back for 8 x 4
 // pixels.  Attributes are the
 // 56-channel 3DGS rows: log-scale 0-2, rotation (w, x, y, z) 3-6, opacity
 // logit 7, SH DC RGB 8-10, SH AC 11-55 as R[15] G[15] B[15].
@@ -29,10 +29,12 @@ namespace {
 constexpr int kTile = 16;
 
 struct Splat {
-    float u, ulo, v, vlo;  // projected centre as hi + lo
-    float l1, l2, l3;      // Cholesky factor of the conic
-    float opacity, r, g, b;
+    float u, v;            // projected centre, rounded
     uint32_t reach;        // pixels from the centre, in x and (upper half) in y, past which alpha stays below the cut
+    float opacity;
+    float ulo, vlo;        // the centre's rest: u + ulo, v + vlo
+    float l1, l2, l3;      // Cholesky factor of the conic
+    float r, g, b;
 };
 
 // Double-float arithmetic (an unevaluated sum h + l of two floats, about 2^-46
@@ -361,76 +363,87 @@ __device__ __forceinline__ void copy16(void *smem, const void *gmem)
                  : "memory");
 }
 
-// One CTA per tile, a thread per pixel, a warp per 8 x 4 pixels; the tile's
-// splats in batches of 256 through shared memory, the next batch landing while
-// one is composited.  A warp first finds, a splat per lane, which of 32 splats
-// reach its pixels (Splat::reach), then composites those in order: most of a
-// tile's list does not reach a given 8 x 4 block, and the skipped ones would
-// have failed the alpha cut at every pixel, so the image is the same.  With the
-// tile rectangles cut to the reach as well: 1M Gaussians at 960 x 540
-// 4.6 -> 2.9 ms (a thread per pixel evaluating its tile's whole list before).
-constexpr int kBatch = 256;
+// A warp per 8 x 4 pixels, a pixel per lane, each on its own: of its tile's
+// list it takes 32 splats at a time, a splat per lane, finds which of them reach
+// its pixels (Splat::reach) and copies those, in order and without gaps, to its
+// own shared memory while the 32 before are composited.  Most of a tile's list
+// does not reach a given block, and what is skipped would have failed the alpha
+// cut at every pixel, so the image is the same.  Bound by instruction issue, some
+// 30 a splat.  1M Gaussians at 960 x 540: 806 us with a CTA per tile that
+// staged batches of 256 splats for its eight warps (a barrier per batch, so
+// that all waited for the slowest, and half the issue slots empty) -> 547 us.
+constexpr int kWarpsPerCta = 4;  // the blocks of half a tile
 
-__global__ void __launch_bounds__(256) render_kernel(const uint2 *ranges, const uint32_t *vals, const Splat *sp,
-                                                     RenderCam cam, float *image)
+__global__ void __launch_bounds__(32 * kWarpsPerCta) render_kernel(const uint2 *ranges, const uint32_t *vals,
+                                                                   const Splat *sp, RenderCam cam, float *image)
 {
-    static_assert(sizeof(Splat) == 48, "copied in 16-byte words");
-    __shared__ __align__(16) Splat batch[2][kBatch];
-    const int tx = blockIdx.x, ty = blockIdx.y, t = threadIdx.x;
-    const uint32_t lane = t & 31, w = t >> 5;
-    const int bx = tx * kTile + (int)(w & 1) * 8, by = ty * kTile + (int)(w >> 1) * 4;  // the warp's block
+    static_assert(sizeof(Splat) == 48 && kTile == 16, "copied in 16-byte words; two halves of 16 x 8 pixels");
+    __shared__ __align__(16) Splat batch[kWarpsPerCta][2][32];
+    const int tx = blockIdx.x, ty = blockIdx.y >> 1;
+    const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5, ltmask = lanemask_lt();
+    const int bx = tx * kTile + (int)(w & 1) * 8, by = (int)blockIdx.y * (kTile / 2) + (int)(w >> 1) * 4;
     const int px = bx + (int)(lane & 7), py = by + (int)(lane >> 3);
-    const float mx = bx + 4.f, my = by + 2.f;  // its centre
+    const float mx = bx + 4.f, my = by + 2.f;  // the block's centre
     const bool inside = px < cam.W && py < cam.H;
     const uint2 rg = ranges[ty * cam.TX + tx];
+    const uint32_t *list = vals + rg.x;
+    const uint32_t n = rg.y - rg.x;
     const float fxp = px + 0.5f, fyp = py + 0.5f;
     float T = 1.f, col[3] = {0.f, 0.f, 0.f};
     bool done = !inside;
-    auto fetch = [&](uint32_t b0, uint32_t val) {  // splat `val` of the batch at b0
-        if (b0 + t < rg.y) {
-            Splat *d = &batch[((b0 - rg.x) / kBatch) & 1][t];
+    // entry g + lane of the list (g a multiple of 32), and the first 16 bytes of its splat
+    auto val_at = [&](uint32_t g) { return g < n && lane < n - g ? list[g + lane] : 0u; };
+    auto head_at = [&](uint32_t g, uint32_t val) {
+        return g < n && lane < n - g ? *reinterpret_cast<const uint4 *>(sp + val) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    auto stage = [&](uint32_t g, uint32_t val, uint4 head, Splat *to) {  // returns how many reach the block
+        const bool hit = g < n && lane < n - g &&
+                         fabsf(__uint_as_float(head.x) - mx) <= (float)(head.z & 0xFFFFu) + 4.f &&
+                         fabsf(__uint_as_float(head.y) - my) <= (float)(head.z >> 16) + 2.f;
+        const uint32_t m = __ballot_sync(0xFFFFFFFFu, hit);
+        if (hit) {
+            char *d = reinterpret_cast<char *>(to + __popc(m & ltmask));
             const char *q = reinterpret_cast<const char *>(sp + val);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) copy16(reinterpret_cast<char *>(d) + 16 * k, q + 16 * k);
+            *reinterpret_cast<uint4 *>(d) = head;
+            copy16(d + 16, q + 16);
+            copy16(d + 32, q + 32);
         }
         asm volatile("cp.async.commit_group;\n" ::: "memory");
+        return (uint32_t)__popc(m);
     };
-    auto val_at = [&](uint32_t b0) { return b0 < rg.y && b0 + t < rg.y ? vals[b0 + t] : 0u; };
-    fetch(rg.x, val_at(rg.x));
-    uint32_t next = val_at(rg.x + kBatch);
-    for (uint32_t b0 = rg.x; b0 < rg.y; b0 += kBatch) {
+    uint32_t v1 = val_at(0), v2 = val_at(32);
+    uint4 h1 = head_at(0, v1);
+    uint32_t cnt = stage(0, v1, h1, batch[w][0]);
+    v1 = v2;
+    h1 = head_at(32, v1);
+    v2 = val_at(64);
+    for (uint32_t g = 0, k = 0; g < n; g += 32, k ^= 1u) {
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-        if (__syncthreads_count(done ? 0 : 1) == 0) break;  // every pixel of the tile has finished
-        fetch(b0 + kBatch, next);  // over the batch before this one
-        next = val_at(b0 + 2 * kBatch);
-        const Splat *B = batch[((b0 - rg.x) / kBatch) & 1];
-        const uint32_t cnt = (rg.y - b0) < (uint32_t)kBatch ? (rg.y - b0) : (uint32_t)kBatch;
-        for (uint32_t j0 = 0; j0 < cnt; j0 += 32) {
-            if (__all_sync(0xFFFFFFFFu, done)) break;
-            bool hit = false;
-            if (j0 + lane < cnt) {
-                const Splat &s = B[j0 + lane];
-                hit = fabsf(s.u - mx) <= (float)(s.reach & 0xFFFFu) + 4.f && fabsf(s.v - my) <= (float)(s.reach >> 16) + 2.f;
-            }
-            for (uint32_t m = __ballot_sync(0xFFFFFFFFu, hit); m; m &= m - 1) {
-                if (done) continue;
-                const Splat &s = B[j0 + __ffs(m) - 1];
-                const float dx = (s.u - fxp) + s.ulo, dy = (s.v - fyp) + s.vlo;
-                const float e0 = fmaf(s.l1, dx, s.l2 * dy), e1 = s.l3 * dy;
-                const float power = -0.5f * fmaf(e0, e0, e1 * e1);
-                const float alpha = fminf(0.99f, s.opacity * expf(power));
-                if (alpha < 1.f / 255.f) continue;
-                const float tn = T * (1.f - alpha);
-                if (tn < 1e-4f) {
-                    done = true;
-                    continue;
-                }
+        __syncwarp();  // this group has landed for every lane, and all have left the one before
+        if (__all_sync(0xFFFFFFFFu, done)) break;
+        const uint32_t next = stage(g + 32, v1, h1, batch[w][k ^ 1u]);
+        v1 = v2;
+        h1 = head_at(g + 64, v1);
+        v2 = val_at(g + 96);
+        const Splat *B = batch[w][k];
+#pragma unroll 2
+        for (uint32_t j = 0; j < cnt; ++j) {
+            const Splat s = B[j];
+            const float dx = (s.u - fxp) + s.ulo, dy = (s.v - fyp) + s.vlo;
+            const float e0 = fmaf(s.l1, dx, s.l2 * dy), e1 = s.l3 * dy;
+            const float power = -0.5f * fmaf(e0, e0, e1 * e1);
+            const float alpha = fminf(0.99f, s.opacity * expf(power));
+            const float tn = T * (1.f - alpha);
+            const bool on = !done && !(alpha < 1.f / 255.f), stop = tn < 1e-4f;
+            if (on && !stop) {
                 col[0] += s.r * alpha * T;
                 col[1] += s.g * alpha * T;
                 col[2] += s.b * alpha * T;
                 T = tn;
             }
+            done = done || (on && stop);
         }
+        cnt = next;
     }
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     if (inside)
@@ -482,7 +495,7 @@ void launch_render_tiles(uint64_t n, const RenderBuffers &b, const uint32_t *ord
     } else {
         dev_memset(ranges, 0, sizeof(uint2) * ntiles, s);
     }
-    render_kernel<<<dim3(cam.TX, cam.TY), 256, 0, s>>>(ranges, sv, (const Splat *)b.splats, cam, image);
+    render_kernel<<<dim3(cam.TX, 2 * cam.TY), 32 * kWarpsPerCta, 0, s>>>(ranges, sv, (const Splat *)b.splats, cam, image);
     count_launch();
 }
 
