@@ -564,6 +564,192 @@ __global__ void __launch_bounds__(512) rlgr_encode_few_kernel(EncJobs E, uint32_
     if (bw.nw > j.slot_words) atomicExch(j.overflow, 1u);
 }
 
+// ---- encoder for very few streams -----------------------------------------------
+// A launch takes as long as one stream does, and a thread that codes a symbol at
+// a time spends 290 cycles on each (65 instructions, one after another).  Only
+// the adaptation is serial, so here a CTA takes kSplitG streams in segments of
+// kSplitSeg symbols and splits the work: one warp walks the adaptation, a lane
+// per stream, and notes the state before each symbol (a fifth of the
+// instructions while no stream is near run mode); a warp per stream then forms
+// the segment's codewords, a lane per symbol, places them by a scan of their
+// lengths and writes whole words, while the first walks the next segment and
+// the one after it is loaded and quantised.  10k Gaussians (1.1k streams): 78 ->
+// 41 us, 30k 79 -> 47; a cloud of 1M points (5.9k streams at most, mostly runs)
+// 58 -> 46.  In all it takes more instructions than the kernels above, and
+// beyond kSplitStreams, when an SM has more than its four CTAs, it loses: 50k
+// Gaussians (5.5k streams) 86 against 80 us, 100k 155, 2M points 80 against 60.
+constexpr uint64_t kSplitStreams = 6144;
+constexpr uint32_t kSplitG = 8, kSplitSeg = 128, kSplitThreads = 32 * (1 + kSplitG);
+constexpr uint32_t kSplitRow = kSplitG + 1;  // of a symbol's row in shared memory: no bank twice down a column
+
+// state before a symbol: K (8 bits), KR (9 bits), pending zeros of an open run (15 bits)
+__device__ __forceinline__ uint32_t split_state(uint32_t K, uint32_t KR, uint32_t z) { return K | KR << 8 | z << 17; }
+
+// adapt_kr; p <= 2^31
+__device__ __forceinline__ uint32_t adapted(uint32_t KR, uint32_t p)
+{
+    const uint32_t down = (uint32_t)max((int)KR - 2, 0), up = min(KR + p + 1u, 384u);
+    return p == 0u ? down : (p == 1u ? KR : up);
+}
+
+// n <= 64 bits c at bit o of a zeroed buffer, least significant first (c < 2^n)
+__device__ __forceinline__ void or_bits(uint32_t *buf, uint32_t o, uint64_t c)
+{
+    const uint32_t s = o & 31u;
+    uint32_t *at = buf + (o >> 5);
+    const uint64_t x = c << s;
+    const uint32_t lo = (uint32_t)x, mid = (uint32_t)(x >> 32), hi = s ? (uint32_t)(c >> (64u - s)) : 0u;
+    if (lo) atomicOr(at, lo);
+    if (mid) atomicOr(at + 1, mid);
+    if (hi) atomicOr(at + 2, hi);
+}
+
+__global__ void __launch_bounds__(kSplitThreads, 4) rlgr_encode_split_kernel(EncJobs E)
+{
+    __shared__ uint32_t sym[3][kSplitSeg * kSplitRow];  // zigzag indices of a segment
+    __shared__ uint32_t pre[2][kSplitSeg * kSplitRow];  // states before its symbols
+    __shared__ uint32_t bits[kSplitG][84];            // 32 codewords of up to 78 bits behind a part of a word
+    __shared__ uint32_t s_len[kSplitG], s_open[kSplitG];
+    const RlgrJob &j = E.j;
+    const uint32_t C = j.C, W = j.R * C, lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    // a lane of the first warp and a whole later warp are a stream's; the loading threads, eight streams a row
+    const uint32_t g = warp == 0 ? lane & (kSplitG - 1u) : warp - 1u, gl = threadIdx.x & (kSplitG - 1u);
+    const auto block_of = [&](uint32_t gg, uint32_t &w) {
+        const uint64_t stream = (uint64_t)blockIdx.x * kSplitG + gg, job = stream / W;
+        w = (uint32_t)(stream - job * W);
+        return enc_block(E, job);
+    };
+    uint32_t w, wl;
+    const EncBlock me = block_of(g, w), ld = block_of(gl, wl);
+    const uint32_t r = w / C, c = w - r * C, rl = wl / C, cl = wl - rl * C;
+    if (warp == 0 && lane < kSplitG) s_len[lane] = me.len;
+    __syncthreads();
+    uint32_t longest = 0;
+#pragma unroll
+    for (uint32_t k = 0; k < kSplitG; ++k) longest = max(longest, s_len[k]);
+    const uint32_t segs = (longest + kSplitSeg - 1) / kSplitSeg;
+    // loading (warps 1 .. kSplitG): symbol at + kSplitSeg / kPer * h of the segment, of stream gl
+    constexpr uint32_t kPer = kSplitSeg * kSplitG / (32 * kSplitG);
+    const uint32_t at = (threadIdx.x - 32u) / kSplitG;
+    const float inv = ld.len ? j.inv_step[rl * C + cl] : 0.f, tau = j.tau;
+    const float *col = j.Y + ld.gbase + cl;
+    float val[kPer];
+    const auto load = [&](uint32_t seg) {
+#pragma unroll
+        for (uint32_t h = 0; h < kPer; ++h) {
+            const uint32_t i = seg * kSplitSeg + at + kSplitSeg / kPer * h;
+            val[h] = i < ld.len ? __ldg(col + (uint64_t)i * C) : 0.f;
+        }
+    };
+    const auto put_symbols = [&](uint32_t seg) {
+        uint32_t *to = sym[seg % 3u];
+#pragma unroll
+        for (uint32_t h = 0; h < kPer; ++h)
+            to[(at + kSplitSeg / kPer * h) * kSplitRow + gl] = quantize_zz_f32(val[h], inv, tau);
+        if (seg == 0 && at == 0 && ld.len && j.dc && ld.b == 0)  // the frame's DC: quantised from its FP64 value
+            to[gl] = zz(quantize_f64(j.dc[(uint64_t)ld.f * C + cl], j.steps_rg[rl * j.G + j.groups[cl]], j.tau64));
+    };
+    if (warp) {
+        load(0);
+        put_symbols(0);
+    }
+    __syncthreads();
+    uint32_t K = 0, KR = 32, z = 0;                // the first warp's, a stream per lane
+    uint32_t words = 0, part = 0, nbits = 0;       // a later warp's stream: whole words written, the bits after them
+    const uint64_t blk = j.blk_off[me.f] + ((uint64_t)r * me.nb + me.b) * C + c;
+    uint32_t *out = j.slots + blk * j.slot_words;
+    for (uint32_t seg = 0; seg <= segs; ++seg) {
+        if (warp == 0) {
+            if (seg < segs && lane < kSplitG) {
+                const uint32_t *u_at = sym[seg % 3u] + lane;
+                uint32_t *pre_at = pre[seg & 1u] + lane;
+                const uint32_t left = me.len > seg * kSplitSeg ? me.len - seg * kSplitSeg : 0u;
+                for (uint32_t i = 0; i < kSplitSeg; i += 4) {
+                    uint32_t u[4];
+#pragma unroll
+                    for (uint32_t h = 0; h < 4; ++h) u[h] = u_at[(i + h) * kSplitRow];
+                    if (__all_sync((1u << kSplitG) - 1u, K < 4u && i + 4 <= left)) {  // four in Golomb-Rice mode: K + 3 each at most
+#pragma unroll
+                        for (uint32_t h = 0; h < 4; ++h) {
+                            pre_at[(i + h) * kSplitRow] = split_state(K, KR, 0u);
+                            const uint32_t p = u[h] >> (KR >> 4);
+                            KR = adapted(KR, p);
+                            K = (uint32_t)max((int)K + (u[h] == 0u ? 3 : -3), 0);
+                        }
+                        continue;
+                    }
+#pragma unroll
+                    for (uint32_t h = 0; h < 4; ++h) {
+                        pre_at[(i + h) * kSplitRow] = split_state(K, KR, z);
+                        if (i + h >= left) continue;  // after the stream's end
+                        const bool run = K >= 16u, zero = u[h] == 0u, quiet = run && zero;
+                        const uint32_t k = K >> 4, z1 = z + 1u, full = z1 >> k;  // z1 <= 2^k in a run
+                        const uint32_t p = (u[h] - (run ? 1u : 0u)) >> (KR >> 4);  // not used when quiet
+                        if (!quiet) KR = adapted(KR, p);
+                        const int dk = quiet ? (full ? 4 : 0) : (run ? -6 : (zero ? 3 : -3));
+                        K = (uint32_t)min(max((int)K + dk, 0), 240);
+                        z = quiet && !full ? z1 : 0u;
+                    }
+                }
+                s_open[lane] = z;
+            }
+        } else {
+            if (seg + 1 < segs) load(seg + 1);
+            for (uint32_t q = 0; seg > 0 && q < kSplitSeg && (seg - 1) * kSplitSeg + q < me.len; q += 32) {
+                const uint32_t i = q + lane;
+                uint32_t n = 0, npre = 0, cpre = 0;
+                uint64_t code = 0;
+                if ((seg - 1) * kSplitSeg + i < me.len) {
+                    const uint32_t u = sym[(seg - 1) % 3u][i * kSplitRow + g], st = pre[(seg - 1) & 1u][i * kSplitRow + g];
+                    const uint32_t k = (st >> 4) & 15u, kr = (st >> 12) & 31u, zr = st >> 17;
+                    if (k && u == 0u) {
+                        n = zr + 1u == 1u << k ? 1u : 0u;  // the 2^k-th zero of a run is bit 0
+                    } else {
+                        if (k) {  // bit 1, then the run length in k bits
+                            npre = 1u + k;
+                            cpre = 1u | zr << 1;
+                        }
+                        const uint32_t v = u - (k ? 1u : 0u), p = v >> kr;
+                        if (p < (uint32_t)kUnaryEsc) {  // as gr_put
+                            n = p + 1u + kr;
+                            code = (((uint64_t)(v & ((1u << kr) - 1u)) << 1 | 1u) << p) - 1u;
+                        } else {
+                            const uint32_t len = 32u - (uint32_t)__clz(v);
+                            n = kUnaryEsc + 6u + len;
+                            code = (uint64_t)v << (kUnaryEsc + 6) | (uint64_t)len << kUnaryEsc | ((1u << kUnaryEsc) - 1u);
+                        }
+                    }
+                }
+                const uint32_t end = nbits + warp_inclusive_sum(npre + n);
+                const uint32_t total = __shfl_sync(0xFFFFFFFFu, end, 31), whole = total >> 5;
+                uint32_t *buf = bits[g];
+                for (uint32_t x = lane; x <= whole; x += 32) buf[x] = x ? 0u : part;
+                __syncwarp();
+                if (npre) or_bits(buf, end - n - npre, cpre);
+                if (n) or_bits(buf, end - n, code);
+                __syncwarp();
+                for (uint32_t x = lane; x < whole; x += 32)
+                    if (words + x < j.slot_words) out[words + x] = buf[x];
+                part = buf[whole];
+                words += whole;
+                nbits = total & 31u;
+                __syncwarp();
+            }
+            if (seg + 1 < segs) put_symbols(seg + 1);
+        }
+        __syncthreads();
+    }
+    if (warp && lane == 0 && me.len) {
+        if (s_open[g]) ++nbits;  // an open run at the end: bit 0
+        if (nbits) {
+            if (words < j.slot_words) out[words] = part;
+            ++words;
+        }
+        j.block_words[blk] = words;
+        if (words > j.slot_words) atomicExch(j.overflow, 1u);
+    }
+}
+
 // ---- decoder ------------------------------------------------------------------
 // Bits are looked at through a 32-bit window over two consecutive words
 // (cur, nxt) at bit offset pos; the word after them (ahead) is in a register
@@ -926,6 +1112,11 @@ void launch_rlgr_encode(const RlgrJob &j, const uint64_t *job_off, uint64_t jobs
     const uint32_t W = j.R * j.C;
     const uint32_t rb = row_blocks_per_cta(W);
     const uint32_t threads = (rb * W + 31) / 32 * 32;
+    if (!j.sq_err && W <= 512 && jobs_bound * W <= kSplitStreams) {
+        rlgr_encode_split_kernel<<<(uint32_t)((jobs_bound * W + kSplitG - 1) / kSplitG), kSplitThreads, 0, s>>>(E);
+        count_launch();
+        return;
+    }
     if (!j.sq_err && jobs_bound * W <= kFewStreams) {
         rlgr_encode_few_kernel<<<(uint32_t)((jobs_bound + rb - 1) / rb), threads, 0, s>>>(E, rb);
         count_launch();
