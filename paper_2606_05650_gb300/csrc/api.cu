@@ -1782,7 +1782,7 @@ gsnfs_status decode_batch_impl(gsnfs_ctx *ctx, cudaStream_t s, uint32_t F, const
         if (P[f].hb > 4096) return GSNFS_ERR_CORRUPT;
     }
     uint32_t C = 0, Jmax = 0;
-    uint64_t N = 0, n_occ = 0, nodes = 0, nblk = 0, jobs = 0, max_occ = 0;
+    uint64_t N = 0, n_occ = 0, tiles = 0, nblk = 0, jobs = 0, max_occ = 0;
     uint32_t max_nch = 0, chunk_max = 0;
     uint64_t n_chunks = 0;
     bool any_rans = false;
@@ -1798,7 +1798,7 @@ gsnfs_status decode_batch_impl(gsnfs_ctx *ctx, cudaStream_t s, uint32_t F, const
         N += P[f].nv;
         n_occ += P[f].n_occ;
         max_occ = std::max(max_occ, P[f].n_occ);
-        for (uint32_t d = 0; d < P[f].J; ++d) nodes += P[f].lsz[d];
+        if (P[f].nv) tiles += octree_tiles(P[f].lsz[P[f].J - 1]);
         if (C && P[f].nv) {
             nblk += (uint64_t)P[f].nb * C;
             jobs += P[f].nb;
@@ -1819,8 +1819,8 @@ gsnfs_status decode_batch_impl(gsnfs_ctx *ctx, cudaStream_t s, uint32_t F, const
     // ---- layout
     struct L_ {
         DecFrame *fr;
-        uint32_t *vstart, *bw_all, *tabs, *tsum, *tile_pref;
-        uint64_t *lvl_pref, *job_off, *blk_pref, *boff_all, *spart, *tbase, *tpart, *nodes, *nvdev;
+        uint32_t *vstart, *bw_all, *tabs, *tsum, *tile_pref, *path, *leaf0, *broken;
+        uint64_t *job_off, *blk_pref, *boff_all, *spart, *tbase, *tpart, *nvdev;
         float *steps, *Y, *pool;
         uint8_t *occ, *gap;
         float *ctab, *klt;
@@ -1837,7 +1837,6 @@ gsnfs_status decode_batch_impl(gsnfs_ctx *ctx, cudaStream_t s, uint32_t F, const
     auto carve = [&](Carve &cv) {
         L.fr = cv.take<DecFrame>(F);
         L.vstart = cv.take<uint32_t>(F + 1);
-        L.lvl_pref = cv.take<uint64_t>((uint64_t)(Jmax + 1) * (F + 1));
         L.job_off = cv.take<uint64_t>(F + 1);
         L.blk_pref = cv.take<uint64_t>(F + 1);
         L.nvdev = cv.take<uint64_t>(1);
@@ -1848,8 +1847,10 @@ gsnfs_status decode_batch_impl(gsnfs_ctx *ctx, cudaStream_t s, uint32_t F, const
         L.tsum = cv.take<uint32_t>(occ_tiles(n_occ) + 1);
         L.tbase = cv.take<uint64_t>(occ_tiles(n_occ) + 2);
         L.tpart = cv.take<uint64_t>(scan_partial_words(occ_tiles(n_occ), ctx->num_sms) + 1);
-        L.tile_pref = cv.take<uint32_t>((uint64_t)Jmax * (F + 1) + 1);
-        L.nodes = cv.take<uint64_t>(nodes + 1);
+        L.tile_pref = cv.take<uint32_t>(F + 1);
+        L.path = cv.take<uint32_t>(octree_path_words(tiles));
+        L.leaf0 = cv.take<uint32_t>(tiles + 1);
+        L.broken = cv.take<uint32_t>(1);
         L.gap = cv.take<uint8_t>(N + 2);
         L.ctab = cv.take<float>(ctab_total + 1);
         L.klt = cv.take<float>((any_color ? (uint64_t)F : 1) * kKltFloats);
@@ -1876,10 +1877,10 @@ gsnfs_status decode_batch_impl(gsnfs_ctx *ctx, cudaStream_t s, uint32_t F, const
 
     // ---- frame tables, packed into pinned memory after the headers
     unsigned char *tp = hp + (size_t)F * 8192;
-    size_t o_fr = 0, o_vs = o_fr + sizeof(DecFrame) * F, o_lp = (o_vs + 4 * (F + 1) + 7) & ~(size_t)7;
-    size_t o_jo = o_lp + 8 * (size_t)(Jmax + 1) * (F + 1), o_bp = o_jo + 8 * (F + 1), o_nv = o_bp + 8 * (F + 1);
+    size_t o_fr = 0, o_vs = o_fr + sizeof(DecFrame) * F, o_jo = (o_vs + 4 * (F + 1) + 7) & ~(size_t)7;
+    size_t o_bp = o_jo + 8 * (F + 1), o_nv = o_bp + 8 * (F + 1);
     size_t o_st = o_nv + 8, o_fc = o_st + 4 * (size_t)F * C, o_tp = o_fc + 4 * (size_t)(F + 1);
-    size_t o_end = o_tp + 4 * ((size_t)Jmax * (F + 1) + 1);
+    size_t o_end = o_tp + 4 * (size_t)(F + 1);
     const size_t need = (size_t)F * 8192 + o_end + 128;  // and the status word after the tables
     if (status ? ctx->aring_cap[ring] < need : ctx->pinned_cap < need) {
         // the headers are parsed by now: the staging buffer holds nothing still needed
@@ -1899,13 +1900,13 @@ gsnfs_status decode_batch_impl(gsnfs_ctx *ctx, cudaStream_t s, uint32_t F, const
     }
     DecFrame *hf = reinterpret_cast<DecFrame *>(tp + o_fr);
     uint32_t *hvs = reinterpret_cast<uint32_t *>(tp + o_vs);
-    uint64_t *hlp = reinterpret_cast<uint64_t *>(tp + o_lp);
     uint64_t *hjo = reinterpret_cast<uint64_t *>(tp + o_jo);
     uint64_t *hbp = reinterpret_cast<uint64_t *>(tp + o_bp);
     float *hst = reinterpret_cast<float *>(tp + o_st);
     uint32_t *hfc = reinterpret_cast<uint32_t *>(tp + o_fc);
     uint32_t *htp = reinterpret_cast<uint32_t *>(tp + o_tp);
-    uint64_t vs = 0, oo = 0, no = 0, bo = 0, jo = 0, co = 0, pb = 0, cho = 0;
+    uint64_t vs = 0, oo = 0, bo = 0, jo = 0, co = 0, pb = 0, cho = 0;
+    uint32_t to = 0;
     for (uint32_t f = 0; f < F; ++f) {
         const ParsedHeader &H = P[f];
         DecFrame d{};
@@ -1943,9 +1944,7 @@ gsnfs_status decode_batch_impl(gsnfs_ctx *ctx, cudaStream_t s, uint32_t F, const
             d.lsz[lv] = H.lsz[lv];
             d.boff[lv] = b2;
             if (lv < H.J) {
-                d.noff[lv] = no;
                 d.pbase[lv] = pb;  // the bytes of a level hold as many set bits as the next level has nodes
-                no += H.lsz[lv];
                 b2 += H.lsz[lv];
                 pb += H.lsz[lv + 1];
             }
@@ -1956,6 +1955,8 @@ gsnfs_status decode_batch_impl(gsnfs_ctx *ctx, cudaStream_t s, uint32_t F, const
         hbp[f] = bo;
         for (uint32_t c = 0; c < C; ++c) hst[(uint64_t)f * C + c] = (float)H.steps[H.groups[c]];
         hfc[f] = H.color;
+        htp[f] = to;
+        if (H.nv) to += octree_tiles(H.lsz[H.J - 1]);
         vs += H.nv;
         oo += H.n_occ;
         if (C && H.nv) {
@@ -1966,37 +1967,17 @@ gsnfs_status decode_batch_impl(gsnfs_ctx *ctx, cudaStream_t s, uint32_t F, const
     hvs[F] = (uint32_t)vs;
     hjo[F] = jo;
     hbp[F] = bo;
-    for (uint32_t lv = 0; lv <= Jmax; ++lv) {
-        uint64_t run = 0;
-        for (uint32_t f = 0; f < F; ++f) {
-            hlp[(uint64_t)lv * (F + 1) + f] = run;
-            if (lv < P[f].J) run += P[f].lsz[lv];
-        }
-        hlp[(uint64_t)lv * (F + 1) + F] = run;
-    }
-    std::vector<uint32_t> level_tiles(Jmax);  // CTAs of each level launch
-    for (uint32_t lv = 0; lv < Jmax; ++lv) {
-        uint32_t run = 0;
-        for (uint32_t f = 0; f < F; ++f) {
-            htp[(uint64_t)lv * (F + 1) + f] = run;
-            if (lv < P[f].J && P[f].lsz[lv]) {
-                const uint64_t a0 = hf[f].occ_off + hf[f].boff[lv];
-                run += (uint32_t)(occ_tile_first(a0 + P[f].lsz[lv] - 1) - occ_tile_first(a0) + 1);
-            }
-        }
-        htp[(uint64_t)lv * (F + 1) + F] = run;
-        level_tiles[lv] = run;
-    }
+    htp[F] = to;
     memcpy(tp + o_nv, &N, 8);
     DevState *dst = ctx->st;
     StageCopies up(s);
     CK(up.add(L.fr, tp + o_fr, sizeof(DecFrame) * F));
     CK(up.add(L.vstart, tp + o_vs, 4 * (F + 1)));
-    CK(up.add(L.lvl_pref, tp + o_lp, 8 * (size_t)(Jmax + 1) * (F + 1)));
     CK(up.add(L.job_off, tp + o_jo, 8 * (F + 1)));
     CK(up.add(L.blk_pref, tp + o_bp, 8 * (F + 1)));
     CK(up.add(L.nvdev, tp + o_nv, 8));
-    if (Jmax) CK(up.add(L.tile_pref, tp + o_tp, 4 * (size_t)Jmax * (F + 1)));
+    CK(up.add(L.tile_pref, tp + o_tp, 4 * (F + 1)));
+    CK(up.add(L.broken, nullptr, 4));
     if (C) CK(up.add(L.steps, tp + o_st, 4 * (size_t)F * C));
     CK(up.add(dst, nullptr, 8));
     if (any_color) {
@@ -2028,11 +2009,9 @@ gsnfs_status decode_batch_impl(gsnfs_ctx *ctx, cudaStream_t s, uint32_t F, const
     stage_end(sg, kStOccDecode);
     stage_begin(sg, kStOctreeDecode);
     if (ctab_total) launch_batch_centre_tables(L.fr, F, Jmax, L.ctab, sms, sg);
-    launch_occ_tile_bases(L.occ, n_occ, L.tsum, L.tbase, L.tpart, sms, sg);
-    launch_batch_roots(L.fr, F, L.nodes, L.gap, N, sg);
-    for (uint32_t lv = 0; lv < Jmax; ++lv)
-        launch_batch_level(L.fr, F, lv, L.tile_pref + (uint64_t)lv * (F + 1), level_tiles[lv], L.occ, n_occ,
-                           L.tbase, L.nodes, L.ctab, d_pos, L.gap, dst, sg);
+    launch_occ_tile_bases(L.occ, n_occ, L.tsum, L.tbase, L.tpart, L.broken, dst, sms, sg);
+    launch_octree_leaves(L.fr, F, Jmax, L.tile_pref, (uint32_t)tiles, L.occ, n_occ, L.tbase, L.path, L.leaf0, L.ctab,
+                         d_pos, L.gap, N, L.broken, dst, sg);
     stage_end(sg, kStOctreeDecode);
     // a12: RAHT schedule, then (after the RLGR branch) the inverse RAHT
     if (attrs) {

@@ -115,25 +115,13 @@ __device__ __forceinline__ uint32_t compact3b(uint64_t m)
     return (uint32_t)m;
 }
 
-__global__ void roots_kernel(const DecFrame *fr, uint32_t F, uint64_t *nodes, uint8_t *gap, uint64_t nv_total)
-{
-    const uint32_t f = blockIdx.x * blockDim.x + threadIdx.x;
-    if (f == 0) gap[nv_total] = (uint8_t)kInfLevel;  // sentinel after the last voxel
-    if (f >= F || fr[f].nv == 0) return;
-    nodes[fr[f].noff[0]] = 0ull;  // implicit root code of Algorithm 2
-}
-
-// ---- octree levels (Algorithm 3) by tiles of the batch occupancy buffer ----
+// ---- octree (Algorithm 3) ------------------------------------------------------
 // P(x) = number of set bits in the batch occupancy bytes before byte x.  Node w
 // of level d of frame f (byte x = occ_off + boff[d] + w) has its children at
-// indices P(x) - P(a0) .. of level d + 1, a0 the level's first byte.  P(a0) is
-// known on the host (a level's popcounts add up to the next level's size);
-// P at every kOccTile-byte boundary comes from a scan of tile popcounts, and
-// a tile's CTA finds P(x) for its bytes with one block scan.  One launch per
-// level covers every frame: its CTAs are the tiles that hold bytes of that
-// level (a tile on a level boundary is visited by both levels' launches).
-// At a frame's last level the leaf codes are not stored: the CTA writes the
-// voxel centres (Sec. 2.1) and the gap levels of consecutive voxels instead.
+// indices P(x) - pbase[d] .. of level d + 1, pbase[d] = P at the level's first
+// byte, which the host knows (a level's popcounts add up to the next level's
+// size).  The bytes are summed in tiles, P at every tile's first byte is one
+// scan.
 constexpr uint32_t kOccTile = 1024;  // bytes per tile
 
 __device__ __forceinline__ uint32_t word_at(const uint8_t *occ, uint64_t n, uint64_t x)  // bytes >= n read 0
@@ -144,15 +132,27 @@ __device__ __forceinline__ uint32_t word_at(const uint8_t *occ, uint64_t n, uint
     return v;
 }
 
+// tsum: set bits per tile; *broken and the error are set when a byte is zero (a node without children)
 __global__ void __launch_bounds__(256) occ_tile_popc_kernel(const uint8_t *__restrict__ occ, uint64_t n,
-                                                            uint64_t ntiles, uint32_t *tsum)
+                                                            uint64_t ntiles, uint32_t *tsum, uint32_t *broken,
+                                                            DevState *st)
 {
     const uint32_t lane = threadIdx.x & 31;
     for (uint64_t t = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < ntiles;
          t += ((uint64_t)gridDim.x * blockDim.x) >> 5) {
-        uint32_t c = 0;
+        uint32_t c = 0, zero = 0;
 #pragma unroll
-        for (uint32_t k = 0; k < kOccTile / 128; ++k) c += __popc(word_at(occ, n, t * kOccTile + 4ull * (lane + 32 * k)));
+        for (uint32_t k = 0; k < kOccTile / 128; ++k) {
+            const uint64_t x = t * kOccTile + 4ull * (lane + 32 * k);
+            uint32_t v = word_at(occ, n, x);
+            c += __popc(v);
+            if (x + 4 > n) v |= x < n ? 0xFFFFFFFFu << (8u * (uint32_t)(n - x)) : 0xFFFFFFFFu;  // bytes past the end
+            zero |= __vcmpeq4(v, 0u);
+        }
+        if (__any_sync(0xFFFFFFFFu, zero != 0u) && lane == 0) {
+            *broken = 1;
+            set_error(&st->err, kErrCorrupt);
+        }
         c = __reduce_add_sync(0xFFFFFFFFu, c);
         if (lane == 0) tsum[t] = c;
     }
@@ -178,147 +178,261 @@ __device__ __forceinline__ void leaf_out(const DecFrame &d, const float *__restr
     }
 }
 
-struct LevelArgs {
+// Going down level by level, every level reads and writes a code per node and
+// waits for a launch.  Instead a CTA takes kLeafTile nodes of the last level and
+// walks down their ancestors only, from the root, the codes in shared memory:
+// global memory sees the occupancy bytes and the voxels' outputs.  A node has at
+// least one child, so that no level has more ancestors than the last has nodes.
+// Where a CTA begins in each level is found first, a warp per CTA going up by
+// rank: the parent of node w of level d + 1 is the byte that holds set bit
+// pbase[d] + w.  A CTA's last node is the next one's first, for that one's last
+// child is the voxel before the next CTA's first (its gap level).
+// 16 frames of 1M voxels, beside the RLGR decode: 1.57 ms in 16 launches, a tile
+// of 1,024 nodes of a level per CTA -> 0.18 + 0.56 ms.  Bound by latency: a
+// level is a scan and a loop over at most eight children between two barriers.
+constexpr uint32_t kLeafTile = 1016, kLeafThreads = 256;
+constexpr uint32_t kLeafNodes = kLeafTile + 1;  // of a level in a CTA at most; with the 3 bytes before, a word a thread
+constexpr uint32_t kLeafStage = 2048;           // voxels gathered at a time
+static_assert(kLeafNodes + 3 <= 4 * kLeafThreads && kLeafNodes <= kLeafStage, "a word of bytes per thread");
+
+struct OctArgs {
     const DecFrame *fr;
-    uint32_t F, d;
-    const uint32_t *tile_pref;  // F + 1: first CTA of each frame at this level
+    uint32_t F, Jmax;
+    const uint32_t *tile_pref;  // F + 1: first CTA of each frame
+    uint32_t tiles;             // tile_pref[F]
     const uint8_t *occ;
     uint64_t n_occ;
-    const uint64_t *tbase;      // P at each tile's first byte
-    uint64_t *nodes;
+    const uint64_t *tbase;      // P at each tile's first byte, and the total
+    uint2 *path;                // per CTA and level: first node, its children that belong to the CTA before
+    uint32_t *leaf0;            // per CTA: voxels of the frame before the first node's
     const float *ctab;
     float *pos;                 // or null: no centres
     uint8_t *gap;
+    uint64_t nv_total;
+    uint32_t *broken;           // set: the bytes are not an octree's with these level sizes
     DevState *st;
 };
 
-// A CTA of kLevelThreads threads takes one tile.  Its bytes are loaded 8 per
-// thread and their set bits scanned; the per-byte prefixes go to shared
-// memory, and the nodes are then taken strided (node j of the tile by thread
-// j mod kLevelThreads), so that code loads and child stores of consecutive
-// threads are consecutive.  Internal level: children codes go straight to
-// the next level.  Leaf level: the children's codes are staged in shared
-// memory at their rank among the tile's set bits, then one child per thread
-// gets its gap level (from the staged code before it) and its centre, with
-// coalesced stores (a tile with more set bits than the stage holds writes its
-// voxels directly).
-constexpr uint32_t kLevelThreads = kOccTile / 8;
-constexpr uint32_t kLeafStage = 2048;
-
-__device__ __forceinline__ uint64_t word8_at(const uint8_t *occ, uint64_t n, uint64_t x)  // bytes >= n read 0
+// P(x), by a warp
+__device__ __forceinline__ uint64_t bits_before(const OctArgs &a, uint64_t x, uint32_t lane)
 {
-    if (x >= n) return 0ull;
-    uint64_t v = *reinterpret_cast<const uint64_t *>(occ + x);  // x % 8 == 0; the buffer has 8 bytes of slack
-    if (x + 8 > n) v &= (1ull << (8u * (uint32_t)(n - x))) - 1ull;
-    return v;
+    const uint64_t t = x / kOccTile;
+    const uint32_t part = (uint32_t)(x % kOccTile);
+    uint32_t c = 0;
+#pragma unroll
+    for (uint32_t k = 0; k < kOccTile / 128; ++k) {
+        const uint32_t o = 4 * (lane + 32 * k);
+        if (o >= part) continue;
+        uint32_t v = word_at(a.occ, a.n_occ, t * kOccTile + o);
+        if (o + 4 > part) v &= (1u << (8u * (part - o))) - 1u;
+        c += __popc(v);
+    }
+    return a.tbase[t] + __reduce_add_sync(0xFFFFFFFFu, c);
 }
 
-// the last child's code of node w (byte b) of a level, shifted to the next level
-__device__ __forceinline__ uint64_t last_child(uint64_t code, uint32_t b)
+// The byte of [a0, a1) that holds set bit r, by a warp: its index from a0 and, in y, the set bits before r in it.
+// (Any r and any bytes: the byte returned lies in the range.)
+__device__ __forceinline__ uint2 byte_of_bit(const OctArgs &a, uint64_t a0, uint64_t a1, uint64_t r, uint32_t lane)
 {
-    return (code << 3) + (b ? 31u - (uint32_t)__clz(b) : 0u);
+    uint64_t t = a0 / kOccTile, n = (a1 - 1) / kOccTile - t + 1;  // the last of n tiles from t that starts at or before r
+    while (n > 1) {
+        const uint64_t step = (n + 31) / 32, probe = lane * step;
+        const uint32_t le = __ballot_sync(0xFFFFFFFFu, probe < n && a.tbase[t + probe] <= r);
+        const uint32_t last = le ? 31u - (uint32_t)__clz(le) : 0u;
+        t += last * step;
+        n = min(step, n - last * step);
+    }
+    const uint64_t tx = t * kOccTile, tb = a.tbase[t];
+    uint32_t rest = r > tb ? (uint32_t)min(r - tb, (uint64_t)(8 * kOccTile)) : 0u;
+    uint32_t c = 0;
+#pragma unroll
+    for (uint32_t k = 0; k < kOccTile / 128; ++k) c += __popc(word_at(a.occ, a.n_occ, tx + lane * (kOccTile / 32) + 4 * k));
+    uint32_t inc = warp_inclusive_sum(c);
+    uint32_t m = __ballot_sync(0xFFFFFFFFu, inc > rest);
+    const uint32_t part = m ? (uint32_t)__ffs(m) - 1u : 31u;  // 32 bytes
+    rest -= min(rest, __shfl_sync(0xFFFFFFFFu, inc - c, part));
+    const uint64_t x = tx + part * (kOccTile / 32) + lane;
+    c = x < a.n_occ ? __popc(a.occ[x]) : 0u;
+    inc = warp_inclusive_sum(c);
+    m = __ballot_sync(0xFFFFFFFFu, inc > rest);
+    const uint32_t byte = m ? (uint32_t)__ffs(m) - 1u : 31u;
+    rest -= min(rest, __shfl_sync(0xFFFFFFFFu, inc - c, byte));
+    const uint64_t y = min(max(tx + part * (kOccTile / 32) + byte, a0), a1 - 1);
+    return make_uint2((uint32_t)(y - a0), min(rest, 8u));
 }
 
-__global__ void __launch_bounds__(kLevelThreads) expand_level_kernel(LevelArgs a)
+// A warp per CTA of octree_leaves_kernel: where it begins in each level.  Then a warp per frame and level: that the
+// level's bytes hold as many set bits as the next level has nodes.
+__global__ void __launch_bounds__(256) octree_paths_kernel(OctArgs a)
 {
-    __shared__ uint64_t sh[33];
-    __shared__ uint64_t s_leaf[kLeafStage];
-    __shared__ uint16_t s_pref[kOccTile];
-    __shared__ uint8_t s_occ[kOccTile];
-    __shared__ uint32_t s_lo, s_hi;
+    const uint32_t lane = threadIdx.x & 31, w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (w == 0 && lane == 0) a.gap[a.nv_total] = (uint8_t)kInfLevel;  // sentinel after the last voxel
+    if (w < a.tiles) {
+        const uint32_t f = find_frame(a.tile_pref, a.F, w), k = w - a.tile_pref[f];
+        const DecFrame &fd = a.fr[f];
+        uint32_t d = fd.J - 1, i = k ? k * kLeafTile - 1 : 0u;  // the last node of the CTA before
+        uint2 *path = a.path + (uint64_t)w * kMaxJ;
+        const uint64_t leaf0 = bits_before(a, fd.occ_off + fd.boff[d] + i, lane) - fd.pbase[d];
+        if (lane == 0) {
+            path[d] = make_uint2(i, 0u);
+            a.leaf0[w] = (uint32_t)min(leaf0, (uint64_t)fd.nv);
+        }
+        while (d > 0) {
+            --d;
+            const uint64_t a0 = fd.occ_off + fd.boff[d];
+            const uint2 p = byte_of_bit(a, a0, a0 + fd.lsz[d], fd.pbase[d] + i, lane);
+            if (lane == 0) path[d] = p;
+            i = p.x;
+        }
+    } else if (w < a.tiles + a.F * a.Jmax) {
+        const uint32_t f = (w - a.tiles) / a.Jmax, d = (w - a.tiles) - f * a.Jmax;
+        const DecFrame &fd = a.fr[f];
+        if (fd.nv == 0 || d >= fd.J) return;
+        const uint64_t a0 = fd.occ_off + fd.boff[d];
+        const uint64_t bits = bits_before(a, a0 + fd.lsz[d], lane) - bits_before(a, a0, lane);
+        if (lane == 0 && bits != fd.lsz[d + 1]) {
+            *a.broken = 1;
+            set_error(&a.st->err, kErrCorrupt);
+        }
+    }
+}
+
+// the set bits of v as children of a node: calls put(rank, code) for each, rank counting from `rank`
+template <typename Put>
+__device__ __forceinline__ void children(uint64_t code, uint32_t v, uint32_t rank, Put put)
+{
+    for (; v; v &= v - 1u) put(rank++, (code << 3) + (uint32_t)(__ffs(v) - 1));
+}
+
+__global__ void __launch_bounds__(kLeafThreads) octree_leaves_kernel(OctArgs a)
+{
+    __shared__ uint64_t s_code[2][kLeafStage];  // a level's codes, the last level's in [0]; then the voxels' in [1]
+    __shared__ uint2 s_path[kMaxJ];             // first node, its children of the CTA before
+    __shared__ uint32_t s_cnt[kMaxJ];           // nodes
+    __shared__ uint32_t s_word[kMaxJ][32];      // the bytes of a level of few nodes
+    __shared__ uint32_t s_scan[2][kLeafThreads / 32];
     __shared__ uint64_t s_prev;
-    __shared__ int s_first;  // the tile holds the level's first node (its first voxel starts a frame)
-    const uint32_t g = blockIdx.x, t = threadIdx.x;
-    const uint32_t f = find_frame(a.tile_pref, a.F, g);
+    const uint32_t g = blockIdx.x, t = threadIdx.x, lane = t & 31;
+    if (*a.broken) {  // nothing to follow: every voxel on its own, for what reads the gap levels next
+        const uint64_t per = (a.nv_total + a.tiles - 1) / a.tiles, lo = g * per, hi = min(lo + per, a.nv_total);
+        for (uint64_t i = lo + t; i < hi; i += kLeafThreads) a.gap[i] = (uint8_t)kInfLevel;
+        return;
+    }
+    const uint32_t f = find_frame(a.tile_pref, a.F, g), k = g - a.tile_pref[f];
+    const bool last = g + 1 == a.tile_pref[f + 1];
     const DecFrame &fd = a.fr[f];
-    const uint32_t d = a.d;
-    const uint64_t a0 = fd.occ_off + fd.boff[d], a1 = a0 + fd.lsz[d];
-    const uint64_t tile = a0 / kOccTile + (g - a.tile_pref[f]);
-    const uint64_t tx = tile * kOccTile;
-    const bool leaf = d + 1 == fd.J;
-    const uint64_t *src = a.nodes + fd.noff[d];
-    const uint64_t wv = word8_at(a.occ, a.n_occ, tx + 8ull * t);
-    // the codes of this thread's nodes (tile bytes t, t + 128, ...) are loaded before the scan
-    uint64_t code[8];
-#pragma unroll
-    for (uint32_t k = 0; k < 8; ++k) {
-        const uint64_t x = tx + k * kLevelThreads + t;
-        code[k] = (x >= a0 && x < a1) ? src[x - a0] : 0ull;
-    }
-    const uint64_t xs = tx > a0 ? tx : a0;  // the tile's first byte of this level
-    if (t == 0) {
-        s_first = xs == a0;
-        s_prev = (leaf && xs > a0 && xs < a1) ? last_child(src[xs - 1 - a0], a.occ[xs - 1]) : 0ull;
-    }
-    const uint64_t tb = a.tbase[tile];
-    uint64_t tot;
-    uint32_t lp = (uint32_t)block_exclusive_sum<uint64_t>((uint64_t)__popcll(wv), sh, &tot);
-#pragma unroll
-    for (uint32_t k = 0; k < 8; ++k) {  // per byte: set bits of the tile before it
-        const uint32_t b = (uint32_t)(wv >> (8u * k)) & 0xFFu;
-        s_pref[8 * t + k] = (uint16_t)lp;
-        s_occ[8 * t + k] = (uint8_t)b;
-        lp += __popc(b);
-    }
-    const uint64_t base = fd.pbase[d];
-    const uint32_t M1 = fd.lsz[d + 1];
-    const bool stage = leaf && tot <= kLeafStage;
-    if (t == 0) {  // the staged range: the tile's bytes of this level
-        s_lo = 0;
-        s_hi = (uint32_t)tot;
+    const uint32_t J = fd.J;
+    if (t < J) {
+        const uint2 p = a.path[(uint64_t)g * kMaxJ + t];
+        const uint32_t e = last ? fd.lsz[t] - 1u : a.path[(uint64_t)(g + 1) * kMaxJ + t].x;
+        s_path[t] = p;
+        s_cnt[t] = e >= p.x ? min(e - p.x + 1u, kLeafNodes) : 0u;
     }
     __syncthreads();
-    bool bad = false;
-#pragma unroll
-    for (uint32_t k = 0; k < 8; ++k) {
-        const uint32_t j = k * kLevelThreads + t;
-        const uint64_t x = tx + j;
-        if (x < a0 || x >= a1) continue;
-        const uint32_t byte = s_occ[j];
-        const uint32_t pj = s_pref[j];
-        if (x == a0) s_lo = pj;
-        if (x + 1 == a1) {
-            if (tb + pj + __popc(byte) - base != M1) bad = true;  // the level's popcounts add up to the next level
-            s_hi = pj + __popc(byte);
-        }
-        const uint64_t cw = tb + pj - base;
-        if (byte == 0 || cw + (uint64_t)__popc(byte) > M1) {
-            bad = true;
-            continue;
-        }
-        const uint64_t c = code[k] << 3;
-        if (!leaf) {
-            uint64_t *dst = a.nodes + fd.noff[d + 1] + cw;
-            for (uint32_t bits = byte; bits; bits &= bits - 1u) *dst++ = c + (uint32_t)(__ffs(bits) - 1);
-        } else if (stage) {
-            uint32_t sl = pj;
-            for (uint32_t bits = byte; bits; bits &= bits - 1u) s_leaf[sl++] = c + (uint32_t)(__ffs(bits) - 1);
-        } else {  // unstaged voxels: the one before comes from node x - 1
-            uint32_t v = fd.vstart + (uint32_t)cw;
-            bool have_prev = x > a0;
-            uint64_t prev = have_prev ? last_child(src[x - 1 - a0], x > tx ? s_occ[j - 1] : a.occ[x - 1]) : 0ull;
-            for (uint32_t bits = byte; bits; bits &= bits - 1u) {
-                const uint64_t m = c + (uint32_t)(__ffs(bits) - 1);
-                a.gap[v] = have_prev ? (uint8_t)gap_level(prev, m, 64) : (uint8_t)kInfLevel;
-                if (a.pos) leaf_out(fd, a.ctab, v, m, a.pos);
-                prev = m;
-                have_prev = true;
-                ++v;
+    // word t of the bytes of this CTA's nodes of level d (aligned: `lead` bytes before the first node), others zero
+    auto lead_of = [&](uint32_t d) { return (uint32_t)((fd.occ_off + fd.boff[d] + s_path[d].x) & 3u); };
+    auto word_of = [&](uint32_t d, uint32_t at) {
+        const uint64_t x = fd.occ_off + fd.boff[d] + s_path[d].x;
+        const uint32_t lead = (uint32_t)(x & 3u), cnt = s_cnt[d], o = 4 * at;
+        if (o >= lead + cnt) return 0u;
+        uint32_t v = *reinterpret_cast<const uint32_t *>(a.occ + (x - lead) + o);  // 8 bytes of slack after the last
+        if (o < lead) v &= 0xFFFFFFFFu << (8u * (lead - o));
+        if (o + 4 > lead + cnt) v &= (1u << (8u * (lead + cnt - o))) - 1u;
+        return v;
+    };
+    auto few = [&](uint32_t d) { return s_cnt[d] + 3u <= 128u; };  // a warp's words
+    for (uint32_t d = t >> 5; d < J; d += kLeafThreads / 32)
+        if (few(d)) s_word[d][lane] = word_of(d, lane);
+    if (t == 0) s_code[(J - 1) & 1u][0] = 0ull;  // the implicit root of Algorithm 2
+    __syncthreads();
+    uint32_t d = 0;
+    while (d + 1 < J && few(d)) ++d;
+    if (t < 32)  // levels of few nodes: one warp, a node per lane
+        for (uint32_t e = 0; e < d; ++e) {
+            const uint8_t *bytes = reinterpret_cast<const uint8_t *>(s_word[e]) + lead_of(e);
+            const uint64_t *from = s_code[(J - 1 - e) & 1u];
+            uint64_t *to = s_code[(J - e) & 1u];
+            const uint32_t cnt = s_cnt[e], cnt1 = s_cnt[e + 1];
+            uint32_t rank = 0u - s_path[e].y;  // of the next child; wraps for the children of the CTA before
+            for (uint32_t n = lane; n < cnt + lane; n += 32) {
+                const uint32_t byte = n < cnt ? bytes[n] : 0u, c = __popc(byte), inc = warp_inclusive_sum(c);
+                children(byte ? from[n] : 0ull, byte, rank + inc - c, [&](uint32_t r, uint64_t m) {
+                    if (r < cnt1) to[r] = m;
+                });
+                rank += __shfl_sync(0xFFFFFFFFu, inc, 31);
             }
+            __syncwarp();
         }
-    }
-    if (bad) set_error(&a.st->err, kErrCorrupt);
-    if (stage) {
+    uint32_t v = word_of(d, t);
+    __syncthreads();
+    // set bits of the CTA's nodes before the thread's word (one barrier), and of all of them
+    auto scan = [&](uint32_t d, uint32_t c, uint32_t *tot) {
+        uint32_t *sh = s_scan[d & 1u];
+        const uint32_t inc = warp_inclusive_sum(c);
+        if (lane == 31) sh[t >> 5] = inc;
         __syncthreads();
-        const uint32_t lo = s_lo, hi = s_hi;
-        const uint64_t vb = (uint64_t)fd.vstart + tb - base;  // voxel row of staged slot i: vb + i
-        for (uint32_t i = lo + t; i < hi; i += kLevelThreads) {
-            const uint64_t m = s_leaf[i];
-            const uint32_t v = (uint32_t)(vb + i);
-            a.gap[v] = (i > lo) ? (uint8_t)gap_level(s_leaf[i - 1], m, 64)
-                                : (s_first ? (uint8_t)kInfLevel : (uint8_t)gap_level(s_prev, m, 64));
-            if (a.pos) leaf_out(fd, a.ctab, v, m, a.pos);
+        uint32_t before = inc - c, all = 0;
+#pragma unroll
+        for (uint32_t w = 0; w < kLeafThreads / 32; ++w) {
+            const uint32_t x = sh[w];
+            before += w < (t >> 5) ? x : 0u;
+            all += x;
         }
+        *tot = all;
+        return before;
+    };
+    uint32_t tot;
+    for (; d + 1 < J; ++d) {  // a word of bytes (four nodes) per thread
+        const uint32_t next = word_of(d + 1, t);  // lands while this level is taken
+        const uint32_t lead = lead_of(d), skip = s_path[d].y, cnt = s_cnt[d], cnt1 = s_cnt[d + 1];
+        const uint64_t *from = s_code[(J - 1 - d) & 1u];
+        uint64_t *to = s_code[(J - d) & 1u];
+        uint32_t rank = scan(d, __popc(v), &tot) - skip;  // wraps for the children of the CTA before
+#pragma unroll
+        for (uint32_t b = 0; b < 4; ++b) {
+            const uint32_t n = 4 * t + b - lead, byte = (v >> (8 * b)) & 0xFFu;  // n wraps before the first node
+            if (n >= cnt) continue;
+            children(from[n], byte, rank, [&](uint32_t r, uint64_t m) {
+                if (r < cnt1) to[r] = m;
+            });
+            rank += __popc(byte);
+        }
+        __syncthreads();
+        v = next;
+    }
+    // last level: the voxels, kLeafStage at a time
+    const uint32_t lead = lead_of(d), cnt = s_cnt[d];
+    const uint32_t before0 = scan(d, __popc(v), &tot);
+    const uint64_t vb = (uint64_t)fd.vstart + a.leaf0[g];
+    const uint64_t vend = (uint64_t)fd.vstart + fd.nv;
+    // the first node's voxels are the CTA's before (but the frame's first CTA's)
+    const uint32_t own = k == 0 ? 0u : (uint32_t)__popc(a.occ[fd.occ_off + fd.boff[d] + s_path[d].x]);
+    uint64_t *out = s_code[1];
+    for (uint32_t base = 0; base < tot; base += kLeafStage) {
+        uint32_t before = before0;
+#pragma unroll
+        for (uint32_t b = 0; b < 4; ++b) {
+            const uint32_t n = 4 * t + b - lead, byte = (v >> (8 * b)) & 0xFFu;
+            if (n >= cnt) continue;
+            children(s_code[0][n], byte, before - base, [&](uint32_t r, uint64_t c) {
+                if (r < kLeafStage) out[r] = c;
+            });
+            before += __popc(byte);
+        }
+        __syncthreads();
+        const uint32_t hi = min(tot - base, kLeafStage);
+        for (uint32_t i = t; i < hi; i += kLeafThreads) {
+            const uint32_t r = base + i;
+            if (r < own || vb + r >= vend) continue;
+            const uint64_t m = out[i];
+            const uint32_t row = (uint32_t)(vb + r);
+            const uint64_t prev = i ? out[i - 1] : s_prev;
+            a.gap[row] = r ? (uint8_t)gap_level(prev, m, 64) : (uint8_t)kInfLevel;
+            if (a.pos) leaf_out(fd, a.ctab, row, m, a.pos);
+        }
+        const uint64_t end = out[hi - 1];
+        __syncthreads();
+        if (t == 0) s_prev = end;
     }
 }
 
@@ -382,38 +496,37 @@ void launch_batch_rans_decode(const DecFrame *fr, uint32_t F, uint32_t max_chunk
     count_launch();
 }
 
-void launch_batch_roots(const DecFrame *fr, uint32_t F, uint64_t *nodes, uint8_t *gap, uint64_t nv_total,
-                        cudaStream_t s)
-{
-    roots_kernel<<<(F + 63) / 64, 64, 0, s>>>(fr, F, nodes, gap, nv_total);
-    count_launch();
-}
-
 uint64_t occ_tiles(uint64_t n_occ) { return (n_occ + kOccTile - 1) / kOccTile; }
 
 void launch_occ_tile_bases(const uint8_t *occ, uint64_t n_occ, uint32_t *tsum, uint64_t *tbase, uint64_t *partials,
-                           int num_sms, cudaStream_t s)
+                           uint32_t *broken, DevState *st, int num_sms, cudaStream_t s)
 {
     const uint64_t nt = occ_tiles(n_occ);
     if (nt) {
         const uint64_t want = (nt + 7) / 8, cap = (uint64_t)num_sms * 8;
-        occ_tile_popc_kernel<<<(uint32_t)(want < cap ? want : cap), 256, 0, s>>>(occ, n_occ, nt, tsum);
+        occ_tile_popc_kernel<<<(uint32_t)(want < cap ? want : cap), 256, 0, s>>>(occ, n_occ, nt, tsum, broken, st);
         count_launch();
     }
     launch_scan_u32_to_u64(tsum, nt, tbase, partials, num_sms, s);
 }
 
-void launch_batch_level(const DecFrame *fr, uint32_t F, uint32_t d, const uint32_t *tile_pref, uint32_t tiles,
-                        const uint8_t *occ, uint64_t n_occ, const uint64_t *tbase, uint64_t *nodes, const float *ctab,
-                        float *pos, uint8_t *gap, DevState *st, cudaStream_t s)
+uint64_t octree_path_words(uint64_t tiles) { return 2 * tiles * kMaxJ; }
+
+uint32_t octree_tiles(uint32_t nodes) { return (nodes + kLeafTile - 1) / kLeafTile; }
+
+void launch_octree_leaves(const DecFrame *fr, uint32_t F, uint32_t Jmax, const uint32_t *tile_pref, uint32_t tiles,
+                          const uint8_t *occ, uint64_t n_occ, const uint64_t *tbase, uint32_t *path, uint32_t *leaf0,
+                          const float *ctab, float *pos, uint8_t *gap, uint64_t nv_total, uint32_t *broken,
+                          DevState *st, cudaStream_t s)
 {
+    OctArgs a{fr, F, Jmax, tile_pref, tiles, occ, n_occ, tbase, reinterpret_cast<uint2 *>(path), leaf0, ctab, pos, gap,
+              nv_total, broken, st};
+    octree_paths_kernel<<<(tiles + F * Jmax + 7) / 8 + 1, 256, 0, s>>>(a);
+    count_launch();
     if (tiles == 0) return;
-    LevelArgs a{fr, F, d, tile_pref, occ, n_occ, tbase, nodes, ctab, pos, gap, st};
-    expand_level_kernel<<<tiles, kLevelThreads, 0, s>>>(a);
+    octree_leaves_kernel<<<tiles, kLeafThreads, 0, s>>>(a);
     count_launch();
 }
-
-uint64_t occ_tile_first(uint64_t byte) { return byte / kOccTile; }
 
 void launch_batch_centre_tables(const DecFrame *fr, uint32_t F, uint32_t Jmax, float *ctab, int num_sms,
                                 cudaStream_t s)

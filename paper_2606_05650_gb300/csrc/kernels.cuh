@@ -201,7 +201,6 @@ struct DecFrame {
     uint32_t B, nb;
     FrameGrid grid;
     uint64_t ctab_off;          // first entry of the frame's centre table (3 x 2^J floats), or ~0: computed directly
-    uint64_t noff[22];          // node-array offset of each level (level J lives in the voxel rows)
     uint64_t boff[22];          // offset of each level's bytes inside the frame's occupancy bytes
     uint64_t pbase[22];         // set bits of the batch occupancy bytes before each level's first byte
     uint32_t lsz[22];
@@ -289,20 +288,20 @@ void launch_batch_occ_bytes(const DecFrame *fr, uint32_t F, uint8_t *occ_all, ui
 // chunks' byte offsets
 void launch_batch_rans_decode(const DecFrame *fr, uint32_t F, uint32_t max_chunks_per_frame, uint32_t chunk_max,
                               uint8_t *occ_all, uint32_t *tabs, uint64_t *cstart, DevState *st, cudaStream_t s);
-// Octree levels of every frame (Algorithm 3), one launch per level: tile popcounts of the batch occupancy
-// bytes and their exclusive scan (tbase, tiles + 1 entries), then per level the CTAs of the tiles holding
-// that level's bytes (tile_pref: F + 1 CTA offsets per frame; a frame's CTAs start at tile
-// occ_tile_first(first byte of the level)).  A frame's last level writes voxel centres and gap levels, not
-// codes.  The roots launch writes every frame's root and the gap sentinel gap[nv_total].
+// Octree of every frame (Algorithm 3): tile popcounts of the batch occupancy bytes and their exclusive scan
+// (tbase, tiles + 1 entries), then the voxels' centres (pos, or null) and gap levels, and the gap sentinel
+// gap[nv_total].  tile_pref: F + 1 CTA offsets, octree_tiles(nodes of the frame's last level) CTAs a frame, tiles in
+// all; path and leaf0: octree_path_words(tiles) and tiles words of scratch.  *broken, zero before, is set (as is the
+// error) where the bytes are not an octree's with the frames' level sizes.
 uint64_t occ_tiles(uint64_t n_occ);
-uint64_t occ_tile_first(uint64_t byte);
+uint32_t octree_tiles(uint32_t nodes);
+uint64_t octree_path_words(uint64_t tiles);
 void launch_occ_tile_bases(const uint8_t *occ, uint64_t n_occ, uint32_t *tsum, uint64_t *tbase, uint64_t *partials,
-                           int num_sms, cudaStream_t s);
-void launch_batch_roots(const DecFrame *fr, uint32_t F, uint64_t *nodes, uint8_t *gap, uint64_t nv_total,
-                        cudaStream_t s);
-void launch_batch_level(const DecFrame *fr, uint32_t F, uint32_t d, const uint32_t *tile_pref, uint32_t tiles,
-                        const uint8_t *occ, uint64_t n_occ, const uint64_t *tbase, uint64_t *nodes, const float *ctab,
-                        float *pos, uint8_t *gap, DevState *st, cudaStream_t s);
+                           uint32_t *broken, DevState *st, int num_sms, cudaStream_t s);
+void launch_octree_leaves(const DecFrame *fr, uint32_t F, uint32_t Jmax, const uint32_t *tile_pref, uint32_t tiles,
+                          const uint8_t *occ, uint64_t n_occ, const uint64_t *tbase, uint32_t *path, uint32_t *leaf0,
+                          const float *ctab, float *pos, uint8_t *gap, uint64_t nv_total, uint32_t *broken,
+                          DevState *st, cudaStream_t s);
 // Voxel-centre tables: a centre coordinate depends only on that axis' voxel
 // coordinate, so frames with 2^J <= N_v evaluate the FP64 expression once per
 // axis value (3 x 2^J) instead of once per voxel.
