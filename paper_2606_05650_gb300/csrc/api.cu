@@ -1443,28 +1443,60 @@ gsnfs_status read_headers(gsnfs_ctx *ctx, cudaStream_t s, const uint8_t *d_in, u
     return parse_sections(hp + 4096, hp + 4096 + 64, P);
 }
 
+// level offsets of a frame whose occupancy bytes follow pb set bits of the frames before; returns those after it
+uint64_t set_levels(DecFrame &d, const uint32_t *lsz, uint64_t pb)
+{
+    uint64_t bytes = 0;
+    for (uint32_t lv = 0; lv <= d.J; ++lv) {
+        d.lsz[lv] = lsz[lv];
+        d.boff[lv] = bytes;
+        if (lv < d.J) {
+            d.pbase[lv] = pb;  // the bytes of a level hold as many set bits as the next level has nodes
+            bytes += lsz[lv];
+            pb += lsz[lv + 1];
+        }
+    }
+    return pb;
+}
+
 struct DecLayout {
     uint8_t *occ, *gap;
     uint64_t *nodes, *codes, *nvdev, *block_off, *spart;
     uint32_t *pref, *ppart;
+    DecFrame *fr;      // without codes: the octree by runs of last-level nodes, as in a batch of one frame
+    uint32_t *tile_pref, *path, *leaf0, *broken, *tsum;
+    uint64_t *tbase, *tpart;
     float *Y, *pool, *step, *ctab, *klt;
     uint32_t *vst;
     FrameGrid *grid;
     RahtPlanDev plan;
 };
 
-size_t carve_decode(Carve &cv, DecLayout &L, const ParsedHeader &P, int num_sms, const uint32_t *tune)
+// codes: the leaf codes are wanted (octree_decode, levels of detail), which come level by level
+size_t carve_decode(Carve &cv, DecLayout &L, const ParsedHeader &P, int num_sms, const uint32_t *tune, bool codes)
 {
     L.grid = cv.take<FrameGrid>(1);
     L.nvdev = cv.take<uint64_t>(1);
     L.step = cv.take<float>(P.C + 1);
     L.occ = cv.take<uint8_t>(P.n_occ + 8);
-    L.pref = cv.take<uint32_t>(P.n_occ + 2);
-    L.ppart = cv.take<uint32_t>(2 * (uint64_t)num_sms + 8);
-    uint64_t nodes = 0;
-    for (uint32_t d = 0; d < P.J; ++d) nodes += P.lsz[d];
-    L.nodes = cv.take<uint64_t>(nodes + 1);
-    L.codes = cv.take<uint64_t>(P.nv + 1);
+    if (codes) {
+        L.pref = cv.take<uint32_t>(P.n_occ + 2);
+        L.ppart = cv.take<uint32_t>(2 * (uint64_t)num_sms + 8);
+        uint64_t nodes = 0;
+        for (uint32_t d = 0; d < P.J; ++d) nodes += P.lsz[d];
+        L.nodes = cv.take<uint64_t>(nodes + 1);
+        L.codes = cv.take<uint64_t>(P.nv + 1);
+    } else {
+        const uint64_t tiles = octree_tiles(P.lsz[P.J - 1]);
+        L.fr = cv.take<DecFrame>(1);
+        L.tile_pref = cv.take<uint32_t>(2);
+        L.path = cv.take<uint32_t>(octree_path_words(tiles));
+        L.leaf0 = cv.take<uint32_t>(tiles + 1);
+        L.broken = cv.take<uint32_t>(1);
+        L.tsum = cv.take<uint32_t>(occ_tiles(P.n_occ) + 1);
+        L.tbase = cv.take<uint64_t>(occ_tiles(P.n_occ) + 2);
+        L.tpart = cv.take<uint64_t>(scan_partial_words(occ_tiles(P.n_occ), num_sms) + 1);
+    }
     L.gap = cv.take<uint8_t>(P.nv + 2);
     L.ctab = cv.take<float>(((1ull << P.J) <= P.nv) ? (3ull << P.J) : 1);
     L.klt = cv.take<float>(kKltFloats);
@@ -1496,8 +1528,7 @@ gsnfs_status lod_from_voxels(gsnfs_ctx *ctx, cudaStream_t s, cudaStream_t cs, co
                              const LodReq &lod);
 
 gsnfs_status decode_impl(gsnfs_ctx *ctx, cudaStream_t s, const uint8_t *d_in, uint64_t bytes, float *d_pos,
-                         float *d_attr, uint64_t capacity_nv, uint64_t *out_nv, const uint64_t **codes_out = nullptr,
-                         const LodReq *lod = nullptr)
+                         float *d_attr, uint64_t capacity_nv, uint64_t *out_nv, const LodReq *lod = nullptr)
 {
     ParsedHeader P{};
     gsnfs_status st = read_headers(ctx, s, d_in, bytes, P);
@@ -1507,12 +1538,11 @@ gsnfs_status decode_impl(gsnfs_ctx *ctx, cudaStream_t s, const uint8_t *d_in, ui
     if (P.nv == 0) return GSNFS_OK;
     DecLayout L;
     Carve m(nullptr);
-    size_t need = carve_decode(m, L, P, ctx->num_sms, ctx->tune);
+    size_t need = carve_decode(m, L, P, ctx->num_sms, ctx->tune, lod != nullptr);
     st = grow_arena(ctx, need, s);
     if (st) return st;
     Carve cv(ctx->arena);
-    carve_decode(cv, L, P, ctx->num_sms, ctx->tune);
-    if (codes_out) *codes_out = L.codes;
+    carve_decode(cv, L, P, ctx->num_sms, ctx->tune, lod != nullptr);
     DevState *dst = ctx->st;
     // host-computed grid and steps
     unsigned char *hp = ctx->pinned;
@@ -1533,6 +1563,26 @@ gsnfs_status decode_impl(gsnfs_ctx *ctx, cudaStream_t s, const uint8_t *d_in, ui
     if (P.color) CK(up.add(L.klt, d_in + P.klt_off, 4 * kKltFloats));
     if (P.C) CK(up.add(L.step, hp + 256, 4 * P.C));
     CK(up.add(dst, nullptr, 8));
+    const uint32_t tiles = octree_tiles(P.lsz[P.J - 1]);
+    if (!lod) {
+        DecFrame f{};
+        f.n_occ = P.n_occ;
+        f.nv = (uint32_t)P.nv;
+        f.J = P.J;
+        f.mode = P.occ_mode;
+        f.aux = P.occ_aux;
+        f.occ_sec = d_in + P.hb;
+        f.grid = g;
+        f.ctab_off = d_pos && (1ull << P.J) <= P.nv ? 0ull : ~0ull;
+        set_levels(f, P.lsz, 0);
+        static_assert(sizeof(DecFrame) <= 1536, "beside the headers in pinned memory");
+        memcpy(hp + 2048, &f, sizeof f);
+        const uint32_t tp_h[2] = {0u, tiles};
+        memcpy(hp + 200, tp_h, 8);
+        CK(up.add(L.fr, hp + 2048, sizeof f));
+        CK(up.add(L.tile_pref, hp + 200, 8));
+        CK(up.add(L.broken, nullptr, 4));
+    }
     CK(up.flush());
     const int sms = ctx->num_sms;
     // a12's RLGR decode needs only the block tables: it runs on s beside a11 and the schedule (the longer
@@ -1556,22 +1606,28 @@ gsnfs_status decode_impl(gsnfs_ctx *ctx, cudaStream_t s, const uint8_t *d_in, ui
     const uint8_t *sec = d_in + P.hb;
     const uint8_t *occ = L.occ;
     stage_begin(sg, kStOccDecode);
-    if (P.occ_mode == 0)
+    if (P.occ_mode == 0 && lod)
         occ = sec + 16;
+    else if (P.occ_mode == 0)  // aligned, for loads of words
+        launch_batch_occ_bytes(L.fr, 1, L.occ, P.n_occ, sms, sg);
     else if (P.occ_mode == 2)
         launch_fill(L.occ, P.n_occ, (uint8_t)P.occ_aux, sg);
     else
         launch_rans_decode(sec, P.occ_bytes, P.n_occ, P.occ_aux, P.chunk, L.occ, dst, sms, sg);
     stage_end(sg, kStOccDecode);
     stage_begin(sg, kStOctreeDecode);
-    launch_octree_decode(occ, P.n_occ, P.J, P.lsz, L.nodes, L.pref, L.ppart, L.codes, dst, sms, sg);
-    if (d_pos) launch_voxel_centres(L.codes, P.nv, P.J, L.grid, d_pos, sg, L.ctab);
+    if (lod) {
+        launch_octree_decode(occ, P.n_occ, P.J, P.lsz, L.nodes, L.pref, L.ppart, L.codes, dst, sms, sg);
+    } else {
+        launch_occ_tile_bases(L.occ, P.n_occ, L.tsum, L.tbase, L.tpart, L.broken, dst, sms, sg);
+        launch_octree_leaves(L.fr, 1, P.J, d_pos && (1ull << P.J) <= P.nv ? P.J : 0u, L.tile_pref, tiles, L.occ, P.n_occ, L.tbase, L.path, L.leaf0, L.ctab, d_pos,
+                             L.gap, P.nv, L.broken, dst, sg);
+    }
     stage_end(sg, kStOctreeDecode);
     if (lod) return lod_from_voxels(ctx, sg, s, P, L, attrs, *lod);
     // a12: schedule, then (after the RLGR branch) the inverse RAHT
     if (attrs) {
         stage_begin(sg, kStPrelude);
-        launch_gap_levels(L.codes, P.nv, L.gap, sg);
         launch_raht_prelude(L.plan, L.gap, dst, L.nvdev, P.nv, sms, sg);
         stage_end(sg, kStPrelude);
         st = stream_wait(ctx, sg, s);  // the coefficients
@@ -1830,10 +1886,14 @@ gsnfs_status decode_batch_impl(gsnfs_ctx *ctx, cudaStream_t s, uint32_t F, const
     } L;
     bool any_color = false;
     for (uint32_t f = 0; f < F; ++f) any_color |= P[f].color != 0;
-    // voxel-centre tables for frames with 2^J <= N_v (see launch_batch_centre_tables)
+    // voxel-centre tables for frames with 2^J <= N_v (see launch_octree_leaves)
     uint64_t ctab_total = 0;
+    uint32_t Jtab = 0;
     for (uint32_t f = 0; f < F; ++f)
-        if (d_pos && P[f].nv && (1ull << P[f].J) <= P[f].nv) ctab_total += 3ull << P[f].J;
+        if (d_pos && P[f].nv && (1ull << P[f].J) <= P[f].nv) {
+            ctab_total += 3ull << P[f].J;
+            Jtab = std::max(Jtab, P[f].J);
+        }
     auto carve = [&](Carve &cv) {
         L.fr = cv.take<DecFrame>(F);
         L.vstart = cv.take<uint32_t>(F + 1);
@@ -1939,16 +1999,7 @@ gsnfs_status decode_batch_impl(gsnfs_ctx *ctx, cudaStream_t s, uint32_t F, const
         d.grid.ext = H.ext;
         d.grid.scale = std::ldexp(1.0, (int)H.J) / H.ext;
         d.grid.cell = H.ext / std::ldexp(1.0, (int)H.J);
-        uint64_t b2 = 0;
-        for (uint32_t lv = 0; lv <= H.J; ++lv) {
-            d.lsz[lv] = H.lsz[lv];
-            d.boff[lv] = b2;
-            if (lv < H.J) {
-                d.pbase[lv] = pb;  // the bytes of a level hold as many set bits as the next level has nodes
-                b2 += H.lsz[lv];
-                pb += H.lsz[lv + 1];
-            }
-        }
+        pb = set_levels(d, H.lsz, pb);
         hf[f] = d;
         hvs[f] = (uint32_t)vs;
         hjo[f] = jo;
@@ -2008,9 +2059,8 @@ gsnfs_status decode_batch_impl(gsnfs_ctx *ctx, cudaStream_t s, uint32_t F, const
     if (any_rans) launch_batch_rans_decode(L.fr, F, max_nch, chunk_max, L.occ, L.tabs, L.cstart, dst, sg);
     stage_end(sg, kStOccDecode);
     stage_begin(sg, kStOctreeDecode);
-    if (ctab_total) launch_batch_centre_tables(L.fr, F, Jmax, L.ctab, sms, sg);
     launch_occ_tile_bases(L.occ, n_occ, L.tsum, L.tbase, L.tpart, L.broken, dst, sms, sg);
-    launch_octree_leaves(L.fr, F, Jmax, L.tile_pref, (uint32_t)tiles, L.occ, n_occ, L.tbase, L.path, L.leaf0, L.ctab,
+    launch_octree_leaves(L.fr, F, Jmax, Jtab, L.tile_pref, (uint32_t)tiles, L.occ, n_occ, L.tbase, L.path, L.leaf0, L.ctab,
                          d_pos, L.gap, N, L.broken, dst, sg);
     stage_end(sg, kStOctreeDecode);
     // a12: RAHT schedule, then (after the RLGR branch) the inverse RAHT
@@ -2371,7 +2421,7 @@ gsnfs_status gsnfs_decode_frame_lod(gsnfs_ctx *ctx, void *stream, const uint8_t 
     }
     LodReq r{depth, d_pos, d_attr, capacity_nodes, out_nodes};
     uint64_t n = 0;
-    return decode_impl(ctx, s, d_bitstream, bytes, nullptr, d_attr, ~0ull, &n, nullptr, &r);
+    return decode_impl(ctx, s, d_bitstream, bytes, nullptr, d_attr, ~0ull, &n, &r);
 }
 
 gsnfs_status gsnfs_decode_batch_async(gsnfs_ctx *ctx, void *stream, uint32_t frames, const uint8_t *d_in,
@@ -2563,10 +2613,10 @@ gsnfs_status gsnfs_octree_decode(gsnfs_ctx *ctx, void *stream, const uint8_t *d_
     P.nb = 0;
     DecLayout L;
     Carve m(nullptr);
-    gsnfs_status st = grow_arena(ctx, carve_decode(m, L, P, ctx->num_sms, ctx->tune), s);
+    gsnfs_status st = grow_arena(ctx, carve_decode(m, L, P, ctx->num_sms, ctx->tune, true), s);
     if (st) return st;
     Carve cv(ctx->arena);
-    carve_decode(cv, L, P, ctx->num_sms, ctx->tune);
+    carve_decode(cv, L, P, ctx->num_sms, ctx->tune, true);
     st = grow_pinned(ctx, 4096);
     if (st) return st;
     CK(dev_memset(ctx->st, 0, 8, s));

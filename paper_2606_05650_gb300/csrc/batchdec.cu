@@ -198,6 +198,7 @@ static_assert(kLeafNodes + 3 <= 4 * kLeafThreads && kLeafNodes <= kLeafStage, "a
 struct OctArgs {
     const DecFrame *fr;
     uint32_t F, Jmax;
+    uint32_t Jtab, tables;      // deepest frame with a centre table, warps for the tables
     const uint32_t *tile_pref;  // F + 1: first CTA of each frame
     uint32_t tiles;             // tile_pref[F]
     const uint8_t *occ;
@@ -205,7 +206,7 @@ struct OctArgs {
     const uint64_t *tbase;      // P at each tile's first byte, and the total
     uint2 *path;                // per CTA and level: first node, its children that belong to the CTA before
     uint32_t *leaf0;            // per CTA: voxels of the frame before the first node's
-    const float *ctab;
+    float *ctab;
     float *pos;                 // or null: no centres
     uint8_t *gap;
     uint64_t nv_total;
@@ -262,7 +263,15 @@ __device__ __forceinline__ uint2 byte_of_bit(const OctArgs &a, uint64_t a0, uint
 }
 
 // A warp per CTA of octree_leaves_kernel: where it begins in each level.  Then a warp per frame and level: that the
-// level's bytes hold as many set bits as the next level has nodes.
+// level's bytes hold as many set bits as the next level has nodes.  Then kTableEntries of a frame's centre table a
+// warp: entry a * 2^J + v = (float)(lo_a + (v + 0.5) * cell), the same FP64 expression as per voxel (Sec. 2.1).
+constexpr uint32_t kTableEntries = 512;
+
+__host__ __device__ inline uint32_t table_warps(uint32_t Jmax)  // of a frame; no table is larger than the voxels
+{
+    return (uint32_t)(((3ull << Jmax) + kTableEntries - 1) / kTableEntries);
+}
+
 __global__ void __launch_bounds__(256) octree_paths_kernel(OctArgs a)
 {
     const uint32_t lane = threadIdx.x & 31, w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -293,6 +302,17 @@ __global__ void __launch_bounds__(256) octree_paths_kernel(OctArgs a)
         if (lane == 0 && bits != fd.lsz[d + 1]) {
             *a.broken = 1;
             set_error(&a.st->err, kErrCorrupt);
+        }
+    } else if (w < a.tiles + a.F * a.Jmax + a.tables) {
+        const uint32_t x = w - a.tiles - a.F * a.Jmax, per = table_warps(a.Jtab), f = x / per;
+        const DecFrame &fd = a.fr[f];
+        if (fd.ctab_off == ~0ull) return;
+        const uint64_t side = 1ull << fd.J, e0 = (uint64_t)(x - f * per) * kTableEntries;
+        float *tab = a.ctab + fd.ctab_off;
+        for (uint64_t e = e0 + lane; e < min(e0 + kTableEntries, 3 * side); e += 32) {
+            const uint32_t axis = (uint32_t)(e >> fd.J);
+            const double off = __dmul_rn(__dadd_rn((double)(e & (side - 1)), 0.5), fd.grid.cell);
+            tab[e] = (float)__dadd_rn(fd.grid.lo[axis], off);
         }
     }
 }
@@ -436,23 +456,6 @@ __global__ void __launch_bounds__(kLeafThreads) octree_leaves_kernel(OctArgs a)
     }
 }
 
-// voxel-centre tables (Sec. 2.1), grid (x, frames): the centre table of frame blockIdx.y, entry a * 2^J + v =
-// (float)(lo_a + (v + 0.5) * cell), the same FP64 expression as per voxel
-__global__ void centre_tables_kernel(const DecFrame *fr, float *ctab)
-{
-    const DecFrame &d = fr[blockIdx.y];
-    if (d.ctab_off == ~0ull) return;
-    const uint64_t side = 1ull << d.J;
-    float *t = ctab + d.ctab_off;
-    for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < 3 * side;
-         e += (uint64_t)gridDim.x * blockDim.x) {
-        const uint32_t a = (uint32_t)(e >> d.J);
-        const uint64_t v = e & (side - 1);
-        const double off = __dmul_rn(__dadd_rn((double)v, 0.5), d.grid.cell);
-        t[e] = (float)__dadd_rn(d.grid.lo[a], off);
-    }
-}
-
 __global__ void block_tables_kernel(const DecFrame *fr, uint32_t F, const uint64_t *blk_pref, uint64_t nblk,
                                     uint32_t *bw_all)
 {
@@ -514,26 +517,17 @@ uint64_t octree_path_words(uint64_t tiles) { return 2 * tiles * kMaxJ; }
 
 uint32_t octree_tiles(uint32_t nodes) { return (nodes + kLeafTile - 1) / kLeafTile; }
 
-void launch_octree_leaves(const DecFrame *fr, uint32_t F, uint32_t Jmax, const uint32_t *tile_pref, uint32_t tiles,
-                          const uint8_t *occ, uint64_t n_occ, const uint64_t *tbase, uint32_t *path, uint32_t *leaf0,
-                          const float *ctab, float *pos, uint8_t *gap, uint64_t nv_total, uint32_t *broken,
+void launch_octree_leaves(const DecFrame *fr, uint32_t F, uint32_t Jmax, uint32_t Jtab, const uint32_t *tile_pref,
+                          uint32_t tiles, const uint8_t *occ, uint64_t n_occ, const uint64_t *tbase, uint32_t *path,
+                          uint32_t *leaf0, float *ctab, float *pos, uint8_t *gap, uint64_t nv_total, uint32_t *broken,
                           DevState *st, cudaStream_t s)
 {
-    OctArgs a{fr, F, Jmax, tile_pref, tiles, occ, n_occ, tbase, reinterpret_cast<uint2 *>(path), leaf0, ctab, pos, gap,
-              nv_total, broken, st};
-    octree_paths_kernel<<<(tiles + F * Jmax + 7) / 8 + 1, 256, 0, s>>>(a);
+    OctArgs a{fr, F, Jmax, Jtab, Jtab ? F * table_warps(Jtab) : 0u, tile_pref, tiles, occ, n_occ, tbase,
+              reinterpret_cast<uint2 *>(path), leaf0, ctab, pos, gap, nv_total, broken, st};
+    octree_paths_kernel<<<(tiles + F * Jmax + a.tables + 7) / 8, 256, 0, s>>>(a);
     count_launch();
     if (tiles == 0) return;
     octree_leaves_kernel<<<tiles, kLeafThreads, 0, s>>>(a);
-    count_launch();
-}
-
-void launch_batch_centre_tables(const DecFrame *fr, uint32_t F, uint32_t Jmax, float *ctab, int num_sms,
-                                cudaStream_t s)
-{
-    if (F == 0) return;
-    uint32_t X = grid_for(3ull << Jmax, num_sms) / F + 1;
-    centre_tables_kernel<<<dim3(X, F), 256, 0, s>>>(fr, ctab);
     count_launch();
 }
 

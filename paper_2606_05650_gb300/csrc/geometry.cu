@@ -478,36 +478,6 @@ __device__ __forceinline__ void centre(uint64_t m, const FrameGrid &g, float *ou
     }
 }
 
-__global__ void centres_kernel(const uint64_t *__restrict__ codes, uint64_t nv, const FrameGrid *grid, float *pos)
-{
-    const FrameGrid g = *grid;
-    for (uint64_t v = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += (uint64_t)gridDim.x * blockDim.x)
-        centre(codes[v], g, pos + 3 * v);
-}
-
-// per-axis centre table of one frame: entry a * 2^J + v = (float)(lo_a + (v + 0.5) cell)
-__global__ void centre_table_kernel(const FrameGrid *grid, uint32_t J, float *ctab)
-{
-    const FrameGrid g = *grid;
-    const uint64_t side = 1ull << J;
-    for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < 3 * side;
-         e += (uint64_t)gridDim.x * blockDim.x) {
-        const uint32_t a = (uint32_t)(e >> J);
-        const double off = __dmul_rn(__dadd_rn((double)(e & (side - 1)), 0.5), g.cell);
-        ctab[e] = (float)__dadd_rn(g.lo[a], off);
-    }
-}
-
-__global__ void centres_table_kernel(const uint64_t *__restrict__ codes, uint64_t nv, uint32_t J,
-                                     const float *__restrict__ ctab, float *pos)
-{
-    for (uint64_t v = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t m = codes[v];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) pos[3 * v + a] = ctab[((uint64_t)a << J) + (uint32_t)compact3(m >> a)];
-    }
-}
-
 __global__ void centres_batch_kernel(const uint64_t *__restrict__ codes, const DevState *st, uint32_t frame_shift,
                                      const FrameGrid *grid, float *pos)
 {
@@ -664,20 +634,6 @@ void launch_octree_decode(const uint8_t *occ, uint64_t n_occ, uint32_t J, const 
 void launch_gap_levels(const uint64_t *codes, uint64_t nv, uint8_t *gap, cudaStream_t s)
 {
     gap_kernel<<<grid_for(nv + 1, 152), kThreads, 0, s>>>(codes, nv, gap);
-    count_launch();
-}
-
-void launch_voxel_centres(const uint64_t *codes, uint64_t nv, uint32_t J, const FrameGrid *grid, float *pos,
-                          cudaStream_t s, float *ctab)
-{
-    if (nv == 0) return;
-    if (ctab && (1ull << J) <= nv) {
-        centre_table_kernel<<<grid_for(3ull << J, 152), kThreads, 0, s>>>(grid, J, ctab);
-        count_launch();
-        centres_table_kernel<<<grid_for(nv, 152), kThreads, 0, s>>>(codes, nv, J, ctab, pos);
-    } else {
-        centres_kernel<<<grid_for(nv, 152), kThreads, 0, s>>>(codes, nv, grid, pos);
-    }
     count_launch();
 }
 

@@ -86,10 +86,6 @@ uint64_t octree_decode_node_words(const uint32_t *h_level_sizes, uint32_t J);
 
 // gap levels of ascending codes (one frame), gap[0] = gap[nv] = kInfLevel
 void launch_gap_levels(const uint64_t *codes, uint64_t nv, uint8_t *gap, cudaStream_t s);
-// voxel centres of the codes of one frame (Sec. 2.1)
-// ctab (3 x 2^J floats, or null): per-axis centre table used when 2^J <= nv
-void launch_voxel_centres(const uint64_t *codes, uint64_t nv, uint32_t J, const FrameGrid *grid, float *pos,
-                          cudaStream_t s, float *ctab = nullptr);
 // voxel centres of a batch: codes carry frame ids above frame_shift
 void launch_voxel_centres_batch(const uint64_t *codes, const DevState *st, uint64_t nv_bound,
                                 uint32_t frame_shift, const uint32_t *J, const FrameGrid *grid, float *pos,
@@ -291,22 +287,19 @@ void launch_batch_rans_decode(const DecFrame *fr, uint32_t F, uint32_t max_chunk
 // Octree of every frame (Algorithm 3): tile popcounts of the batch occupancy bytes and their exclusive scan
 // (tbase, tiles + 1 entries), then the voxels' centres (pos, or null) and gap levels, and the gap sentinel
 // gap[nv_total].  tile_pref: F + 1 CTA offsets, octree_tiles(nodes of the frame's last level) CTAs a frame, tiles in
-// all; path and leaf0: octree_path_words(tiles) and tiles words of scratch.  *broken, zero before, is set (as is the
-// error) where the bytes are not an octree's with the frames' level sizes.
+// all; path and leaf0: octree_path_words(tiles) and tiles words of scratch.  ctab: room for the centre tables
+// (DecFrame::ctab_off): a centre coordinate depends only on that axis' voxel coordinate, so frames with 2^J <= N_v
+// evaluate the FP64 expression once per axis value (3 x 2^J); Jtab: the deepest such frame's J, or 0.  *broken, zero
+// before, is set (as is the error) where the bytes are not an octree's with the frames' level sizes.
 uint64_t occ_tiles(uint64_t n_occ);
 uint32_t octree_tiles(uint32_t nodes);
 uint64_t octree_path_words(uint64_t tiles);
 void launch_occ_tile_bases(const uint8_t *occ, uint64_t n_occ, uint32_t *tsum, uint64_t *tbase, uint64_t *partials,
                            uint32_t *broken, DevState *st, int num_sms, cudaStream_t s);
-void launch_octree_leaves(const DecFrame *fr, uint32_t F, uint32_t Jmax, const uint32_t *tile_pref, uint32_t tiles,
-                          const uint8_t *occ, uint64_t n_occ, const uint64_t *tbase, uint32_t *path, uint32_t *leaf0,
-                          const float *ctab, float *pos, uint8_t *gap, uint64_t nv_total, uint32_t *broken,
+void launch_octree_leaves(const DecFrame *fr, uint32_t F, uint32_t Jmax, uint32_t Jtab, const uint32_t *tile_pref,
+                          uint32_t tiles, const uint8_t *occ, uint64_t n_occ, const uint64_t *tbase, uint32_t *path,
+                          uint32_t *leaf0, float *ctab, float *pos, uint8_t *gap, uint64_t nv_total, uint32_t *broken,
                           DevState *st, cudaStream_t s);
-// Voxel-centre tables: a centre coordinate depends only on that axis' voxel
-// coordinate, so frames with 2^J <= N_v evaluate the FP64 expression once per
-// axis value (3 x 2^J) instead of once per voxel.
-void launch_batch_centre_tables(const DecFrame *fr, uint32_t F, uint32_t Jmax, float *ctab, int num_sms,
-                                cudaStream_t s);
 void launch_batch_block_tables(const DecFrame *fr, uint32_t F, const uint64_t *blk_pref, uint64_t nblk,
                                uint32_t *bw_all, int num_sms, cudaStream_t s);
 
