@@ -895,6 +895,7 @@ __device__ __forceinline__ uint32_t gr_read(WinReader &r, uint32_t k, int &KR, b
 // codeword the table holds takes the short path; run mode (runs are kept as
 // pending zeros, and the nonzero that ends a partial run as a pending value)
 // and longer codewords the general one.
+constexpr uint32_t kDecThreads = 512, kDecSmall = 256;
 constexpr int kRunLeft = 1 << 16;  // flags in K: zeros or a value of an earlier run are still to be written,
 constexpr int kDrained = 1 << 17;  // the ring may not hold the next words: only the general path, which checks
 
@@ -988,20 +989,18 @@ __device__ __forceinline__ void decode_stream(const DecTable &tab, uint32_t *rin
 // b = x * rb + jl of channel c.  Streams at block_off[b*C+c] (words) when
 // block_off is given, else at (b*C+c) * stride.
 template <bool TO_INT>
-__global__ void __launch_bounds__(512, 2) rlgr_decode_kernel(const uint32_t *payload, uint64_t payload_words,
+__global__ void __launch_bounds__(kDecThreads, 2) rlgr_decode_kernel(const uint32_t *payload, uint64_t payload_words,
                                                           const uint32_t *block_words, const uint64_t *block_off,
                                                           uint32_t stride, uint32_t nv, uint32_t C, uint32_t B,
-                                                          uint32_t rb, const float *step, float *Y, int32_t *qout,
+                                                          const float *step, float *Y, int32_t *qout,
                                                           DevState *st)
 {
     extern __shared__ __align__(128) uint32_t ring[];  // kRingWords per thread
     __shared__ __align__(16) DecTable tab;
     stage_table(&tab, &g_dec_table);
     __syncthreads();
-    const uint32_t jl = threadIdx.x / C;
-    if (jl >= rb) return;
-    const uint32_t c = threadIdx.x - jl * C;
-    const uint64_t b = (uint64_t)blockIdx.x * rb + jl;
+    const uint64_t stream = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, b = stream / C;
+    const uint32_t c = (uint32_t)(stream - b * C);
     const uint64_t row0 = b * B;
     if (row0 >= nv) return;
     const uint32_t len = (nv - row0) < B ? (uint32_t)(nv - row0) : B;
@@ -1013,24 +1012,22 @@ __global__ void __launch_bounds__(512, 2) rlgr_decode_kernel(const uint32_t *pay
         nw = 0;
         off = 0;
     }
-    decode_stream<TO_INT>(tab, ring + threadIdx.x * kRingWords, payload + off, nw, len, C, TO_INT ? 0.f : step[c], TO_INT ? nullptr : Y + row0 * C + c,
-                          TO_INT ? qout + row0 * C + c : nullptr, st);
+    decode_stream<TO_INT>(tab, ring + threadIdx.x * kRingWords, payload + off, nw, len, C, TO_INT ? 0.f : step[c],
+                          TO_INT ? nullptr : Y + row0 * C + c, TO_INT ? qout + row0 * C + c : nullptr, st);
 }
 
 // All frames of a batch: row blocks numbered across frames (job_off), rb per CTA.
-__global__ void __launch_bounds__(512, 2) rlgr_decode_batch_kernel(const DecFrame *fr, uint32_t F,
+__global__ void __launch_bounds__(kDecThreads, 2) rlgr_decode_batch_kernel(const DecFrame *fr, uint32_t F,
                                                                 const uint64_t *job_off, const uint32_t *bw_all,
                                                                 const uint64_t *boff_all, const float *steps_all,
-                                                                uint32_t C, uint32_t rb, float *Y, DevState *st)
+                                                                uint32_t C, float *Y, DevState *st)
 {
     extern __shared__ __align__(128) uint32_t ring[];  // kRingWords per thread
     __shared__ __align__(16) DecTable tab;
     stage_table(&tab, &g_dec_table);
     __syncthreads();
-    const uint32_t jl = threadIdx.x / C;
-    if (jl >= rb) return;
-    const uint32_t c = threadIdx.x - jl * C;
-    const uint64_t job = (uint64_t)blockIdx.x * rb + jl;
+    const uint64_t stream = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, job = stream / C;
+    const uint32_t c = (uint32_t)(stream - job * C);
     if (job >= job_off[F]) return;
     uint32_t lo = 0, hi = F;
     while (hi - lo > 1) {
@@ -1150,17 +1147,27 @@ void launch_rlgr_encode_indices(const int32_t *q, const uint32_t *vstart, uint32
     launch_encode<true, false>(E, q, rb, threads, jobs_bound, s);
 }
 
+// Threads per CTA: a CTA has a copy of the table (32 KB) beside 64 bytes a thread, and many streams are bound by the
+// integer pipe once 32 warps are resident: 16 x 1M frames, beside the same geometry kernels, 2.14 ms with 224 threads
+// (28 warps), 1.83 with 512 (32), 1.74 with 640 (40), which slows the geometry, the longer branch, by more.  Streams
+// that do not fill every SM twice that way take smaller CTAs, for the sake of all SMs.
+template <typename Kernel, typename Launch>
+static void launch_decode(Kernel k, uint64_t streams, Launch launch)
+{
+    const uint32_t threads = streams < 152 * 2 * kDecThreads ? kDecSmall : kDecThreads;
+    launch(k, (uint32_t)((streams + threads - 1) / threads), threads, ring_smem(k, 4 * (size_t)kRingWords * threads));
+    count_launch();
+}
+
 void launch_rlgr_decode(const uint32_t *payload, uint64_t payload_words, const uint32_t *block_words,
                         const uint64_t *block_off, uint64_t nv, uint32_t C, uint32_t B, const float *step, float *Y,
                         DevState *st, cudaStream_t s)
 {
     if (nv == 0 || C == 0) return;
-    const uint64_t nb = (nv + B - 1) / B;
-    const uint32_t rb = row_blocks_per_cta(C);
-    const size_t smem = ring_smem(rlgr_decode_kernel<false>, 4 * kRingWords * rb * C);
-    rlgr_decode_kernel<false><<<(uint32_t)((nb + rb - 1) / rb), rb * C, smem, s>>>(
-        payload, payload_words, block_words, block_off, 0u, (uint32_t)nv, C, B, rb, step, Y, nullptr, st);
-    count_launch();
+    launch_decode(rlgr_decode_kernel<false>, (nv + B - 1) / B * C, [&](auto k, uint32_t grid, uint32_t threads, size_t smem) {
+        k<<<grid, threads, smem, s>>>(payload, payload_words, block_words, block_off, 0u, (uint32_t)nv, C, B, step, Y,
+                                      nullptr, st);
+    });
 }
 
 void launch_rlgr_decode_batch(const DecFrame *fr, uint32_t F, const uint64_t *job_off, uint64_t jobs_bound,
@@ -1168,23 +1175,19 @@ void launch_rlgr_decode_batch(const DecFrame *fr, uint32_t F, const uint64_t *jo
                               float *Y, DevState *st, cudaStream_t s)
 {
     if (jobs_bound == 0 || C == 0) return;
-    const uint32_t rb = row_blocks_per_cta(C);
-    const size_t smem = ring_smem(rlgr_decode_batch_kernel, 4 * kRingWords * rb * C);
-    rlgr_decode_batch_kernel<<<(uint32_t)((jobs_bound + rb - 1) / rb), rb * C, smem, s>>>(
-        fr, F, job_off, bw_all, boff_all, steps_all, C, rb, Y, st);
-    count_launch();
+    launch_decode(rlgr_decode_batch_kernel, jobs_bound * C, [&](auto k, uint32_t grid, uint32_t threads, size_t smem) {
+        k<<<grid, threads, smem, s>>>(fr, F, job_off, bw_all, boff_all, steps_all, C, Y, st);
+    });
 }
 
 void launch_rlgr_decode_indices(const uint32_t *words, uint64_t total_words, const uint32_t *bw, uint32_t stride,
                                 uint64_t nv, uint32_t C, uint32_t B, int32_t *q, DevState *st, cudaStream_t s)
 {
     if (nv == 0 || C == 0) return;
-    const uint64_t nb = (nv + B - 1) / B;
-    const uint32_t rb = row_blocks_per_cta(C);
-    const size_t smem = ring_smem(rlgr_decode_kernel<true>, 4 * kRingWords * rb * C);
-    rlgr_decode_kernel<true><<<(uint32_t)((nb + rb - 1) / rb), rb * C, smem, s>>>(
-        words, total_words, bw, nullptr, stride, (uint32_t)nv, C, B, rb, nullptr, nullptr, q, st);
-    count_launch();
+    launch_decode(rlgr_decode_kernel<true>, (nv + B - 1) / B * C, [&](auto k, uint32_t grid, uint32_t threads, size_t smem) {
+        k<<<grid, threads, smem, s>>>(words, total_words, bw, nullptr, stride, (uint32_t)nv, C, B, nullptr, nullptr, q,
+                                      st);
+    });
 }
 
 }  // namespace gsnfs
