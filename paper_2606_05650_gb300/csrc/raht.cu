@@ -1677,6 +1677,13 @@ void launch_finish(const XformArgs<S> &A, int q0, size_t smem, cudaStream_t s)
     count_launch();
 }
 
+// CTAs of a later pass, three per SM; a pass has at most a quarter of the tiles of the one before
+uint32_t later_grid(uint64_t tiles, int q, int num_sms)
+{
+    const uint64_t t = (tiles >> (2 * q)) + 1, cap = 3 * (uint64_t)num_sms;
+    return (uint32_t)(t < cap ? t : cap);
+}
+
 template <typename S, int VEC>
 void forward_all(const XformArgs<S> &A, uint64_t nv_bound, int num_sms, cudaStream_t s)
 {
@@ -1687,7 +1694,7 @@ void forward_all(const XformArgs<S> &A, uint64_t nv_bound, int num_sms, cudaStre
     uint32_t grid0 = (uint32_t)(tiles < 1 ? 1 : (tiles < gcap ? tiles : gcap));
     const int wide = grid_passes(nv_bound, T);
     for (int q = 0; q < wide; ++q) {
-        uint32_t g = q == 0 ? grid0 : (grid0 < (uint32_t)num_sms ? grid0 : (uint32_t)num_sms);
+        const uint32_t g = q == 0 ? grid0 : later_grid(tiles, q, num_sms);
         if (q == 0) stage_begin(s, kStRahtFwd0);
         size_t psm = 0;
         if constexpr (std::is_same<S, float>::value) {
@@ -1725,7 +1732,7 @@ void inverse_all(const XformArgs<S> &A, uint64_t nv_bound, int num_sms, cudaStre
     else
         launch_finish<S, true, VEC, false>(A, wide, smem, s);
     for (int q = wide - 1; q >= 0; --q) {
-        uint32_t g = q == 0 ? grid0 : (grid0 < (uint32_t)num_sms ? grid0 : (uint32_t)num_sms);
+        const uint32_t g = q == 0 ? grid0 : later_grid(tiles, q, num_sms);
         if (q == 0) stage_begin(s, kStRahtInv0);
         size_t psm = 0;
         if constexpr (std::is_same<S, float>::value) {
