@@ -895,7 +895,7 @@ __device__ __forceinline__ uint32_t gr_read(WinReader &r, uint32_t k, int &KR, b
 // codeword the table holds takes the short path; run mode (runs are kept as
 // pending zeros, and the nonzero that ends a partial run as a pending value)
 // and longer codewords the general one.
-constexpr uint32_t kDecThreads = 512, kDecSmall = 256;
+constexpr uint32_t kDecThreads = 512, kDecSmall = 128;
 constexpr int kRunLeft = 1 << 16;  // flags in K: zeros or a value of an earlier run are still to be written,
 constexpr int kDrained = 1 << 17;  // the ring may not hold the next words: only the general path, which checks
 
