@@ -3046,8 +3046,14 @@ gsnfs_status gsnfs_render(gsnfs_ctx *ctx, void *stream, const float *d_pos, cons
         for (int c = 0; c < 3; ++c) rc.R[3 * r + c] = V[4 * r + c];
         rc.t[r] = V[4 * r + 3];
     }
-    for (int c = 0; c < 3; ++c)  // camera centre -R^T t
+    for (int c = 0; c < 3; ++c) {  // camera centre -R^T t
         rc.campos[c] = -(V[c] * V[3] + V[4 + c] * V[7] + V[8 + c] * V[11]);
+        double rest = rc.campos[c];
+        for (int k = 0; k < 3; ++k) {
+            rc.campos3[c][k] = (float)rest;
+            rest -= (double)rc.campos3[c][k];
+        }
+    }
     rc.fx = cam->fx;
     rc.fy = cam->fy;
     rc.cx = cam->cx;

@@ -323,6 +323,7 @@ void launch_lod_centres(const uint64_t *codes, const uint64_t *starts, const uin
 // ---- render.cu: splat rasteriser ------------------------------------------------
 struct RenderCam {  // camera in FP64: the per-Gaussian projection is evaluated in FP64
     double R[9], t[3], campos[3];
+    float campos3[3][3];  // campos as sums of three floats
     double fx, fy, cx, cy, znear;
     int W, H, TX, TY;
     float bg[3];
