@@ -14,6 +14,7 @@
 //     (32 u32 states + u16 words, padded to 4); rANS only when smaller.
 //   attribute section (C > 0 and N_v > 0): u32 B, u32 nb, u32
 //     block_words[nb*C] (block-major: b*C + c), payload words, pad 8.
+#include <optional>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -74,6 +75,8 @@ thread_local std::vector<Profiler::Rec> *t_capture_stages = nullptr;
 thread_local std::vector<Profiler::Rec> t_capture_open;
 
 namespace gsnfs {
+thread_local int LateLaunches::depth = 0;
+
 void count_launch()
 {
     if (t_capture_launches)
@@ -351,6 +354,7 @@ struct CopyList {
 
 __global__ void __launch_bounds__(256) stage_copy_kernel(CopyList l)
 {
+    if (after_previous()) return;
     const CopyList::Item c = l.item[blockIdx.y];
     const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (uint64_t)gridDim.x * blockDim.x;
     if ((((uintptr_t)c.dst | (uintptr_t)c.src | c.n) & 3) == 0) {
@@ -380,7 +384,7 @@ public:
     {
         if (!l_.count) return cudaSuccess;
         const uint64_t blocks = std::min<uint64_t>((longest_ / 4 + 255) / 256, 128);
-        stage_copy_kernel<<<dim3((uint32_t)std::max<uint64_t>(blocks, 1), l_.count), 256, 0, s_>>>(l_);
+        launch_after(stage_copy_kernel, dim3((uint32_t)std::max<uint64_t>(blocks, 1), l_.count), 256, 0, s_, l_);
         count_launch();
         l_.count = 0;
         longest_ = 0;
@@ -551,6 +555,7 @@ __global__ void __launch_bounds__(kMaxFrames * kMaxRungs) sizes_kernel(HdrParams
                                                                        const uint64_t *block_off, StreamInfo *si,
                                                                        DevState *st)
 {
+    if (after_previous()) return;
     __shared__ uint64_t sh[33];
     const uint32_t i = threadIdx.x;
     StreamInfo x{0, 0, 0, 0};
@@ -580,6 +585,7 @@ __global__ void header_kernel(HdrParams hp, const uint32_t *J, const uint32_t *v
                               const uint32_t *lsz, const uint8_t *groups, const double *steps_rg,
                               const float *klt, const StreamInfo *si, const DevState *st, uint8_t *out)
 {
+    if (after_previous()) return;
     if (st->total_bytes > hp.capacity) return;
     const uint32_t s = blockIdx.x, f = s / hp.R, r = s % hp.R;
     const StreamInfo x = si[s];
@@ -627,6 +633,7 @@ struct OccCopyArgs {
 
 __global__ void occ_copy_kernel(HdrParams hp, OccCopyArgs a, const StreamInfo *si, const DevState *st, uint8_t *out)
 {
+    if (after_previous()) return;
     if (st->total_bytes > hp.capacity) return;
     const uint32_t s = blockIdx.y, f = s / hp.R;
     const StreamInfo x = si[s];
@@ -699,6 +706,7 @@ struct AttrCopyArgs {
 
 __global__ void attr_copy_kernel(HdrParams hp, AttrCopyArgs a, const StreamInfo *si, const DevState *st, uint8_t *out)
 {
+    if (after_previous()) return;
     if (st->total_bytes > hp.capacity) return;
     const uint32_t s = blockIdx.y, f = s / hp.R, r = s % hp.R;
     const StreamInfo x = si[s];
@@ -742,24 +750,24 @@ __global__ void attr_copy_kernel(HdrParams hp, AttrCopyArgs a, const StreamInfo 
                 w[q] = __shfl_sync(0xFFFFFFFFu, wl, j);
                 o[q] = __shfl_sync(0xFFFFFFFFu, ol, j);
                 if (j0 + q >= cnt) w[q] = 0;
-                const uint32_t *__restrict__ src = a.slots + (b0 + k0 + j0 + q) * a.slot_words;
+                const uint32_t *src = a.slots + (b0 + k0 + j0 + q) * a.slot_words;
 #pragma unroll
                 for (uint32_t u = 0; u < kPerLane; ++u) {
                     const uint32_t i = lane + 32 * u;
-                    v[q][u] = i < w[q] ? __ldg(src + i) : 0u;
+                    v[q][u] = i < w[q] ? *(src + i) : 0u;
                 }
             }
 #pragma unroll
             for (uint32_t q = 0; q < kGroup; ++q) {
-                uint32_t *__restrict__ dst = pay + o[q];
+                uint32_t *dst = pay + o[q];
 #pragma unroll
                 for (uint32_t u = 0; u < kPerLane; ++u) {
                     const uint32_t i = lane + 32 * u;
                     if (i < w[q]) dst[i] = v[q][u];
                 }
                 // the rest of a longer stream
-                const uint32_t *__restrict__ src = a.slots + (b0 + k0 + j0 + q) * a.slot_words;
-                for (uint32_t i = 32 * kPerLane + lane; i < w[q]; i += 32) dst[i] = __ldg(src + i);
+                const uint32_t *src = a.slots + (b0 + k0 + j0 + q) * a.slot_words;
+                for (uint32_t i = 32 * kPerLane + lane; i < w[q]; i += 32) dst[i] = *(src + i);
             }
         }
     }
@@ -1099,6 +1107,8 @@ gsnfs_status encode_impl(gsnfs_ctx *ctx, cudaStream_t s, EncodeReq &rq, bool wor
         // the attributes' centres and colour transforms depend on the input rows alone: beside a1-a3, on the
         // high-priority stream that a6-a9 follow on
         cudaStream_t sa = s;
+        std::optional<LateLaunches> late;  // beside the colour KLT, the longer chain (1M Gaussians with reconstruction:
+        if (C && q->color) late.emplace(true);  // 1.47 ms, else 1.56)
         if (C) {
             gsnfs_status fst = fork_hi_begin(ctx, s, &sa);
             if (fst) return fst;
@@ -1155,6 +1165,7 @@ gsnfs_status encode_impl(gsnfs_ctx *ctx, cudaStream_t s, EncodeReq &rq, bool wor
             if (q->color) {
                 CK(cudaEventRecord(ctx->ev_join_klt, ctx->aux_klt));
                 CK(cudaStreamWaitEvent(sa, ctx->ev_join_klt, 0));
+                late.reset();
             }
             RahtIO io{};
             io.C = C;
@@ -1208,19 +1219,19 @@ gsnfs_status encode_impl(gsnfs_ctx *ctx, cudaStream_t s, EncodeReq &rq, bool wor
         }
         // a10: container
         stage_begin(s, kStContainer);
-        sizes_kernel<<<1, (F * R + 31) / 32 * 32, 0, s>>>(hpar, L.Jd, L.vstart, L.sec_bytes, L.blk_off, L.block_off, L.si, dst);
+        launch_after(sizes_kernel, 1, (F * R + 31) / 32 * 32, 0, s, hpar, L.Jd, L.vstart, L.sec_bytes, L.blk_off, L.block_off, L.si, dst);
         count_launch();
-        header_kernel<<<F * R, 128, 0, s>>>(hpar, L.Jd, L.vstart, L.grid, L.lsz, L.groups, L.steps_rg, L.klt, L.si, dst,
+        launch_after(header_kernel, F * R, 128, 0, s, hpar, L.Jd, L.vstart, L.grid, L.lsz, L.groups, L.steps_rg, L.klt, L.si, dst,
                                             rq.out);
         count_launch();
         OccCopyArgs oa{L.occ, L.occ_off, L.mode, L.chunk_off, L.freq, L.chunk_words, L.chunk_top, L.chunk_pos,
                        L.chunk_slots, rans_chunk_slot_bytes(q->rans_chunk)};
-        occ_copy_kernel<<<dim3(std::max<uint32_t>(1, (uint32_t)sms * 4 / (F * R)), F * R), 256, 0, s>>>(hpar, oa, L.si,
+        launch_after(occ_copy_kernel, dim3(std::max<uint32_t>(1, (uint32_t)sms * 4 / (F * R)), F * R), 256, 0, s, hpar, oa, L.si,
                                                                                                       dst, rq.out);
         count_launch();
         if (C) {
             AttrCopyArgs aa{L.vstart, L.blk_off, L.block_off, L.block_words, L.slots, L.slot_words};
-            attr_copy_kernel<<<dim3(std::max<uint32_t>(1, (uint32_t)sms * 8 / (F * R)), F * R), 256, 0, s>>>(
+            launch_after(attr_copy_kernel, dim3(std::max<uint32_t>(1, (uint32_t)sms * 8 / (F * R)), F * R), 256, 0, s, 
                 hpar, aa, L.si, dst, rq.out);
             count_launch();
         }
@@ -2677,7 +2688,7 @@ gsnfs_status gsnfs_occupancy_section_encode(gsnfs_ctx *ctx, void *stream, const 
     count_launch();
     HdrParams hpar{1, 1, 0, 0, 1, rans_chunk, 0u, 0.5, capacity};
     OccCopyArgs oa{d_in, occ_off, mode, chunk_off, freq, cw, ct, cp, slots, rans_chunk_slot_bytes(rans_chunk)};
-    occ_copy_kernel<<<dim3(ctx->num_sms, 1), 256, 0, s>>>(hpar, oa, si, ctx->st, d_out);
+    launch_after(occ_copy_kernel, dim3(ctx->num_sms, 1), 256, 0, s, hpar, oa, si, ctx->st, d_out);
     count_launch();
     CK(cudaMemcpyAsync(hp + 8, sec, 8, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));

@@ -27,6 +27,7 @@ __device__ __forceinline__ uint32_t find_frame(const T *pref, uint32_t F, uint64
 // raw and constant occupancy sections: bytes straight into the batch buffer
 __global__ void occ_bytes_kernel(const DecFrame *fr, uint8_t *occ_all)
 {
+    if (after_previous()) return;
     const DecFrame &d = fr[blockIdx.y];
     if (d.mode == 1) return;
     uint8_t *dst = occ_all + d.occ_off;
@@ -39,6 +40,7 @@ __global__ void occ_bytes_kernel(const DecFrame *fr, uint8_t *occ_all)
 __global__ void __launch_bounds__(1024) tables_kernel(const DecFrame *fr, uint32_t *tabs, uint64_t tab_words,
                                                       uint64_t *cstart, DevState *st)
 {
+    if (after_previous()) return;
     const DecFrame &d = fr[blockIdx.x];
     if (d.mode != 1) return;
     uint32_t *tab = tabs + (uint64_t)blockIdx.x * tab_words;
@@ -74,6 +76,7 @@ __global__ void __launch_bounds__(32 * kRansWarps) rans_batch_kernel(const DecFr
                                                                      uint64_t tab_words, const uint64_t *cstart,
                                                                      uint8_t *occ_all, DevState *st)
 {
+    if (after_previous()) return;
     using namespace ransdec;
     extern __shared__ __align__(16) unsigned char dsm[];
     const DecFrame &d = fr[blockIdx.y];
@@ -133,10 +136,11 @@ __device__ __forceinline__ uint32_t word_at(const uint8_t *occ, uint64_t n, uint
 }
 
 // tsum: set bits per tile; *broken and the error are set when a byte is zero (a node without children)
-__global__ void __launch_bounds__(256) occ_tile_popc_kernel(const uint8_t *__restrict__ occ, uint64_t n,
+__global__ void __launch_bounds__(256) occ_tile_popc_kernel(const uint8_t *occ, uint64_t n,
                                                             uint64_t ntiles, uint32_t *tsum, uint32_t *broken,
                                                             DevState *st)
 {
+    if (after_previous()) return;
     const uint32_t lane = threadIdx.x & 31;
     for (uint64_t t = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < ntiles;
          t += ((uint64_t)gridDim.x * blockDim.x) >> 5) {
@@ -158,14 +162,14 @@ __global__ void __launch_bounds__(256) occ_tile_popc_kernel(const uint8_t *__res
     }
 }
 
-__device__ __forceinline__ void leaf_out(const DecFrame &d, const float *__restrict__ ctab, uint32_t v, uint64_t m,
+__device__ __forceinline__ void leaf_out(const DecFrame &d, const float *ctab, uint32_t v, uint64_t m,
                                          float *pos)
 {
     if (d.ctab_off != ~0ull) {
         const float *t = ctab + d.ctab_off;
         float c[3];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) c[a] = __ldg(t + ((uint64_t)a << d.J) + compact3b(m >> a));
+        for (int a = 0; a < 3; ++a) c[a] = *(t + ((uint64_t)a << d.J) + compact3b(m >> a));
 #pragma unroll
         for (int a = 0; a < 3; ++a) pos[3ull * v + a] = c[a];
     } else {
@@ -274,6 +278,7 @@ __host__ __device__ inline uint32_t table_warps(uint32_t Jmax)  // of a frame; n
 
 __global__ void __launch_bounds__(256) octree_paths_kernel(OctArgs a)
 {
+    if (after_previous()) return;
     const uint32_t lane = threadIdx.x & 31, w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (w == 0 && lane == 0) a.gap[a.nv_total] = (uint8_t)kInfLevel;  // sentinel after the last voxel
     if (w < a.tiles) {
@@ -326,6 +331,7 @@ __device__ __forceinline__ void children(uint64_t code, uint32_t v, uint32_t ran
 
 __global__ void __launch_bounds__(kLeafThreads) octree_leaves_kernel(OctArgs a)
 {
+    if (after_previous()) return;
     __shared__ uint64_t s_code[2][kLeafStage];  // a level's codes, the last level's in [0]; then the voxels' in [1]
     __shared__ uint2 s_path[kMaxJ];             // first node, its children of the CTA before
     __shared__ uint32_t s_cnt[kMaxJ];           // nodes
@@ -459,6 +465,7 @@ __global__ void __launch_bounds__(kLeafThreads) octree_leaves_kernel(OctArgs a)
 __global__ void block_tables_kernel(const DecFrame *fr, uint32_t F, const uint64_t *blk_pref, uint64_t nblk,
                                     uint32_t *bw_all)
 {
+    if (after_previous()) return;
     for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nblk; k += (uint64_t)gridDim.x * blockDim.x) {
         const uint32_t f = find_frame(blk_pref, F, k);
         bw_all[k] = fr[f].bw[k - blk_pref[f]];
@@ -480,7 +487,7 @@ void launch_batch_occ_bytes(const DecFrame *fr, uint32_t F, uint8_t *occ_all, ui
 {
     if (max_occ == 0) return;
     uint32_t X = grid_for(max_occ, num_sms) / F + 1;
-    occ_bytes_kernel<<<dim3(X, F), 256, 0, s>>>(fr, occ_all);
+    launch_after(occ_bytes_kernel, dim3(X, F), 256, 0, s, fr, occ_all);
     count_launch();
 }
 
@@ -490,12 +497,12 @@ void launch_batch_rans_decode(const DecFrame *fr, uint32_t F, uint32_t max_chunk
     (void)chunk_max;
     if (max_chunks_per_frame == 0) return;
     const uint64_t tab_words = kM / 4 + 256 + 4;
-    tables_kernel<<<F, 1024, 0, s>>>(fr, tabs, tab_words, cstart, st);
+    launch_after(tables_kernel, F, 1024, 0, s, fr, tabs, tab_words, cstart, st);
     count_launch();
     const size_t smem = (size_t)ransdec::kTabWords * 4;
     cudaFuncSetAttribute(rans_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const uint32_t X = (max_chunks_per_frame + kRansWarps - 1) / kRansWarps;
-    rans_batch_kernel<<<dim3(X, F), 32 * kRansWarps, smem, s>>>(fr, tabs, tab_words, cstart, occ_all, st);
+    launch_after(rans_batch_kernel, dim3(X, F), 32 * kRansWarps, smem, s, fr, tabs, tab_words, cstart, occ_all, st);
     count_launch();
 }
 
@@ -507,7 +514,7 @@ void launch_occ_tile_bases(const uint8_t *occ, uint64_t n_occ, uint32_t *tsum, u
     const uint64_t nt = occ_tiles(n_occ);
     if (nt) {
         const uint64_t want = (nt + 7) / 8, cap = (uint64_t)num_sms * 8;
-        occ_tile_popc_kernel<<<(uint32_t)(want < cap ? want : cap), 256, 0, s>>>(occ, n_occ, nt, tsum, broken, st);
+        launch_after(occ_tile_popc_kernel, (uint32_t)(want < cap ? want : cap), 256, 0, s, occ, n_occ, nt, tsum, broken, st);
         count_launch();
     }
     launch_scan_u32_to_u64(tsum, nt, tbase, partials, num_sms, s);
@@ -524,10 +531,10 @@ void launch_octree_leaves(const DecFrame *fr, uint32_t F, uint32_t Jmax, uint32_
 {
     OctArgs a{fr, F, Jmax, Jtab, Jtab ? F * table_warps(Jtab) : 0u, tile_pref, tiles, occ, n_occ, tbase,
               reinterpret_cast<uint2 *>(path), leaf0, ctab, pos, gap, nv_total, broken, st};
-    octree_paths_kernel<<<(tiles + F * Jmax + a.tables + 7) / 8, 256, 0, s>>>(a);
+    launch_after(octree_paths_kernel, (tiles + F * Jmax + a.tables + 7) / 8, 256, 0, s, a);
     count_launch();
     if (tiles == 0) return;
-    octree_leaves_kernel<<<tiles, kLeafThreads, 0, s>>>(a);
+    launch_after(octree_leaves_kernel, tiles, kLeafThreads, 0, s, a);
     count_launch();
 }
 
@@ -535,7 +542,7 @@ void launch_batch_block_tables(const DecFrame *fr, uint32_t F, const uint64_t *b
                                uint32_t *bw_all, int num_sms, cudaStream_t s)
 {
     if (nblk == 0) return;
-    block_tables_kernel<<<grid_for(nblk, num_sms), 256, 0, s>>>(fr, F, blk_pref, nblk, bw_all);
+    launch_after(block_tables_kernel, grid_for(nblk, num_sms), 256, 0, s, fr, F, blk_pref, nblk, bw_all);
     count_launch();
 }
 

@@ -40,6 +40,19 @@ struct DevState {
     uint32_t hist[kMaxFrames][256];  // occupancy byte histograms
 };
 
+// First in a kernel that launch_after() launches: waits for everything the
+// stream did before, then lets the next such kernel's CTAs take their places.
+// Returns 0; a kernel returns when it is not, which it never is, so that no
+// load of the kernel is moved before the wait.  Such a kernel reads what other
+// kernels wrote by ordinary loads only (no __ldg, no const __restrict__): the
+// read-only path may hold a line from before the wait.
+__device__ __forceinline__ uint32_t after_previous()
+{
+    uint32_t zero;
+    asm volatile("griddepcontrol.wait;\ngriddepcontrol.launch_dependents;\nmov.u32 %0, 0;\n" : "=r"(zero)::"memory");
+    return zero;
+}
+
 __device__ __forceinline__ void set_error(uint32_t *err, uint32_t code)
 {
     atomicCAS(err, 0u, code);

@@ -38,9 +38,10 @@ __device__ __forceinline__ Range cta_range(uint64_t vs, uint64_t ve, uint32_t x,
 }
 
 // ---------------------------------------------------------------- dedup ---
-__global__ void __launch_bounds__(kThreads) dedup_up_kernel(const uint64_t *__restrict__ keys, uint64_t n,
+__global__ void __launch_bounds__(kThreads) dedup_up_kernel(const uint64_t *keys, uint64_t n,
                                                             uint64_t chunk, uint32_t *partials)
 {
+    if (after_previous()) return;
     uint64_t b = (uint64_t)blockIdx.x * chunk, e = b + chunk;
     if (e > n) e = n;
     uint32_t c = 0;
@@ -51,12 +52,13 @@ __global__ void __launch_bounds__(kThreads) dedup_up_kernel(const uint64_t *__re
     if (threadIdx.x == 0) partials[blockIdx.x] = tot;
 }
 
-__global__ void __launch_bounds__(kThreads) dedup_down_kernel(const uint64_t *__restrict__ keys, uint64_t n,
+__global__ void __launch_bounds__(kThreads) dedup_down_kernel(const uint64_t *keys, uint64_t n,
                                                               uint64_t chunk, const uint32_t *partials,
                                                               uint32_t frame_shift, uint64_t *codes,
                                                               uint32_t *seg, uint8_t *gap, uint32_t *vstart,
-                                                              const uint32_t *__restrict__ vals, uint32_t *row0)
+                                                              const uint32_t *vals, uint32_t *row0)
 {
+    if (after_previous()) return;
     __shared__ uint32_t sh[33];
     uint64_t b = (uint64_t)blockIdx.x * chunk, e = b + chunk;
     if (e > n) e = n;
@@ -90,6 +92,7 @@ __global__ void __launch_bounds__(kThreads) dedup_down_kernel(const uint64_t *__
 __global__ void __launch_bounds__(32) dedup_fix_kernel(const uint32_t *partials, uint32_t P, uint32_t *vstart,
                                                        uint32_t F, DevState *st)
 {
+    if (after_previous()) return;
     // partials were scanned in place; the total is the last prefix plus the last count
     const uint32_t nv = partials[P], lane = threadIdx.x;
     uint32_t next = nv;  // start of the frame after the group
@@ -111,6 +114,7 @@ __global__ void __launch_bounds__(32) dedup_fix_kernel(const uint32_t *partials,
 // exclusive scan of P words with the total appended at [P] (one CTA)
 __global__ void __launch_bounds__(1024) scan_total_kernel(uint32_t *a, uint32_t m)
 {
+    if (after_previous()) return;
     __shared__ uint32_t sh[33];
     uint32_t per = (m + 1023) / 1024;
     uint32_t b = per * threadIdx.x, e = b + per;
@@ -134,10 +138,11 @@ __device__ __forceinline__ int height_of(uint8_t g, uint32_t J)
     return (g >= kInfLevel) ? (int)J : ((int)g - 1) / 3;
 }
 
-__global__ void __launch_bounds__(kThreads) occ_up_kernel(const uint8_t *__restrict__ gap,
-                                                          const uint32_t *__restrict__ vstart,
-                                                          const uint32_t *__restrict__ Jarr, uint32_t *partials)
+__global__ void __launch_bounds__(kThreads) occ_up_kernel(const uint8_t *gap,
+                                                          const uint32_t *vstart,
+                                                          const uint32_t *Jarr, uint32_t *partials)
 {
+    if (after_previous()) return;
     const uint32_t f = blockIdx.y, x = blockIdx.x, X = gridDim.x;
     const uint32_t J = Jarr[f];
     __shared__ uint32_t cnt[kH];
@@ -155,10 +160,11 @@ __global__ void __launch_bounds__(kThreads) occ_up_kernel(const uint8_t *__restr
 // one CTA of 32 x kH threads per frame: warp h scans the CTA counts of height h
 // (exclusive, in place), then level sizes and byte offsets of the frame
 __global__ void __launch_bounds__(32 * kH) occ_scan_kernel(uint32_t *partials, uint32_t X,
-                                                           const uint32_t *__restrict__ vstart,
-                                                           const uint32_t *__restrict__ Jarr, uint32_t *lsz,
+                                                           const uint32_t *vstart,
+                                                           const uint32_t *Jarr, uint32_t *lsz,
                                                            uint32_t *hoff, uint64_t *nocc)
 {
+    if (after_previous()) return;
     __shared__ uint32_t tot[kH];
     const uint32_t f = blockIdx.x, lane = threadIdx.x & 31, h = threadIdx.x >> 5;
     uint32_t *row = partials + ((uint64_t)f * kH + h) * X;
@@ -195,6 +201,7 @@ __global__ void __launch_bounds__(32 * kH) occ_scan_kernel(uint32_t *partials, u
 
 __global__ void __launch_bounds__(kMaxFrames) occ_offsets_kernel(const uint64_t *nocc, uint32_t F, uint64_t *occ_off)
 {
+    if (after_previous()) return;
     __shared__ uint64_t sh[33];
     const uint32_t f = threadIdx.x;
     uint64_t tot;
@@ -205,6 +212,7 @@ __global__ void __launch_bounds__(kMaxFrames) occ_offsets_kernel(const uint64_t 
 
 __global__ void zero_words_kernel(uint32_t *p, const uint64_t *nbytes_at, uint64_t cap_words)
 {
+    if (after_previous()) return;
     uint64_t nw = (*nbytes_at + 3) / 4;
     if (nw > cap_words) nw = cap_words;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nw; i += (uint64_t)gridDim.x * blockDim.x)
@@ -222,16 +230,17 @@ __global__ void zero_words_kernel(uint32_t *p, const uint64_t *nbytes_at, uint64
 // tile's range is shared with its neighbours).
 constexpr int kOccWords = kThreads / 4 + 2;  // per height: bytes 0 .. kThreads, word-aligned either way
 
-__global__ void __launch_bounds__(kThreads) occ_down_kernel(const uint64_t *__restrict__ codes,
-                                                            const uint8_t *__restrict__ gap,
-                                                            const uint32_t *__restrict__ vstart,
-                                                            const uint32_t *__restrict__ Jarr,
-                                                            const uint32_t *__restrict__ partials,
-                                                            const uint32_t *__restrict__ hoff,
-                                                            const uint64_t *__restrict__ occ_off,
+__global__ void __launch_bounds__(kThreads) occ_down_kernel(const uint64_t *codes,
+                                                            const uint8_t *gap,
+                                                            const uint32_t *vstart,
+                                                            const uint32_t *Jarr,
+                                                            const uint32_t *partials,
+                                                            const uint32_t *hoff,
+                                                            const uint64_t *occ_off,
                                                             uint32_t *occ_words, uint64_t occ_capacity,
                                                             DevState *st)
 {
+    if (after_previous()) return;
     const uint32_t f = blockIdx.y, x = blockIdx.x, X = gridDim.x;
     const uint32_t J = Jarr[f];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -335,7 +344,7 @@ __device__ __forceinline__ void load16(const uint8_t *p, uint64_t i, uint64_t e,
     }
 }
 
-__global__ void __launch_bounds__(kThreads) popc_up_kernel(const uint8_t *__restrict__ occ, uint64_t n,
+__global__ void __launch_bounds__(kThreads) popc_up_kernel(const uint8_t *occ, uint64_t n,
                                                            uint64_t chunk, uint32_t *partials)
 {
     uint64_t b = (uint64_t)blockIdx.x * chunk, e = b + chunk;
@@ -353,7 +362,7 @@ __global__ void __launch_bounds__(kThreads) popc_up_kernel(const uint8_t *__rest
     if (threadIdx.x == 0) partials[blockIdx.x] = tot;
 }
 
-__global__ void __launch_bounds__(kThreads) popc_down_kernel(const uint8_t *__restrict__ occ, uint64_t n,
+__global__ void __launch_bounds__(kThreads) popc_down_kernel(const uint8_t *occ, uint64_t n,
                                                              uint64_t chunk, const uint32_t *partials,
                                                              uint32_t *pref)
 {
@@ -392,9 +401,9 @@ __global__ void __launch_bounds__(kThreads) popc_down_kernel(const uint8_t *__re
 __global__ void root_kernel(uint64_t *nodes) { nodes[0] = 0ull; }
 
 // one level of Algorithm 3: node p of L_d writes (code << 3) + i for each set bit i
-__global__ void __launch_bounds__(kThreads) expand_kernel(const uint64_t *__restrict__ Ld, uint32_t Md,
-                                                          const uint8_t *__restrict__ occ, uint64_t boff,
-                                                          const uint32_t *__restrict__ pref, uint64_t *Ld1,
+__global__ void __launch_bounds__(kThreads) expand_kernel(const uint64_t *Ld, uint32_t Md,
+                                                          const uint8_t *occ, uint64_t boff,
+                                                          const uint32_t *pref, uint64_t *Ld1,
                                                           uint32_t Md1, DevState *st)
 {
     const uint32_t base = pref[boff];
@@ -423,8 +432,8 @@ struct LevelTable {
 };
 
 __global__ void __launch_bounds__(1024) expand_top_kernel(LevelTable lt, uint32_t d_end, uint64_t *nodes,
-                                                          const uint8_t *__restrict__ occ,
-                                                          const uint32_t *__restrict__ pref, DevState *st)
+                                                          const uint8_t *occ,
+                                                          const uint32_t *pref, DevState *st)
 {
     for (uint32_t d = 0; d < d_end; ++d) {
         const uint32_t Md = lt.M[d], Md1 = lt.M[d + 1];
@@ -451,8 +460,9 @@ __global__ void __launch_bounds__(1024) expand_top_kernel(LevelTable lt, uint32_
     }
 }
 
-__global__ void gap_kernel(const uint64_t *__restrict__ codes, uint64_t nv, uint8_t *gap)
+__global__ void gap_kernel(const uint64_t *codes, uint64_t nv, uint8_t *gap)
 {
+    if (after_previous()) return;
     for (uint64_t v = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; v <= nv; v += (uint64_t)gridDim.x * blockDim.x)
         gap[v] = (v == 0 || v == nv) ? (uint8_t)kInfLevel : (uint8_t)gap_level(codes[v - 1], codes[v], 64);
 }
@@ -478,9 +488,10 @@ __device__ __forceinline__ void centre(uint64_t m, const FrameGrid &g, float *ou
     }
 }
 
-__global__ void centres_batch_kernel(const uint64_t *__restrict__ codes, const DevState *st, uint32_t frame_shift,
+__global__ void centres_batch_kernel(const uint64_t *codes, const DevState *st, uint32_t frame_shift,
                                      const FrameGrid *grid, float *pos)
 {
+    if (after_previous()) return;
     const uint64_t nv = st->nv_total;
     const uint64_t mask = (frame_shift < 64) ? ((1ull << frame_shift) - 1) : ~0ull;
     for (uint64_t v = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += (uint64_t)gridDim.x * blockDim.x) {
@@ -552,15 +563,15 @@ void launch_dedup(const uint64_t *keys, uint64_t n, uint32_t frame_shift, uint32
         dev_memset(seg, 0, sizeof(uint32_t), s);
         dev_memset(gap, (int)kInfLevel, 1, s);
     } else {
-        dedup_up_kernel<<<c.P, kThreads, 0, s>>>(keys, n, c.chunk, partials);
+        launch_after(dedup_up_kernel, c.P, kThreads, 0, s, keys, n, c.chunk, partials);
         count_launch();
-        scan_total_kernel<<<1, 1024, 0, s>>>(partials, c.P);
+        launch_after(scan_total_kernel, 1, 1024, 0, s, partials, c.P);
         count_launch();
-        dedup_down_kernel<<<c.P, kThreads, 0, s>>>(keys, n, c.chunk, partials, frame_shift, codes, seg, gap,
+        launch_after(dedup_down_kernel, c.P, kThreads, 0, s, keys, n, c.chunk, partials, frame_shift, codes, seg, gap,
                                                    vstart, vals, row0);
         count_launch();
     }
-    dedup_fix_kernel<<<1, 32, 0, s>>>(partials, c.P, vstart, F, st);
+    launch_after(dedup_fix_kernel, 1, 32, 0, s, partials, c.P, vstart, F, st);
     count_launch();
 }
 
@@ -571,16 +582,16 @@ void launch_occupancy(const uint64_t *codes, const uint8_t *gap, const uint32_t 
 {
     uint32_t X = occ_x(F, num_sms, n_max);
     dim3 grid(X, F);
-    occ_up_kernel<<<grid, kThreads, 0, s>>>(gap, vstart, J, o.partials);
+    launch_after(occ_up_kernel, grid, kThreads, 0, s, gap, vstart, J, o.partials);
     count_launch();
     uint64_t *nocc = reinterpret_cast<uint64_t *>(o.partials + (uint64_t)F * X * kH + ((F * X * kH) & 1u));
-    occ_scan_kernel<<<F, 32 * kH, 0, s>>>(o.partials, X, vstart, J, o.level_sizes, o.hoff, nocc);
+    launch_after(occ_scan_kernel, F, 32 * kH, 0, s, o.partials, X, vstart, J, o.level_sizes, o.hoff, nocc);
     count_launch();
-    occ_offsets_kernel<<<1, kMaxFrames, 0, s>>>(nocc, F, o.occ_off);
+    launch_after(occ_offsets_kernel, 1, kMaxFrames, 0, s, nocc, F, o.occ_off);
     count_launch();
-    zero_words_kernel<<<num_sms * 2, 256, 0, s>>>((uint32_t *)o.occ, o.occ_off + F, o.occ_capacity / 4);
+    launch_after(zero_words_kernel, num_sms * 2, 256, 0, s, (uint32_t *)o.occ, o.occ_off + F, o.occ_capacity / 4);
     count_launch();
-    occ_down_kernel<<<grid, kThreads, 0, s>>>(codes, gap, vstart, J, o.partials, o.hoff, o.occ_off,
+    launch_after(occ_down_kernel, grid, kThreads, 0, s, codes, gap, vstart, J, o.partials, o.hoff, o.occ_off,
                                               (uint32_t *)o.occ, o.occ_capacity, st);
     count_launch();
 }
@@ -600,7 +611,7 @@ void launch_octree_decode(const uint8_t *occ, uint64_t n_occ, uint32_t J, const 
     Chunks c = popc_chunks(n_occ, num_sms);
     popc_up_kernel<<<c.P, kThreads, 0, s>>>(occ, n_occ, c.chunk, partials);
     count_launch();
-    scan_total_kernel<<<1, 1024, 0, s>>>(partials, c.P);
+    launch_after(scan_total_kernel, 1, 1024, 0, s, partials, c.P);
     count_launch();
     popc_down_kernel<<<c.P, kThreads, 0, s>>>(occ, n_occ, c.chunk, partials, pref);
     count_launch();
@@ -633,7 +644,7 @@ void launch_octree_decode(const uint8_t *occ, uint64_t n_occ, uint32_t J, const 
 
 void launch_gap_levels(const uint64_t *codes, uint64_t nv, uint8_t *gap, cudaStream_t s)
 {
-    gap_kernel<<<grid_for(nv + 1, 152), kThreads, 0, s>>>(codes, nv, gap);
+    launch_after(gap_kernel, grid_for(nv + 1, 152), kThreads, 0, s, codes, nv, gap);
     count_launch();
 }
 
@@ -643,7 +654,7 @@ void launch_voxel_centres_batch(const uint64_t *codes, const DevState *st, uint6
 {
     (void)J;
     if (nv_bound == 0) return;
-    centres_batch_kernel<<<grid_for(nv_bound, 152), kThreads, 0, s>>>(codes, st, frame_shift, grid, pos);
+    launch_after(centres_batch_kernel, grid_for(nv_bound, 152), kThreads, 0, s, codes, st, frame_shift, grid, pos);
     count_launch();
 }
 

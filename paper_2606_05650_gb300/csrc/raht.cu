@@ -302,6 +302,7 @@ __device__ void prelude_tile(const PreludeArgs &a, PreludeSmem<TMAX> &S, int q, 
 __global__ void __launch_bounds__(kThreads) prelude_init_kernel(RahtPlanDev p, const DevState *st,
                                                                  const uint64_t *nv_override)
 {
+    if (after_previous()) return;
     if (threadIdx.x == 0) {
         uint32_t n = (uint32_t)(nv_override ? *nv_override : st->nv_total);
         RahtPass ps = {};
@@ -354,6 +355,7 @@ __device__ __forceinline__ uint32_t tiles_per_cta(uint32_t ntiles, uint32_t ctas
 template <int TMAX, bool WARP>
 __global__ void __launch_bounds__(kThreads) prelude_tiles_kernel(PreludeArgs a, int q)
 {
+    if (after_previous()) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint32_t sh[33];
     __shared__ bool last;
@@ -455,6 +457,7 @@ __device__ void prelude_compact_body(const PreludeArgs &a, int q, uint32_t warp0
 
 __global__ void __launch_bounds__(kThreads) prelude_compact_kernel(PreludeArgs a, int q, uint32_t tile_ctas)
 {
+    if (after_previous()) return;
     if (a.p.passes[q].n == 0 || q + 1 >= kRahtMaxPasses) return;
     prelude_compact_body(a, q, blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5), gridDim.x * (kThreads / 32),
                          tiles_per_cta(a.p.passes[q].ntiles, tile_ctas));
@@ -465,6 +468,7 @@ __global__ void __launch_bounds__(kThreads) prelude_compact_kernel(PreludeArgs a
 template <int TMAX>
 __global__ void __launch_bounds__(kThreads) prelude_finish_kernel(PreludeArgs a, int q0)
 {
+    if (after_previous()) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     PreludeSmem<TMAX> *S = reinterpret_cast<PreludeSmem<TMAX> *>(smem_raw);
     for (int q = q0; q + 1 < kRahtMaxPasses; ++q) {
@@ -912,6 +916,7 @@ __device__ void xform_tile(const XformArgs<S> &A, const XformSmem<S> &X, TileSch
 template <typename S, bool INV, int VEC, bool GATHER, bool QDQ>
 __global__ void __launch_bounds__(kXThreads, 3) xform_pass_kernel(XformArgs<S> A, int q)
 {
+    if (after_previous()) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ TileSched sch;
     const XformSmem<S> X = carve_xform<S>(smem_raw, A.p.T, A.Cg);
@@ -925,6 +930,7 @@ __global__ void __launch_bounds__(kXThreads, 3) xform_pass_kernel(XformArgs<S> A
 template <typename S, bool INV, int VEC, bool QDQ>
 __global__ void __launch_bounds__(kXThreads, 3) xform_finish_kernel(XformArgs<S> A, int q0)
 {
+    if (after_previous()) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ TileSched sch;
     const XformSmem<S> X = carve_xform<S>(smem_raw, A.p.T, A.Cg);
@@ -1319,6 +1325,7 @@ __device__ __forceinline__ FirstStage first_stage(unsigned char *base, uint32_t 
 template <bool INV, bool GATHER, bool QDQ, bool COLOR, int THREADS>
 __global__ void __launch_bounds__(THREADS, 3) xform_first_kernel(XformArgs<float> A, uint32_t slots)
 {
+    if (after_previous()) return;
     typedef Vec<float, 4> V4;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint32_t s_claim[4];
@@ -1619,11 +1626,11 @@ void launch_first(const XformArgs<float> &A, uint64_t tiles, size_t smem, int nu
     if (slots * L <= 448) {
         auto k = xform_first_kernel<INV, GATHER, QDQ, COLOR, 448>;
         const uint32_t grid = one_wave(k, 448, tiles, smem, num_sms);
-        k<<<grid, 448, smem, s>>>(A, slots);
+        launch_after(k, grid, 448, smem, s, A, slots);
     } else {
         auto k = xform_first_kernel<INV, GATHER, QDQ, COLOR, 512>;
         const uint32_t grid = one_wave(k, 512, tiles, smem, num_sms);
-        k<<<grid, 512, smem, s>>>(A, slots);
+        launch_after(k, grid, 512, smem, s, A, slots);
     }
     count_launch();
 }
@@ -1664,7 +1671,7 @@ void launch_pass(const XformArgs<S> &A, int q, uint32_t grid, size_t smem, cudaS
 {
     auto k = xform_pass_kernel<S, INV, VEC, GATHER, QDQ>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<grid, kXThreads, smem, s>>>(A, q);
+    launch_after(k, grid, kXThreads, smem, s, A, q);
     count_launch();
 }
 
@@ -1673,7 +1680,7 @@ void launch_finish(const XformArgs<S> &A, int q0, size_t smem, cudaStream_t s)
 {
     auto k = xform_finish_kernel<S, INV, VEC, QDQ>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<1, kXThreads, smem, s>>>(A, q0);
+    launch_after(k, 1, kXThreads, smem, s, A, q0);
     count_launch();
 }
 
@@ -1782,7 +1789,7 @@ void prelude_tiles(const PreludeArgs &a, int q, uint32_t grid, cudaStream_t s)
 {
     const size_t smem = prelude_smem_bytes<TMAX, WARP>();
     cudaFuncSetAttribute(prelude_tiles_kernel<TMAX, WARP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    prelude_tiles_kernel<TMAX, WARP><<<grid, kThreads, smem, s>>>(a, q);
+    launch_after(prelude_tiles_kernel<TMAX, WARP>, grid, kThreads, smem, s, a, q);
     count_launch();
 }
 
@@ -1792,7 +1799,7 @@ void prelude_launches(const PreludeArgs &a, const RahtPlanDev &p, const DevState
 {
     const size_t smem = prelude_smem_bytes<TMAX, kWarpTiles<TMAX>>();
     cudaFuncSetAttribute(prelude_finish_kernel<TMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    prelude_init_kernel<<<1, 32, 0, s>>>(p, st, nv_dev);
+    launch_after(prelude_init_kernel, 1, 32, 0, s, p, st, nv_dev);
     count_launch();
     const uint32_t grid = (uint32_t)num_sms * (p.pgrid_mult ? p.pgrid_mult : 8u);
     // A pass's sequence is about a fifth of the one before it (its length is known on the device only).  A CTA per
@@ -1809,10 +1816,10 @@ void prelude_launches(const PreludeArgs &a, const RahtPlanDev &p, const DevState
             prelude_tiles<TMAX, kWarpTiles<TMAX>>(a, q, g, s);
         else
             prelude_tiles<TMAX, false>(a, q, g, s);
-        prelude_compact_kernel<<<g, kThreads, 0, s>>>(a, q, g);
+        launch_after(prelude_compact_kernel, g, kThreads, 0, s, a, q, g);
         count_launch();
     }
-    prelude_finish_kernel<TMAX><<<1, kThreads, smem, s>>>(a, wide);
+    launch_after(prelude_finish_kernel<TMAX>, 1, kThreads, smem, s, a, wide);
     count_launch();
 }
 
@@ -1892,7 +1899,7 @@ __global__ void __launch_bounds__(256) frame_centres_kernel(const float *const *
         for (; r + (kAhead - 1) * lanes < m; r += kAhead * lanes) {
             float x[kAhead];
 #pragma unroll
-            for (uint32_t u = 0; u < kAhead; ++u) x[u] = __ldg(a + (uint64_t)(r + u * lanes) * C + c);
+            for (uint32_t u = 0; u < kAhead; ++u) x[u] = *(a + (uint64_t)(r + u * lanes) * C + c);
 #pragma unroll
             for (uint32_t u = 0; u < kAhead; ++u) sum = __fadd_rn(sum, x[u]);
         }
@@ -1910,6 +1917,7 @@ __global__ void __launch_bounds__(256) frame_centres_kernel(const float *const *
 __global__ void frame_dc_kernel(float *Y, const uint32_t *vstart, uint32_t C, const float *center,
                                 const double *steps_rg, const uint8_t *groups, uint32_t G, double tau, double *dc)
 {
+    if (after_previous()) return;
     const uint32_t f = blockIdx.x;
     const uint32_t v0 = vstart[f], nv = vstart[f + 1] - v0;
     for (uint32_t c = threadIdx.x; c < C; c += blockDim.x) {
@@ -1941,7 +1949,7 @@ void launch_frame_dc(float *Y, const uint32_t *vstart, uint32_t F, uint32_t C, c
                      const double *steps_rg, const uint8_t *groups, uint32_t G, double tau, double *dc, cudaStream_t s)
 {
     if (F == 0 || C == 0) return;
-    frame_dc_kernel<<<F, 64, 0, s>>>(Y, vstart, C, center, steps_rg, groups, G, tau, dc);
+    launch_after(frame_dc_kernel, F, 64, 0, s, Y, vstart, C, center, steps_rg, groups, G, tau, dc);
     count_launch();
 }
 

@@ -24,9 +24,10 @@ constexpr uint32_t kL = 1u << 16;
 // bytes of a 16-byte word are counted from registers, so every thread keeps
 // several loads in flight), counted into per-warp sub-histograms in shared
 // memory (fewer lanes contend for a bin), added up per CTA.
-__global__ void __launch_bounds__(256) hist_kernel(const uint8_t *__restrict__ occ, const uint64_t *occ_off,
+__global__ void __launch_bounds__(256) hist_kernel(const uint8_t *occ, const uint64_t *occ_off,
                                                    DevState *st)
 {
+    if (after_previous()) return;
     __shared__ uint32_t h[8][256];
     const uint32_t f = blockIdx.y, t = threadIdx.x, wid = t >> 5;
     for (uint32_t k = t; k < 8 * 256; k += 256) (&h[0][0])[k] = 0;
@@ -41,7 +42,7 @@ __global__ void __launch_bounds__(256) hist_kernel(const uint8_t *__restrict__ o
     for (uint64_t i = gt; i < n16; i += 4 * gs) {
         uint4 x[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = (i + u * gs < n16) ? __ldg(v + i + u * gs) : make_uint4(0, 0, 0, 0);
+        for (int u = 0; u < 4; ++u) x[u] = (i + u * gs < n16) ? *(v + i + u * gs) : make_uint4(0, 0, 0, 0);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             if (i + u * gs >= n16) break;
@@ -70,6 +71,7 @@ __global__ void __launch_bounds__(256) hist_kernel(const uint8_t *__restrict__ o
 __global__ void __launch_bounds__(256) norm_kernel(const uint64_t *occ_off, DevState *st, uint16_t *freq,
                                                    uint32_t *cum, uint32_t *mode)
 {
+    if (after_previous()) return;
     const uint32_t f = blockIdx.x, s = threadIdx.x;
     const uint64_t n = occ_off[f + 1] - occ_off[f];
     const uint32_t cnt = st->hist[f][s];
@@ -102,6 +104,7 @@ __global__ void __launch_bounds__(256) norm_kernel(const uint64_t *occ_off, DevS
 __global__ void __launch_bounds__(kMaxFrames) chunk_offsets_kernel(const uint64_t *occ_off, const uint32_t *mode, uint32_t F,
                                                                    uint32_t chunk, uint64_t *chunk_off)
 {
+    if (after_previous()) return;
     __shared__ uint64_t sh[33];
     const uint32_t f = threadIdx.x;
     const uint64_t c = f < F && mode[f] == 1 ? (occ_off[f + 1] - occ_off[f] + chunk - 1) / chunk : 0ull;
@@ -118,12 +121,13 @@ __global__ void __launch_bounds__(kMaxFrames) chunk_offsets_kernel(const uint64_
 constexpr int kEncWarps = 4;
 constexpr uint32_t kStageSyms = 4096;  // symbols staged per pass
 
-__global__ void __launch_bounds__(32 * kEncWarps) encode_kernel(const uint8_t *__restrict__ occ, const uint64_t *occ_off,
+__global__ void __launch_bounds__(32 * kEncWarps) encode_kernel(const uint8_t *occ, const uint64_t *occ_off,
                                                                const uint64_t *chunk_off, uint32_t F, uint32_t chunk,
                                                                const uint16_t *freq, const uint32_t *cum, uint8_t *slots,
                                                                uint64_t slot_bytes, uint32_t *chunk_words,
                                                                uint32_t *chunk_top)
 {
+    if (after_previous()) return;
     __shared__ __align__(16) uint8_t s_sym[kEncWarps][kStageSyms];
     __shared__ uint32_t s_fc[256];   // freq << 16 | cum (cum < 2^15)
     __shared__ uint32_t s_rcp[256];  // ceil(2^32 / freq) for freq >= 2 (0 for freq < 2)
@@ -162,7 +166,7 @@ __global__ void __launch_bounds__(32 * kEncWarps) encode_kernel(const uint8_t *_
                 const uint4 *v = reinterpret_cast<const uint4 *>(sym + b0 + head);
                 uint8_t *dst = &s_sym[wl][0];
                 for (uint32_t k = lane; k < nvec; k += 32) {
-                    const uint4 w = __ldg(v + k);
+                    const uint4 w = *(v + k);
                     uint32_t *d32 = reinterpret_cast<uint32_t *>(dst + head + 16 * k);  // byte-addressed smem
                     const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
@@ -222,6 +226,7 @@ __global__ void __launch_bounds__(512) section_size_kernel(const uint64_t *occ_o
                                                            const uint32_t *chunk_words, uint32_t *chunk_pos,
                                                            uint32_t *mode, uint64_t *sec_bytes)
 {
+    if (after_previous()) return;
     __shared__ uint64_t sh[33];
     const uint32_t f = blockIdx.x;
     const uint64_t n = occ_off[f + 1] - occ_off[f];
@@ -256,10 +261,11 @@ __global__ void __launch_bounds__(512) section_size_kernel(const uint64_t *occ_o
 // building the tables for all of them in a launch before: 19 us more.)
 constexpr uint32_t kSmemChunks = 4096;
 
-__global__ void __launch_bounds__(32 * ransdec::kMaxWarps) decode_kernel(const uint8_t *__restrict__ sec,
+__global__ void __launch_bounds__(32 * ransdec::kMaxWarps) decode_kernel(const uint8_t *sec,
                                                                          uint64_t sec_bytes, uint64_t n, uint32_t nch,
                                                                          uint32_t chunk, uint8_t *out, DevState *st)
 {
+    if (after_previous()) return;
     using namespace ransdec;
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ uint32_t sh[33], cum[257];
@@ -320,11 +326,11 @@ void launch_rans_encode(const RansFrames &r, DevState *st, uint64_t max_chunks, 
     dev_memset(&st->hist[0][0], 0, sizeof(uint32_t) * 256 * r.F, s);
     dim3 g(num_sms, r.F);
     if (r.F > 8) g.x = (num_sms * 8 + r.F - 1) / r.F;
-    hist_kernel<<<g, 256, 0, s>>>(r.occ, r.occ_off, st);
+    launch_after(hist_kernel, g, 256, 0, s, r.occ, r.occ_off, st);
     count_launch();
-    norm_kernel<<<r.F, 256, 0, s>>>(r.occ_off, st, r.freq, r.cum, r.mode);
+    launch_after(norm_kernel, r.F, 256, 0, s, r.occ_off, st, r.freq, r.cum, r.mode);
     count_launch();
-    chunk_offsets_kernel<<<1, kMaxFrames, 0, s>>>(r.occ_off, r.mode, r.F, r.chunk, r.chunk_off);
+    launch_after(chunk_offsets_kernel, 1, kMaxFrames, 0, s, r.occ_off, r.mode, r.F, r.chunk, r.chunk_off);
     count_launch();
     if (max_chunks) {
         // per frame: enough CTAs to fill the GPU when every frame has chunks, at most one chunk per warp
@@ -332,12 +338,12 @@ void launch_rans_encode(const RansFrames &r, DevState *st, uint64_t max_chunks, 
         const uint64_t need = (max_chunks + kEncWarps - 1) / kEncWarps;
         if (per > need) per = need;
         if (per < 1) per = 1;
-        encode_kernel<<<dim3((uint32_t)per, r.F), 32 * kEncWarps, 0, s>>>(r.occ, r.occ_off, r.chunk_off, r.F, r.chunk, r.freq, r.cum,
+        launch_after(encode_kernel, dim3((uint32_t)per, r.F), 32 * kEncWarps, 0, s, r.occ, r.occ_off, r.chunk_off, r.F, r.chunk, r.freq, r.cum,
                                                         r.chunk_slots, rans_chunk_slot_bytes(r.chunk), r.chunk_words,
                                                         r.chunk_top);
         count_launch();
     }
-    section_size_kernel<<<r.F, 512, 0, s>>>(r.occ_off, r.chunk_off, r.chunk_words, r.chunk_pos, r.mode, r.sec_bytes);
+    launch_after(section_size_kernel, r.F, 512, 0, s, r.occ_off, r.chunk_off, r.chunk_words, r.chunk_pos, r.mode, r.sec_bytes);
     count_launch();
 }
 
@@ -352,7 +358,7 @@ void launch_rans_decode(const uint8_t *sec, uint64_t sec_bytes, uint64_t n, uint
     if (blocks > (uint32_t)num_sms * 4) blocks = (uint32_t)num_sms * 4;
     const size_t smem = (size_t)ransdec::kTabWords * 4 + 4 * (size_t)kSmemChunks;
     cudaFuncSetAttribute(decode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    decode_kernel<<<blocks, 32 * warps, smem, s>>>(sec, sec_bytes, n, nch, chunk, out, st);
+    launch_after(decode_kernel, blocks, 32 * warps, smem, s, sec, sec_bytes, n, nch, chunk, out, st);
     count_launch();
 }
 

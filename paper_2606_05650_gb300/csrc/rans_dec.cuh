@@ -77,7 +77,7 @@ __device__ __forceinline__ bool decode_chunk(const uint8_t *slot2sym, const uint
 {
     const uint32_t *words = reinterpret_cast<const uint32_t *>(src + 128);
     const uint32_t n32 = W / 2;
-    auto word = [&](uint32_t i) { return i < n32 ? __ldg(words + i) : 0u; };
+    auto word = [&](uint32_t i) { return i < n32 ? words[i] : 0u; };
     uint32_t x = reinterpret_cast<const uint32_t *>(src)[lane];
     const uint32_t ltm = lanemask_lt();
     uint32_t line = 0, c0 = word(lane), c1 = word(32 + lane), c2 = word(64 + lane), c3 = word(96 + lane);

@@ -212,11 +212,12 @@ __device__ __forceinline__ void view_direction(const float *p, const RenderCam &
     for (int c = 0; c < 3; ++c) dir[c] = d[c] * id;
 }
 
-__global__ void __launch_bounds__(256) preprocess_kernel(const float *__restrict__ pos,
-                                                         const float *__restrict__ attr, uint64_t n, RenderCam cam,
+__global__ void __launch_bounds__(256) preprocess_kernel(const float *pos,
+                                                         const float *attr, uint64_t n, RenderCam cam,
                                                          Splat *sp, uint32_t *depth, uint32_t *idx,
                                                          ushort4 *rect, uint32_t *count)
 {
+    if (after_previous()) return;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
         count[i] = 0;
         depth[i] = 0xFFFFFFFFu;
@@ -324,6 +325,7 @@ __global__ void __launch_bounds__(256) preprocess_kernel(const float *__restrict
 
 __global__ void gather_counts_kernel(const uint32_t *order, const uint32_t *count, uint64_t n, uint32_t *out)
 {
+    if (after_previous()) return;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
         out[i] = count[order[i]];
 }
@@ -334,6 +336,7 @@ __global__ void gather_counts_kernel(const uint32_t *order, const uint32_t *coun
 __global__ void __launch_bounds__(256) emit_kernel(uint64_t n, const uint32_t *order, const ushort4 *rect,
                                                    const uint64_t *offs, int TX, uint32_t *tiles, uint32_t *vals)
 {
+    if (after_previous()) return;
     const uint32_t lane = threadIdx.x & 31;
     const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
     for (uint64_t w = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w * 32 < n; w += warps) {
@@ -367,8 +370,9 @@ __global__ void __launch_bounds__(256) emit_kernel(uint64_t n, const uint32_t *o
 // Entries [x, y) of the sorted list per tile, by binary search: a thread per
 // tile and some twenty-five dependent loads, against a pass over the whole list
 // (1M Gaussians at 960 x 540: 85 -> 17 us).
-__global__ void ranges_kernel(const uint32_t *__restrict__ tiles, uint64_t total, uint32_t ntiles, uint2 *ranges)
+__global__ void ranges_kernel(const uint32_t *tiles, uint64_t total, uint32_t ntiles, uint2 *ranges)
 {
+    if (after_previous()) return;
     const uint32_t tile = blockIdx.x * blockDim.x + threadIdx.x;
     if (tile >= ntiles) return;
     auto first = [&](uint32_t key) {  // the first entry with a tile of at least key
@@ -402,6 +406,7 @@ constexpr int kWarpsPerCta = 4;  // the blocks of half a tile
 __global__ void __launch_bounds__(32 * kWarpsPerCta) render_kernel(const uint2 *ranges, const uint32_t *vals,
                                                                    const Splat *sp, RenderCam cam, float *image)
 {
+    if (after_previous()) return;
     static_assert(sizeof(Splat) == 48 && kTile == 16, "copied in 16-byte words; two halves of 16 x 8 pixels");
     __shared__ __align__(16) Splat batch[kWarpsPerCta][2][32];
     const int tx = blockIdx.x, ty = blockIdx.y >> 1;
@@ -489,7 +494,7 @@ size_t render_splat_bytes() { return sizeof(Splat); }
 void launch_render_prepare(const float *pos, const float *attr, uint64_t n, const RenderCam &cam,
                            const RenderBuffers &b, const uint32_t **order, int num_sms, cudaStream_t s)
 {
-    preprocess_kernel<<<rgrid(n, num_sms), 256, 0, s>>>(pos, attr, n, cam, (Splat *)b.splats, b.depth, b.idx, b.rect,
+    launch_after(preprocess_kernel, rgrid(n, num_sms), 256, 0, s, pos, attr, n, cam, (Splat *)b.splats, b.depth, b.idx, b.rect,
                                                         b.count);
     count_launch();
     // Depth first, over the Gaussians; then only the tile bits over the many times longer list of their tiles.
@@ -497,7 +502,7 @@ void launch_render_prepare(const float *pos, const float *attr, uint64_t n, cons
     // 1M Gaussians and 960 x 540 (24M entries); the whole call was 4.6 ms this way.
     const bool alt = radix_sort(b.depth, b.idx, b.depth_alt, b.idx_alt, b.hist, n, 32u, num_sms, s);
     *order = alt ? b.idx_alt : b.idx;
-    gather_counts_kernel<<<rgrid(n, num_sms), 256, 0, s>>>(*order, b.count, n, b.count_sorted);
+    launch_after(gather_counts_kernel, rgrid(n, num_sms), 256, 0, s, *order, b.count, n, b.count_sorted);
     count_launch();
     launch_scan_u32_to_u64(b.count_sorted, n, b.offs, b.partials, num_sms, s);
 }
@@ -509,18 +514,18 @@ void launch_render_tiles(uint64_t n, const RenderBuffers &b, const uint32_t *ord
     const uint32_t ntiles = (uint32_t)(cam.TX * cam.TY);
     const uint32_t *sv = vals;
     if (total) {
-        emit_kernel<<<rgrid(n, num_sms), 256, 0, s>>>(n, order, b.rect, b.offs, cam.TX, tiles, vals);
+        launch_after(emit_kernel, rgrid(n, num_sms), 256, 0, s, n, order, b.rect, b.offs, cam.TX, tiles, vals);
         count_launch();
         uint32_t tb = 0;
         while ((1u << tb) < ntiles) ++tb;
         const bool alt = radix_sort(tiles, vals, tiles_alt, vals_alt, hist, total, tb, num_sms, s);
         if (alt) sv = vals_alt;
-        ranges_kernel<<<(ntiles + 63) / 64, 64, 0, s>>>(alt ? tiles_alt : tiles, total, ntiles, ranges);
+        launch_after(ranges_kernel, (ntiles + 63) / 64, 64, 0, s, alt ? tiles_alt : tiles, total, ntiles, ranges);
         count_launch();
     } else {
         dev_memset(ranges, 0, sizeof(uint2) * ntiles, s);
     }
-    render_kernel<<<dim3(cam.TX, 2 * cam.TY), 32 * kWarpsPerCta, 0, s>>>(ranges, sv, (const Splat *)b.splats, cam, image);
+    launch_after(render_kernel, dim3(cam.TX, 2 * cam.TY), 32 * kWarpsPerCta, 0, s, ranges, sv, (const Splat *)b.splats, cam, image);
     count_launch();
 }
 

@@ -369,6 +369,7 @@ __device__ __forceinline__ EncBlock enc_block(const EncJobs &E, uint64_t job)
 template <bool FROM_INT, bool DIST, uint32_t PITCH>
 __global__ void __launch_bounds__(PITCH, 1024 / PITCH) rlgr_encode_kernel(EncJobs E, const int32_t *qin, uint32_t rb)
 {
+    if (after_previous()) return;
     extern __shared__ uint32_t ring[];  // kRing x PITCH
     __shared__ EncBlock blk_info[32];
     __shared__ __align__(16) EncTable tab;
@@ -471,7 +472,7 @@ __global__ void __launch_bounds__(PITCH, 1024 / PITCH) rlgr_encode_kernel(EncJob
     if (i < len) {  // fewer than kPrefetch rows
         uint32_t x[kPrefetch - 1];
 #pragma unroll
-        for (uint32_t d = 0; d + 1 < kPrefetch; ++d) x[d] = i + d < len ? __ldg(col + (uint64_t)(i + d) * C) : 0u;
+        for (uint32_t d = 0; d + 1 < kPrefetch; ++d) x[d] = i + d < len ? *(col + (uint64_t)(i + d) * C) : 0u;
 #pragma unroll 1
         for (uint32_t d = 0; i < len; ++i, ++d) {
             const uint32_t y = d == 0 ? x[0] : (d == 1 ? x[1] : x[2]);
@@ -521,6 +522,7 @@ struct RlgrFew {
 
 __global__ void __launch_bounds__(512) rlgr_encode_few_kernel(EncJobs E, uint32_t rb)
 {
+    if (after_previous()) return;
     __shared__ EncBlock blk_info[32];
     const RlgrJob &j = E.j;
     const uint32_t C = j.C, W = j.R * C, t = threadIdx.x;
@@ -544,12 +546,12 @@ __global__ void __launch_bounds__(512) rlgr_encode_few_kernel(EncJobs E, uint32_
     }
     float cur[kPrefetch];
 #pragma unroll
-    for (uint32_t d = 0; d < kPrefetch; ++d) cur[d] = (i + d < len) ? __ldg(col + (uint64_t)(i + d) * C) : 0.f;
+    for (uint32_t d = 0; d < kPrefetch; ++d) cur[d] = (i + d < len) ? *(col + (uint64_t)(i + d) * C) : 0.f;
     for (; i + kPrefetch <= len; i += kPrefetch) {
         float nx[kPrefetch];
         const float *q = col + (uint64_t)(i + kPrefetch) * C;
 #pragma unroll
-        for (uint32_t d = 0; d < kPrefetch; ++d) nx[d] = (i + kPrefetch + d < len) ? __ldg(q + d * C) : 0.f;
+        for (uint32_t d = 0; d < kPrefetch; ++d) nx[d] = (i + kPrefetch + d < len) ? *(q + d * C) : 0.f;
 #pragma unroll
         for (uint32_t d = 0; d < kPrefetch; ++d) st.code(bw, quantize_zz_f32(cur[d], inv, tau));
 #pragma unroll
@@ -606,6 +608,7 @@ __device__ __forceinline__ void or_bits(uint32_t *buf, uint32_t o, uint64_t c)
 
 __global__ void __launch_bounds__(kSplitThreads, 4) rlgr_encode_split_kernel(EncJobs E)
 {
+    if (after_previous()) return;
     __shared__ uint32_t sym[3][kSplitSeg * kSplitRow];  // zigzag indices of a segment
     __shared__ uint32_t pre[2][kSplitSeg * kSplitRow];  // states before its symbols
     __shared__ uint32_t bits[kSplitG][84];            // 32 codewords of up to 78 bits behind a part of a word
@@ -638,7 +641,7 @@ __global__ void __launch_bounds__(kSplitThreads, 4) rlgr_encode_split_kernel(Enc
 #pragma unroll
         for (uint32_t h = 0; h < kPer; ++h) {
             const uint32_t i = seg * kSplitSeg + at + kSplitSeg / kPer * h;
-            val[h] = i < ld.len ? __ldg(col + (uint64_t)i * C) : 0.f;
+            val[h] = i < ld.len ? *(col + (uint64_t)i * C) : 0.f;
         }
     };
     const auto put_symbols = [&](uint32_t seg) {
@@ -995,6 +998,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) rlgr_decode_kernel(const uint3
                                                           const float *step, float *Y, int32_t *qout,
                                                           DevState *st)
 {
+    if (after_previous()) return;
     extern __shared__ __align__(128) uint32_t ring[];  // kRingWords per thread
     __shared__ __align__(16) DecTable tab;
     stage_table(&tab, &g_dec_table);
@@ -1022,6 +1026,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) rlgr_decode_batch_kernel(const
                                                                 const uint64_t *boff_all, const float *steps_all,
                                                                 uint32_t C, float *Y, DevState *st)
 {
+    if (after_previous()) return;
     extern __shared__ __align__(128) uint32_t ring[];  // kRingWords per thread
     __shared__ __align__(16) DecTable tab;
     stage_table(&tab, &g_dec_table);
@@ -1054,6 +1059,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) rlgr_decode_batch_kernel(const
 __global__ void __launch_bounds__(kMaxFrames) job_offsets_kernel(const uint32_t *vstart, uint32_t F, uint32_t B, uint32_t R,
                                                                  uint32_t C, uint64_t *job_off, uint64_t *blk_off)
 {
+    if (after_previous()) return;
     __shared__ uint64_t sh[33];
     const uint32_t f = threadIdx.x;
     const uint64_t nb = f < F ? ((uint64_t)(vstart[f + 1] - vstart[f]) + B - 1) / B : 0ull;
@@ -1084,7 +1090,7 @@ static void launch_encode(const EncJobs &E, const int32_t *q, uint32_t rb, uint3
 {
     const uint32_t grid = (uint32_t)((jobs + rb - 1) / rb);
     auto k = threads <= 256 ? rlgr_encode_kernel<FROM_INT, DIST, 256> : rlgr_encode_kernel<FROM_INT, DIST, 512>;
-    k<<<grid, threads, ring_smem(k, 4 * (size_t)kRing * (threads <= 256 ? 256 : 512)), s>>>(E, q, rb);
+    launch_after(k, grid, threads, ring_smem(k, 4 * (size_t)kRing * (threads <= 256 ? 256 : 512)), s, E, q, rb);
     count_launch();
 }
 
@@ -1098,7 +1104,7 @@ uint32_t rlgr_slot_words(uint32_t B, bool worst_case)
 void launch_rlgr_offsets(const uint32_t *vstart, uint32_t F, uint32_t B, uint32_t R, uint32_t C, uint64_t *job_off,
                          uint64_t *blk_off, cudaStream_t s)
 {
-    job_offsets_kernel<<<1, kMaxFrames, 0, s>>>(vstart, F, B, R, C, job_off, blk_off);
+    launch_after(job_offsets_kernel, 1, kMaxFrames, 0, s, vstart, F, B, R, C, job_off, blk_off);
     count_launch();
 }
 
@@ -1110,12 +1116,12 @@ void launch_rlgr_encode(const RlgrJob &j, const uint64_t *job_off, uint64_t jobs
     const uint32_t rb = row_blocks_per_cta(W);
     const uint32_t threads = (rb * W + 31) / 32 * 32;
     if (!j.sq_err && W <= 512 && jobs_bound * W <= kSplitStreams) {
-        rlgr_encode_split_kernel<<<(uint32_t)((jobs_bound * W + kSplitG - 1) / kSplitG), kSplitThreads, 0, s>>>(E);
+        launch_after(rlgr_encode_split_kernel, (uint32_t)((jobs_bound * W + kSplitG - 1) / kSplitG), kSplitThreads, 0, s, E);
         count_launch();
         return;
     }
     if (!j.sq_err && jobs_bound * W <= kFewStreams) {
-        rlgr_encode_few_kernel<<<(uint32_t)((jobs_bound + rb - 1) / rb), threads, 0, s>>>(E, rb);
+        launch_after(rlgr_encode_few_kernel, (uint32_t)((jobs_bound + rb - 1) / rb), threads, 0, s, E, rb);
         count_launch();
         return;
     }
@@ -1165,7 +1171,7 @@ void launch_rlgr_decode(const uint32_t *payload, uint64_t payload_words, const u
 {
     if (nv == 0 || C == 0) return;
     launch_decode(rlgr_decode_kernel<false>, (nv + B - 1) / B * C, [&](auto k, uint32_t grid, uint32_t threads, size_t smem) {
-        k<<<grid, threads, smem, s>>>(payload, payload_words, block_words, block_off, 0u, (uint32_t)nv, C, B, step, Y,
+        launch_after(k, grid, threads, smem, s, payload, payload_words, block_words, block_off, 0u, (uint32_t)nv, C, B, step, Y,
                                       nullptr, st);
     });
 }
@@ -1176,7 +1182,7 @@ void launch_rlgr_decode_batch(const DecFrame *fr, uint32_t F, const uint64_t *jo
 {
     if (jobs_bound == 0 || C == 0) return;
     launch_decode(rlgr_decode_batch_kernel, jobs_bound * C, [&](auto k, uint32_t grid, uint32_t threads, size_t smem) {
-        k<<<grid, threads, smem, s>>>(fr, F, job_off, bw_all, boff_all, steps_all, C, Y, st);
+        launch_after(k, grid, threads, smem, s, fr, F, job_off, bw_all, boff_all, steps_all, C, Y, st);
     });
 }
 
@@ -1185,7 +1191,7 @@ void launch_rlgr_decode_indices(const uint32_t *words, uint64_t total_words, con
 {
     if (nv == 0 || C == 0) return;
     launch_decode(rlgr_decode_kernel<true>, (nv + B - 1) / B * C, [&](auto k, uint32_t grid, uint32_t threads, size_t smem) {
-        k<<<grid, threads, smem, s>>>(words, total_words, bw, nullptr, stride, (uint32_t)nv, C, B, nullptr, nullptr, q,
+        launch_after(k, grid, threads, smem, s, words, total_words, bw, nullptr, stride, (uint32_t)nv, C, B, nullptr, nullptr, q,
                                       st);
     });
 }

@@ -28,6 +28,7 @@ Geom geom(uint64_t n, int num_sms)
 
 __global__ void __launch_bounds__(kThreads) up_kernel(const uint32_t *in, uint64_t n, uint64_t chunk, uint64_t *part)
 {
+    if (after_previous()) return;
     uint64_t b = (uint64_t)blockIdx.x * chunk, e = b + chunk;
     if (e > n) e = n;
     uint64_t s = 0;
@@ -40,6 +41,7 @@ __global__ void __launch_bounds__(kThreads) up_kernel(const uint32_t *in, uint64
 
 __global__ void __launch_bounds__(1024) mid_kernel(uint64_t *part, uint32_t P)
 {
+    if (after_previous()) return;
     __shared__ uint64_t sh[33];
     uint64_t v = (threadIdx.x < P) ? part[threadIdx.x] : 0ull;
     uint64_t tot;
@@ -51,6 +53,7 @@ __global__ void __launch_bounds__(1024) mid_kernel(uint64_t *part, uint32_t P)
 __global__ void __launch_bounds__(kThreads) down_kernel(const uint32_t *in, uint64_t n, uint64_t chunk,
                                                         const uint64_t *part, uint64_t *out)
 {
+    if (after_previous()) return;
     __shared__ uint64_t sh[33];
     uint64_t b = (uint64_t)blockIdx.x * chunk, e = b + chunk;
     if (e > n) e = n;
@@ -73,8 +76,9 @@ __global__ void __launch_bounds__(kThreads) down_kernel(const uint32_t *in, uint
 // a frame of 10k Gaussians went from 438 to 428 us (encode) and from 355 to 347
 // us (decode), the 8 x 5 ladder from 3630 to 3587 us.
 constexpr uint64_t kSmallScan = 8192;
-__global__ void __launch_bounds__(1024) small_kernel(const uint32_t *__restrict__ in, uint32_t n, uint64_t *__restrict__ out)
+__global__ void __launch_bounds__(1024) small_kernel(const uint32_t *in, uint32_t n, uint64_t *out)
 {
+    if (after_previous()) return;
     __shared__ uint64_t sh[33];
     constexpr uint32_t kPer = kSmallScan / 1024;
     const uint32_t b = threadIdx.x * kPer;
@@ -108,15 +112,15 @@ void launch_scan_u32_to_u64(const uint32_t *in, uint64_t n, uint64_t *out, uint6
         return;
     }
     if (n <= kSmallScan) {
-        small_kernel<<<1, 1024, 0, s>>>(in, (uint32_t)n, out);
+        launch_after(small_kernel, 1, 1024, 0, s, in, (uint32_t)n, out);
         count_launch();
         return;
     }
-    up_kernel<<<g.P, kThreads, 0, s>>>(in, n, g.chunk, partials);
+    launch_after(up_kernel, g.P, kThreads, 0, s, in, n, g.chunk, partials);
     count_launch();
-    mid_kernel<<<1, 1024, 0, s>>>(partials, g.P);
+    launch_after(mid_kernel, 1, 1024, 0, s, partials, g.P);
     count_launch();
-    down_kernel<<<g.P, kThreads, 0, s>>>(in, n, g.chunk, partials, out);
+    launch_after(down_kernel, g.P, kThreads, 0, s, in, n, g.chunk, partials, out);
     count_launch();
 }
 
@@ -126,6 +130,7 @@ void launch_scan_u32_to_u64(const uint32_t *in, uint64_t n, uint64_t *out, uint6
 namespace {
 __global__ void memset_kernel(unsigned char *p, uint32_t v4, unsigned char v, uint64_t n)
 {
+    if (after_previous()) return;
     const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (uint64_t)gridDim.x * blockDim.x;
     const uint64_t head = (16 - ((uintptr_t)p & 15)) & 15;
     const uint64_t h = head < n ? head : n;
@@ -144,7 +149,7 @@ cudaError_t dev_memset(void *p, int value, size_t bytes, cudaStream_t s)
     const uint32_t v4 = 0x01010101u * v;
     const uint64_t units = (bytes + 15) / 16;
     const uint32_t blocks = (uint32_t)std::min<uint64_t>((units + 255) / 256, 1024);
-    memset_kernel<<<blocks, 256, 0, s>>>(static_cast<unsigned char *>(p), v4, v, bytes);
+    launch_after(memset_kernel, blocks, 256, 0, s, static_cast<unsigned char *>(p), v4, v, bytes);
     count_launch();
     return cudaGetLastError();
 }

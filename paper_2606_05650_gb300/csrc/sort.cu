@@ -103,10 +103,11 @@ __device__ __forceinline__ uint32_t same_digit(uint32_t d, bool ok, uint32_t mas
 }
 
 template <typename Key, int kThreads>
-__global__ void __launch_bounds__(kThreads) upsweep_kernel(const Key *__restrict__ keys, uint64_t n,
+__global__ void __launch_bounds__(kThreads) upsweep_kernel(const Key *keys, uint64_t n,
                                                            uint32_t shift, uint32_t mask, uint64_t chunk, uint32_t *hist,
-                                                           const uint64_t *__restrict__ cta_lo)
+                                                           const uint64_t *cta_lo)
 {
+    if (after_previous()) return;
     __shared__ uint32_t h[kRadix];
     if (threadIdx.x < kRadix) h[threadIdx.x] = 0;
     __syncthreads();
@@ -129,6 +130,7 @@ __global__ void __launch_bounds__(kThreads) upsweep_kernel(const Key *__restrict
 // stores the digit total at hist[256 * P + d]
 __global__ void __launch_bounds__(256) scan_cols_kernel(uint32_t *hist, uint32_t P)
 {
+    if (after_previous()) return;
     const uint32_t d = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     uint32_t *row = hist + (uint64_t)d * P;
     uint32_t run = 0;
@@ -155,15 +157,16 @@ struct DownSmem {
 };
 
 template <typename Key, typename Cfg>
-__global__ void __launch_bounds__(Cfg::threads, Cfg::ctas) downsweep_kernel(const Key *__restrict__ keys,
-                                                             const uint32_t *__restrict__ vals, uint64_t n,
+__global__ void __launch_bounds__(Cfg::threads, Cfg::ctas) downsweep_kernel(const Key *keys,
+                                                             const uint32_t *vals, uint64_t n,
                                                              uint32_t shift, uint32_t mask, uint64_t chunk,
-                                                             const uint32_t *__restrict__ hist,
-                                                             Key *__restrict__ keys_out,
-                                                             uint32_t *__restrict__ vals_out,
-                                                             const uint64_t *__restrict__ cta_lo,
-                                                             const uint32_t *__restrict__ cta_seg)
+                                                             const uint32_t *hist,
+                                                             Key *keys_out,
+                                                             uint32_t *vals_out,
+                                                             const uint64_t *cta_lo,
+                                                             const uint32_t *cta_seg)
 {
+    if (after_previous()) return;
     constexpr int kWarps = Cfg::warps, kPairs = Cfg::kpt, kTile = Cfg::tile;
     extern __shared__ __align__(16) unsigned char sort_raw[];
     DownSmem<Key, Cfg> &S = *reinterpret_cast<DownSmem<Key, Cfg> *>(sort_raw);
@@ -281,12 +284,13 @@ struct SmallSmem {
 };
 
 template <typename Key>
-__global__ void __launch_bounds__(kSmallThreads, 1) small_sort_kernel(const Key *__restrict__ keys,
-                                                                      const uint32_t *__restrict__ vals, uint32_t n,
+__global__ void __launch_bounds__(kSmallThreads, 1) small_sort_kernel(const Key *keys,
+                                                                      const uint32_t *vals, uint32_t n,
                                                                       uint32_t nbits, uint32_t width, uint32_t rounds,
-                                                                      Key *__restrict__ keys_out,
-                                                                      uint32_t *__restrict__ vals_out)
+                                                                      Key *keys_out,
+                                                                      uint32_t *vals_out)
 {
+    if (after_previous()) return;
     extern __shared__ __align__(16) unsigned char small_raw[];
     SmallSmem<Key> &S = *reinterpret_cast<SmallSmem<Key> *>(small_raw);
     const uint32_t tid = threadIdx.x, lane = tid & 31, w = tid >> 5, at0 = w * rounds * 32 + lane;
@@ -367,7 +371,7 @@ void small_sort(const Key *keys, const uint32_t *vals, Key *keys_out, uint32_t *
                 cudaStream_t s)
 {
     cudaFuncSetAttribute(small_sort_kernel<Key>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallSmem<Key>));
-    small_sort_kernel<Key><<<1, kSmallThreads, sizeof(SmallSmem<Key>), s>>>(
+    launch_after(small_sort_kernel<Key>, 1, kSmallThreads, sizeof(SmallSmem<Key>), s, 
         keys, vals, n, nbits, digit_width(nbits), (n + kSmallThreads - 1) / kSmallThreads, keys_out, vals_out);
     count_launch();
 }
@@ -405,7 +409,7 @@ static void launch_down(const Key *keys, const uint32_t *vals, uint64_t n, uint3
 {
     constexpr size_t smem = sizeof(DownSmem<Key, Cfg>);
     cudaFuncSetAttribute(downsweep_kernel<Key, Cfg>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    downsweep_kernel<Key, Cfg><<<P, Cfg::threads, smem, s>>>(keys, vals, n, shift, mask, chunk, hist, keys_out, vals_out,
+    launch_after(downsweep_kernel<Key, Cfg>, P, Cfg::threads, smem, s, keys, vals, n, shift, mask, chunk, hist, keys_out, vals_out,
                                                              cta_lo, cta_seg);
     count_launch();
 }
@@ -422,11 +426,11 @@ static bool sort_passes(Key *keys, uint32_t *vals, Key *keys_alt, uint32_t *vals
     const uint32_t width = digit_width(nbits), mask = (1u << width) - 1u;
     for (uint32_t shift = 0; shift < nbits; shift += width) {
         if (large)
-            upsweep_kernel<Key, SortLarge::threads><<<P, SortLarge::threads, 0, s>>>(ki, n, shift, mask, chunk, hist, cta_lo);
+            launch_after(upsweep_kernel<Key, SortLarge::threads>, P, SortLarge::threads, 0, s, ki, n, shift, mask, chunk, hist, cta_lo);
         else
-            upsweep_kernel<Key, SortSmall::threads><<<P, SortSmall::threads, 0, s>>>(ki, n, shift, mask, chunk, hist, cta_lo);
+            launch_after(upsweep_kernel<Key, SortSmall::threads>, P, SortSmall::threads, 0, s, ki, n, shift, mask, chunk, hist, cta_lo);
         count_launch();
-        scan_cols_kernel<<<kRadix / 8, 256, 0, s>>>(hist, P);
+        launch_after(scan_cols_kernel, kRadix / 8, 256, 0, s, hist, P);
         count_launch();
         if (large)
             launch_down<Key, SortLarge>(ki, vi, n, shift, mask, chunk, hist, ko, vo, cta_lo, cta_seg, P, s);

@@ -17,6 +17,7 @@ constexpr int kThreads = 256;
 
 __global__ void init_bbox_kernel(DevState *st, uint32_t F)
 {
+    if (after_previous()) return;
     int t = threadIdx.x;
     if (t == 0) {
         st->err = 0;
@@ -33,6 +34,7 @@ __global__ void init_bbox_kernel(DevState *st, uint32_t F)
 // grid (X, F): block (x, f) reduces a strided share of frame f's points
 __global__ void __launch_bounds__(kThreads) bbox_kernel(FrameSet fs, DevState *st)
 {
+    if (after_previous()) return;
     const uint32_t f = blockIdx.y;
     const float *pos = fs.pos[f];
     const uint64_t n = fs.poff[f + 1] - fs.poff[f];
@@ -44,7 +46,7 @@ __global__ void __launch_bounds__(kThreads) bbox_kernel(FrameSet fs, DevState *s
 #pragma unroll
         for (int k = 0; k < 4; ++k)
 #pragma unroll
-            for (int a = 0; a < 3; ++a) p[k][a] = __ldg(pos + 3 * (i + k * step) + a);
+            for (int a = 0; a < 3; ++a) p[k][a] = *(pos + 3 * (i + k * step) + a);
 #pragma unroll
         for (int k = 0; k < 4; ++k)
 #pragma unroll
@@ -56,7 +58,7 @@ __global__ void __launch_bounds__(kThreads) bbox_kernel(FrameSet fs, DevState *s
     for (; i < n; i += step) {
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            float p = __ldg(pos + 3 * i + a);
+            float p = *(pos + 3 * i + a);
             mn[a] = fminf(mn[a], p);
             mx[a] = fmaxf(mx[a], p);
         }
@@ -90,6 +92,7 @@ __global__ void __launch_bounds__(kThreads) bbox_kernel(FrameSet fs, DevState *s
 
 __global__ void grid_kernel(FrameSet fs, DevState *st)
 {
+    if (after_previous()) return;
     uint32_t f = blockIdx.x * blockDim.x + threadIdx.x;
     if (f >= fs.F) return;
     FrameGrid g;
@@ -194,6 +197,7 @@ __device__ __forceinline__ uint32_t voxel_index(float p, const AxisGrid &g, uint
 // of 1M points 532 -> 524 us.
 __global__ void __launch_bounds__(kThreads) morton_kernel(FrameSet fs, uint64_t *keys, uint32_t *vals)
 {
+    if (after_previous()) return;
     const uint32_t f = blockIdx.y;
     const float *pos = fs.pos[f];
     const uint64_t base = fs.poff[f];
@@ -219,12 +223,12 @@ __global__ void __launch_bounds__(kThreads) morton_kernel(FrameSet fs, uint64_t 
 #pragma unroll
         for (int k = 0; k < 4; ++k)
 #pragma unroll
-            for (int a = 0; a < 3; ++a) p[k][a] = __ldg(pos + 3 * (i + k * step) + a);
+            for (int a = 0; a < 3; ++a) p[k][a] = *(pos + 3 * (i + k * step) + a);
 #pragma unroll
         for (int k = 0; k < 4; ++k) put(i + k * step, p[k]);
     }
     for (; i < n; i += step) {
-        const float p[3] = {__ldg(pos + 3 * i), __ldg(pos + 3 * i + 1), __ldg(pos + 3 * i + 2)};
+        const float p[3] = {*(pos + 3 * i), *(pos + 3 * i + 1), *(pos + 3 * i + 2)};
         put(i, p);
     }
 }
@@ -234,7 +238,7 @@ __global__ void __launch_bounds__(kThreads) morton_kernel(FrameSet fs, uint64_t 
 void launch_voxelize(const FrameSet &fs, DevState *st, uint64_t n_total, uint64_t n_max, uint64_t *keys,
                      uint32_t *vals, int num_sms, cudaStream_t s)
 {
-    init_bbox_kernel<<<1, 256, 0, s>>>(st, fs.F);
+    launch_after(init_bbox_kernel, 1, 256, 0, s, st, fs.F);
     count_launch();
     // X blocks per frame: enough for the largest frame, ~4 CTAs per SM overall
     uint64_t want = (n_max + kThreads - 1) / kThreads;
@@ -243,13 +247,13 @@ void launch_voxelize(const FrameSet &fs, DevState *st, uint64_t n_total, uint64_
     uint32_t X = (uint32_t)(want < 1 ? 1 : (want > cap ? cap : want));
     dim3 grid(X, fs.F);
     if (n_total > 0) {
-        bbox_kernel<<<grid, kThreads, 0, s>>>(fs, st);
+        launch_after(bbox_kernel, grid, kThreads, 0, s, fs, st);
         count_launch();
     }
-    grid_kernel<<<1, 64, 0, s>>>(fs, st);
+    launch_after(grid_kernel, 1, 64, 0, s, fs, st);
     count_launch();
     if (n_total > 0) {
-        morton_kernel<<<grid, kThreads, 0, s>>>(fs, keys, vals);
+        launch_after(morton_kernel, grid, kThreads, 0, s, fs, keys, vals);
         count_launch();
     }
 }
