@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(kThreads) prelude_finish_kernel(PreludeArgs a,
 
 // Passes launched grid-wide, the rest run in one CTA: a pass has about a 26th
 // of the tiles of the one before, so that with at most 64 tiles in the first
-// the later ones are one to three tiles, for which a launch (three in the
+// the later ones are one to three tiles, for which a launch (two in the
 // prelude) costs more than it saves.  10k Gaussians: encode 412 -> 390 us,
 // decode 347 -> 328 us.  Two wide passes up to 2000 tiles lost: the last kernel
 // then walks up to three tiles of 56 channels one by one (500k rows, two
