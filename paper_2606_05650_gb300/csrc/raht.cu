@@ -490,17 +490,18 @@ __global__ void __launch_bounds__(kThreads) prelude_finish_kernel(PreludeArgs a,
     }
 }
 
-// Passes launched grid-wide, the rest run in one CTA: a pass has about a 26th
-// of the tiles of the one before, so that with at most 64 tiles in the first
-// the later ones are one to three tiles, for which a launch (two in the
-// prelude) costs more than it saves.  10k Gaussians: encode 412 -> 390 us,
-// decode 347 -> 328 us.  Two wide passes up to 2000 tiles lost: the last kernel
-// then walks up to three tiles of 56 channels one by one (500k rows, two
-// forward and two inverse transforms: 375 -> 425 us).
+// Passes launched grid-wide, the rest run in one CTA: a pass has at most a
+// quarter of the tiles of the one before, mostly a twentieth, so that with at
+// most 64 tiles in the first the third is one tile, for which a launch (two in
+// the prelude) costs more than it saves.  10k Gaussians, wide passes one / two /
+// three: encode 300 / 291 / 300 us, decode 298 / 287 / 298 us.  Two wide passes
+// up to 2000 tiles lost: the last kernel then walks up to three tiles of 56
+// channels one by one (500k rows, two forward and two inverse transforms: 375
+// -> 425 us).
 int grid_passes(uint64_t nv_bound, uint32_t T)
 {
     const uint64_t tiles = (nv_bound + T - 1) / T;
-    return tiles <= 64 ? 1 : kRahtMultiPasses;
+    return tiles <= 64 ? 2 : kRahtMultiPasses;
 }
 
 // ----------------------------------------------------------- transform ---
