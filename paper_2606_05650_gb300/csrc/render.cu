@@ -30,12 +30,16 @@ constexpr int kTile = 16;
 
 struct Splat {
     float u, v;            // projected centre, rounded
-    uint32_t reach;        // pixels from the centre, in x and (upper half) in y, past which alpha stays below the cut
+    uint32_t reach;        // pixels from the centre, in x (upper half) and in y, past which alpha stays below the cut: the
+                           // upper halves of floats, rounded up, infinite where there is no such bound
     float opacity;
     float ulo, vlo;        // the centre's rest: u + ulo, v + vlo
     float l1, l2, l3;      // Cholesky factor of the conic
     float r, g, b;
 };
+
+// upper half of a float's bits, rounded up (x >= 0 or infinite)
+__device__ __forceinline__ uint32_t upper_half(float x) { return (__float_as_uint(x) + 0xFFFFu) >> 16; }
 
 // Double-float arithmetic (an unevaluated sum h + l of two floats, about 2^-46
 // relative; the error-free sums of Knuth and products of Dekker, by FMA).  An
@@ -282,7 +286,7 @@ __global__ void __launch_bounds__(256) preprocess_kernel(const float *pos,
         // margins cover the FP32 rounding of the per-pixel exponent, whose relative error grows with
         // cov_xx cov_yy / det (1e-7 sqrt(of it)): very elongated footprints keep the square of radius rad alone.
         double rx = rad, ry = rad;
-        float reach_x = 65535.f, reach_y = 65535.f;
+        float reach_x = INFINITY, reach_y = INFINITY;
         if (ca * cc < 1e8 * det) {
             if (opacity * 255.f < 0.9999f) continue;
             const float c = 2.04f * fmaxf(logf(opacity * 255.f), 0.f) + 0.1f;
@@ -315,7 +319,7 @@ __global__ void __launch_bounds__(256) preprocess_kernel(const float *pos,
         s.r = col[0];
         s.g = col[1];
         s.b = col[2];
-        s.reach = (uint32_t)fminf(ceilf(reach_x) + 1.f, 65535.f) | ((uint32_t)fminf(ceilf(reach_y) + 1.f, 65535.f) << 16);
+        s.reach = upper_half(ceilf(reach_x) + 1.f) << 16 | upper_half(ceilf(reach_y) + 1.f);
         sp[i] = s;
         depth[i] = __float_as_uint((float)z);  // positive: integer order = float order
         rect[i] = make_ushort4((unsigned short)tx0, (unsigned short)tx1, (unsigned short)ty0, (unsigned short)ty1);
@@ -428,8 +432,8 @@ __global__ void __launch_bounds__(32 * kWarpsPerCta) render_kernel(const uint2 *
     };
     auto stage = [&](uint32_t g, uint32_t val, uint4 head, Splat *to) {  // returns how many reach the block
         const bool hit = g < n && lane < n - g &&
-                         fabsf(__uint_as_float(head.x) - mx) <= (float)(head.z & 0xFFFFu) + 4.f &&
-                         fabsf(__uint_as_float(head.y) - my) <= (float)(head.z >> 16) + 2.f;
+                         fabsf(__uint_as_float(head.x) - mx) <= __uint_as_float(head.z & 0xFFFF0000u) + 4.f &&
+                         fabsf(__uint_as_float(head.y) - my) <= __uint_as_float(head.z << 16) + 2.f;
         const uint32_t m = __ballot_sync(0xFFFFFFFFu, hit);
         if (hit) {
             char *d = reinterpret_cast<char *>(to + __popc(m & ltmask));
