@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(256) preprocess_kernel(const float *pos,
         // cov_xx cov_yy / det (1e-7 sqrt(of it)): very elongated footprints keep the square of radius rad alone.
         double rx = rad, ry = rad;
         float reach_x = INFINITY, reach_y = INFINITY;
-        if (ca * cc < 1e8 * det) {
+        if (ca * cc < 1e8 * det && opacity >= 0.f) {  // a NaN opacity draws 0.99 wherever its tiles lie
             if (opacity * 255.f < 0.9999f) continue;
             const float c = 2.04f * fmaxf(logf(opacity * 255.f), 0.f) + 0.1f;
             reach_x = sqrtf(c * caf) * 1.0001f;
