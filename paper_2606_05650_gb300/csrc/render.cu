@@ -12,8 +12,8 @@
 //
 // Precision: everything per Gaussian (projection, covariance, conic, tile
 // rectangle, opacity, colour) is evaluated in FP64, or in double-float where
-// nothing cancels, and rounded once to FP32 for the per-pixel loop, which runs
-// in FP32.  The projected centre is kept as an unevaluated sum of two floats,
+// that certainly rounds to the same float, and rounded once to FP32 for the
+// per-pixel loop, which runs in FP32.  The projected centre is kept as an unevaluated sum of two floats,
 // so a pixel's offset from it is exact to FP32 rounding of the offset itself (a
 // single float would carry an absolute error of its ulp at hundreds of pixels).  The conic enters the
 // loop through its Cholesky factor, conic = L^T L with
@@ -45,12 +45,13 @@ __device__ __forceinline__ uint32_t upper_half(float x) { return (__float_as_uin
 // relative; the error-free sums of Knuth and products of Dekker, by FMA).  An
 // SM issues an FP64 warp instruction in 16 cycles and four FP32 ones a cycle,
 // and the projection was bound by its FP64 instructions (some 640 a Gaussian):
-// what stays in FP64 is what cancels or decides (camera coordinates,
-// covariance, determinant, footprint), some 190; viewing direction, colour,
-// scales and opacity are double-float and round to the same floats as the FP64
-// expressions but for about one in a million.  1M Gaussians at 960 x 540: this
-// kernel 334 us (381 with the direction in FP64), the whole call 2.86 -> 2.03 ms
-// when the rest was as before.
+// what is rounded to FP32 next, and is not the difference of nearly equal
+// numbers, is double-float (viewing direction, colour, opacity), evaluated in
+// FP64 after all where double-float cannot tell which float FP64 rounds to; the
+// rest stays in FP64 (camera coordinates, squared scales, covariance,
+// determinant, footprint), some 240.  1M Gaussians at 960 x 540: this kernel
+// 1,024 us all in FP64, 413 us now (332 us with the squared scales in
+// double-float too, which kept 46 of their 53 bits).
 struct Df {
     float h, l;
 };
@@ -83,6 +84,11 @@ __device__ __forceinline__ Df operator*(Df a, float b)
 {
     const float p = __fmul_rn(a.h, b);
     return df_quick(p, __fmaf_rn(a.l, b, __fmaf_rn(a.h, b, -p)));
+}
+// whether every number within err of h + l rounds to h (err counts some 2^-40 of h: its own rounding is nothing to it)
+__device__ __forceinline__ bool rounds_to_high(Df a, float err)
+{
+    return __fadd_rn(a.h, __fadd_rn(a.l, err)) == a.h && __fadd_rn(a.h, __fsub_rn(a.l, err)) == a.h;
 }
 __device__ __forceinline__ Df df_of(double x)
 {
@@ -118,31 +124,23 @@ __device__ __forceinline__ Df df_exp(float x, int &k)
     return s * r + Df{1.f, 0.f};
 }
 
-// e^(2 a) in FP64 from a float
-__device__ __forceinline__ double exp_twice(float a)
-{
-    if (!(fabsf(a) <= 40.f)) return exp(2.0 * (double)a);
-    int k;
-    const Df e = df_exp(2.f * a, k);
-    const double d = (double)e.h + (double)e.l;  // in [0.7, 1.42]: the exponent has room for k
-    return __hiloint2double(__double2hiint(d) + k * 0x100000, __double2loint(d));
-}
-
-// 1 / (1 + e^-a), rounded once
+// 1 / (1 + e^-a), rounded once: in double-float (within 2^-40) unless that is too near the middle of two floats to
+// tell, one in some 30,000
 __device__ __forceinline__ float sigmoid(float a)
 {
-    if (!(fabsf(a) <= 60.f)) return (float)(1.0 / (1.0 + exp(-(double)a)));
-    int k;
-    Df e = df_exp(-a, k);
-    const float sc = __int_as_float((127 + k) << 23);  // |k| <= 87
-    e = Df{1.f, 0.f} + Df{__fmul_rn(e.h, sc), __fmul_rn(e.l, sc)};
-    const float q = __frcp_rn(e.h);
-    const Df r = Df{1.f, 0.f} - e * q;  // 1 / e = q + q r + ...
-    return df_quick(q, __fmul_rn(q, r.h)).h;
+    if (fabsf(a) <= 60.f) {
+        int k;
+        Df e = df_exp(-a, k);
+        const float sc = __int_as_float((127 + k) << 23);  // |k| <= 87
+        e = Df{1.f, 0.f} + Df{__fmul_rn(e.h, sc), __fmul_rn(e.l, sc)};
+        const float q = __frcp_rn(e.h);
+        const Df r = Df{1.f, 0.f} - e * q;  // 1 / e = q + q r + ...
+        const Df s = df_quick(q, __fmul_rn(q, r.h));
+        if (rounds_to_high(s, __fmul_rn(s.h, 0x1p-40f))) return s.h;
+    }
+    return (float)(1.0 / (1.0 + exp(-(double)a)));
 }
 
-// degree-3 real SH basis at the unit direction (x, y, z), times the three
-// colours' coefficients (DC at a[8 + c], AC at a[11 + 15 c]), plus 0.5
 constexpr double kPi = 3.14159265358979323846;
 __host__ __device__ constexpr double csqrt_(double x)
 {
@@ -151,7 +149,11 @@ __host__ __device__ constexpr double csqrt_(double x)
     return r;
 }
 
-__device__ __forceinline__ void sh_colour(Df x, Df y, Df z, const float *a, float col[3])
+// Degree-3 real SH basis at the unit direction (x, y, z), times the three colours' coefficients (DC at a[8 + c], AC at
+// a[11 + 15 c]), plus 0.5, cut off below at 0.  False where a sum is too near the middle of two floats to be rounded, or
+// not finite: colour_f64.  The direction is within 41 2^-48, the basis functions are within 2^-41, a sum is within 2^-40
+// times 0.5 and its coefficients' magnitudes: one Gaussian in some 4,000.
+__device__ __forceinline__ bool sh_colour(Df x, Df y, Df z, const float *a, float col[3])
 {
     constexpr Df c0 = df_const(0.5 / csqrt_(kPi)), c1 = df_const(csqrt_(3.0 / (4.0 * kPi)));
     constexpr Df c2a = df_const(0.5 * csqrt_(15.0 / kPi)), c2b = df_const(0.25 * csqrt_(5.0 / kPi)),
@@ -162,14 +164,19 @@ __device__ __forceinline__ void sh_colour(Df x, Df y, Df z, const float *a, floa
     const Df xx = x * x, yy = y * y, zz = z * z, xy = x * y;
     const Df dm = xx - yy, dz = zz * 4.f - xx - yy;
     Df sum[3];
+    float mag[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) sum[c] = c0 * a[8 + c] + Df{0.5f, 0.f};
+    for (int c = 0; c < 3; ++c) {
+        sum[c] = c0 * a[8 + c] + Df{0.5f, 0.f};
+        mag[c] = 0.5f + fabsf(a[8 + c]);
+    }
     auto add = [&](int k, Df Y) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const float v = a[11 + 15 * c + (k - 1)], p = __fmul_rn(Y.h, v);
             const Df s = df_sum(sum[c].h, p);
             sum[c] = df_quick(s.h, __fadd_rn(__fadd_rn(s.l, sum[c].l), __fmaf_rn(Y.l, v, __fmaf_rn(Y.h, v, -p))));
+            mag[c] += fabsf(v);
         }
     };
     add(1, -(c1 * y));
@@ -187,8 +194,38 @@ __device__ __forceinline__ void sh_colour(Df x, Df y, Df z, const float *a, floa
     add(13, -(c3c * (x * dz)));
     add(14, c3e * (z * dm));
     add(15, -(c3a * (x * (xx - yy * 3.f))));
+    bool ok = true;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) col[c] = sum[c].h > 0.f ? sum[c].h : 0.f;
+    for (int c = 0; c < 3; ++c) {
+        ok = ok && rounds_to_high(sum[c], __fmul_rn(mag[c], 0x1p-40f));
+        col[c] = sum[c].h > 0.f ? sum[c].h : 0.f;
+    }
+    return ok;
+}
+
+// the same in FP64, from the Gaussian's position
+__device__ __noinline__ void colour_f64(const float *p, const float *a, double cam0, double cam1, double cam2,
+                                        float col[3])
+{
+    const double d[3] = {(double)p[0] - cam0, (double)p[1] - cam1, (double)p[2] - cam2};
+    const double dn = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]), id = dn > 0.0 ? 1.0 / dn : 1.0;
+    const double x = d[0] * id, y = d[1] * id, z = d[2] * id;
+    const double c0 = 0.5 / sqrt(kPi), c1 = sqrt(3.0 / (4.0 * kPi)), c2a = 0.5 * sqrt(15.0 / kPi),
+                 c2b = 0.25 * sqrt(5.0 / kPi), c2c = 0.25 * sqrt(15.0 / kPi), c3a = 0.25 * sqrt(35.0 / (2.0 * kPi)),
+                 c3b = 0.5 * sqrt(105.0 / kPi), c3c = 0.25 * sqrt(21.0 / (2.0 * kPi)), c3d = 0.25 * sqrt(7.0 / kPi),
+                 c3e = 0.25 * sqrt(105.0 / kPi);
+    const double Y[16] = {c0, -c1 * y, c1 * z, -c1 * x, c2a * x * y, -c2a * y * z, c2b * (2.0 * z * z - x * x - y * y),
+                          -c2a * x * z, c2c * (x * x - y * y), -c3a * y * (3.0 * x * x - y * y), c3b * x * y * z,
+                          -c3c * y * (4.0 * z * z - x * x - y * y), c3d * z * (2.0 * z * z - 3.0 * x * x - 3.0 * y * y),
+                          -c3c * x * (4.0 * z * z - x * x - y * y), c3e * z * (x * x - y * y),
+                          -c3a * x * (x * x - 3.0 * y * y)};
+    for (int c = 0; c < 3; ++c) {
+        double v = Y[0] * (double)a[8 + c];
+#pragma unroll
+        for (int k = 1; k < 16; ++k) v += Y[k] * (double)a[11 + 15 * c + (k - 1)];
+        v += 0.5;
+        col[c] = v > 0.0 ? (float)v : 0.f;
+    }
 }
 
 // (p - camera) / |p - camera|, the camera's position as a sum of three floats;
@@ -246,7 +283,7 @@ __global__ void __launch_bounds__(256) preprocess_kernel(const float *pos,
                      wy = sy * qw, wz = sz * qw;
         const double Rq[9] = {1 - (yy + zz), xy - wz, xz + wy, xy + wz, 1 - (xx + zz), yz - wx, xz - wy, yz + wx,
                               1 - (xx + yy)};
-        const double v2[3] = {exp_twice(a[0]), exp_twice(a[1]), exp_twice(a[2])};  // squared scales
+        const double v2[3] = {exp(2.0 * a[0]), exp(2.0 * a[1]), exp(2.0 * a[2])};  // squared scales
         // 2-D covariance N diag(v2) N^T, N = J W Rq
         const double iz = 1.0 / z, jx = cam.fx * iz, jy = cam.fy * iz;
         const double ux = jx * pc[0], vy = jy * pc[1], jxz = -ux * iz, jyz = -vy * iz;
@@ -315,7 +352,7 @@ __global__ void __launch_bounds__(256) preprocess_kernel(const float *pos,
         Df dir[3];
         view_direction(p, cam, dir);
         float col[3];
-        sh_colour(dir[0], dir[1], dir[2], a, col);
+        if (!sh_colour(dir[0], dir[1], dir[2], a, col)) colour_f64(p, a, cam.campos[0], cam.campos[1], cam.campos[2], col);
         s.r = col[0];
         s.g = col[1];
         s.b = col[2];
