@@ -2301,7 +2301,7 @@ static gsnfs_status encode_batch_impl(gsnfs_ctx *ctx, void *stream, uint32_t fra
         return GSNFS_ERR_INVALID_ARG;
     gsnfs_status st = check_quant(q);
     if (st) return st;
-    if ((uint64_t)rungs * q->num_channels > 1024) return GSNFS_ERR_UNSUPPORTED;  // rungs x channels threads per block
+    if ((uint64_t)rungs * q->num_channels > 1024) return GSNFS_ERR_UNSUPPORTED;  // streams of a row block
     for (uint32_t f = 0; f < frames; ++f) {
         if (h_J[f] < 1 || h_J[f] > 19) return GSNFS_ERR_INVALID_ARG;
         if (h_n[f] > 0 && !h_pos[f]) return GSNFS_ERR_INVALID_ARG;

@@ -18,6 +18,8 @@
 //            p == 0 -> KR -= 2 (floor 0); p > 1 -> KR += p + 1 (cap 384).
 //   Bits are packed least-significant first into 32-bit words; a block ends
 //   on a word boundary.  At most 78 bits per coefficient.
+#include <algorithm>
+
 #include "kernels.cuh"
 
 namespace gsnfs {
@@ -297,6 +299,7 @@ struct Rlgr {
 struct EncJobs {
     RlgrJob j;
     const uint64_t *job_off;  // F + 1: first job (row block) of each frame
+    uint32_t w0, ws;          // the launch codes streams w0 .. w0 + ws - 1 of each row block (kernels of a thread a stream)
 };
 
 constexpr uint32_t kPrefetch = 4;  // rows copied and coded at a time; even, for the rows are coded in pairs
@@ -378,13 +381,13 @@ __global__ void __launch_bounds__(PITCH, 1024 / PITCH) rlgr_encode_kernel(EncJob
     __shared__ __align__(16) EncTable tab;
     stage_table(&tab, &g_enc_table);
     const RlgrJob &j = E.j;
-    const uint32_t C = j.C, W = j.R * C;
+    const uint32_t C = j.C, W = E.ws;
     const uint32_t t = threadIdx.x;
     if (t < rb) blk_info[t] = enc_block(E, (uint64_t)blockIdx.x * rb + t);
     __syncthreads();
     // lanes past the last stream do that stream's work once more and write nothing
     const bool spare = t >= rb * W;
-    const uint32_t tt = spare ? rb * W - 1u : t, jl = tt / W, w = tt - jl * W;
+    const uint32_t tt = spare ? rb * W - 1u : t, jl = tt / W, w = E.w0 + tt - jl * W;
     const EncBlock me = blk_info[jl];
     const uint32_t r = w / C, c = w - r * C;
     const uint64_t blk = j.blk_off[me.f] + ((uint64_t)r * me.nb + me.b) * C + c;
@@ -529,14 +532,14 @@ __global__ void __launch_bounds__(512) rlgr_encode_few_kernel(EncJobs E, uint32_
     if (after_previous()) return;
     __shared__ EncBlock blk_info[32];
     const RlgrJob &j = E.j;
-    const uint32_t C = j.C, W = j.R * C, t = threadIdx.x;
+    const uint32_t C = j.C, W = E.ws, t = threadIdx.x;
     if (t < rb) blk_info[t] = enc_block(E, (uint64_t)blockIdx.x * rb + t);
     __syncthreads();
     const uint32_t jl = t / W;
     if (jl >= rb) return;
     const EncBlock me = blk_info[jl];
     if (me.len == 0) return;
-    const uint32_t w = t - jl * W, r = w / C, c = w - r * C;
+    const uint32_t w = E.w0 + t - jl * W, r = w / C, c = w - r * C;
     const uint64_t blk = j.blk_off[me.f] + ((uint64_t)r * me.nb + me.b) * C + c;
     BitWriter bw(j.slots + blk * j.slot_words, j.slot_words);
     RlgrFew st{0, 32, 0u};
@@ -1089,13 +1092,26 @@ size_t ring_smem(Kernel k, size_t bytes)
 
 }  // namespace
 
-template <bool FROM_INT, bool DIST>
-static void launch_encode(const EncJobs &E, const int32_t *q, uint32_t rb, uint32_t threads, uint64_t jobs, cudaStream_t s)
+// launch(E, row blocks per CTA, CTAs, threads) for each slice of at most 512 of a row block's W streams
+template <typename Launch>
+static void launch_slices(EncJobs E, uint32_t W, uint64_t jobs, Launch launch)
 {
-    const uint32_t grid = (uint32_t)((jobs + rb - 1) / rb);
-    auto k = threads <= 256 ? rlgr_encode_kernel<FROM_INT, DIST, 256> : rlgr_encode_kernel<FROM_INT, DIST, 512>;
-    launch_after(k, grid, threads, ring_smem(k, 4 * (size_t)kRing * (threads <= 256 ? 256 : 512)), s, E, q, rb);
-    count_launch();
+    const uint32_t slices = (W + 511) / 512, most = (W + slices - 1) / slices;
+    for (E.w0 = 0; E.w0 < W; E.w0 += most) {
+        E.ws = std::min(most, W - E.w0);
+        const uint32_t rb = row_blocks_per_cta(E.ws);
+        launch(E, rb, (uint32_t)((jobs + rb - 1) / rb), (rb * E.ws + 31) / 32 * 32);
+        count_launch();
+    }
+}
+
+template <bool FROM_INT, bool DIST>
+static void launch_encode(const EncJobs &E, const int32_t *q, uint32_t W, uint64_t jobs, cudaStream_t s)
+{
+    launch_slices(E, W, jobs, [&](const EncJobs &S, uint32_t rb, uint32_t grid, uint32_t threads) {
+        auto k = threads <= 256 ? rlgr_encode_kernel<FROM_INT, DIST, 256> : rlgr_encode_kernel<FROM_INT, DIST, 512>;
+        launch_after(k, grid, threads, ring_smem(k, 4 * (size_t)kRing * (threads <= 256 ? 256 : 512)), s, S, q, rb);
+    });
 }
 
 // A slot holds 16 bits per coefficient on average (ample for quantised
@@ -1115,24 +1131,20 @@ void launch_rlgr_offsets(const uint32_t *vstart, uint32_t F, uint32_t B, uint32_
 void launch_rlgr_encode(const RlgrJob &j, const uint64_t *job_off, uint64_t jobs_bound, cudaStream_t s)
 {
     if (jobs_bound == 0 || j.C == 0) return;
-    EncJobs E{j, job_off};
     const uint32_t W = j.R * j.C;
-    const uint32_t rb = row_blocks_per_cta(W);
-    const uint32_t threads = (rb * W + 31) / 32 * 32;
-    if (!j.sq_err && W <= 512 && jobs_bound * W <= kSplitStreams) {
+    const EncJobs E{j, job_off, 0, W};
+    if (!j.sq_err && jobs_bound * W <= kSplitStreams) {
         launch_after(rlgr_encode_split_kernel, (uint32_t)((jobs_bound * W + kSplitG - 1) / kSplitG), kSplitThreads, 0, s, E);
         count_launch();
-        return;
+    } else if (!j.sq_err && jobs_bound * W <= kFewStreams) {
+        launch_slices(E, W, jobs_bound, [&](const EncJobs &S, uint32_t rb, uint32_t grid, uint32_t threads) {
+            launch_after(rlgr_encode_few_kernel, grid, threads, 0, s, S, rb);
+        });
+    } else if (j.sq_err) {
+        launch_encode<false, true>(E, nullptr, W, jobs_bound, s);
+    } else {
+        launch_encode<false, false>(E, nullptr, W, jobs_bound, s);
     }
-    if (!j.sq_err && jobs_bound * W <= kFewStreams) {
-        launch_after(rlgr_encode_few_kernel, (uint32_t)((jobs_bound + rb - 1) / rb), threads, 0, s, E, rb);
-        count_launch();
-        return;
-    }
-    if (j.sq_err)
-        launch_encode<false, true>(E, nullptr, rb, threads, jobs_bound, s);
-    else
-        launch_encode<false, false>(E, nullptr, rb, threads, jobs_bound, s);
 }
 
 void launch_rlgr_encode_indices(const int32_t *q, const uint32_t *vstart, uint32_t C, uint32_t B, uint32_t *slots,
@@ -1151,10 +1163,7 @@ void launch_rlgr_encode_indices(const int32_t *q, const uint32_t *vstart, uint32
     j.blk_off = blk_off;
     j.slot_words = slot_words;
     j.overflow = overflow;
-    EncJobs E{j, job_off};
-    const uint32_t rb = row_blocks_per_cta(C);
-    const uint32_t threads = (rb * C + 31) / 32 * 32;
-    launch_encode<true, false>(E, q, rb, threads, jobs_bound, s);
+    launch_encode<true, false>(EncJobs{j, job_off, 0, C}, q, C, jobs_bound, s);
 }
 
 // Threads per CTA: a CTA has a copy of the table (32 KB) beside 64 bytes a thread, and many streams are bound by the
