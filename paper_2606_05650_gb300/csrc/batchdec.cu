@@ -500,7 +500,7 @@ void launch_batch_rans_decode(const DecFrame *fr, uint32_t F, uint32_t max_chunk
     launch_after(tables_kernel, F, 1024, 0, s, fr, tabs, tab_words, cstart, st);
     count_launch();
     const size_t smem = (size_t)ransdec::kTabWords * 4;
-    cudaFuncSetAttribute(rans_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_shared<rans_batch_kernel>();
     const uint32_t X = (max_chunks_per_frame + kRansWarps - 1) / kRansWarps;
     launch_after(rans_batch_kernel, dim3(X, F), 32 * kRansWarps, smem, s, fr, tabs, tab_words, cstart, occ_all, st);
     count_launch();

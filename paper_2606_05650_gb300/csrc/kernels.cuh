@@ -45,6 +45,23 @@ void launch_after(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStrea
     cudaLaunchKernelEx(&c, k, static_cast<P>(args)...);
 }
 
+// Opts a kernel in to all the dynamic shared memory that a CTA can have beside its static arrays.  The limit is the
+// kernel's, shared by every thread of the process: set to each call's own size it would be lowered by a smaller call of
+// another thread (another context) between that and the launch.
+template <auto Kernel>
+void allow_shared()
+{
+    static const int room = [] {
+        int dev = 0, most = 0;
+        cudaFuncAttributes a{};
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        cudaFuncGetAttributes(&a, Kernel);
+        return most - (int)a.sharedSizeBytes;
+    }();
+    cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, room);
+}
+
 // Optional per-stage timing with CUDA events on the launching stream.
 enum StageId {
     kStVoxelize, kStSort, kStDedup, kStOccupancy, kStRans, kStPrelude, kStRahtFwd, kStRahtFwd0, kStRlgrEnc,

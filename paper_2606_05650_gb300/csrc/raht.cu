@@ -1606,12 +1606,12 @@ int pipe_depth(const XformArgs<S> &A, size_t *smem)
     return *smem <= (size_t)max_optin_smem() ? nr : 0;
 }
 
-template <typename Kernel>
-uint32_t one_wave(Kernel k, int threads, uint64_t tiles, size_t smem, int num_sms)  // and the kernel's opt-in
+template <auto Kernel>
+uint32_t one_wave(int threads, uint64_t tiles, size_t smem, int num_sms)  // and the kernel's opt-in
 {
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_shared<Kernel>();
     int per_sm = 0;  // resident CTAs per SM with this shared memory
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem) != cudaSuccess || per_sm < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, Kernel, threads, smem) != cudaSuccess || per_sm < 1)
         per_sm = 1;
     const uint64_t cap = (uint64_t)num_sms * (uint64_t)per_sm;
     return (uint32_t)(tiles < 1 ? 1 : (tiles < cap ? tiles : cap));
@@ -1625,12 +1625,12 @@ void launch_first(const XformArgs<float> &A, uint64_t tiles, size_t smem, int nu
     while (2 * pow2 <= slots) pow2 *= 2;
     if (pow2 * L >= 384) slots = pow2;  // whole sweeps over a tile's rows
     if (slots * L <= 448) {
-        auto k = xform_first_kernel<INV, GATHER, QDQ, COLOR, 448>;
-        const uint32_t grid = one_wave(k, 448, tiles, smem, num_sms);
+        constexpr auto k = xform_first_kernel<INV, GATHER, QDQ, COLOR, 448>;
+        const uint32_t grid = one_wave<k>(448, tiles, smem, num_sms);
         launch_after(k, grid, 448, smem, s, A, slots);
     } else {
-        auto k = xform_first_kernel<INV, GATHER, QDQ, COLOR, 512>;
-        const uint32_t grid = one_wave(k, 512, tiles, smem, num_sms);
+        constexpr auto k = xform_first_kernel<INV, GATHER, QDQ, COLOR, 512>;
+        const uint32_t grid = one_wave<k>(512, tiles, smem, num_sms);
         launch_after(k, grid, 512, smem, s, A, slots);
     }
     count_launch();
@@ -1641,8 +1641,8 @@ void launch_pipe_nr(int nr, const XformArgs<float> &A, uint64_t nv_bound, size_t
 {
     const uint64_t tiles = (nv_bound + A.p.T - 1) / A.p.T;
     if (nr == 3) {
-        auto k = xform_pipe_kernel<3, INV, GATHER, QDQ>;
-        const uint32_t grid = one_wave(k, kXThreads, tiles, smem, num_sms);
+        constexpr auto k = xform_pipe_kernel<3, INV, GATHER, QDQ>;
+        const uint32_t grid = one_wave<k>(kXThreads, tiles, smem, num_sms);
         k<<<grid, kXThreads, smem, s>>>(A);
         count_launch();
     } else if (A.io.klt && (INV || GATHER)) {
@@ -1670,8 +1670,8 @@ size_t xform_smem(uint32_t T, uint32_t Cg, bool color)
 template <typename S, bool INV, int VEC, bool GATHER, bool QDQ>
 void launch_pass(const XformArgs<S> &A, int q, uint32_t grid, size_t smem, cudaStream_t s)
 {
-    auto k = xform_pass_kernel<S, INV, VEC, GATHER, QDQ>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    constexpr auto k = xform_pass_kernel<S, INV, VEC, GATHER, QDQ>;
+    allow_shared<k>();
     launch_after(k, grid, kXThreads, smem, s, A, q);
     count_launch();
 }
@@ -1679,8 +1679,8 @@ void launch_pass(const XformArgs<S> &A, int q, uint32_t grid, size_t smem, cudaS
 template <typename S, bool INV, int VEC, bool QDQ>
 void launch_finish(const XformArgs<S> &A, int q0, size_t smem, cudaStream_t s)
 {
-    auto k = xform_finish_kernel<S, INV, VEC, QDQ>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    constexpr auto k = xform_finish_kernel<S, INV, VEC, QDQ>;
+    allow_shared<k>();
     launch_after(k, 1, kXThreads, smem, s, A, q0);
     count_launch();
 }
@@ -1789,7 +1789,7 @@ template <int TMAX, bool WARP>
 void prelude_tiles(const PreludeArgs &a, int q, uint32_t grid, cudaStream_t s)
 {
     const size_t smem = prelude_smem_bytes<TMAX, WARP>();
-    cudaFuncSetAttribute(prelude_tiles_kernel<TMAX, WARP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_shared<prelude_tiles_kernel<TMAX, WARP>>();
     launch_after(prelude_tiles_kernel<TMAX, WARP>, grid, kThreads, smem, s, a, q);
     count_launch();
 }
@@ -1799,7 +1799,7 @@ void prelude_launches(const PreludeArgs &a, const RahtPlanDev &p, const DevState
                       uint64_t nv_bound, int num_sms, cudaStream_t s)
 {
     const size_t smem = prelude_smem_bytes<TMAX, kWarpTiles<TMAX>>();
-    cudaFuncSetAttribute(prelude_finish_kernel<TMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_shared<prelude_finish_kernel<TMAX>>();
     launch_after(prelude_init_kernel, 1, 32, 0, s, p, st, nv_dev);
     count_launch();
     const uint32_t grid = (uint32_t)num_sms * (p.pgrid_mult ? p.pgrid_mult : 8u);

@@ -357,7 +357,7 @@ void launch_rans_decode(const uint8_t *sec, uint64_t sec_bytes, uint64_t n, uint
     uint32_t blocks = (nch + warps - 1) / warps;
     if (blocks > (uint32_t)num_sms * 4) blocks = (uint32_t)num_sms * 4;
     const size_t smem = (size_t)ransdec::kTabWords * 4 + 4 * (size_t)kSmemChunks;
-    cudaFuncSetAttribute(decode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_shared<decode_kernel>();
     launch_after(decode_kernel, blocks, 32 * warps, smem, s, sec, sec_bytes, n, nch, chunk, out, st);
     count_launch();
 }

@@ -1082,14 +1082,6 @@ __global__ void __launch_bounds__(kMaxFrames) job_offsets_kernel(const uint32_t 
     }
 }
 
-// dynamic shared memory of a kernel's rings (beside its table it may pass the 48 KB that need no opt-in)
-template <typename Kernel>
-size_t ring_smem(Kernel k, size_t bytes)
-{
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    return bytes;
-}
-
 }  // namespace
 
 // launch(E, row blocks per CTA, CTAs, threads) for each slice of at most 512 of a row block's W streams
@@ -1109,8 +1101,13 @@ template <bool FROM_INT, bool DIST>
 static void launch_encode(const EncJobs &E, const int32_t *q, uint32_t W, uint64_t jobs, cudaStream_t s)
 {
     launch_slices(E, W, jobs, [&](const EncJobs &S, uint32_t rb, uint32_t grid, uint32_t threads) {
-        auto k = threads <= 256 ? rlgr_encode_kernel<FROM_INT, DIST, 256> : rlgr_encode_kernel<FROM_INT, DIST, 512>;
-        launch_after(k, grid, threads, ring_smem(k, 4 * (size_t)kRing * (threads <= 256 ? 256 : 512)), s, S, q, rb);
+        if (threads <= 256) {
+            allow_shared<rlgr_encode_kernel<FROM_INT, DIST, 256>>();
+            launch_after(rlgr_encode_kernel<FROM_INT, DIST, 256>, grid, threads, 4 * (size_t)kRing * 256, s, S, q, rb);
+        } else {
+            allow_shared<rlgr_encode_kernel<FROM_INT, DIST, 512>>();
+            launch_after(rlgr_encode_kernel<FROM_INT, DIST, 512>, grid, threads, 4 * (size_t)kRing * 512, s, S, q, rb);
+        }
     });
 }
 
@@ -1170,11 +1167,12 @@ void launch_rlgr_encode_indices(const int32_t *q, const uint32_t *vstart, uint32
 // integer pipe once 32 warps are resident: 16 x 1M frames, beside the same geometry kernels, 2.14 ms with 224 threads
 // (28 warps), 1.83 with 512 (32), 1.74 with 640 (40), which slows the geometry, the longer branch, by more.  Streams
 // that do not fill every SM twice that way take smaller CTAs, for the sake of all SMs.
-template <typename Kernel, typename Launch>
-static void launch_decode(Kernel k, uint64_t streams, Launch launch)
+template <auto Kernel, typename... A>
+static void launch_decode(uint64_t streams, cudaStream_t s, A... args)
 {
     const uint32_t threads = streams < 152 * 2 * kDecThreads ? kDecSmall : kDecThreads;
-    launch(k, (uint32_t)((streams + threads - 1) / threads), threads, ring_smem(k, 4 * (size_t)kRingWords * threads));
+    allow_shared<Kernel>();
+    launch_after(Kernel, (uint32_t)((streams + threads - 1) / threads), threads, 4 * (size_t)kRingWords * threads, s, args...);
     count_launch();
 }
 
@@ -1183,10 +1181,8 @@ void launch_rlgr_decode(const uint32_t *payload, uint64_t payload_words, const u
                         DevState *st, cudaStream_t s)
 {
     if (nv == 0 || C == 0) return;
-    launch_decode(rlgr_decode_kernel<false>, (nv + B - 1) / B * C, [&](auto k, uint32_t grid, uint32_t threads, size_t smem) {
-        launch_after(k, grid, threads, smem, s, payload, payload_words, block_words, block_off, 0u, (uint32_t)nv, C, B, step, Y,
-                                      nullptr, st);
-    });
+    launch_decode<rlgr_decode_kernel<false>>((nv + B - 1) / B * C, s, payload, payload_words, block_words, block_off, 0u,
+                                             (uint32_t)nv, C, B, step, Y, nullptr, st);
 }
 
 void launch_rlgr_decode_batch(const DecFrame *fr, uint32_t F, const uint64_t *job_off, uint64_t jobs_bound,
@@ -1194,19 +1190,15 @@ void launch_rlgr_decode_batch(const DecFrame *fr, uint32_t F, const uint64_t *jo
                               float *Y, DevState *st, cudaStream_t s)
 {
     if (jobs_bound == 0 || C == 0) return;
-    launch_decode(rlgr_decode_batch_kernel, jobs_bound * C, [&](auto k, uint32_t grid, uint32_t threads, size_t smem) {
-        launch_after(k, grid, threads, smem, s, fr, F, job_off, bw_all, boff_all, steps_all, C, Y, st);
-    });
+    launch_decode<rlgr_decode_batch_kernel>(jobs_bound * C, s, fr, F, job_off, bw_all, boff_all, steps_all, C, Y, st);
 }
 
 void launch_rlgr_decode_indices(const uint32_t *words, uint64_t total_words, const uint32_t *bw, uint32_t stride,
                                 uint64_t nv, uint32_t C, uint32_t B, int32_t *q, DevState *st, cudaStream_t s)
 {
     if (nv == 0 || C == 0) return;
-    launch_decode(rlgr_decode_kernel<true>, (nv + B - 1) / B * C, [&](auto k, uint32_t grid, uint32_t threads, size_t smem) {
-        launch_after(k, grid, threads, smem, s, words, total_words, bw, nullptr, stride, (uint32_t)nv, C, B, nullptr, nullptr, q,
-                                      st);
-    });
+    launch_decode<rlgr_decode_kernel<true>>((nv + B - 1) / B * C, s, words, total_words, bw, nullptr, stride, (uint32_t)nv, C, B,
+                                            nullptr, nullptr, q, st);
 }
 
 }  // namespace gsnfs

@@ -370,7 +370,7 @@ template <typename Key>
 void small_sort(const Key *keys, const uint32_t *vals, Key *keys_out, uint32_t *vals_out, uint32_t n, uint32_t nbits,
                 cudaStream_t s)
 {
-    cudaFuncSetAttribute(small_sort_kernel<Key>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallSmem<Key>));
+    allow_shared<small_sort_kernel<Key>>();
     launch_after(small_sort_kernel<Key>, 1, kSmallThreads, sizeof(SmallSmem<Key>), s, 
         keys, vals, n, nbits, digit_width(nbits), (n + kSmallThreads - 1) / kSmallThreads, keys_out, vals_out);
     count_launch();
@@ -408,7 +408,7 @@ static void launch_down(const Key *keys, const uint32_t *vals, uint64_t n, uint3
                         const uint32_t *cta_seg, uint32_t P, cudaStream_t s)
 {
     constexpr size_t smem = sizeof(DownSmem<Key, Cfg>);
-    cudaFuncSetAttribute(downsweep_kernel<Key, Cfg>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_shared<downsweep_kernel<Key, Cfg>>();
     launch_after(downsweep_kernel<Key, Cfg>, P, Cfg::threads, smem, s, keys, vals, n, shift, mask, chunk, hist, keys_out, vals_out,
                                                              cta_lo, cta_seg);
     count_launch();
