@@ -168,18 +168,26 @@ __global__ void __launch_bounds__(32 * kH) occ_scan_kernel(uint32_t *partials, u
     __shared__ uint32_t tot[kH];
     const uint32_t f = blockIdx.x, lane = threadIdx.x & 31, h = threadIdx.x >> 5;
     uint32_t *row = partials + ((uint64_t)f * kH + h) * X;
-    // a contiguous run of counts per lane: all its loads in flight, one warp scan, then its prefixes
-    const uint32_t per = (X + 31) / 32, b0 = min(lane * per, X), b1 = min(b0 + per, X);
-    uint32_t sum = 0;
-#pragma unroll 8
-    for (uint32_t x = b0; x < b1; ++x) sum += row[x];
-    const uint32_t inc = warp_inclusive_sum(sum), run = __shfl_sync(0xFFFFFFFFu, inc, 31);
-    uint32_t pre = inc - sum;
-#pragma unroll 8
-    for (uint32_t x = b0; x < b1; ++x) {
-        const uint32_t v = __ldcg(row + x);
-        row[x] = pre;
-        pre += v;
+    // 256 counts at a time, eight consecutive ones per lane: all loads of a turn in flight, one warp scan, then the stores.
+    // (With a lane's whole run at once, its second reading of a count waited for the store before it: 1M voxels, 1,216
+    // counts a height, this kernel and its wait for the one before 34 -> 12 us, octree encoding of their codes 203 -> 176.)
+    uint32_t run = 0;
+    for (uint32_t b = 0; b < X; b += 256) {
+        const uint32_t x0 = b + 8 * lane;
+        uint32_t v[8], sum = 0;
+#pragma unroll
+        for (uint32_t k = 0; k < 8; ++k) {
+            v[k] = x0 + k < X ? row[x0 + k] : 0u;
+            sum += v[k];
+        }
+        const uint32_t inc = warp_inclusive_sum(sum);
+        uint32_t pre = run + inc - sum;
+#pragma unroll
+        for (uint32_t k = 0; k < 8; ++k) {
+            if (x0 + k < X) row[x0 + k] = pre;
+            pre += v[k];
+        }
+        run += __shfl_sync(0xFFFFFFFFu, inc, 31);
     }
     if (lane == 0) tot[h] = run;
     __syncthreads();
