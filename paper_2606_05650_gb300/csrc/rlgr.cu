@@ -213,10 +213,38 @@ __device__ __forceinline__ uint32_t column_i32(int32_t q)
     return kColBias + 2u * min(m, kEncMax) + (q < 0 ? 1u : 0u);
 }
 
-// RLGR coder of one block.
-struct Rlgr {
+// RLGR state of one block; code() takes any symbol, by its zigzag index, each lane on its own path.
+struct RlgrState {
     int K, KR;
-    uint32_t z;    // pending zeros of an open run
+    uint32_t z;  // pending zeros of an open run
+    __device__ __forceinline__ void code(BitWriter &bw, uint32_t u)
+    {
+        const uint32_t k = (uint32_t)K >> 4;
+        if (__builtin_expect(k == 0, 1)) {  // Golomb-Rice mode
+            gr_put(bw, u, (uint32_t)KR >> 4, KR);
+            K = max(K + (u == 0 ? 3 : -3), 0);
+        } else if (u == 0) {
+            if (++z == (1u << k)) {
+                bw.put(0, 1);
+                K = min(K + 4, 240);
+                z = 0;
+            }
+        } else {
+            bw.put(1u | (z << 1), 1u + k);  // bit 1, then the run length in k bits (z < 2^k, k <= 15)
+            gr_put(bw, u - 1u, (uint32_t)KR >> 4, KR);
+            K = max(K - 6, 0);
+            z = 0;
+        }
+    }
+    __device__ __forceinline__ void finish(BitWriter &bw)
+    {
+        if (z) bw.put(0, 1);
+        bw.flush();
+    }
+};
+
+// RLGR coder of one block by table.
+struct Rlgr : RlgrState {
     uint32_t tab;  // shared-memory address of the table, less the bias of its columns
     __device__ __forceinline__ void init(const EncTable &t)
     {
@@ -229,10 +257,13 @@ struct Rlgr {
     {
         return __viaddmin_s32_relu(kr, signed_byte<2>(e), 384);
     }
+    // Parameters at which so many symbols lie past the table that a warp is better off without it (deviations of some
+    // 50 steps; 100k rows of 45 / 60 steps, with the line 8 lower: 95 / 100 us, here 71 / 95).
+    __device__ __forceinline__ bool large() const { return KR >= 16 * (int)kEncRows - 16; }
     // Two symbols in Golomb-Rice mode (K < 16: no cap at 240), appended by one write; false, with nothing changed,
     // when the table does not hold one of the codewords.  Wants ready(): the first symbol raises K by 3 and KR by 16
     // at most, which leaves the second in Golomb-Rice mode and in the table's rows.
-    __device__ __forceinline__ bool ready() const { return K < 13 && KR < 16 * (int)kEncRows - 16; }
+    __device__ __forceinline__ bool ready() const { return K < 13 && !large(); }
     __device__ __forceinline__ bool pair(BitWriter &bw, uint32_t a, uint32_t b)
     {
         const uint32_t e0 = table_load((uint32_t)(KR & 0x1F0) * (kEncCols / 4) + tab + 4u * a);
@@ -263,28 +294,6 @@ struct Rlgr {
         z = more && !full ? z1 : 0u;
         bw.put(more ? 0u : c, more ? full : n);
         return true;
-    }
-    // any symbol, by its zigzag index
-    __device__ __forceinline__ void any(BitWriter &bw, uint32_t u)
-    {
-        const uint32_t k = (uint32_t)K >> 4;
-        if (k != 0 && u == 0) {
-            if (++z == (1u << k)) {
-                bw.put(0, 1);
-                K = min(K + 4, 240);
-                z = 0;
-            }
-            return;
-        }
-        if (k != 0) bw.put(1u | (z << 1), 1u + k);
-        gr_put(bw, k ? u - 1u : u, (uint32_t)KR >> 4, KR);
-        K = max(k ? K - 6 : K + (u == 0 ? 3 : -3), 0);
-        z = 0;
-    }
-    __device__ __forceinline__ void finish(BitWriter &bw)
-    {
-        if (z) bw.put(0, 1);
-        bw.flush();
     }
 };
 
@@ -405,7 +414,7 @@ __global__ void __launch_bounds__(PITCH, 1024 / PITCH) rlgr_encode_kernel(EncJob
     if (!FROM_INT && j.dc && me.b == 0 && me.len) {  // the frame's DC: quantised from its FP64 value
         const double y = j.dc[(uint64_t)me.f * C + c], st64 = j.steps_rg[r * j.G + j.groups[c]];
         const int32_t q = quantize_f64(y, st64, j.tau64);
-        st.any(bw, zz(q));
+        st.code(bw, zz(q));
         if (DIST) {
             const double e = __dsub_rn(y, __dmul_rn((double)q, st64));
             dc_err = __dmul_rn(e, e);
@@ -450,18 +459,22 @@ __global__ void __launch_bounds__(PITCH, 1024 / PITCH) rlgr_encode_kernel(EncJob
         const uint32_t x[kPrefetch] = {ring_load<0>(from), ring_load<kRow>(from), ring_load<2 * kRow>(from),
                                        ring_load<3 * kRow>(from)};
         copy_group();  // over the group before this one
+        // One lane whose parameter is large takes its warp through the general path, one in run mode (or near it)
+        // through the path for either mode; what the table does not hold is left to the general path too, by each lane.
+        // (With the table tried again for every such symbol, a warp of large coefficients went through all the paths:
+        // 100k rows of 56 channels of 120 steps 201 us, now 95; 1M rows of 100 steps 416 -> 221; a frame of 250k
+        // Gaussians at the base steps 78 -> 57, the 8 x 5 ladder 1.78 -> 1.69 ms.)
+        const bool large = __any_sync(0xFFFFFFFFu, live && st.large());
 #pragma unroll
         for (uint32_t d = 0; d < kPrefetch; d += 2) {
-            // one lane in run mode (or near it) takes its warp through the path for either mode
             bool done = __all_sync(0xFFFFFFFFu, !live || st.ready());
             if (!live) continue;
             const uint32_t a = column_of(x[d]), b = column_of(x[d + 1]);
             if (done) done = st.pair(bw, a, b);
             if (!done) {
-                uint32_t h = st.one(bw, a) ? (st.one(bw, b) ? 2u : 1u) : 0u;
-#pragma unroll 1
-                for (; h < 2u; ++h)  // what the table does not hold: rare
-                    if (!st.one(bw, h ? b : a)) st.any(bw, index_of(h ? x[d + 1] : x[d]));
+                const uint32_t coded = large ? 0u : st.one(bw, a) ? (st.one(bw, b) ? 2u : 1u) : 0u;
+                if (coded == 0u) st.code(bw, index_of(x[d]));
+                if (coded != 2u) st.code(bw, index_of(x[d + 1]));
             }
             if (DIST) {
                 distort(x[d]);
@@ -482,7 +495,7 @@ __global__ void __launch_bounds__(PITCH, 1024 / PITCH) rlgr_encode_kernel(EncJob
 #pragma unroll 1
         for (uint32_t d = 0; i < len; ++i, ++d) {
             const uint32_t y = d == 0 ? x[0] : (d == 1 ? x[1] : x[2]);
-            if (!st.one(bw, column_of(y))) st.any(bw, index_of(y));
+            if (!st.one(bw, column_of(y))) st.code(bw, index_of(y));
             if (DIST) distort(y);
         }
     }
@@ -503,30 +516,6 @@ __global__ void __launch_bounds__(PITCH, 1024 / PITCH) rlgr_encode_kernel(EncJob
 // (Fewer streams than kSplitStreams take the kernel after this one.)
 constexpr uint64_t kFewStreams = 20000;
 
-struct RlgrFew {
-    int K, KR;
-    uint32_t z;  // pending zeros of an open run
-    __device__ __forceinline__ void code(BitWriter &bw, uint32_t u)
-    {
-        const uint32_t k = (uint32_t)K >> 4;
-        if (__builtin_expect(k == 0, 1)) {  // Golomb-Rice mode
-            gr_put(bw, u, (uint32_t)KR >> 4, KR);
-            K = max(K + (u == 0 ? 3 : -3), 0);
-        } else if (u == 0) {
-            if (++z == (1u << k)) {
-                bw.put(0, 1);
-                K = min(K + 4, 240);
-                z = 0;
-            }
-        } else {
-            bw.put(1u | (z << 1), 1u + k);  // bit 1, then the run length in k bits (z < 2^k, k <= 15)
-            gr_put(bw, u - 1u, (uint32_t)KR >> 4, KR);
-            K = max(K - 6, 0);
-            z = 0;
-        }
-    }
-};
-
 __global__ void __launch_bounds__(512) rlgr_encode_few_kernel(EncJobs E, uint32_t rb)
 {
     if (after_previous()) return;
@@ -542,7 +531,7 @@ __global__ void __launch_bounds__(512) rlgr_encode_few_kernel(EncJobs E, uint32_
     const uint32_t w = E.w0 + t - jl * W, r = w / C, c = w - r * C;
     const uint64_t blk = j.blk_off[me.f] + ((uint64_t)r * me.nb + me.b) * C + c;
     BitWriter bw(j.slots + blk * j.slot_words, j.slot_words);
-    RlgrFew st{0, 32, 0u};
+    RlgrState st{0, 32, 0u};
     const float inv = j.inv_step[r * C + c], tau = j.tau;
     const float *col = j.Y + me.gbase + c;  // row i of this channel at col[i * C]
     const uint32_t len = me.len;
@@ -567,8 +556,7 @@ __global__ void __launch_bounds__(512) rlgr_encode_few_kernel(EncJobs E, uint32_
 #pragma unroll
     for (uint32_t d = 0; d < kPrefetch; ++d)
         if (i + d < len) st.code(bw, quantize_zz_f32(cur[d], inv, tau));
-    if (st.z) bw.put(0, 1);
-    bw.flush();
+    st.finish(bw);
     j.block_words[blk] = bw.nw;
     if (bw.nw > j.slot_words) atomicExch(j.overflow, 1u);
 }
