@@ -1610,7 +1610,7 @@ gsnfs_status decode_impl(gsnfs_ctx *ctx, cudaStream_t s, const uint8_t *d_in, ui
         const uint64_t payload_words = (P.attr_bytes - 8 - 4 * nblk) / 4;
         launch_scan_u32_to_u64(bw, nblk, L.block_off, L.spart, sms, s);
         stage_begin(s, kStRlgrDec);
-        launch_rlgr_decode(payload, payload_words, bw, L.block_off, P.nv, P.C, P.B, L.step, L.Y, dst, s);
+        launch_rlgr_decode(payload, payload_words, bw, L.block_off, P.nv, P.C, P.B, L.step, L.Y, dst, sms, s);
         stage_end(s, kStRlgrDec);
     }
     // a11: occupancy bytes
@@ -1976,7 +1976,7 @@ gsnfs_status decode_batch_impl(gsnfs_ctx *ctx, cudaStream_t s, uint32_t F, const
     float *hst = reinterpret_cast<float *>(tp + o_st);
     uint32_t *hfc = reinterpret_cast<uint32_t *>(tp + o_fc);
     uint32_t *htp = reinterpret_cast<uint32_t *>(tp + o_tp);
-    uint64_t vs = 0, oo = 0, bo = 0, jo = 0, co = 0, pb = 0, cho = 0;
+    uint64_t vs = 0, oo = 0, bo = 0, jo = 0, co = 0, pb = 0, cho = 0, payload_words = 0;
     uint32_t to = 0;
     for (uint32_t f = 0; f < F; ++f) {
         const ParsedHeader &H = P[f];
@@ -1993,6 +1993,7 @@ gsnfs_status decode_batch_impl(gsnfs_ctx *ctx, cudaStream_t s, uint32_t F, const
         d.bw = reinterpret_cast<const uint32_t *>(as + 8);
         d.payload = d.bw + (uint64_t)H.nb * C;
         d.payload_words = (C && H.nv) ? (H.attr_bytes - 8 - 4ull * C * H.nb) / 4 : 0;
+        payload_words += d.payload_words;
         d.occ_off = oo;
         d.n_occ = H.n_occ;
         d.chunk_off = cho;
@@ -2061,7 +2062,7 @@ gsnfs_status decode_batch_impl(gsnfs_ctx *ctx, cudaStream_t s, uint32_t F, const
         stage_begin(s, kStRlgrDec);
         launch_batch_block_tables(L.fr, F, L.blk_pref, nblk, L.bw_all, sms, s);
         launch_scan_u32_to_u64(L.bw_all, nblk, L.boff_all, L.spart, sms, s);
-        launch_rlgr_decode_batch(L.fr, F, L.job_off, jobs, L.bw_all, L.boff_all, L.steps, C, L.Y, dst, s);
+        launch_rlgr_decode_batch(L.fr, F, L.job_off, jobs, payload_words, N, L.bw_all, L.boff_all, L.steps, C, L.Y, dst, sms, s);
         stage_end(s, kStRlgrDec);
     }
     // a11: occupancy bytes of every frame, octree levels, voxel centres

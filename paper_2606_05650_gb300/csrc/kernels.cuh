@@ -298,10 +298,11 @@ void launch_rlgr_encode_indices(const int32_t *q, const uint32_t *vstart, uint32
                                 uint64_t jobs_bound, uint32_t *overflow, cudaStream_t s);
 void launch_rlgr_decode(const uint32_t *payload, uint64_t payload_words, const uint32_t *block_words,
                         const uint64_t *block_off, uint64_t nv, uint32_t C, uint32_t B, const float *step, float *Y,
-                        DevState *st, cudaStream_t s);
+                        DevState *st, int num_sms, cudaStream_t s);
+// payload_words, nv_total: of all frames
 void launch_rlgr_decode_batch(const DecFrame *fr, uint32_t F, const uint64_t *job_off, uint64_t jobs_bound,
-                              const uint32_t *bw_all, const uint64_t *boff_all, const float *steps_all, uint32_t C,
-                              float *Y, DevState *st, cudaStream_t s);
+                              uint64_t payload_words, uint64_t nv_total, const uint32_t *bw_all, const uint64_t *boff_all,
+                              const float *steps_all, uint32_t C, float *Y, DevState *st, int num_sms, cudaStream_t s);
 void launch_rlgr_decode_indices(const uint32_t *words, uint64_t total_words, const uint32_t *bw, uint32_t stride,
                                 uint64_t nv, uint32_t C, uint32_t B, int32_t *q, DevState *st, cudaStream_t s);
 

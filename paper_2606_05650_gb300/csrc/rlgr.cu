@@ -890,15 +890,15 @@ __device__ __forceinline__ uint32_t gr_read(WinReader &r, uint32_t k, int &KR, b
 
 // Decodes one block stream (len coefficients of one channel) to out[i * C],
 // i < len: dequantised (times sc) or as indices.  A Golomb-Rice symbol whose
-// codeword the table holds takes the short path; run mode (runs are kept as
-// pending zeros, and the nonzero that ends a partial run as a pending value)
-// and longer codewords the general one.
+// codeword the table holds (TABLE), or whose codeword lies in the window (else),
+// takes the short path; run mode (runs are kept as pending zeros, and the nonzero
+// that ends a partial run as a pending value) and longer codewords the general one.
 constexpr uint32_t kDecThreads = 512, kDecSmall = 128;
 constexpr int kRunLeft = 1 << 16;  // flags in K: zeros or a value of an earlier run are still to be written,
 constexpr int kDrained = 1 << 17;  // the ring may not hold the next words: only the general path, which checks
 
-template <bool TO_INT>
-__device__ __forceinline__ void decode_stream(const DecTable &tab, uint32_t *ring, const uint32_t *wp, uint32_t nw,
+template <bool TO_INT, bool TABLE>
+__device__ __forceinline__ void decode_stream(const DecTable *tab, uint32_t *ring, const uint32_t *wp, uint32_t nw,
                                               uint32_t len, uint32_t C, float sc, float *yout, int32_t *qout,
                                               DevState *st)
 {
@@ -947,8 +947,8 @@ __device__ __forceinline__ void decode_stream(const DecTable &tab, uint32_t *rin
         if (zeros | (uint32_t)pending) K |= kRunLeft;
         return 0;
     };
-    const uint32_t ta = shared_address(tab.e);
-    auto symbol = [&](uint32_t i) {
+    const uint32_t ta = TABLE ? shared_address(tab->e) : 0u;
+    auto by_table = [&](uint32_t i) {
         const uint32_t e = table_load((uint32_t)(KR & 0x70) * (4u << (kDecBits - 4)) + ta +
                                       4u * (r.peek() & ((1u << kDecBits) - 1u)));
         int32_t q;
@@ -970,6 +970,32 @@ __device__ __forceinline__ void decode_stream(const DecTable &tab, uint32_t *rin
         else
             yout[(uint64_t)i * C] = __fmul_rn(y, sc);
     };
+    auto by_arithmetic = [&](uint32_t i) {
+        const uint32_t x = r.peek(), k = (uint32_t)KR >> 4;
+        const uint32_t p = (uint32_t)__ffs(~x) - 1u, n = p + 1u + k;  // leading ones (all ones: wraps)
+        int32_t q;
+        // Golomb-Rice mode (K < 16, no flag set), a codeword inside the window
+        if (__builtin_expect(K < 16 && p < (uint32_t)kUnaryEsc && n <= 32u, 1)) {
+            const uint32_t u = (p << k) | ((x >> (p + 1u)) & ((1u << k) - 1u));
+            q = unzz(u);
+            adapt_kr(p, KR);
+            K = max(K + (u == 0 ? 3 : -3), 0);
+            r.skip_ready(n);
+        } else {
+            q = general(len - i);
+        }
+        if (!r.stocked()) K |= kDrained;  // up to 32 bits a symbol: looked after at each
+        if (TO_INT)
+            qout[(uint64_t)i * C] = q;
+        else
+            yout[(uint64_t)i * C] = __fmul_rn((float)q, sc);
+    };
+    auto symbol = [&](uint32_t i) {
+        if constexpr (TABLE)
+            by_table(i);
+        else
+            by_arithmetic(i);
+    };
     uint32_t i = 0;
     for (; i + 4 <= len; i += 4) {
         K = r.top_up() ? K & ~kDrained : K | kDrained;
@@ -983,10 +1009,23 @@ __device__ __forceinline__ void decode_stream(const DecTable &tab, uint32_t *rin
     if (bad || r.overrun()) set_error(&st->err, kErrCorrupt);
 }
 
+// whole CTA: the decoder's table in shared memory, or null
+template <bool TABLE>
+__device__ __forceinline__ const DecTable *dec_table()
+{
+    if constexpr (TABLE) {
+        __shared__ __align__(16) DecTable tab;
+        stage_table(&tab, &g_dec_table);
+        __syncthreads();
+        return &tab;
+    }
+    return nullptr;
+}
+
 // One frame: thread (local row block jl, channel c) of CTA x decodes block
 // b = x * rb + jl of channel c.  Streams at block_off[b*C+c] (words) when
 // block_off is given, else at (b*C+c) * stride.
-template <bool TO_INT>
+template <bool TO_INT, bool TABLE>
 __global__ void __launch_bounds__(kDecThreads, 2) rlgr_decode_kernel(const uint32_t *payload, uint64_t payload_words,
                                                           const uint32_t *block_words, const uint64_t *block_off,
                                                           uint32_t stride, uint32_t nv, uint32_t C, uint32_t B,
@@ -995,9 +1034,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) rlgr_decode_kernel(const uint3
 {
     if (after_previous()) return;
     extern __shared__ __align__(128) uint32_t ring[];  // kRingWords per thread
-    __shared__ __align__(16) DecTable tab;
-    stage_table(&tab, &g_dec_table);
-    __syncthreads();
+    const DecTable *tab = dec_table<TABLE>();
     const uint64_t stream = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, b = stream / C;
     const uint32_t c = (uint32_t)(stream - b * C);
     const uint64_t row0 = b * B;
@@ -1011,11 +1048,12 @@ __global__ void __launch_bounds__(kDecThreads, 2) rlgr_decode_kernel(const uint3
         nw = 0;
         off = 0;
     }
-    decode_stream<TO_INT>(tab, ring + threadIdx.x * kRingWords, payload + off, nw, len, C, TO_INT ? 0.f : step[c],
+    decode_stream<TO_INT, TABLE>(tab, ring + threadIdx.x * kRingWords, payload + off, nw, len, C, TO_INT ? 0.f : step[c],
                           TO_INT ? nullptr : Y + row0 * C + c, TO_INT ? qout + row0 * C + c : nullptr, st);
 }
 
 // All frames of a batch: row blocks numbered across frames (job_off), rb per CTA.
+template <bool TABLE>
 __global__ void __launch_bounds__(kDecThreads, 2) rlgr_decode_batch_kernel(const DecFrame *fr, uint32_t F,
                                                                 const uint64_t *job_off, const uint32_t *bw_all,
                                                                 const uint64_t *boff_all, const float *steps_all,
@@ -1023,9 +1061,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) rlgr_decode_batch_kernel(const
 {
     if (after_previous()) return;
     extern __shared__ __align__(128) uint32_t ring[];  // kRingWords per thread
-    __shared__ __align__(16) DecTable tab;
-    stage_table(&tab, &g_dec_table);
-    __syncthreads();
+    const DecTable *tab = dec_table<TABLE>();
     const uint64_t stream = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, job = stream / C;
     const uint32_t c = (uint32_t)(stream - job * C);
     if (job >= job_off[F]) return;
@@ -1047,7 +1083,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) rlgr_decode_batch_kernel(const
         nw = 0;
         off = 0;
     }
-    decode_stream<false>(tab, ring + threadIdx.x * kRingWords, d.payload + off, nw, len, C, steps_all[(uint64_t)lo * C + c],
+    decode_stream<false, TABLE>(tab, ring + threadIdx.x * kRingWords, d.payload + off, nw, len, C, steps_all[(uint64_t)lo * C + c],
                          Y + ((uint64_t)d.vstart + row0) * C + c, nullptr, st);
 }
 
@@ -1164,29 +1200,50 @@ static void launch_decode(uint64_t streams, cudaStream_t s, A... args)
     count_launch();
 }
 
+// By table, or by arithmetic: the table's path takes fewer instructions while the codewords are short; a warp with a lane
+// whose codeword is not in it goes through the general path too, which arithmetic seldom needs.  4 frames of 1M
+// Gaussians (whole decode, ms, by table / by arithmetic): 4.3 bits of payload a coefficient 1.29 / 1.40, 5.6 1.34 /
+// 1.40, 6.0 1.44 / 1.41, 6.6 1.57 / 1.41, 10.1 1.70 / 1.41.  And it takes many streams: with few the arithmetic kernel is
+// done sooner, but holds up the geometry beside it, the longer branch (6.6 bits: 250k Gaussians 411 / 461 us, 550k 527 /
+// 524, 700k 569 / 547).
+static bool decode_by_table(uint64_t streams, uint64_t payload_words, uint64_t coefficients, int num_sms)
+{
+    return streams < (uint64_t)num_sms * 448 || 32 * payload_words < 5.9 * coefficients;
+}
+
 void launch_rlgr_decode(const uint32_t *payload, uint64_t payload_words, const uint32_t *block_words,
                         const uint64_t *block_off, uint64_t nv, uint32_t C, uint32_t B, const float *step, float *Y,
-                        DevState *st, cudaStream_t s)
+                        DevState *st, int num_sms, cudaStream_t s)
 {
     if (nv == 0 || C == 0) return;
-    launch_decode<rlgr_decode_kernel<false>>((nv + B - 1) / B * C, s, payload, payload_words, block_words, block_off, 0u,
-                                             (uint32_t)nv, C, B, step, Y, nullptr, st);
+    const uint64_t streams = (nv + B - 1) / B * C;
+    auto go = [&](auto launch) {
+        launch(streams, s, payload, payload_words, block_words, block_off, 0u, (uint32_t)nv, C, B, step, Y, nullptr, st);
+    };
+    if (decode_by_table(streams, payload_words, nv * C, num_sms))
+        go([](auto... a) { launch_decode<rlgr_decode_kernel<false, true>>(a...); });
+    else
+        go([](auto... a) { launch_decode<rlgr_decode_kernel<false, false>>(a...); });
 }
 
 void launch_rlgr_decode_batch(const DecFrame *fr, uint32_t F, const uint64_t *job_off, uint64_t jobs_bound,
-                              const uint32_t *bw_all, const uint64_t *boff_all, const float *steps_all, uint32_t C,
-                              float *Y, DevState *st, cudaStream_t s)
+                              uint64_t payload_words, uint64_t nv_total, const uint32_t *bw_all, const uint64_t *boff_all,
+                              const float *steps_all, uint32_t C, float *Y, DevState *st, int num_sms, cudaStream_t s)
 {
     if (jobs_bound == 0 || C == 0) return;
-    launch_decode<rlgr_decode_batch_kernel>(jobs_bound * C, s, fr, F, job_off, bw_all, boff_all, steps_all, C, Y, st);
+    if (decode_by_table(jobs_bound * C, payload_words, nv_total * C, num_sms))
+        launch_decode<rlgr_decode_batch_kernel<true>>(jobs_bound * C, s, fr, F, job_off, bw_all, boff_all, steps_all, C, Y, st);
+    else
+        launch_decode<rlgr_decode_batch_kernel<false>>(jobs_bound * C, s, fr, F, job_off, bw_all, boff_all, steps_all, C, Y, st);
 }
 
+// (how many bits the streams hold is known on the device only: by arithmetic, which is done sooner but for many short ones)
 void launch_rlgr_decode_indices(const uint32_t *words, uint64_t total_words, const uint32_t *bw, uint32_t stride,
                                 uint64_t nv, uint32_t C, uint32_t B, int32_t *q, DevState *st, cudaStream_t s)
 {
     if (nv == 0 || C == 0) return;
-    launch_decode<rlgr_decode_kernel<true>>((nv + B - 1) / B * C, s, words, total_words, bw, nullptr, stride, (uint32_t)nv, C, B,
-                                            nullptr, nullptr, q, st);
+    launch_decode<rlgr_decode_kernel<true, false>>((nv + B - 1) / B * C, s, words, total_words, bw, nullptr, stride, (uint32_t)nv,
+                                                   C, B, nullptr, nullptr, q, st);
 }
 
 }  // namespace gsnfs
