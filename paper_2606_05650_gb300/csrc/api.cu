@@ -1209,7 +1209,7 @@ gsnfs_status encode_impl(gsnfs_ctx *ctx, cudaStream_t s, EncodeReq &rq, bool wor
             j.G = G;
             j.tau64 = q->tau;
             stage_begin(sa, kStRlgrEnc);
-            launch_rlgr_encode(j, L.job_off, L.jobs_bound, sa);
+            launch_rlgr_encode(j, L.job_off, L.jobs_bound, sms, sa);
             stage_end(sa, kStRlgrEnc);
             launch_scan_u32_to_u64(L.block_words, L.blocks_bound, L.block_off, L.spart, sms, sa);
         }

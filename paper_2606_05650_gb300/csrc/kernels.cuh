@@ -292,7 +292,7 @@ void launch_frame_dc(float *Y, const uint32_t *vstart, uint32_t F, uint32_t C, c
 uint32_t rlgr_slot_words(uint32_t B, bool worst_case);
 void launch_rlgr_offsets(const uint32_t *vstart, uint32_t F, uint32_t B, uint32_t R, uint32_t C, uint64_t *job_off,
                          uint64_t *blk_off, cudaStream_t s);
-void launch_rlgr_encode(const RlgrJob &j, const uint64_t *job_off, uint64_t jobs_bound, cudaStream_t s);
+void launch_rlgr_encode(const RlgrJob &j, const uint64_t *job_off, uint64_t jobs_bound, int num_sms, cudaStream_t s);
 void launch_rlgr_encode_indices(const int32_t *q, const uint32_t *vstart, uint32_t C, uint32_t B, uint32_t *slots,
                                 uint32_t slot_words, uint32_t *bw, const uint64_t *job_off, const uint64_t *blk_off,
                                 uint64_t jobs_bound, uint32_t *overflow, cudaStream_t s);

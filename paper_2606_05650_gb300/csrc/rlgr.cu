@@ -308,7 +308,13 @@ struct Rlgr : RlgrState {
 struct EncJobs {
     RlgrJob j;
     const uint64_t *job_off;  // F + 1: first job (row block) of each frame
-    uint32_t w0, ws;          // the launch codes streams w0 .. w0 + ws - 1 of each row block (kernels of a thread a stream)
+    uint32_t w0, ws;          // the launch codes streams w0 .. w0 + ws - 1 of each row block (kernel of a thread a stream)
+    uint64_t least, most;     // and nothing unless the streams, known on the device only, number least .. most
+    __device__ __forceinline__ bool concerned() const
+    {
+        const uint64_t n = job_off[j.F] * j.R * j.C;
+        return n >= least && n <= most;
+    }
 };
 
 constexpr uint32_t kPrefetch = 4;  // rows copied and coded at a time; even, for the rows are coded in pairs
@@ -385,6 +391,7 @@ template <bool FROM_INT, bool DIST, uint32_t PITCH>
 __global__ void __launch_bounds__(PITCH, 1024 / PITCH) rlgr_encode_kernel(EncJobs E, const int32_t *qin, uint32_t rb)
 {
     if (after_previous()) return;
+    if (!E.concerned()) return;
     extern __shared__ uint32_t ring[];  // kRing x PITCH
     __shared__ EncBlock blk_info[32];
     __shared__ __align__(16) EncTable tab;
@@ -507,75 +514,23 @@ __global__ void __launch_bounds__(PITCH, 1024 / PITCH) rlgr_encode_kernel(EncJob
 }
 
 // ---- encoder for few streams ----------------------------------------------------
-// Where the streams do not fill the GPU, a launch takes as long as one thread
-// takes for its block, and what counts is the length of a symbol's dependent
-// chain, not its instructions over all paths: each lane branches to its own
-// path, and a zero of a run is three instructions.  A point cloud of 1M points
-// (C = 3, 2,900 streams, mostly runs): 88 us against 129 us by the kernel
-// above; a frame of 250k Gaussians (27k streams, few runs): 90 against 81 us.
-// (Fewer streams than kSplitStreams take the kernel after this one.)
-constexpr uint64_t kFewStreams = 20000;
-
-__global__ void __launch_bounds__(512) rlgr_encode_few_kernel(EncJobs E, uint32_t rb)
-{
-    if (after_previous()) return;
-    __shared__ EncBlock blk_info[32];
-    const RlgrJob &j = E.j;
-    const uint32_t C = j.C, W = E.ws, t = threadIdx.x;
-    if (t < rb) blk_info[t] = enc_block(E, (uint64_t)blockIdx.x * rb + t);
-    __syncthreads();
-    const uint32_t jl = t / W;
-    if (jl >= rb) return;
-    const EncBlock me = blk_info[jl];
-    if (me.len == 0) return;
-    const uint32_t w = E.w0 + t - jl * W, r = w / C, c = w - r * C;
-    const uint64_t blk = j.blk_off[me.f] + ((uint64_t)r * me.nb + me.b) * C + c;
-    BitWriter bw(j.slots + blk * j.slot_words, j.slot_words);
-    RlgrState st{0, 32, 0u};
-    const float inv = j.inv_step[r * C + c], tau = j.tau;
-    const float *col = j.Y + me.gbase + c;  // row i of this channel at col[i * C]
-    const uint32_t len = me.len;
-    uint32_t i = 0;
-    if (j.dc && me.b == 0) {  // the frame's DC: quantised from its FP64 value
-        st.code(bw, zz(quantize_f64(j.dc[(uint64_t)me.f * C + c], j.steps_rg[r * j.G + j.groups[c]], j.tau64)));
-        i = 1;
-    }
-    float cur[kPrefetch];
-#pragma unroll
-    for (uint32_t d = 0; d < kPrefetch; ++d) cur[d] = (i + d < len) ? *(col + (uint64_t)(i + d) * C) : 0.f;
-    for (; i + kPrefetch <= len; i += kPrefetch) {
-        float nx[kPrefetch];
-        const float *q = col + (uint64_t)(i + kPrefetch) * C;
-#pragma unroll
-        for (uint32_t d = 0; d < kPrefetch; ++d) nx[d] = (i + kPrefetch + d < len) ? *(q + d * C) : 0.f;
-#pragma unroll
-        for (uint32_t d = 0; d < kPrefetch; ++d) st.code(bw, quantize_zz_f32(cur[d], inv, tau));
-#pragma unroll
-        for (uint32_t d = 0; d < kPrefetch; ++d) cur[d] = nx[d];
-    }
-#pragma unroll
-    for (uint32_t d = 0; d < kPrefetch; ++d)
-        if (i + d < len) st.code(bw, quantize_zz_f32(cur[d], inv, tau));
-    st.finish(bw);
-    j.block_words[blk] = bw.nw;
-    if (bw.nw > j.slot_words) atomicExch(j.overflow, 1u);
-}
-
-// ---- encoder for very few streams -----------------------------------------------
 // A launch takes as long as one stream does, and a thread that codes a symbol at
-// a time spends 290 cycles on each (65 instructions, one after another).  Only
+// a time spends some 200 cycles on each, one instruction after another.  Only
 // the adaptation is serial, so here a CTA takes kSplitG streams in segments of
 // kSplitSeg symbols and splits the work: one warp walks the adaptation, a lane
 // per stream, and notes the state before each symbol (a fifth of the
 // instructions while no stream is near run mode); a warp per stream then forms
 // the segment's codewords, a lane per symbol, places them by a scan of their
 // lengths and writes whole words, while the first walks the next segment and
-// the one after it is loaded and quantised.  10k Gaussians (1.1k streams): 78 ->
-// 41 us, 30k 79 -> 47; a cloud of 1M points (5.9k streams at most, mostly runs)
-// 58 -> 46.  In all it takes more instructions than the kernels above, and
-// beyond kSplitStreams, when an SM has more than its four CTAs, it loses: 50k
-// Gaussians (5.5k streams) 86 against 80 us, 100k 155, 2M points 80 against 60.
-constexpr uint64_t kSplitStreams = 6144;
+// the one after it is loaded and quantised.  By the kernel above / by this one:
+// 10k Gaussians (1.1k streams) 57 / 42 us, 30k 57 / 47, 40k 57 / 50; a cloud of 1M
+// points (mostly runs) 84 / 47.  In all it takes more instructions, and where an
+// SM has more than its four CTAs it loses: 45k Gaussians (4.9k streams) 57 / 80,
+// 100k 57 / 130.  How many streams there are is known on the device (a cloud has
+// far fewer voxels than points): up to kSplitBound times as many points as would
+// make four CTAs an SM, both kernels are launched and the streams' number says
+// which one works (encode of a cloud of 1.3M points 543 -> 482 us).
+constexpr uint32_t kSplitCtas = 4, kSplitBound = 4;
 constexpr uint32_t kSplitG = 8, kSplitSeg = 128, kSplitThreads = 32 * (1 + kSplitG);
 constexpr uint32_t kSplitRow = kSplitG + 1;  // of a symbol's row in shared memory: no bank twice down a column
 
@@ -604,6 +559,7 @@ __device__ __forceinline__ void or_bits(uint32_t *buf, uint32_t o, uint64_t c)
 __global__ void __launch_bounds__(kSplitThreads, 4) rlgr_encode_split_kernel(EncJobs E)
 {
     if (after_previous()) return;
+    if (!E.concerned()) return;
     __shared__ uint32_t sym[3][kSplitSeg * kSplitRow];  // zigzag indices of a segment
     __shared__ uint32_t pre[2][kSplitSeg * kSplitRow];  // states before its symbols
     __shared__ uint32_t bits[kSplitG][84];            // 32 codewords of up to 78 bits behind a part of a word
@@ -1149,23 +1105,25 @@ void launch_rlgr_offsets(const uint32_t *vstart, uint32_t F, uint32_t B, uint32_
     count_launch();
 }
 
-void launch_rlgr_encode(const RlgrJob &j, const uint64_t *job_off, uint64_t jobs_bound, cudaStream_t s)
+void launch_rlgr_encode(const RlgrJob &j, const uint64_t *job_off, uint64_t jobs_bound, int num_sms, cudaStream_t s)
 {
     if (jobs_bound == 0 || j.C == 0) return;
     const uint32_t W = j.R * j.C;
-    const EncJobs E{j, job_off, 0, W};
-    if (!j.sq_err && jobs_bound * W <= kSplitStreams) {
-        launch_after(rlgr_encode_split_kernel, (uint32_t)((jobs_bound * W + kSplitG - 1) / kSplitG), kSplitThreads, 0, s, E);
+    const uint64_t streams = jobs_bound * W;  // at most: the host knows the points, the device the voxels
+    const uint64_t split = (uint64_t)kSplitG * kSplitCtas * num_sms;
+    EncJobs E{j, job_off, 0, W, 0, ~0ull};
+    if (!j.sq_err && streams <= kSplitBound * split) {
+        E.most = split;
+        launch_after(rlgr_encode_split_kernel, (uint32_t)((std::min(streams, split) + kSplitG - 1) / kSplitG), kSplitThreads, 0, s, E);
         count_launch();
-    } else if (!j.sq_err && jobs_bound * W <= kFewStreams) {
-        launch_slices(E, W, jobs_bound, [&](const EncJobs &S, uint32_t rb, uint32_t grid, uint32_t threads) {
-            launch_after(rlgr_encode_few_kernel, grid, threads, 0, s, S, rb);
-        });
-    } else if (j.sq_err) {
-        launch_encode<false, true>(E, nullptr, W, jobs_bound, s);
-    } else {
-        launch_encode<false, false>(E, nullptr, W, jobs_bound, s);
+        if (streams <= split) return;
+        E.least = split + 1;
+        E.most = ~0ull;
     }
+    if (j.sq_err)
+        launch_encode<false, true>(E, nullptr, W, jobs_bound, s);
+    else
+        launch_encode<false, false>(E, nullptr, W, jobs_bound, s);
 }
 
 void launch_rlgr_encode_indices(const int32_t *q, const uint32_t *vstart, uint32_t C, uint32_t B, uint32_t *slots,
@@ -1184,7 +1142,7 @@ void launch_rlgr_encode_indices(const int32_t *q, const uint32_t *vstart, uint32
     j.blk_off = blk_off;
     j.slot_words = slot_words;
     j.overflow = overflow;
-    launch_encode<true, false>(EncJobs{j, job_off, 0, C}, q, C, jobs_bound, s);
+    launch_encode<true, false>(EncJobs{j, job_off, 0, C, 0, ~0ull}, q, C, jobs_bound, s);
 }
 
 // Threads per CTA: a CTA has a copy of the table (32 KB) beside 64 bytes a thread, and many streams are bound by the
