@@ -2990,7 +2990,7 @@ gsnfs_status gsnfs_rlgr_decode_indices(gsnfs_ctx *ctx, void *stream, const uint3
     CK(dev_memset(ctx->st, 0, 8, s));
     const uint32_t sw = rlgr_slot_words(B, true);
     const uint64_t nb = (nv + B - 1) / B;
-    launch_rlgr_decode_indices(d_slots, (uint64_t)C * nb * sw, d_block_words, sw, nv, C, B, d_q, ctx->st, s);
+    launch_rlgr_decode_indices(d_slots, (uint64_t)C * nb * sw, d_block_words, sw, nv, C, B, d_q, ctx->st, ctx->num_sms, s);
     CK(cudaMemcpyAsync(ctx->pinned, ctx->st, 4, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     CK(cudaGetLastError());

@@ -304,7 +304,7 @@ void launch_rlgr_decode_batch(const DecFrame *fr, uint32_t F, const uint64_t *jo
                               uint64_t payload_words, uint64_t nv_total, const uint32_t *bw_all, const uint64_t *boff_all,
                               const float *steps_all, uint32_t C, float *Y, DevState *st, int num_sms, cudaStream_t s);
 void launch_rlgr_decode_indices(const uint32_t *words, uint64_t total_words, const uint32_t *bw, uint32_t stride,
-                                uint64_t nv, uint32_t C, uint32_t B, int32_t *q, DevState *st, cudaStream_t s);
+                                uint64_t nv, uint32_t C, uint32_t B, int32_t *q, DevState *st, int num_sms, cudaStream_t s);
 
 // ---- rans.cu: occupancy entropy stage ------------------------------------
 struct RansFrames {

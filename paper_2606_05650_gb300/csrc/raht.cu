@@ -490,10 +490,11 @@ __global__ void __launch_bounds__(kThreads) prelude_finish_kernel(PreludeArgs a,
     }
 }
 
-// Passes launched grid-wide, the rest run in one CTA: a pass has at most a
-// quarter of the tiles of the one before, mostly a twentieth, so that with at
-// most 64 tiles in the first the third is one tile, for which a launch (two in
-// the prelude) costs more than it saves.  10k Gaussians, wide passes one / two /
+// Passes launched grid-wide, the rest run in one CTA: a tile carries at most 128
+// elements on (kRahtCarrySlots), so that a pass has at most half of the tiles of
+// the one before where a tile is 256 elements, mostly a twentieth; with at most
+// 64 tiles in the first the third is mostly one tile (16 at worst), for which a
+// launch (two in the prelude) costs more than it saves.  10k Gaussians, wide passes one / two /
 // three: encode 300 / 291 / 300 us, decode 298 / 287 / 298 us.  Two wide passes
 // up to 2000 tiles lost: the last kernel then walks up to three tiles of 56
 // channels one by one (500k rows, two forward and two inverse transforms: 375
@@ -1685,7 +1686,8 @@ void launch_finish(const XformArgs<S> &A, int q0, size_t smem, cudaStream_t s)
     count_launch();
 }
 
-// CTAs of a later pass, three per SM; a pass has at most a quarter of the tiles of the one before
+// CTAs of a later pass, three per SM at most, for a quarter of the tiles of the one before (an estimate, mostly a high
+// one: a CTA takes its tiles by stride)
 uint32_t later_grid(uint64_t tiles, int q, int num_sms)
 {
     const uint64_t t = (tiles >> (2 * q)) + 1, cap = 3 * (uint64_t)num_sms;

@@ -1150,9 +1150,9 @@ void launch_rlgr_encode_indices(const int32_t *q, const uint32_t *vstart, uint32
 // (28 warps), 1.83 with 512 (32), 1.74 with 640 (40), which slows the geometry, the longer branch, by more.  Streams
 // that do not fill every SM twice that way take smaller CTAs, for the sake of all SMs.
 template <auto Kernel, typename... A>
-static void launch_decode(uint64_t streams, cudaStream_t s, A... args)
+static void launch_decode(uint64_t streams, int num_sms, cudaStream_t s, A... args)
 {
-    const uint32_t threads = streams < 152 * 2 * kDecThreads ? kDecSmall : kDecThreads;
+    const uint32_t threads = streams < (uint64_t)num_sms * 2 * kDecThreads ? kDecSmall : kDecThreads;
     allow_shared<Kernel>();
     launch_after(Kernel, (uint32_t)((streams + threads - 1) / threads), threads, 4 * (size_t)kRingWords * threads, s, args...);
     count_launch();
@@ -1176,7 +1176,7 @@ void launch_rlgr_decode(const uint32_t *payload, uint64_t payload_words, const u
     if (nv == 0 || C == 0) return;
     const uint64_t streams = (nv + B - 1) / B * C;
     auto go = [&](auto launch) {
-        launch(streams, s, payload, payload_words, block_words, block_off, 0u, (uint32_t)nv, C, B, step, Y, nullptr, st);
+        launch(streams, num_sms, s, payload, payload_words, block_words, block_off, 0u, (uint32_t)nv, C, B, step, Y, nullptr, st);
     };
     if (decode_by_table(streams, payload_words, nv * C, num_sms))
         go([](auto... a) { launch_decode<rlgr_decode_kernel<false, true>>(a...); });
@@ -1190,18 +1190,18 @@ void launch_rlgr_decode_batch(const DecFrame *fr, uint32_t F, const uint64_t *jo
 {
     if (jobs_bound == 0 || C == 0) return;
     if (decode_by_table(jobs_bound * C, payload_words, nv_total * C, num_sms))
-        launch_decode<rlgr_decode_batch_kernel<true>>(jobs_bound * C, s, fr, F, job_off, bw_all, boff_all, steps_all, C, Y, st);
+        launch_decode<rlgr_decode_batch_kernel<true>>(jobs_bound * C, num_sms, s, fr, F, job_off, bw_all, boff_all, steps_all, C, Y, st);
     else
-        launch_decode<rlgr_decode_batch_kernel<false>>(jobs_bound * C, s, fr, F, job_off, bw_all, boff_all, steps_all, C, Y, st);
+        launch_decode<rlgr_decode_batch_kernel<false>>(jobs_bound * C, num_sms, s, fr, F, job_off, bw_all, boff_all, steps_all, C, Y, st);
 }
 
 // (how many bits the streams hold is known on the device only: by arithmetic, which is done sooner but for many short ones)
 void launch_rlgr_decode_indices(const uint32_t *words, uint64_t total_words, const uint32_t *bw, uint32_t stride,
-                                uint64_t nv, uint32_t C, uint32_t B, int32_t *q, DevState *st, cudaStream_t s)
+                                uint64_t nv, uint32_t C, uint32_t B, int32_t *q, DevState *st, int num_sms, cudaStream_t s)
 {
     if (nv == 0 || C == 0) return;
-    launch_decode<rlgr_decode_kernel<true, false>>((nv + B - 1) / B * C, s, words, total_words, bw, nullptr, stride, (uint32_t)nv,
-                                                   C, B, nullptr, nullptr, q, st);
+    launch_decode<rlgr_decode_kernel<true, false>>((nv + B - 1) / B * C, num_sms, s, words, total_words, bw, nullptr, stride,
+                                                   (uint32_t)nv, C, B, nullptr, nullptr, q, st);
 }
 
 }  // namespace gsnfs
