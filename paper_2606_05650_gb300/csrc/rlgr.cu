@@ -72,8 +72,9 @@ struct BitWriter {
 // of it on the half-rate integer pipe: one serial stream per thread, every
 // stream slot of the SM filled.  With the tables 44 (encoder) and 51 (decoder)
 // warp instructions per 32 symbols, 64 each before: 16 x 1M frames, encode 1.78
-// -> 1.36 ms; a ladder of eight frames and five rungs 2.25 -> 1.75 ms; decode,
-// at 32 warps per SM, 1.45 ms alone.
+// -> 1.36 ms; a ladder of eight frames and five rungs 2.25 -> 1.69 ms; decode,
+// at 32 warps per SM, 1.45 ms alone.  Large coefficients are past the tables, and
+// so past their gain: what codes them without is chosen below.
 constexpr uint32_t kEncRows = 8, kEncCols = 256;   // per mode: k 0 .. 7
 constexpr uint32_t kEncMax = kEncCols / 2 - 1;     // magnitudes below; kEncMax stands for every larger one
 constexpr uint32_t kEncMode = kEncRows * kEncCols;  // entries of one mode
