@@ -269,10 +269,12 @@ __global__ void __launch_bounds__(Cfg::threads, Cfg::ctas) downsweep_kernel(cons
 // Few pairs: every pass in one CTA, the keys and the pairs' original places in
 // shared memory (a launch instead of three per pass, and no trips through L2).
 // A warp owns `rounds` x 32 consecutive pairs, in registers while a pass moves
-// them; the values are fetched by place at the end.  A frame of 10k Gaussians
-// (30-bit keys, 12 launches before): encode 427 -> 412 us.  Above kSmallMax the
-// pairs do not fit one SM's shared memory.
-constexpr uint32_t kSmallMax = 16384, kSmallThreads = 1024, kSmallRounds = kSmallMax / kSmallThreads;
+// them; the values are fetched by place at the end.  By the launches of all
+// passes / by this one, voxelisation and sort (us): 30-bit keys (12 launches), 2k
+// points 121 / 109, 6k 129 / 121, 8k 130 / 123, 10k 131 / 134, 16k 131 / 159; 63
+// bits (24 launches), 2k 158 / 120, 8k 171 / 158, 10k 169 / 171, 16k 172 / 210;
+// 32-bit keys of a render, 3k Gaussians 171 / 155, 8k 211 / 209, 16k 240 / 260.
+constexpr uint32_t kSmallMax = 8192, kSmallThreads = 1024, kSmallRounds = kSmallMax / kSmallThreads;
 
 template <typename Key>
 struct SmallSmem {
