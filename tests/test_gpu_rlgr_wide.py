@@ -21,7 +21,8 @@ def G():
     return gsnfs
 
 
-# streams in all (row blocks of 512 x rungs x channels): up to 6,144, up to 20,000, more
+# streams in all (row blocks of 512 x rungs x channels): 1,500 to 61,440, on both sides of the limit (4,864) of the
+# kernel that splits the work, and of four times that by points
 @pytest.mark.parametrize("n", [700, 4500, 20_000])
 @pytest.mark.parametrize("C,rungs", [(171, 3), (129, 4), (65, 8), (256, 3), (128, 8), (256, 4)])
 def test_wide_ladder(G, n, C, rungs):
